@@ -72,18 +72,41 @@ struct Bucket {
     int64_t rows = 0, cols = 0, s = 0, l = 0, e = 0;
     int grad_dtype = 0, state_dtype = 0;
     bool tall = false, tc_ok = false;
+    bool paired = false;        // takes its first two iterations together on the s x s side (see ns_pair_pays)
     std::vector<MatRef> mats;
     // bytes from the state base of the three blocks: M (fp32), A and G_prev (fp32, or bf16 with MONA-Lite storage)
     size_t off_M = 0, off_A = 0, off_G = 0;
     int Cb = 1, Cf = 1;         // chunk capacity: bf16 tensor-core mode / fp32 mode
     int slabs = 1;
     int64_t slab_len = 0;
-    size_t off_x[2] = {0, 0}, off_a = 0, off_b = 0;          // bf16 mode, bytes from the slot's iterate base
+    size_t off_x[2] = {0, 0}, off_a = 0, off_b = 0, off_delta = 0;   // bf16 mode, bytes from the slot's iterate base
     size_t off32_x[2] = {0, 0}, off32_a = 0, off32_b = 0;    // fp32 mode
     size_t data_bytes = 0;
-    NsMaps maps[NSLOTS] = {};      // per workspace slot: X ping, X pong, A, B' of a chunk of this bucket
+    NsMaps maps[NSLOTS] = {};      // per workspace slot: X ping, X pong, A, B', C of a chunk of this bucket
 };
-constexpr int MAP_X0 = 0, MAP_A = 2, MAP_B = 3;
+constexpr int MAP_X0 = 0, MAP_A = 2, MAP_B = 3, MAP_C = 4;
+
+// The first two iterations can be taken on the s x s side without forming the iterate between them:
+//     A = X X^T, P = b A + c A^2 + a I, A' = P (P A), P' = b A' + c A'^2 + a I, Q = P' P, X'' = Q X
+// (A, P and their products are polynomials in A: they commute and are symmetric, lower-triangle tiles all).  Against two plain
+// iterations this saves one X X^T and one B' X and costs three s x s products.  It pays where that is clearly less tensor work
+// (tile-k-slices of the pair against two plain iterations, one step before -> after: 1024 x 4096 0.68, 21.7 -> 20.1 ms; 768 x 2048
+// 0.76, 20.2 -> 19.6 ms; 256 x 768 0.79, 3.87 -> 3.79 ms; but 512 x 1024 0.85, 4.05 -> 4.12 ms; 1024 x 1536 0.91, 6.93 -> 6.95 ms),
+// and only with enough tiles per product to fill the machine twice over: on a few tiles the launch is bound by its chain of
+// dependent products, which gets one longer (16 instead of 15).
+bool ns_pair_pays(int64_t s, int64_t l, int64_t count) {
+    const int64_t ts = (s + TC_BM - 1) / TC_BM, tl = (l + TC_BM - 1) / TC_BM, ks = (s + TC_BK - 1) / TC_BK, kl = (l + TC_BK - 1) / TC_BK;
+    const int64_t sym = ts * (ts + 1) / 2;
+    const int64_t plain = 2 * (sym * kl + sym * ks + ts * tl * ks), paired = sym * kl + 5 * sym * ks + ts * tl * ks;
+    return paired * 100 <= plain * 80 && sym * count >= 150;
+}
+// Whether a T-step run takes its first two iterations together.  Rounding A to bf16 perturbs A' by up to a^2 |A| 2^-9 in the
+// directions of small singular values, so only the first two are, where |A| is small (the iterate has Frobenius norm 1).
+// Relative error of O_5 against fp64 at 256 x 768 (bf16 emulation; every iteration apart -> first two together, both with the
+// diagonal correction): Gaussian 0.0081 -> 0.0082, training-like 0.0085 -> 0.0085, condition number 100 0.0279 -> 0.0228, 1000
+// 0.0536 -> 0.0424 (without the correction, apart: 0.0086, 0.0097, 0.0279, 0.0536).  With the last two together as well the
+// ill-conditioned ones get worse (0.030), and for T < 4 an error of the first two has no iterations left to shrink in.
+bool ns_first_two_together(const bool pair_pays, int T) { return pair_pays && T >= 4; }
 
 struct Plan {
     std::vector<mona_matrix_desc> descs;
@@ -148,10 +171,12 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         cb = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cb, MAXC), count));
         b.Cb = (int)cb;
         b.Cf = (int)std::max<int64_t>(1, cb / 2);
+        b.paired = b.tc_ok && ns_pair_pays(b.s, b.l, count);
         size_t off = 0;
         for (int i = 0; i < 2; ++i) { b.off_x[i] = off; off += align_up((size_t)b.Cb * b.e * 2, 1024); }
         b.off_a = off; off += align_up((size_t)b.Cb * b.s * b.s * 2, 1024);
         b.off_b = off; off += align_up((size_t)b.Cb * b.s * b.s * 2, 1024);
+        b.off_delta = off; off += align_up((size_t)b.Cb * b.s * sizeof(float), 1024);
         size_t off32 = 0;
         for (int i = 0; i < 2; ++i) { b.off32_x[i] = off32; off32 += align_up((size_t)b.Cf * b.e * 4, 1024); }
         b.off32_a = off32; off32 += align_up((size_t)b.Cf * b.s * b.s * 4, 1024);
@@ -169,10 +194,11 @@ typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t,
                                   const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
                                   CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
 
-// bf16 tensor [C][outer][inner] (inner contiguous) cut into boxes of 64 x box_rows with the 128-byte swizzle.
-bool encode_map(EncodeTiledFn fn, CUtensorMap* map, void* base, int64_t inner, int64_t outer, int64_t C, int box_rows) {
+// bf16 tensor [C][outer][inner] (inner contiguous, matrices `mat_stride` elements apart) cut into boxes of 64 x box_rows with the
+// 128-byte swizzle.
+bool encode_map(EncodeTiledFn fn, CUtensorMap* map, void* base, int64_t inner, int64_t outer, int64_t C, int box_rows, int64_t mat_stride) {
     cuuint64_t dims[3] = {(cuuint64_t)inner, (cuuint64_t)outer, (cuuint64_t)C};
-    cuuint64_t strides[2] = {(cuuint64_t)inner * 2, (cuuint64_t)inner * (cuuint64_t)outer * 2};
+    cuuint64_t strides[2] = {(cuuint64_t)inner * 2, (cuuint64_t)mat_stride * 2};
     cuuint32_t box[3] = {(cuuint32_t)TC_BOX, (cuuint32_t)box_rows, 1};
     cuuint32_t estr[3] = {1, 1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3, base, dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
@@ -339,9 +365,12 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
             uint8_t* data = h->ws + WS_DATA_OFF + sl * h->plan.slot_bytes;
             for (int big = 0; big < 2; ++big) {     // 64-row boxes, then 128-row boxes
                 const int rows = big ? 2 * TC_BOX : TC_BOX, at = big * NS_TENSORS;
-                for (int i = 0; i < 2; ++i) ok = ok && encode_map(encode, &b.maps[sl].m[at + MAP_X0 + i], data + b.off_x[i], b.cols, b.rows, b.Cb, rows);
-                ok = ok && encode_map(encode, &b.maps[sl].m[at + MAP_A], data + b.off_a, b.s, b.s, b.Cb, rows);
-                ok = ok && encode_map(encode, &b.maps[sl].m[at + MAP_B], data + b.off_b, b.s, b.s, b.Cb, rows);
+                for (int i = 0; i < 2; ++i) ok = ok && encode_map(encode, &b.maps[sl].m[at + MAP_X0 + i], data + b.off_x[i], b.cols, b.rows, b.Cb, rows, b.e);
+                ok = ok && encode_map(encode, &b.maps[sl].m[at + MAP_A], data + b.off_a, b.s, b.s, b.Cb, rows, b.s * b.s);
+                ok = ok && encode_map(encode, &b.maps[sl].m[at + MAP_B], data + b.off_b, b.s, b.s, b.Cb, rows, b.s * b.s);
+                // C of a matrix lives in the second iterate of the SAME matrix, which nothing holds until the first pair's Q X is
+                // stored there - after the last read of C, by the order of the matrix's own phases
+                ok = ok && encode_map(encode, &b.maps[sl].m[at + MAP_C], data + b.off_x[1], b.s, b.s, b.Cb, rows, b.e);
             }
         }
         if (!ok) return h->fail(MONA_ERR_CUDA, "cuTensorMapEncodeTiled failed for bucket %lldx%lld", (long long)b.rows, (long long)b.cols);
@@ -362,6 +391,48 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
 }
 
 }  // extern "C"
+
+// Appends to `g` the phases of one iteration (or of two taken together) of a chunk of bucket `b`.  X is read from tensor
+// MAP_X0 + x_cur and written to the other one; `first`: X is still un-normalised.
+static void ns_plan_group(NsProgram& g, const Bucket& b, bool together, bool first, int x_cur, const __nv_bfloat16* a_data, float* delta,
+                          float ns_a, float ns_b, float ns_c, int macro_tile_min_k, bool fuse_update) {
+    const int s = (int)b.s, l = (int)b.l;
+    // D = product of two symmetric s x s matrices, operands and result lower-block-stored
+    auto small = [&](int a_map, int b_map, int d_map) -> NsPhase& {
+        NsPhase& p = g.ph[g.P++];
+        p.M = p.N = p.K = s; p.a_map = a_map; p.b_map = b_map; p.a_sym = p.b_sym = 1; p.symmetric = p.small_sym = 1; p.ab_same = a_map == b_map;
+        p.d_map = d_map; p.ld = s; p.mat_stride = (long long)s * s; p.c2 = 1.f;
+        ns_phase_plan(p);
+        return p;
+    };
+    // D = b A + c A A + a I
+    auto poly = [&](int d_map) {
+        NsPhase& p = small(MAP_A, MAP_A, d_map);
+        p.cin = a_data; p.c1 = ns_b; p.c2 = ns_c; p.diag_add = ns_a; p.delta_in = delta;
+    };
+    NsPhase& g1 = g.ph[g.P++];      // A = X X^T (wide) or X^T X (tall): lower-triangle tiles only
+    g1.M = g1.N = s; g1.K = l; g1.a_map = g1.b_map = MAP_X0 + x_cur; g1.a_mn = g1.b_mn = b.tall ? 1 : 0;
+    g1.symmetric = 1; g1.ab_same = 1; g1.d_map = MAP_A; g1.ld = s; g1.mat_stride = (long long)s * s;
+    g1.c2 = 1.f; g1.post_mode = first ? 2 : 0; g1.delta_out = delta;
+    ns_phase_plan(g1);
+    poly(MAP_B);                                        // P
+    if (together) {
+        small(MAP_B, MAP_A, MAP_C);                     // P A
+        small(MAP_B, MAP_C, MAP_A).delta_out = delta;   // A' = P (P A)
+        poly(MAP_C);                                    // P'
+        small(MAP_C, MAP_B, MAP_A);                     // Q = P' P
+    }
+    const int q_map = together ? MAP_A : MAP_B;
+    NsPhase& g3 = g.ph[g.P++];      // X' = Q X (wide) or X Q (tall); 256 x 512 macro-tiles when the inner dimension is long
+    g3.K = s; g3.wide = s >= macro_tile_min_k ? 1 : 0; g3.d_map = MAP_X0 + (x_cur ^ 1); g3.ld = b.cols; g3.mat_stride = b.e;
+    g3.c2 = 1.f; g3.post_mode = first ? 1 : 0; g3.fuse_update = fuse_update ? 1 : 0;
+    if (!b.tall) {   // Q is the symmetric "A" operand, X the MN-major "B" operand
+        g3.M = s; g3.N = l; g3.a_map = q_map; g3.a_sym = 1; g3.b_map = MAP_X0 + x_cur; g3.b_mn = 1;
+    } else {         // X is K-major, the symmetric Q serves as its own transpose
+        g3.M = l; g3.N = s; g3.a_map = MAP_X0 + x_cur; g3.a_mn = 0; g3.b_map = q_map; g3.b_sym = 1;
+    }
+    ns_phase_plan(g3);
+}
 
 // One optimizer step.  With `params_host` set (mona_step_host) every chunk first waits for the gradient copies of
 // the descriptors it touches, and a descriptor whose last matrix has been updated is copied back right away
@@ -471,6 +542,8 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             const void* o_final = nullptr;
             bool update_fused = false;
             if (tc) {
+                const bool together = ns_first_two_together(b.paired, T);
+                const int groups = together ? T - 1 : T;      // each reads one iterate and writes the other
                 if (phase_mask & 2u) {
                     NvtxRange range("mona.newton_schulz");
                     // the last X' = B' X applies the parameter update in its epilogue when this call runs both phases and the
@@ -479,46 +552,29 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                     for (int c = 0; c < C && update_fused; ++c)
                         if (((uintptr_t)ptrs.w[c] & 31) || ((uintptr_t)ptrs.o[c] & 31)) update_fused = false;
                     unsigned int* sched = (unsigned int*)(ctrl + CTRL_SCHED_OFF);
-                    for (int t0 = 0; t0 < T; t0 += NS_MAX_PHASES / 3) {
-                        const int t1 = std::min(T, t0 + NS_MAX_PHASES / 3);
+                    for (int gi = 0; gi < groups;) {
                         NsProgram g{};
-                        g.C = C; g.P = 3 * (t1 - t0); g.delay = h->opt.ns_delay;
+                        g.C = C; g.delay = h->opt.ns_delay;
                         g.inv_norm = inv_norm; g.work_counter = sched; g.done = sched + 64;
                         g.eta_lambda = eta_lambda; g.eta_gamma = eta_gamma;
-                        for (int t = t0; t < t1; ++t) {
-                            const int cur = t & 1, nxt = cur ^ 1;
-                            NsPhase& g1 = g.ph[3 * (t - t0)];      // A = X X^T (wide) or X^T X (tall): lower-triangle tiles only
-                            g1.M = g1.N = (int)b.s; g1.K = (int)b.l; g1.a_map = g1.b_map = MAP_X0 + cur; g1.a_mn = g1.b_mn = b.tall ? 1 : 0;
-                            g1.symmetric = 1; g1.ab_same = 1; g1.d_map = MAP_A; g1.ld = b.s; g1.mat_stride = b.s * b.s;
-                            g1.c1 = 0.f; g1.c2 = 1.f; g1.post_mode = t == 0 ? 2 : 0;
-                            ns_phase_plan(g1);
-                            NsPhase& g2 = g.ph[3 * (t - t0) + 1];  // B' = b A + c A A + a I, operands and result lower-block-stored
-                            g2.M = g2.N = g2.K = (int)b.s; g2.a_map = g2.b_map = MAP_A; g2.a_sym = g2.b_sym = 1; g2.symmetric = 1; g2.ab_same = 1;
-                            g2.cin = ab; g2.d_map = MAP_B; g2.ld = b.s; g2.mat_stride = b.s * b.s; g2.c1 = ns_b; g2.c2 = ns_c; g2.diag_add = ns_a;
-                            ns_phase_plan(g2);
-                            NsPhase& g3 = g.ph[3 * (t - t0) + 2];  // X' = B' X (wide) or X B' (tall); 256 x 512 macro-tiles when the inner dimension is long
-                            g3.K = (int)b.s; g3.wide = b.s >= h->opt.macro_tile_min_k ? 1 : 0; g3.d_map = MAP_X0 + nxt; g3.ld = b.cols; g3.mat_stride = b.e;
-                            g3.c1 = 0.f; g3.c2 = 1.f; g3.post_mode = t == 0 ? 1 : 0;
-                            g3.fuse_update = (update_fused && t == T - 1) ? 1 : 0;
-                            if (!b.tall) {   // B' is the symmetric "A" operand, X the MN-major "B" operand
-                                g3.M = (int)b.s; g3.N = (int)b.l; g3.a_map = MAP_B; g3.a_sym = 1; g3.b_map = MAP_X0 + cur; g3.b_mn = 1;
-                            } else {         // X is K-major, the symmetric B' serves as its own transpose
-                                g3.M = (int)b.l; g3.N = (int)b.s; g3.a_map = MAP_X0 + cur; g3.a_mn = 0; g3.b_map = MAP_B; g3.b_sym = 1;
-                            }
-                            ns_phase_plan(g3);
-                            h->flops_exec += (double)C * (ns_phase_executed_flops(g1) + ns_phase_executed_flops(g2) + ns_phase_executed_flops(g3));
-                            h->flops_dense += (double)C * (4.0 * b.s * b.s * b.l + 2.0 * (double)b.s * b.s * b.s);
-                            h->flops_useful += (double)C * (3.0 * b.s * b.s * b.l + (double)b.s * b.s * b.s);
+                        bool last = false;
+                        for (; gi < groups && g.P + (gi == 0 && together ? 7 : 3) <= NS_MAX_PHASES; ++gi) {
+                            last = gi + 1 == groups;
+                            ns_plan_group(g, b, gi == 0 && together, gi == 0, gi & 1, ab, (float*)(data + b.off_delta), ns_a, ns_b, ns_c,
+                                          h->opt.macro_tile_min_k, update_fused && last);
                         }
+                        for (int q = 0; q < g.P; ++q) h->flops_exec += (double)C * ns_phase_executed_flops(g.ph[q]);
                         ns_program_plan(g);
                         MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(C, g.P), stream));
                         NsUpdatePtrs up{};
-                        if (update_fused && t1 == T) { up.w = ptrs.w; up.o = ptrs.o; }
+                        if (update_fused && last) { up.w = ptrs.w; up.o = ptrs.o; }
                         MONA_CUDA(h, launch_ns_program(b.maps[slot], g, up, h->max_pairs, dstatus, stream));
                         ++h->launches;
                     }
+                    h->flops_dense += (double)T * C * (4.0 * b.s * b.s * b.l + 2.0 * (double)b.s * b.s * b.s);
+                    h->flops_useful += (double)T * C * (3.0 * b.s * b.s * b.l + (double)b.s * b.s * b.s);
                 }
-                o_final = xb[T & 1];
+                o_final = xb[groups & 1];
             } else if (small_ns_eligible(b.rows, b.cols)) {
                 // short side <= 64 (routers): the whole iteration in one launch, one block per matrix
                 if (phase_mask & 2u) {
@@ -726,7 +782,7 @@ static_assert(MONA_TRACE_ROWS == mona::NS_TRACE_ROWS && MONA_TRACE_SLOTS == mona
 
 mona_status mona_work_order(int32_t n_matrices, int32_t n_phases, int32_t delay, const uint32_t* items_per_phase,
                             uint32_t start, uint32_t stride, int32_t* out_cqt, size_t capacity, size_t* n_written) {
-    if (!n_written) return MONA_ERR_INVALID_ARG;
+    if (!n_written || n_phases > 15) return MONA_ERR_INVALID_ARG;      // the documented range
     const int n = mona::ns_work_order(n_matrices, n_phases, delay, items_per_phase, start, stride, out_cqt, capacity);
     if (n < 0) return MONA_ERR_INVALID_ARG;
     *n_written = (size_t)n;

@@ -632,8 +632,8 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 }
                 if (tc.nsub == 1) acc_next ^= 1u;
 #ifdef MONA_TRACE
-                {   // kind of tile: 0/1 X X^T off/on the diagonal, 2/3 b A + c A^2 + a I off/on the diagonal, 4 macro-tile, 5 single tile of X' = B' X
-                    const int kind = !p.symmetric ? (tc.nsub == 2 ? 4 : 5) : ((p.cin ? 2 : 0) + (shared_ab ? 1 : 0));
+                {   // kind of tile: 0/1 X X^T off/on the diagonal, 2/3 a product of s x s matrices off/on the diagonal, 4 macro-tile, 5 single tile of X' = B' X
+                    const int kind = !p.symmetric ? (tc.nsub == 2 ? 4 : 5) : ((p.small_sym ? 2 : 0) + (shared_ab ? 1 : 0));
                     const int slot = NS_TRACE_TILE0 + 4 * kind;
                     trace_add(slot, trace_clock() - t_item0); trace_add(slot + 1, (uint32_t)num_kb);
                     trace_add(slot + 2, w_full); trace_add(slot + 3, w_acc);
@@ -798,10 +798,12 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             const long long row_off = (long long)it.c * p.mat_stride + (long long)gr * p.ld;
             float post = 1.0f;
             if (p.post_mode) { const float sc = g.inv_norm[it.c]; post = p.post_mode == 2 ? sc * sc : sc; }
-            const float c1 = p.c1 * post, c2 = p.c2 * post;
+            // correction of this row's diagonal element of A (written earlier in this launch by another CTA: read from L2)
+            const float delta = row_ok && p.delta_in ? __ldcg(p.delta_in + (size_t)it.c * p.M + gr) : 0.0f;
+            const float c2 = p.c2 * post, c1 = fmaf(2.0f * c2, delta, p.c1 * post);
             const uint32_t acc0 = tc.nsub == 2 ? 0u : acc_next;
-            if (!p.cin && !p.fuse_update && p.diag_add == 0.f) {
-                // No axpy operand, no diagonal term (X X^T and X' = B' X).  A thread's share of an accumulator is 128 values,
+            if (!p.cin && !p.fuse_update) {
+                // No axpy operand, no diagonal term (X X^T, products of s x s matrices, X' = B' X).  A thread's share of an accumulator is 128 values,
                 // 64 registers once packed: read and pack every accumulator of the item first, handing each back to the MMA
                 // issuer as soon as it has been read, and only then stage.  Nothing hides the epilogue of a macro-tile, so
                 // the time the tensor cores wait is the time of these reads.  The item widths are separate instances whose packed
@@ -828,6 +830,15 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                                 tmem_ld_wait();
                                 #pragma unroll
                                 for (int j = 0; j < 32; ++j) v[j] *= c2;
+                                if (NSUB == 1 && p.delta_out) {
+                                    const int dj = gr - ((tc.tn + u) * TC_BN + ph * EPI_COLS + half * 64 + 32 * h);
+                                    if (row_ok && dj >= 0 && dj < 32) {       // this row's diagonal element is among the 32
+                                        float d = 0.f;
+                                        #pragma unroll
+                                        for (int j = 0; j < 32; ++j) d = j == dj ? v[j] : d;
+                                        p.delta_out[(size_t)it.c * p.M + gr] = d - __bfloat162float(__float2bfloat16_rn(d));
+                                    }
+                                }
                                 #pragma unroll
                                 for (int q = 0; q < 4; ++q) pk[u][ph][4 * h + q] = pack8(v + 8 * q);
                             }
@@ -898,14 +909,16 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                             v[2 * h] = fmaf(c1, __uint_as_float(cin_w[h] << 16), c2 * v[2 * h]);
                             v[2 * h + 1] = fmaf(c1, __uint_as_float(cin_w[h] & 0xffff0000u), c2 * v[2 * h + 1]);
                         }
+                        if (gr >= gc0 && gr < gc0 + 64) {
+                            // the row's diagonal element: + a, and b A(i,i) with the exact A(i,i)
+                            const float d = fmaf(p.c1, delta, p.diag_add);
+                            #pragma unroll
+                            for (int j = 0; j < 64; ++j) v[j] += (gc0 + j == gr) ? d : 0.f;
+                        }
                         if (ph + 1 < nphases) load_cin(ph + 1);
                     } else {
                         #pragma unroll
                         for (int j = 0; j < 64; ++j) v[j] *= c2;
-                    }
-                    if (p.diag_add != 0.f && gr >= gc0 && gr < gc0 + 64) {
-                        #pragma unroll
-                        for (int j = 0; j < 64; ++j) v[j] += (gc0 + j == gr) ? p.diag_add : 0.f;
                     }
                     if (!p.fuse_update) {
                         uint4 pk[8];
@@ -936,7 +949,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             if (lane == 0) {      // one lane per warp: the table holds sums over the eight epilogue warps
                 trace_add(NS_TRACE_EPI_RING, w_ring); trace_add(NS_TRACE_EPI_ACC_FULL, w_accf); trace_add(NS_TRACE_EPI_STAGE_EMPTY, w_stge);
                 const bool diag = p.ab_same && tc.tm == tc.tn && tc.nsub == 1;
-                const int kind = !p.symmetric ? (tc.nsub == 2 ? 4 : 5) : ((p.cin ? 2 : 0) + (diag ? 1 : 0));
+                const int kind = !p.symmetric ? (tc.nsub == 2 ? 4 : 5) : ((p.small_sym ? 2 : 0) + (diag ? 1 : 0));
                 const int slot = NS_TRACE_EPI_TILE0 + 4 * kind;
                 trace_add(slot, trace_clock() - t_item0); trace_add(slot + 1, 1u); trace_add(slot + 2, w_accf); trace_add(slot + 3, w_stge);
             }

@@ -12,8 +12,8 @@ constexpr int TC_BM = 256;      // rows of D per tile: one CTA pair, 128 rows pe
 constexpr int TC_BN = 256;      // columns of D per tile (UMMA N = 256, each CTA stages 128 of them)
 constexpr int TC_BK = 64;       // k-slice per pipeline stage: 64 bf16 = one 128-byte swizzle row
 constexpr int TC_BOX = 64;      // every TMA box is 64 bf16 wide (one 128-byte swizzle row) and 64 or 128 rows high
-constexpr int NS_MAX_PHASES = 15;   // 3 GEMMs x 5 iterations per launch; longer iterations take several launches
-constexpr int NS_TENSORS = 4;       // operand tensors of a chunk: X ping, X pong, A, B'
+constexpr int NS_MAX_PHASES = 16;   // five iterations: 3 GEMMs each, 7 for two iterations taken together; longer ones take several launches
+constexpr int NS_TENSORS = 5;       // operand tensors of a chunk: X ping, X pong, A, B', C (in the memory of X pong)
 constexpr int NS_MAPS = 2 * NS_TENSORS;   // each with 64-row boxes (index t) and with 128-row boxes (index t + NS_TENSORS)
 
 // One batched GEMM ("phase") of the iteration of Eq. newton_schulz over the C matrices of a chunk:
@@ -36,6 +36,7 @@ struct NsPhase {
     int a_mn, b_mn;             // 1: operand is MN-major (ignored for an operand flagged *_sym)
     int a_sym, b_sym;           // 1: operand is a symmetric matrix stored as its lower block triangle
     int symmetric;              // 1: D = D^T, compute lower-triangle tiles only
+    int small_sym;              // 1: symmetric D from s x s operands (not X X^T); only the profiling build reads it
     int ab_same;                // 1: both operands are the same tensor in the same form (X X^T, A A): a diagonal
                                 //    tile stages its operand rows once and uses them on both sides
     int wide;                   // 1 (non-symmetric D only): a work item is a 256 x 512 macro-tile, two tiles that share
@@ -48,6 +49,11 @@ struct NsPhase {
     float diag_add;             // added to D(i,i): folds the a*X term of the quintic into B' = b A + c A^2 + a I
     int post_mode;              // 0: post = 1, 1: post = inv_norm[c], 2: post = inv_norm[c]^2
     int fuse_update;            // 1: epilogue applies the parameter update instead of storing D
+    // Diagonal correction of A, null or [C][M] fp32.  The diagonal of A is its largest entry by far, so its rounding to bf16 is
+    // most of what rounding A costs.  The phase that stores A keeps delta_out[i] = exact - stored diagonal element; the phase
+    // that forms b A + c A^2 + a I from it uses A + diag(delta) to first order (in A^2 the row's delta stands for both sides).
+    float* delta_out;
+    const float* delta_in;
 };
 
 // Everything one launch needs: the phases in execution order and the scheduler state.  Work items are handed

@@ -111,6 +111,9 @@ bool ns_first_two_together(const bool pair_pays, int T) { return pair_pays && T 
 struct Plan {
     std::vector<mona_matrix_desc> descs;
     std::vector<Bucket> buckets;
+    // Buckets in the order in which a step takes them: matrices small enough for one block cluster each first, so that their
+    // few-block launches run beside the first big prologue; last, they were the step's tail with the machine idle.
+    std::vector<int> order;
     std::vector<int> desc_bucket;          // bucket of descriptor i
     std::vector<int64_t> desc_pos;         // position of descriptor i's matrix 0 inside its bucket
     std::vector<int64_t> desc_first_gid;   // global matrix index (descriptor order) of matrix 0
@@ -170,7 +173,10 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         int64_t cb = (int64_t)(chunk_budget / per_mat_bf16);
         cb = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cb, MAXC), count));
         b.Cb = (int)cb;
-        b.Cf = (int)std::max<int64_t>(1, cb / 2);
+        // fp32 iterates take twice the bytes.  A bucket that has no other path gets whole chunks; in validation mode one that
+        // also has the bf16 path must not make the workspace larger than that path needs.
+        const int64_t cf = b.tc_ok ? cb / 2 : std::min<int64_t>(cb, (int64_t)(chunk_budget / (2 * per_mat_bf16)));
+        b.Cf = (int)std::max<int64_t>(1, cf);
         b.paired = b.tc_ok && ns_pair_pays(b.s, b.l, count);
         size_t off = 0;
         for (int i = 0; i < 2; ++i) { b.off_x[i] = off; off += align_up((size_t)b.Cb * b.e * 2, 1024); }
@@ -184,6 +190,11 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         b.data_bytes = std::max(off, off32);
         max_data = std::max(max_data, b.data_bytes);
     }
+    for (int small = 1; small >= 0; --small)
+        for (int i = 0; i < (int)plan.buckets.size(); ++i) {
+            const Bucket& b = plan.buckets[i];
+            if ((!b.tc_ok && small_ns_eligible(b.rows, b.cols)) == (small != 0)) plan.order.push_back(i);
+        }
     plan.state_bytes = state_bytes;
     plan.slot_bytes = align_up(max_data, 1024);
     plan.workspace_bytes = WS_DATA_OFF + NSLOTS * plan.slot_bytes;
@@ -487,7 +498,8 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
     h->flops_dense = 0.0;
     h->flops_useful = 0.0;
 
-    for (const Bucket& b : plan.buckets) {
+    for (int bucket_index : plan.order) {
+        const Bucket& b = plan.buckets[bucket_index];
         const bool tc = (hp->ns_precision == 0) && b.tc_ok && T >= 1;
         const int cap = tc ? b.Cb : b.Cf;
         const int64_t count = (int64_t)b.mats.size();
@@ -576,7 +588,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                 }
                 o_final = xb[groups & 1];
             } else if (small_ns_eligible(b.rows, b.cols)) {
-                // short side <= 64 (routers): the whole iteration in one launch, one block per matrix
+                // short side <= 64 (routers): the whole iteration in one launch, one block cluster per matrix
                 if (phase_mask & 2u) {
                     NvtxRange range("mona.newton_schulz.small");
                     MONA_CUDA(h, launch_small_ns(Mc, xf[0], inv_norm, C, (int)b.rows, (int)b.cols, T, ns_a, ns_b, ns_c, stream));
@@ -688,7 +700,8 @@ mona_status mona_step_host(mona_handle* h, const mona_hparams* hp, void* const* 
     MONA_CUDA(h, cudaStreamWaitEvent(h->h2d, h->ev_hfork, 0));
     MONA_CUDA(h, cudaStreamWaitEvent(h->d2h, h->ev_hfork, 0));
     // gradients travel in the order in which the chunks will want them: bucket by bucket, descriptor by descriptor
-    for (const Bucket& b : h->plan.buckets) {
+    for (int bucket_index : h->plan.order) {
+        const Bucket& b = h->plan.buckets[bucket_index];
         int prev = -1;
         for (const MatRef& mr : b.mats) {
             if (mr.desc == prev) continue;

@@ -9,21 +9,26 @@ namespace mona {
 
 // A chunk is the unit that goes through prologue -> Newton-Schulz -> update together: up to MAXC
 // same-shape matrices whose bf16 iterates fit the chunk budget (sized for full machine occupancy, not for cache).
-constexpr int MAXC = 512;   // the pointer table below travels as a kernel argument (14 KiB of the 32 KiB CUDA 12 allows)
-// Each matrix is cut into at most MAX_SLABS contiguous slabs for the elementwise passes; every slab
+constexpr int MAXC = 512;   // per-matrix pointers travel as kernel arguments (at most 8 KiB of the 32 KiB CUDA 12 allows)
+// Each matrix is cut into at most MAX_SLABS contiguous slabs for the prologue; every slab
 // owns one partial sum of squares, so the Frobenius norm is reduced in a fixed order.
 constexpr int MAX_SLABS = 256;
 
-// Slab decomposition of a matrix of e elements: ~16 K elements per slab, at most MAX_SLABS slabs, slab length a
-// multiple of 1024 once the cap binds.
-inline void slab_plan(long long e, long long* slab_len, int* slabs) {
-    long long slab = 16384;
-    if ((e + slab - 1) / slab > MAX_SLABS) slab = ((e + MAX_SLABS - 1) / MAX_SLABS + 1023) / 1024 * 1024;
+// Slab decomposition of `count` matrices of e elements that go through one launch.  A slab is one block's work: a multiple of
+// `unit` elements (one trip of its loop), 16 K of them at most (longer slabs leave fewer blocks than the device holds at
+// once), as short as it takes to give every SM its eleven blocks - with 16 K always, a 256 x 512 matrix ran on 8 blocks and its
+// prologue took 10.6 us, 128 blocks take 4.1 - and long enough for at most MAX_SLABS per matrix.
+inline void slab_plan(long long e, long long count, long long unit, long long* slab_len, int* slabs) {
+    const long long resident = 148 * 11;
+    long long slab = (e * count + resident - 1) / resident;
+    slab = slab < 16384 ? slab : 16384;
+    if ((e + slab - 1) / slab > MAX_SLABS) slab = (e + MAX_SLABS - 1) / MAX_SLABS;
+    slab = (slab + unit - 1) / unit * unit;
     *slab_len = slab;
     *slabs = (int)((e + slab - 1) / slab);
 }
 
-// Per-chunk pointer table passed by value to the elementwise kernels.
+// Per-chunk pointers, filled on the host; the elementwise kernels take the parts they need in tables of their own size.
 struct ChunkPtrs {
     const void* g[MAXC];   // gradient of matrix c (fp32 or bf16)
     float* w[MAXC];        // parameter of matrix c

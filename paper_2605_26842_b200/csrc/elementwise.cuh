@@ -4,6 +4,9 @@
 
 namespace mona {
 
+// Elements one block handles per trip of its loop: slab lengths are multiples (see slab_plan).
+constexpr int PROLOGUE_UNIT = 1024, UPDATE_UNIT = 2048;
+
 // Fused prologue over a chunk of C same-shape matrices (state stored densely, e elements each):
 // updates A, M, G_prev in place from the gradient, optionally writes bf16(M) to `xhat` (null to skip),
 // and leaves 1/(||M||_F + eps) of matrix c in inv_norm[c].  `state_kind` says how the acceleration state is kept:

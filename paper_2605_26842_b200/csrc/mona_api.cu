@@ -77,8 +77,8 @@ struct Bucket {
     // bytes from the state base of the three blocks: M (fp32), A and G_prev (fp32, or bf16 with MONA-Lite storage)
     size_t off_M = 0, off_A = 0, off_G = 0;
     int Cb = 1, Cf = 1;         // chunk capacity: bf16 tensor-core mode / fp32 mode
-    int slabs = 1;
-    int64_t slab_len = 0;
+    int slabs = 1, up_slabs = 1;                // of the prologue; of the update and scale passes
+    int64_t slab_len = 0, up_slab_len = 0;
     size_t off_x[2] = {0, 0}, off_a = 0, off_b = 0, off_delta = 0;   // bf16 mode, bytes from the slot's iterate base
     size_t off32_x[2] = {0, 0}, off32_a = 0, off32_b = 0;    // fp32 mode
     size_t data_bytes = 0;
@@ -165,9 +165,6 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         b.off_A = state_bytes; state_bytes += align_up((size_t)count * b.e * aux, 256);
         b.off_G = state_bytes;                                              // the single-buffer form has no G_prev block
         if (b.state_dtype != MONA_STATE_COMBINED) state_bytes += align_up((size_t)count * b.e * aux, 256);
-        long long slab = 0;
-        slab_plan(b.e, &slab, &b.slabs);
-        b.slab_len = slab;
         // chunk capacity
         const size_t per_mat_bf16 = (size_t)(2 * b.e + 2 * b.s * b.s) * 2;
         int64_t cb = (int64_t)(chunk_budget / per_mat_bf16);
@@ -177,6 +174,11 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         // also has the bf16 path must not make the workspace larger than that path needs.
         const int64_t cf = b.tc_ok ? cb / 2 : std::min<int64_t>(cb, (int64_t)(chunk_budget / (2 * per_mat_bf16)));
         b.Cf = (int)std::max<int64_t>(1, cf);
+        long long slab = 0;
+        slab_plan(b.e, cb, PROLOGUE_UNIT, &slab, &b.slabs);
+        b.slab_len = slab;
+        slab_plan(b.e, cb, UPDATE_UNIT, &slab, &b.up_slabs);
+        b.up_slab_len = slab;
         b.paired = b.tc_ok && ns_pair_pays(b.s, b.l, count);
         size_t off = 0;
         for (int i = 0; i < 2; ++i) { b.off_x[i] = off; off += align_up((size_t)b.Cb * b.e * 2, 1024); }
@@ -599,7 +601,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             } else {
                 if (phase_mask & 2u) {
                     NvtxRange range("mona.newton_schulz.fp32");
-                    MONA_CUDA(h, launch_scale(Mc, xf[0], inv_norm, C, b.e, b.slab_len, b.slabs, stream));
+                    MONA_CUDA(h, launch_scale(Mc, xf[0], inv_norm, C, b.e, b.up_slab_len, b.up_slabs, stream));
                     ++h->launches;
                     for (int t = 0; t < T; ++t) {
                         const int cur = t & 1, nxt = cur ^ 1;
@@ -637,7 +639,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             }
             if ((phase_mask & 4u) && !update_fused) {
                 NvtxRange range("mona.update");
-                MONA_CUDA(h, launch_update(ptrs, C, tc, vec4, o_final, b.e, b.slab_len, b.slabs, eta_lambda, eta_gamma, stream));
+                MONA_CUDA(h, launch_update(ptrs, C, tc, vec4, o_final, b.e, b.up_slab_len, b.up_slabs, eta_lambda, eta_gamma, stream));
                 ++h->launches;
             }
             if (params_host) {

@@ -27,10 +27,12 @@ using namespace mona;
 namespace {
 
 // ---- workspace layout -------------------------------------------------------------------------------
-// [status word | control block of slot 0 | control block of slot 1 | iterates of slot 0 | iterates of slot 1]
-// Consecutive chunks alternate between two slots (and two streams), so that the last wave of each GEMM
-// launch is filled by the other chunk's tiles and launch gaps of one chunk are covered by the other.
-constexpr int NSLOTS = 2;
+// [status word | control blocks of the slots | iterates of slot 0 | 1 | 2 | 3]
+// Consecutive large chunks alternate between slots 0 and 1 (and two streams), so that the last wave of each GEMM
+// launch is filled by the other chunk's tiles and launch gaps of one chunk are covered by the other.  Small chunks, whose
+// products have too few tiles for the machine, go to slots 2 and 3 beside them, or to all four when there is nothing else.
+constexpr int NSLOTS = 4;
+constexpr int BIG_SLOTS = 2;
 constexpr size_t WS_STATUS_OFF = 0;
 constexpr size_t WS_CTRL_OFF = 4096;                 // first control block
 constexpr size_t WS_CTRL_BYTES = 1024 * 1024;        // per slot
@@ -72,6 +74,7 @@ struct Bucket {
     int64_t rows = 0, cols = 0, s = 0, l = 0, e = 0;
     int grad_dtype = 0, state_dtype = 0;
     bool tall = false, tc_ok = false;
+    bool small = false;         // its products do not fill the machine: runs beside other chunks (see bucket_is_small)
     bool paired = false;        // takes its first two iterations together on the s x s side (see ns_pair_pays)
     std::vector<MatRef> mats;
     // bytes from the state base of the three blocks: M (fp32), A and G_prev (fp32, or bf16 with MONA-Lite storage)
@@ -108,6 +111,23 @@ bool ns_pair_pays(int64_t s, int64_t l, int64_t count) {
 // ill-conditioned ones get worse (0.030), and for T < 4 an error of the first two has no iterations left to shrink in.
 bool ns_first_two_together(const bool pair_pays, int T) { return pair_pays && T >= 4; }
 
+// A bucket whose symmetric products are at most four waves of tiles over the machine's 74 CTA pairs, and whose iterates are
+// small enough to hold twice more, does not get the machine to itself: a launch of it is a chain of dependent products with many
+// pairs idle at the end of each, so such buckets run side by side on streams and SM pairs of their own.  Measured: buckets of four
+// 1024 x 1024, two 2816 x 1024 and one 1024 x 2816 928 -> 372 us per step; sixteen, eight and four of 1160 and 3096 (240, 120 and 60
+// tiles; with the line at two waves 2.03 ms) -> 1.75 ms; from five waves on (six tried) nothing changes.  Everything on the
+// fp32 path that takes one block cluster per matrix is small too.
+constexpr size_t SMALL_BUCKET_BYTES = 400ull << 20;
+bool bucket_is_small(int64_t s, int64_t e, int64_t count, bool tc_ok, bool one_cluster) {
+    const int64_t ts = (s + TC_BM - 1) / TC_BM;
+    if (!tc_ok && !one_cluster) return false;
+    return (one_cluster || ts * (ts + 1) / 2 * count <= 4 * 74) && (size_t)(2 * e + 2 * s * s) * 2 * count <= SMALL_BUCKET_BYTES;
+}
+// NARROW_ROUNDS: a launch on a share of the pairs looks at other tile widths for phases of at most this many rounds of items (1 to 8
+// measured equal within 2 %).  GATE_ROUNDS: the claim gate (NsProgram::gate) pays while a phase leaves pairs idle (mixed small set 151 ->
+// 124 us) and costs a round trip per item where every pair has several (12 dense blocks, a bucket at 1.6 rounds: 1-2 %).
+constexpr double NARROW_ROUNDS = 4.0, GATE_ROUNDS = 1.5;
+
 struct Plan {
     std::vector<mona_matrix_desc> descs;
     std::vector<Bucket> buckets;
@@ -117,7 +137,9 @@ struct Plan {
     std::vector<int> desc_bucket;          // bucket of descriptor i
     std::vector<int64_t> desc_pos;         // position of descriptor i's matrix 0 inside its bucket
     std::vector<int64_t> desc_first_gid;   // global matrix index (descriptor order) of matrix 0
-    size_t state_bytes = 0, workspace_bytes = 0, slot_bytes = 0;
+    bool all_small = true;                 // no large bucket: small ones use all slots
+    size_t state_bytes = 0, workspace_bytes = 0;
+    size_t slot_off[NSLOTS] = {};          // bytes from the workspace base
 };
 
 mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chunk_budget, Plan& plan, std::string& err) {
@@ -157,7 +179,7 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         gid += d.batch;
     }
     size_t state_bytes = 0;
-    size_t max_data = 0;
+    size_t max_data[2] = {0, 0};        // of all buckets, of the small ones
     for (Bucket& b : plan.buckets) {
         const int64_t count = (int64_t)b.mats.size();
         const size_t aux = b.state_dtype == MONA_BF16 ? 2 : 4;              // every block starts 256-byte aligned
@@ -190,16 +212,26 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         b.off32_a = off32; off32 += align_up((size_t)b.Cf * b.s * b.s * 4, 1024);
         b.off32_b = off32; off32 += align_up((size_t)b.Cf * b.s * b.s * 4, 1024);
         b.data_bytes = std::max(off, off32);
-        max_data = std::max(max_data, b.data_bytes);
+        b.small = bucket_is_small(b.s, b.e, count, b.tc_ok, !b.tc_ok && small_ns_eligible(b.rows, b.cols)) && cb == count;
+        plan.all_small = plan.all_small && b.small;
+        max_data[0] = std::max(max_data[0], b.data_bytes);
+        if (b.small) max_data[1] = std::max(max_data[1], b.data_bytes);
     }
+    // slots 2 and 3 exist when there are small buckets to fill them with
+    int64_t n_small = 0;
+    for (const Bucket& b : plan.buckets) n_small += b.small ? 1 : 0;
+    const int64_t extra = plan.all_small ? std::max<int64_t>(0, n_small - BIG_SLOTS) : n_small;
     for (int small = 1; small >= 0; --small)
         for (int i = 0; i < (int)plan.buckets.size(); ++i) {
             const Bucket& b = plan.buckets[i];
             if ((!b.tc_ok && small_ns_eligible(b.rows, b.cols)) == (small != 0)) plan.order.push_back(i);
         }
     plan.state_bytes = state_bytes;
-    plan.slot_bytes = align_up(max_data, 1024);
-    plan.workspace_bytes = WS_DATA_OFF + NSLOTS * plan.slot_bytes;
+    plan.workspace_bytes = WS_DATA_OFF;
+    for (int sl = 0; sl < NSLOTS; ++sl) {
+        plan.slot_off[sl] = plan.workspace_bytes;
+        plan.workspace_bytes += align_up(sl < BIG_SLOTS ? max_data[0] : sl - BIG_SLOTS < extra ? max_data[1] : 0, 1024);
+    }
     return MONA_OK;
 }
 
@@ -234,13 +266,13 @@ struct mona_handle {
     int device = 0, max_pairs = 0;
     uint8_t* state = nullptr;
     uint8_t* ws = nullptr;
-    cudaStream_t side = nullptr;
-    cudaEvent_t ev_fork = nullptr, ev_join = nullptr;
+    cudaStream_t side[NSLOTS] = {};        // stream of slot 1 .. NSLOTS - 1 (slot 0 uses the caller's)
+    cudaEvent_t ev_fork = nullptr, ev_join[NSLOTS] = {};
     // host-to-host pipeline of mona_step_host(): copy streams and per-descriptor events, created on first use
     cudaStream_t h2d = nullptr, d2h = nullptr;
     cudaEvent_t ev_hfork = nullptr, ev_hjoin = nullptr;
     std::vector<cudaEvent_t> ev_in;     // gradient of descriptor i has arrived on the device
-    std::vector<cudaEvent_t> ev_out;    // 2 per descriptor: its chunks on slot stream 0 / 1 have been updated
+    std::vector<cudaEvent_t> ev_out;    // NSLOTS per descriptor: its chunks on that slot's stream have been updated
     DeviceStatus* host_status = nullptr;   // pinned
     std::string last_error;
     int64_t launches = 0;
@@ -375,7 +407,8 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
         if (!b.tc_ok) continue;
         bool ok = true;
         for (int sl = 0; sl < NSLOTS; ++sl) {
-            uint8_t* data = h->ws + WS_DATA_OFF + sl * h->plan.slot_bytes;
+            if (sl >= BIG_SLOTS && !b.small) continue;
+            uint8_t* data = h->ws + h->plan.slot_off[sl];
             for (int big = 0; big < 2; ++big) {     // 64-row boxes, then 128-row boxes
                 const int rows = big ? 2 * TC_BOX : TC_BOX, at = big * NS_TENSORS;
                 for (int i = 0; i < 2; ++i) ok = ok && encode_map(encode, &b.maps[sl].m[at + MAP_X0 + i], data + b.off_x[i], b.cols, b.rows, b.Cb, rows, b.e);
@@ -390,9 +423,11 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
     }
     MONA_CUDA(h, ns_configure(&h->max_pairs));
     MONA_CUDA(h, small_ns_configure());
-    MONA_CUDA(h, cudaStreamCreateWithFlags(&h->side, cudaStreamNonBlocking));
     MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
-    MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming));
+    for (int sl = 1; sl < NSLOTS; ++sl) {
+        MONA_CUDA(h, cudaStreamCreateWithFlags(&h->side[sl], cudaStreamNonBlocking));
+        MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_join[sl], cudaEventDisableTiming));
+    }
     MONA_CUDA(h, cudaMallocHost((void**)&h->host_status, sizeof(DeviceStatus)));
     // M_0 = A_0 = G_0 = 0; control block cleared
     MONA_CUDA(h, cudaMemset(h->state, 0, h->plan.state_bytes));
@@ -447,6 +482,48 @@ static void ns_plan_group(NsProgram& g, const Bucket& b, bool together, bool fir
     ns_phase_plan(g3);
 }
 
+// Tile work of a bucket's iteration, in k-slices of 256 x 256 tiles.
+static double bucket_work(const Bucket& b) {
+    const double ts = (double)((b.s + TC_BM - 1) / TC_BM), tl = (double)((b.l + TC_BM - 1) / TC_BM);
+    const double ks = (double)((b.s + TC_BK - 1) / TC_BK), kl = (double)((b.l + TC_BK - 1) / TC_BK);
+    return (double)b.mats.size() * (ts * (ts + 1) / 2 * (kl + ks) + ts * tl * ks);
+}
+// SM pairs of a small chunk: its share of the work when only small chunks run; beside large ones four times that, and eight
+// at least, so that it is through long before they are.  (Pairs that a launch does not find free simply come later: items are
+// handed out to whichever pairs run.)
+static int pairs_share(int max_pairs, double work, double work_total, bool all_small) {
+    const double share = max_pairs * work / work_total;
+    return std::max(1, std::min(max_pairs, (int)(all_small ? share + 0.5 : std::max(8.0, 4.0 * share))));
+}
+// Fits a launch to `pairs` SM pairs: tile widths by estimated time, the claim gate, no more pairs than a phase has items.
+// (`shared`: beside other launches on a part of the pairs.)  A launch that has all pairs looks at other tile widths only for phases
+// that do not fill them once; macro-tiles move the fewest bytes per flop.
+static void ns_fit_launch(NsProgram& g, int pairs, bool shared) {
+    int most = 0;
+    bool fused = false;
+    for (int q = 0; q < g.P; ++q) fused = fused || g.ph[q].fuse_update;
+    for (int q = 0; q < g.P; ++q) {
+        NsPhase& p = g.ph[q];
+        NsPhase best = p;
+        double best_cycles = ns_phase_cycles(p, std::ceil((double)g.C * p.items_per_mat / pairs));
+        if (!fused && (double)g.C * p.items_per_mat <= (shared ? NARROW_ROUNDS : 1.0) * pairs) {
+            for (int narrow = 0; narrow < 2; ++narrow) {
+                NsPhase alt = p;
+                alt.wide = 0; alt.narrow = narrow;
+                ns_phase_plan(alt);
+                const double cycles = ns_phase_cycles(alt, std::ceil((double)g.C * alt.items_per_mat / pairs));
+                if (cycles < best_cycles) { best_cycles = cycles; best = alt; }
+            }
+        }
+        p = best;
+        most = std::max(most, p.items_per_mat * g.C);
+    }
+    g.gate = !fused && most < GATE_ROUNDS * pairs ? 1 : 0;
+    g.few = g.gate;
+    for (int q = 0; q < g.P; ++q) g.few |= g.ph[q].narrow;
+    g.max_pairs = std::min(pairs, most);
+}
+
 // One optimizer step.  With `params_host` set (mona_step_host) every chunk first waits for the gradient copies of
 // the descriptors it touches, and a descriptor whose last matrix has been updated is copied back right away
 // on the handle's device-to-host stream, so transfers in both directions overlap the remaining chunks.
@@ -487,13 +564,16 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
         total_chunks += ((int64_t)b.mats.size() + capb - 1) / capb;
     }
     const bool overlap = h->opt.chunk_overlap && total_chunks > 1;
-    cudaStream_t slot_stream[NSLOTS] = {(cudaStream_t)stream_v, overlap ? h->side : (cudaStream_t)stream_v};
-    if (overlap) {
-        MONA_CUDA(h, cudaEventRecord(h->ev_fork, slot_stream[0]));
-        MONA_CUDA(h, cudaStreamWaitEvent(h->side, h->ev_fork, 0));
-    }
-    int64_t chunk_index = 0;
-    std::vector<char> out_recorded(params_host ? 2 * plan.descs.size() : 0, 0);
+    cudaStream_t slot_stream[NSLOTS] = {(cudaStream_t)stream_v};
+    bool slot_used[NSLOTS] = {true};
+    for (int sl = 1; sl < NSLOTS; ++sl) slot_stream[sl] = overlap ? h->side[sl] : (cudaStream_t)stream_v;
+    if (overlap) MONA_CUDA(h, cudaEventRecord(h->ev_fork, slot_stream[0]));
+    int64_t big_index = 0, small_index = 0;
+    // estimated tensor work of the buckets, by which chunks that run side by side share the SM pairs
+    double work_total = 0.0;
+    for (const Bucket& b : plan.buckets)
+        if (hp->ns_precision == 0 && b.tc_ok) work_total += bucket_work(b);
+    std::vector<char> out_recorded(params_host ? NSLOTS * plan.descs.size() : 0, 0);
     std::vector<int> chunk_descs;
     h->launches = 0;
     h->flops_exec = 0.0;
@@ -505,6 +585,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
         const bool tc = (hp->ns_precision == 0) && b.tc_ok && T >= 1;
         const int cap = tc ? b.Cb : b.Cf;
         const int64_t count = (int64_t)b.mats.size();
+        const bool small = b.small && cap >= count;       // one chunk: the extra slots are made for whole buckets
         const double gamma = hp->scale_mode == 0 ? hp->scale_value * std::sqrt((double)b.l) : hp->scale_value;
         const float eta_gamma = (float)(hp->lr * gamma);
         const size_t gsz = b.grad_dtype == MONA_BF16 ? 2 : 4;
@@ -526,11 +607,17 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                 ptrs.o[c] = (o_out && o_out[mr.desc]) ? (float*)o_out[mr.desc] + mr.b * d.batch_stride : nullptr;
                 ptrs.gid[c] = (int)(plan.desc_first_gid[mr.desc] + mr.b);
             }
-            const int slot = overlap ? (int)(chunk_index % NSLOTS) : 0;
-            ++chunk_index;
+            int slot = 0;
+            if (overlap) {
+                if (!small) slot = (int)(big_index++ % BIG_SLOTS);
+                else slot = plan.all_small ? (int)(small_index++ % NSLOTS) : BIG_SLOTS + (int)(small_index++ % (NSLOTS - BIG_SLOTS));
+                if (!slot_used[slot]) MONA_CUDA(h, cudaStreamWaitEvent(slot_stream[slot], h->ev_fork, 0));
+                slot_used[slot] = true;
+            }
             cudaStream_t stream = slot_stream[slot];
             uint8_t* ctrl = h->ws + WS_CTRL_OFF + slot * WS_CTRL_BYTES;
-            uint8_t* data = h->ws + WS_DATA_OFF + slot * plan.slot_bytes;
+            uint8_t* data = h->ws + plan.slot_off[slot];
+            unsigned int* sched = (unsigned int*)(ctrl + CTRL_SCHED_OFF);
             unsigned int* counters = (unsigned int*)(ctrl + CTRL_COUNTERS_OFF);
             float* inv_norm = (float*)(ctrl + CTRL_INVNORM_OFF);
             float* partials = (float*)(ctrl + CTRL_PARTIALS_OFF);
@@ -545,12 +632,13 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
 
             if (params_host)
                 for (int dsc : chunk_descs) MONA_CUDA(h, cudaStreamWaitEvent(stream, h->ev_in[dsc], 0));
+            const bool cleared_by_prologue = tc && small;
             if (phase_mask & 1u) {
                 NvtxRange range("mona.prologue");
                 MONA_CUDA(h, launch_prologue(ptrs, C, b.grad_dtype == MONA_BF16,
                                              hp->algorithm == 1 ? PROLOGUE_NO_AUX : (b.state_dtype == MONA_BF16 ? PROLOGUE_AUX_BF16 :
                                                  b.state_dtype == MONA_STATE_COMBINED ? PROLOGUE_AUX_COMBINED : PROLOGUE_AUX_F32), vec4, Mc, Ac, Gc, tc ? xb[0] : nullptr, partials,
-                                             counters, inv_norm, dstatus, b.e, b.slab_len, b.slabs, ps, stream));
+                                             counters, inv_norm, dstatus, b.e, b.slab_len, b.slabs, ps, sched, cleared_by_prologue ? (int)ns_sched_words(C, NS_MAX_PHASES) : 0, stream));
                 ++h->launches;
             }
             const void* o_final = nullptr;
@@ -565,10 +653,10 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                     update_fused = h->opt.fuse_update && (phase_mask & 4u) != 0u;
                     for (int c = 0; c < C && update_fused; ++c)
                         if (((uintptr_t)ptrs.w[c] & 31) || ((uintptr_t)ptrs.o[c] & 31)) update_fused = false;
-                    unsigned int* sched = (unsigned int*)(ctrl + CTRL_SCHED_OFF);
+                    bool launched = false;
                     for (int gi = 0; gi < groups;) {
                         NsProgram g{};
-                        g.C = C; g.delay = h->opt.ns_delay;
+                        g.C = C; g.delay = std::min(h->opt.ns_delay, C);       // beyond C matrices the order is the same
                         g.inv_norm = inv_norm; g.work_counter = sched; g.done = sched + 64;
                         g.eta_lambda = eta_lambda; g.eta_gamma = eta_gamma;
                         bool last = false;
@@ -577,9 +665,16 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                             ns_plan_group(g, b, gi == 0 && together, gi == 0, gi & 1, ab, (float*)(data + b.off_delta), ns_a, ns_b, ns_c,
                                           h->opt.macro_tile_min_k, update_fused && last);
                         }
+                        const bool shared = overlap && small;
+                        ns_fit_launch(g, shared ? pairs_share(h->max_pairs, bucket_work(b), work_total, plan.all_small) : h->max_pairs, shared);
                         for (int q = 0; q < g.P; ++q) h->flops_exec += (double)C * ns_phase_executed_flops(g.ph[q]);
                         ns_program_plan(g);
-                        MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(C, g.P), stream));
+                        // For a small chunk the prologue of this call has cleared the scheduler words of the first launch: one
+                        // operation less in a short chain (one 256 x 512 matrix 102 -> 100 us, a mixed small set 126 -> 124).
+                        // Between a large prologue and its launch the memset stays: without it the launch takes the SMs
+                        // before the other stream's prologue has started on them (12 dense blocks 3.20 -> 3.36 ms).
+                        if (!(cleared_by_prologue && (phase_mask & 1u)) || launched) MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(C, g.P), stream));
+                        launched = true;
                         NsUpdatePtrs up{};
                         if (update_fused && last) { up.w = ptrs.w; up.o = ptrs.o; }
                         MONA_CUDA(h, launch_ns_program(b.maps[slot], g, up, h->max_pairs, dstatus, stream));
@@ -644,24 +739,25 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             }
             if (params_host) {
                 for (int dsc : chunk_descs) {
-                    MONA_CUDA(h, cudaEventRecord(h->ev_out[2 * dsc + slot], stream));
-                    out_recorded[2 * dsc + slot] = 1;
+                    MONA_CUDA(h, cudaEventRecord(h->ev_out[NSLOTS * dsc + slot], stream));
+                    out_recorded[NSLOTS * dsc + slot] = 1;
                 }
                 const MatRef& last = b.mats[start + C - 1];
                 for (int dsc : chunk_descs) {
                     const mona_matrix_desc& d = plan.descs[dsc];
                     if (dsc == last.desc && last.b != d.batch - 1) continue;    // descriptor continues in the next chunk
                     for (int sl = 0; sl < NSLOTS; ++sl)
-                        if (out_recorded[2 * dsc + sl]) MONA_CUDA(h, cudaStreamWaitEvent(h->d2h, h->ev_out[2 * dsc + sl], 0));
+                        if (out_recorded[NSLOTS * dsc + sl]) MONA_CUDA(h, cudaStreamWaitEvent(h->d2h, h->ev_out[NSLOTS * dsc + sl], 0));
                     const size_t bytes = (size_t)((d.batch - 1) * d.batch_stride + d.rows * d.cols) * 4;
                     MONA_CUDA(h, cudaMemcpyAsync(params_host[dsc], params[dsc], bytes, cudaMemcpyDeviceToHost, h->d2h));
                 }
             }
         }
     }
-    if (overlap) {
-        MONA_CUDA(h, cudaEventRecord(h->ev_join, h->side));
-        MONA_CUDA(h, cudaStreamWaitEvent(slot_stream[0], h->ev_join, 0));
+    for (int sl = 1; sl < NSLOTS; ++sl) {
+        if (!slot_used[sl]) continue;
+        MONA_CUDA(h, cudaEventRecord(h->ev_join[sl], slot_stream[sl]));
+        MONA_CUDA(h, cudaStreamWaitEvent(slot_stream[0], h->ev_join[sl], 0));
     }
     return MONA_OK;
 }
@@ -693,7 +789,7 @@ mona_status mona_step_host(mona_handle* h, const mona_hparams* hp, void* const* 
         MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_hfork, cudaEventDisableTiming));
         MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_hjoin, cudaEventDisableTiming));
         h->ev_in.assign((size_t)n_desc, nullptr);
-        h->ev_out.assign((size_t)(2 * n_desc), nullptr);
+        h->ev_out.assign((size_t)(NSLOTS * n_desc), nullptr);
         for (auto& e : h->ev_in) MONA_CUDA(h, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
         for (auto& e : h->ev_out) MONA_CUDA(h, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     }
@@ -816,7 +912,7 @@ const char* mona_last_error(const mona_handle* h) { return h ? h->last_error.c_s
 
 void mona_destroy(mona_handle* h) {
     if (!h) return;
-    if (h->side) cudaStreamDestroy(h->side);
+    for (cudaStream_t s : h->side) if (s) cudaStreamDestroy(s);
     if (h->ev_fork) cudaEventDestroy(h->ev_fork);
     if (h->h2d) cudaStreamDestroy(h->h2d);
     if (h->d2h) cudaStreamDestroy(h->d2h);
@@ -824,7 +920,7 @@ void mona_destroy(mona_handle* h) {
     if (h->ev_hjoin) cudaEventDestroy(h->ev_hjoin);
     for (cudaEvent_t e : h->ev_in) if (e) cudaEventDestroy(e);
     for (cudaEvent_t e : h->ev_out) if (e) cudaEventDestroy(e);
-    if (h->ev_join) cudaEventDestroy(h->ev_join);
+    for (cudaEvent_t e : h->ev_join) if (e) cudaEventDestroy(e);
     if (h->host_status) cudaFreeHost(h->host_status);
     delete h;
 }

@@ -280,6 +280,8 @@ constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);
 // the pair, N = 256); bits 15 / 16 say that A / B is MN-major.
 constexpr uint32_t IDESC_BASE = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(TC_BN >> 3) << 17) | ((uint32_t)(TC_BM >> 4) << 24);
 
+constexpr uint32_t IDESC_NARROW = IDESC_BASE - ((uint32_t)(TC_BN >> 4) << 17);     // N = 128
+
 // ---- tcgen05 --------------------------------------------------------------------------------------
 __device__ __forceinline__ void tmem_alloc(uint32_t dst_smem, uint32_t cols) {
     asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(dst_smem), "r"(cols) : "memory");
@@ -334,10 +336,11 @@ struct Item {
 };
 
 struct TileCoord {
-    int tm, tn;      // tile row, first tile column
-    int nsub;        // 256-column tiles in this item: 1 or 2
+    int tm, tn;      // tile row, first tile column (in units of the phase's tile width)
+    int nsub;        // tiles in this item: 1 or 2
 };
 
+template <bool FEW>
 __device__ __forceinline__ TileCoord decode_tile(const NsPhase& p, int r) {
     TileCoord tc;
     tc.nsub = 1;
@@ -347,10 +350,11 @@ __device__ __forceinline__ TileCoord decode_tile(const NsPhase& p, int r) {
         tc.tn = 2 * (r - tc.tm * macro_n);
         tc.nsub = tc.tn + 1 < p.tiles_n ? 2 : 1;
     } else if (p.symmetric) {
+        const int half = FEW && p.narrow ? 1 : 0;      // lower block triangle, row by row: tm + 1 blocks of 1 or 2 tiles
         int tm = 0;
-        while ((tm + 1) * (tm + 2) / 2 <= r) ++tm;     // lower triangle, row by row
+        while (((tm + 1) * (tm + 2) / 2 << half) <= r) ++tm;
         tc.tm = tm;
-        tc.tn = r - tm * (tm + 1) / 2;
+        tc.tn = r - (tm * (tm + 1) / 2 << half);
     } else {
         tc.tm = r / p.tiles_n;
         tc.tn = r - tc.tm * p.tiles_n;
@@ -395,7 +399,9 @@ struct UpdateTable {
     float* o[CAP];
 };
 
-template <int CAP>
+// FEW: the instance for launches of few tiles per phase, which knows narrow tiles and the claim gate.  As run-time branches in the one
+// kernel they cost the large launches 3-7 % (more live values in the single-thread loops of the producer and the MMA issuer).
+template <int CAP, bool FEW>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(TC_MAX_REGS)
 ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsProgram g,
                 const __grid_constant__ UpdateTable<CAP> upd, DeviceStatus* __restrict__ status) {
@@ -472,22 +478,24 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     const uint32_t full_leader = map_to_cta(bar_full, 0);
     auto produce = [&](const Item& it) -> bool {
         const NsPhase& p = g.ph[it.q];
-        const TileCoord tc = decode_tile(p, it.t);
+        const TileCoord tc = decode_tile<FEW>(p, it.t);
         // K-major operands come as one box of 128 rows, MN-major ones as two boxes of 64 (the swizzle row is 64 elements)
         const CUtensorMap* a_box64 = &maps.m[p.a_map];
         const CUtensorMap* a_box128 = &maps.m[p.a_map + NS_TENSORS];
         const CUtensorMap* b_box64 = &maps.m[p.b_map];
         const CUtensorMap* b_box128 = &maps.m[p.b_map + NS_TENSORS];
         const int m0 = tc.tm * TC_BM + (int)rank * CTA_M;      // this CTA's rows of the A operand
-        const int n0 = tc.tn * TC_BN + (int)rank * CTA_N;      // this CTA's rows of the B operand (first sub-tile)
+        const bool narrow = FEW && p.narrow;
+        const int bn = narrow ? TC_BN / 2 : TC_BN;
+        const int n0 = tc.tn * bn + (int)rank * (bn / 2);      // this CTA's rows of the B operand (first sub-tile)
         // diagonal tile of X X^T or A A: both operands are the same rows, staged once
-        const bool shared_ab = p.ab_same && tc.tm == tc.tn && tc.nsub == 1;
+        const bool shared_ab = p.ab_same && !narrow && tc.tm == tc.tn && tc.nsub == 1;
         const int nb = shared_ab ? 0 : tc.nsub;
-        const uint32_t tx_bytes = 2u * (A_STAGE_BYTES + (uint32_t)nb * B_SUB_BYTES) + (uint32_t)g.selftest_extra_tx;
+        const uint32_t tx_bytes = 2u * (A_STAGE_BYTES + (uint32_t)nb * (narrow ? B_SUB_BYTES / 2 : B_SUB_BYTES)) + (uint32_t)g.selftest_extra_tx;
         const int num_kb = (p.K + TC_BK - 1) / TC_BK;
         // from k-slice `switch` on the operand is MN-major (see the MMA issuer)
         const int a_switch = p.a_sym ? (tc.tm + 1) * (TC_BM / TC_BK) : (p.a_mn ? 0 : num_kb);
-        const int b_switch0 = p.b_sym ? (tc.tn + 1) * (TC_BN / TC_BK) : (p.b_mn ? 0 : num_kb);
+        const int b_switch0 = p.b_sym ? ((narrow ? tc.tn >> 1 : tc.tn) + 1) * (TC_BN / TC_BK) : (p.b_mn ? 0 : num_kb);
         const int b_switch1 = p.b_sym ? (tc.tn + 2) * (TC_BN / TC_BK) : (p.b_mn ? 0 : num_kb);
         const uint32_t nslab = 1u + (uint32_t)nb;
         for (int kb = 0; kb < num_kb; ++kb) {
@@ -519,7 +527,10 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             }
             if (nb > 0) {
                 const uint32_t sb = sa + A_STAGE_BYTES;
-                if (kb >= b_switch0) {
+                if (narrow) {                 // 64 rows of B per CTA: one box in either form
+                    const bool mn = kb >= b_switch0;
+                    tma_load_3d(sb, b_box64, full, mn ? n0 : k0, mn ? k0 : n0, it.c);
+                } else if (kb >= b_switch0) {
                     tma_load_3d(sb, b_box64, full, n0, k0, it.c);
                     tma_load_3d(sb + BOX_BYTES, b_box64, full, n0 + TC_BOX, k0, it.c);
                 } else {
@@ -571,8 +582,9 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 if (!(ok = take_item(n, it, 9, true, TRACE_PTR(w_ring))) || it.stop) break;
                 TRACE_ONLY(const uint32_t t_item0 = trace_clock(); uint32_t w_full = 0, w_acc = 0;)
                 const NsPhase& p = g.ph[it.q];
-                const TileCoord tc = decode_tile(p, it.t);
-                const bool shared_ab = p.ab_same && tc.tm == tc.tn && tc.nsub == 1;
+                const TileCoord tc = decode_tile<FEW>(p, it.t);
+                const bool shared_ab = p.ab_same && !(FEW && p.narrow) && tc.tm == tc.tn && tc.nsub == 1;
+                const uint32_t idesc_base = FEW && p.narrow ? IDESC_NARROW : IDESC_BASE;
                 const uint32_t acc0 = tc.nsub == 2 ? 0u : acc_next;
                 const int num_kb = (p.K + TC_BK - 1) / TC_BK;
                 // This one thread feeds both tensor cores, so the loop over k-slices is kept to a few dozen instructions:
@@ -582,7 +594,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 int b_switch[2];
                 #pragma unroll
                 for (int u = 0; u < 2; ++u)
-                    b_switch[u] = shared_ab ? a_switch : (p.b_sym ? (tc.tn + u + 1) * (TC_BN / TC_BK) : (p.b_mn ? 0 : num_kb));
+                    b_switch[u] = shared_ab ? a_switch : (p.b_sym ? ((FEW && p.narrow ? tc.tn >> 1 : tc.tn) + u + 1) * (TC_BN / TC_BK) : (p.b_mn ? 0 : num_kb));
                 const uint32_t b_off0 = shared_ab ? 0u : (A_STAGE_BYTES >> 4);             // operand offsets inside a stage, in 16-byte units
                 const uint32_t b_off1 = (A_STAGE_BYTES + B_SUB_BYTES) >> 4;
                 // an accumulator must have been drained by the epilogue of its previous tile before the first MMA into it
@@ -606,7 +618,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                     const uint32_t a_step = a_mn ? (2048u >> 4) : (32u >> 4), b_step0 = b_mn0 ? (2048u >> 4) : (32u >> 4);
                     const uint32_t a_lo = stage_lo | (a_mn ? DESC_LBO_MN : DESC_LBO_K);
                     const uint32_t b_lo0 = (stage_lo + b_off0) | (b_mn0 ? DESC_LBO_MN : DESC_LBO_K);
-                    const uint32_t idesc0 = IDESC_BASE | (a_mn << 15) | (b_mn0 << 16);
+                    const uint32_t idesc0 = idesc_base | (a_mn << 15) | (b_mn0 << 16);
                     #pragma unroll
                     for (int k = 0; k < TC_BK / 16; ++k) {
                         tc_mma_bf16(d0, a_lo + k * a_step, b_lo0 + k * b_step0, idesc0, accum);
@@ -663,15 +675,15 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 const NsPhase& p = g.ph[it.q];
                 if (p.fuse_update) continue;               // the epilogue writes the parameters itself; nothing is staged
                 const CUtensorMap* tma_d = &maps.m[p.d_map + NS_TENSORS];     // 64 columns x 128 rows per store
-                const TileCoord tc = decode_tile(p, it.t);
+                const TileCoord tc = decode_tile<FEW>(p, it.t);
                 const int m0 = tc.tm * TC_BM + (int)rank * CTA_M;
                 // The two 64-column halves of the staging buffer are separate buffers with their own barriers, filled by
                 // different warps: each half is stored as soon as it is full and handed back as soon as its own store has
                 // read it, the first half while the second store is still reading.
                 for (int u = 0; u < tc.nsub && ok; ++u) {
                     for (int ph = 0; ph < 2 && ok; ++ph) {
-                        const int x0 = (tc.tn + u) * TC_BN + ph * EPI_COLS;
-                        if (x0 >= p.N) continue;
+                        const int x0 = (tc.tn + u) * (FEW ? ns_tile_cols(p) : TC_BN) + ph * EPI_COLS;
+                        if (x0 >= p.N || (FEW && ph && p.narrow)) continue;
                         if (!MONA_IN_BOUNDS(m0 < p.M + CTA_M && it.c < g.C && tc.tm < p.tiles_m, status, 106)) { ok = false; break; }
                         #pragma unroll
                         for (int bx = 0; bx < 2; ++bx) {
@@ -724,12 +736,18 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             // The counter is always asked for one item more than has been published, so that its round trip (as long as that
             // of the dependency check) runs beside the dependency wait of the item before.  An item claimed early is still
             // published in order and only after everything it depends on, all of it with smaller indices, is complete.
+            // With `gate` the next item is asked for only once the accumulator of the last one is full.
             unsigned next_idx = atomicAdd(g.work_counter, 1u);
+            uint32_t acc_next = 0, acc_par = 0, last_acc = 0;      // the accumulators' use, as the MMA issuer keeps it
             while (ok) {
                 const uint32_t slot = published % RING, par = (published / RING) & 1u;
                 if (!(ok = mbar_wait<true>(bar_ring_empty + 8 * slot, par ^ 1u, abort_flag, status, 7, TRACE_PTR(w_slot)))) break;
+                if (FEW && g.gate && published > 0) {
+                    if (!(ok = mbar_wait(bar_acc_full + 8 * last_acc, ((acc_par >> last_acc) & 1u) ^ 1u, abort_flag, status, 14, TRACE_PTR(w_slot)))) break;
+                    next_idx = atomicAdd(g.work_counter, 1u);
+                }
                 const unsigned idx = next_idx;
-                if (idx < g.total_items) next_idx = atomicAdd(g.work_counter, 1u);
+                if (!(FEW && g.gate) && idx < g.total_items) next_idx = atomicAdd(g.work_counter, 1u);
                 Item it;
                 const bool found = decode(idx, it);
                 if (!found || !it.stop && !MONA_IN_BOUNDS(it.c >= 0 && it.c < g.C && it.q >= 0 && it.q < P && it.t >= 0 && (unsigned)it.t < phase_first[it.q + 1] - phase_first[it.q], status, 101)) {
@@ -746,6 +764,12 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 mbar_arrive_relaxed_cluster(ring_full_own + 8 * slot);
                 mbar_arrive_relaxed_cluster(ring_full_peer + 8 * slot);
                 ++published;
+                if (FEW && g.gate && !it.stop) {
+                    const int nsub = decode_tile<FEW>(g.ph[it.q], it.t).nsub;
+                    last_acc = nsub == 2 ? 1u : acc_next;
+                    acc_par ^= nsub == 2 ? 3u : 1u << acc_next;
+                    if (nsub == 1) acc_next ^= 1u;
+                }
                 TRACE_ONLY(trace_add(NS_TRACE_SCHED_SLOT, w_slot); trace_add(NS_TRACE_SCHED_DEPENDENCY, w_dep); w_slot = w_dep = 0;)
                 if (it.stop) break;
             }
@@ -795,7 +819,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             if (it.stop) break;
             TRACE_ONLY(const uint32_t t_item0 = trace_clock();)
             const NsPhase& p = g.ph[it.q];
-            const TileCoord tc = decode_tile(p, it.t);
+            const TileCoord tc = decode_tile<FEW>(p, it.t);
             const int m0 = tc.tm * TC_BM + (int)rank * CTA_M;
             const int gr = m0 + row_in_cta;
             const bool row_ok = gr < p.M;
@@ -815,9 +839,9 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 // conditional writes the array stayed live through the other epilogue path and every item spilled 61 registers
                 // per thread.  Measured, before -> after: one 256 x 512 matrix 150 -> 134 us per step, 12 dense blocks 3.80 ->
                 // 3.65 ms, three layers of 768 x 2048 experts 21.3 -> 20.4 ms.
-                auto pack_and_stage = [&](auto nsub_c) -> bool {
-                    constexpr int NSUB = decltype(nsub_c)::value;
-                    uint4 pk[NSUB][2][8];
+                auto pack_and_stage = [&](auto nsub_c, auto nph_c) -> bool {
+                    constexpr int NSUB = decltype(nsub_c)::value, NPH = decltype(nph_c)::value;
+                    uint4 pk[NSUB][NPH][8];
                     #pragma unroll
                     for (int u = 0; u < NSUB; ++u) {
                         const uint32_t acc = acc0 + u;
@@ -826,7 +850,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                         acc_par ^= 1u << acc;
                         const uint32_t t_base = tmem_base + lane_base + acc * TC_BN + half * 64;
                         #pragma unroll
-                        for (int ph = 0; ph < 2; ++ph) {
+                        for (int ph = 0; ph < NPH; ++ph) {
                             #pragma unroll
                             for (int h = 0; h < 2; ++h) {
                                 float v[32];
@@ -835,7 +859,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                                 #pragma unroll
                                 for (int j = 0; j < 32; ++j) v[j] *= c2;
                                 if (NSUB == 1 && p.delta_out) {
-                                    const int dj = gr - ((tc.tn + u) * TC_BN + ph * EPI_COLS + half * 64 + 32 * h);
+                                    const int dj = gr - ((tc.tn + u) * (EPI_COLS * NPH) + ph * EPI_COLS + half * 64 + 32 * h);
                                     if (row_ok && dj >= 0 && dj < 32) {       // this row's diagonal element is among the 32
                                         float d = 0.f;
                                         #pragma unroll
@@ -854,16 +878,19 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                     #pragma unroll
                     for (int u = 0; u < NSUB; ++u)
                         #pragma unroll
-                        for (int ph = 0; ph < 2; ++ph)
-                            if ((tc.tn + u) * TC_BN + ph * EPI_COLS < p.N && !put_phase(pk[u][ph])) return false;
+                        for (int ph = 0; ph < NPH; ++ph)
+                            if ((tc.tn + u) * (EPI_COLS * NPH) + ph * EPI_COLS < p.N && !put_phase(pk[u][ph])) return false;
                     return true;
                 };
-                alive = tc.nsub == 2 ? pack_and_stage(std::integral_constant<int, 2>{}) : pack_and_stage(std::integral_constant<int, 1>{});
+                using std::integral_constant;
+                if (tc.nsub == 2) alive = pack_and_stage(integral_constant<int, 2>{}, integral_constant<int, 2>{});
+                else if (!(FEW && p.narrow)) alive = pack_and_stage(integral_constant<int, 1>{}, integral_constant<int, 2>{});
+                else alive = pack_and_stage(integral_constant<int, 1>{}, integral_constant<int, FEW ? 1 : 2>{});
             } else
             for (int u = 0; u < tc.nsub && alive; ++u) {
                 const uint32_t acc = acc0 + u;
-                const int n0 = (tc.tn + u) * TC_BN;
-                const int nphases = (p.N - n0 > EPI_COLS) ? 2 : 1;
+                const int n0 = (tc.tn + u) * (FEW ? ns_tile_cols(p) : TC_BN);
+                const int nphases = (p.N - n0 > EPI_COLS && !(FEW && p.narrow)) ? 2 : 1;
                 // Operand of the axpy term: this thread's 64 values of a phase (128 bytes), requested before the accumulator is
                 // ready (first phase) or before the previous phase is staged (second), so that the round trip is hidden.  It was written by other CTAs of this
                 // launch, so it is read from L2 (.cg), never from a line L1 may still hold from an earlier iteration.  A thread
@@ -952,7 +979,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
 #ifdef MONA_TRACE
             if (lane == 0) {      // one lane per warp: the table holds sums over the eight epilogue warps
                 trace_add(NS_TRACE_EPI_RING, w_ring); trace_add(NS_TRACE_EPI_ACC_FULL, w_accf); trace_add(NS_TRACE_EPI_STAGE_EMPTY, w_stge);
-                const bool diag = p.ab_same && tc.tm == tc.tn && tc.nsub == 1;
+                const bool diag = p.ab_same && !(FEW && p.narrow) && tc.tm == tc.tn && tc.nsub == 1;
                 const int kind = !p.symmetric ? (tc.nsub == 2 ? 4 : 5) : ((p.small_sym ? 2 : 0) + (diag ? 1 : 0));
                 const int slot = NS_TRACE_EPI_TILE0 + 4 * kind;
                 trace_add(slot, trace_clock() - t_item0); trace_add(slot + 1, 1u); trace_add(slot + 2, w_accf); trace_add(slot + 3, w_stge);
@@ -1014,18 +1041,33 @@ int ns_work_order(int C, int P, int delay, const unsigned int* items_per_phase, 
     return (int)n;
 }
 
+// Tiles of the lower block triangle.  The last narrow tile is left out when its columns are all beyond N: every item must have
+// something to stage.
+static int lower_tiles(const NsPhase& p) {
+    const int blocks = p.tiles_m * (p.tiles_m + 1) / 2;
+    return p.narrow ? 2 * blocks - (2 * p.tiles_m - p.tiles_n) : blocks;
+}
+
 void ns_phase_plan(NsPhase& p) {
     p.tiles_m = (p.M + TC_BM - 1) / TC_BM;
-    p.tiles_n = (p.N + TC_BN - 1) / TC_BN;
-    if (p.symmetric || p.tiles_n < 2) p.wide = 0;      // a macro-tile needs two tile columns to pay
+    p.tiles_n = (p.N + ns_tile_cols(p) - 1) / ns_tile_cols(p);
+    if (p.symmetric || p.narrow || p.tiles_n < 2) p.wide = 0;      // a macro-tile needs two tile columns to pay
     if (p.wide) p.items_per_mat = p.tiles_m * ((p.tiles_n + 1) / 2);
-    else p.items_per_mat = p.symmetric ? p.tiles_m * (p.tiles_m + 1) / 2 : p.tiles_m * p.tiles_n;
+    else p.items_per_mat = p.symmetric ? lower_tiles(p) : p.tiles_m * p.tiles_n;
 }
 
 double ns_phase_executed_flops(const NsPhase& p) {
     const double kpad = (double)((p.K + TC_BK - 1) / TC_BK * TC_BK);
-    const double tiles256 = p.symmetric ? p.tiles_m * (p.tiles_m + 1) / 2 : p.tiles_m * p.tiles_n;
-    return 2.0 * TC_BM * TC_BN * kpad * tiles256;
+    const double tiles = p.symmetric ? lower_tiles(p) : p.tiles_m * p.tiles_n;
+    return 2.0 * TC_BM * ns_tile_cols(p) * kpad * tiles;
+}
+
+// Figures: a k-slice takes the tensor pipe 512 cycles per 256 x 256 x 64; a narrow tile's is bound by its copies (24 KiB per CTA), not
+// its 256.  The constant is what an item adds on a pair with nothing else to do - first copies, epilogue, stores, completion count,
+// the next claim - from the wait breakdown (an epilogue of 4400 cycles per plain tile, half of it per 128 columns).
+double ns_phase_cycles(const NsPhase& p, double rounds) {
+    const double ks = (p.K + TC_BK - 1) / TC_BK;
+    return rounds * (p.wide ? 1024.0 * ks + 9000.0 : p.narrow ? 340.0 * ks + 4500.0 : 512.0 * ks + 6500.0);
 }
 
 void ns_program_plan(NsProgram& g) {
@@ -1039,8 +1081,9 @@ cudaError_t ns_configure(int* max_pairs) {
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<MAXC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<MAXC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sms / 2 * 2));
     cfg.blockDim = dim3(TC_THREADS);
@@ -1051,7 +1094,7 @@ cudaError_t ns_configure(int* max_pairs) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int clusters = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(&clusters, ns_chunk_kernel<1>, &cfg)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveClusters(&clusters, ns_chunk_kernel<1, false>, &cfg)) != cudaSuccess) return e;
     if (clusters < 1) return cudaErrorInvalidConfiguration;
     *max_pairs = clusters < sms / 2 ? clusters : sms / 2;
     return cudaSuccess;
@@ -1060,13 +1103,16 @@ cudaError_t ns_configure(int* max_pairs) {
 cudaError_t launch_ns_program(const NsMaps& maps, const NsProgram& g, const NsUpdatePtrs& up, int max_pairs,
                               DeviceStatus* status, cudaStream_t stream) {
     if (g.total_items == 0) return cudaSuccess;
+    if (g.max_pairs > 0 && g.max_pairs < max_pairs) max_pairs = g.max_pairs;
     const int pairs = (long long)g.total_items < (long long)max_pairs ? (int)g.total_items : max_pairs;
     if (up.w) {
         UpdateTable<MAXC> table;
         for (int c = 0; c < g.C; ++c) { table.w[c] = up.w[c]; table.o[c] = up.o ? up.o[c] : nullptr; }
-        ns_chunk_kernel<MAXC><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, table, status);
+        ns_chunk_kernel<MAXC, false><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, table, status);
+    } else if (g.few) {
+        ns_chunk_kernel<1, true><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
     } else {
-        ns_chunk_kernel<1><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
+        ns_chunk_kernel<1, false><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
     }
     return cudaGetLastError();
 }

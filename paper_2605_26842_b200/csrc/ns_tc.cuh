@@ -41,6 +41,7 @@ struct NsPhase {
                                 //    tile stages its operand rows once and uses them on both sides
     int wide;                   // 1 (non-symmetric D only): a work item is a 256 x 512 macro-tile, two tiles that share
                                 //    one staged slice of the A operand, one per tensor-memory accumulator
+    int narrow;                 // 1: tiles of 128 instead of 256 columns (not with `wide`)
     int tiles_m, tiles_n, items_per_mat;   // filled by ns_phase_plan(); items are macro-tiles when `wide`
     const __nv_bfloat16* cin;   // may be null; [C][M][N] like D; lower-block-stored when D is symmetric
     long long ld, mat_stride;   // leading dimension and per-matrix stride of cin (and of the fp32 parameter when
@@ -71,6 +72,11 @@ struct NsProgram {
     unsigned int* work_counter; // zero at launch
     unsigned int* done;         // C * P words, zero at launch
     float eta_lambda, eta_gamma;    // fuse_update: eta * lambda and eta * gamma
+    int few;                    // 1: the launch runs the kernel instance that knows narrow phases and the gate (not with fuse_update)
+    int gate;                   // 1: a pair takes its next item only when the MMAs of the last one are complete.  0: a few items
+                                //    ahead.  For launches of about one round of items per phase, where pairs that come first
+                                //    would hoard items that others are idle for
+    int max_pairs;              // CTA pairs the launch may use (0: all that the device holds)
     int selftest_extra_tx;      // 0 in normal use.  The time-out self-test sets it: every stage then expects this many
                                 //    bytes more than its copies deliver, so the "full" wait runs out and the kernel must
                                 //    report STATUS_TIMEOUT and leave cleanly (all copies still complete; nothing faults)
@@ -151,9 +157,13 @@ struct NsUpdatePtrs {
     float* const* o;            // entries may be null; the array itself may be null
 };
 
-// Fills the tile counts of `p` from M, N, symmetric, wide.
+// Columns of D per tile.
+__host__ __device__ inline int ns_tile_cols(const NsPhase& p) { return p.narrow ? TC_BN / 2 : TC_BN; }
+// Fills the tile counts of `p` from M, N, symmetric, wide, narrow.
 void ns_phase_plan(NsPhase& p);
-// Tensor-core flops one matrix costs in phase `p`: executed (2*M*N*K per issued 256 x 256 tile MMA, padded
+// Estimated SM cycles of `rounds` items of a phase one after the other on a pair (see the definition for where the figures come from).
+double ns_phase_cycles(const NsPhase& p, double rounds);
+// Tensor-core flops one matrix costs in phase `p`: executed (2*M*N*K per issued tile MMA, padded
 // extents and the upper halves of diagonal tiles included).
 double ns_phase_executed_flops(const NsPhase& p);
 // Fills total_items from C, P, the phases' item counts.

@@ -1,0 +1,49 @@
+"""Newton-Schulz launches of few tiles per product: narrow (256 x 128) tiles, the claim gate, several buckets side by side on
+streams and SM pairs of their own.  Sizes around the edges of a narrow tile (a last tile of 8 to 128 columns, or none), one and many
+tile rows, both orientations; more buckets than there are slots; results must not depend on the overlap."""
+import pytest
+import torch
+
+import paper_2605_26842_b200 as pkg
+from tests.parity_util import TOL_O_BF16, TOL_O_MAX_BF16, TOL_STATE, TOL_W, run_case
+
+pytestmark = pytest.mark.gpu
+
+
+def check(errs):
+    assert errs["M"] <= TOL_STATE, errs
+    assert errs["O"] <= TOL_O_BF16 and errs["O_max"] <= TOL_O_MAX_BF16 and errs["dW"] <= TOL_W, errs
+
+
+@pytest.mark.parametrize("shape", [(1, 64, 64), (1, 120, 136), (1, 128, 512), (1, 136, 128), (1, 256, 264), (1, 264, 376), (1, 392, 384),
+                                   (2, 520, 648), (1, 1032, 1160), (30, 256, 256), (40, 128, 384)])
+def test_one_bucket(shape):
+    check(run_case([shape], steps=2, seed=51, sample={0: sorted({0, shape[0] - 1})}))
+
+
+def test_more_buckets_than_slots():
+    shapes = [(1, 256, 512), (1, 512, 256), (2, 384, 640), (1, 72, 200), (1, 1000, 136), (3, 192, 320), (1, 32, 512), (1, 33, 17)]
+    check(run_case(shapes, steps=3, seed=52))
+
+
+def test_small_buckets_beside_a_large_one_match_a_single_stream():
+    """Parameters and state agree bit for bit (a tile of any width accumulates over k in the same order), also in validation mode,
+    whose chunks are smaller than a bucket."""
+    dev = torch.device("cuda", 0)
+    gen = torch.Generator().manual_seed(53)
+    shapes = [(400, 256, 256), (2, 264, 520), (1, 520, 264), (2, 32, 256)]
+    W0 = [torch.randn(s, generator=gen) * 0.02 for s in shapes]
+    G = [[torch.randn(s, generator=gen) * 1e-3 for s in shapes] for _ in range(2)]
+    for precision in (0, 1):
+        def run(overlap):
+            p = [w.clone().to(dev) for w in W0]
+            opt = pkg.MonaOptimizer(p, options=pkg.default_options(chunk_overlap=overlap, chunk_budget_bytes=64 << 20))
+            hp = pkg.default_hparams(ns_precision=precision)
+            for k in range(2):
+                opt.step(hp, p, [g.to(dev) for g in G[k]])
+            assert opt.poll_status()[0] == 0
+            out = [t.clone() for t in p] + [opt.state.clone()]
+            opt.close()
+            return out
+        for x, y in zip(run(1), run(0)):
+            assert torch.equal(x, y)

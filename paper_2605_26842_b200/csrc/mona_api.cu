@@ -74,6 +74,7 @@ struct Bucket {
     int64_t rows = 0, cols = 0, s = 0, l = 0, e = 0;
     int grad_dtype = 0, state_dtype = 0;
     bool tall = false, tc_ok = false;
+    double chain_us = 0.0;      // rough time of a small bucket's step, for ordering and slots only
     bool small = false;         // its products do not fill the machine: runs beside other chunks (see bucket_is_small)
     bool paired = false;        // takes its first two iterations together on the s x s side (see ns_pair_pays)
     std::vector<MatRef> mats;
@@ -119,9 +120,8 @@ bool ns_first_two_together(const bool pair_pays, int T) { return pair_pays && T 
 // fp32 path that takes one block cluster per matrix is small too.
 constexpr size_t SMALL_BUCKET_BYTES = 400ull << 20;
 bool bucket_is_small(int64_t s, int64_t e, int64_t count, bool tc_ok, bool one_cluster) {
-    const int64_t ts = (s + TC_BM - 1) / TC_BM;
-    if (!tc_ok && !one_cluster) return false;
-    return (one_cluster || ts * (ts + 1) / 2 * count <= 4 * 74) && (size_t)(2 * e + 2 * s * s) * 2 * count <= SMALL_BUCKET_BYTES;
+    const int64_t tile = tc_ok ? TC_BM : 64, ts = (s + tile - 1) / tile;       // the fp32 GEMM: 64 x 64 tiles, one block per SM
+    return (one_cluster || ts * (ts + 1) / 2 * count <= 4 * (tc_ok ? 74 : 148)) && (size_t)(2 * e + 2 * s * s) * (tc_ok ? 2 : 4) * count <= SMALL_BUCKET_BYTES;
 }
 // NARROW_ROUNDS: a launch on a share of the pairs looks at other tile widths for phases of at most this many rounds of items (1 to 8
 // measured equal within 2 %).  GATE_ROUNDS: the claim gate (NsProgram::gate) pays while a phase leaves pairs idle (mixed small set 151 ->
@@ -131,13 +131,14 @@ constexpr double NARROW_ROUNDS = 4.0, GATE_ROUNDS = 1.5;
 struct Plan {
     std::vector<mona_matrix_desc> descs;
     std::vector<Bucket> buckets;
-    // Buckets in the order in which a step takes them: matrices small enough for one block cluster each first, so that their
-    // few-block launches run beside the first big prologue; last, they were the step's tail with the machine idle.
+    // Buckets in the order in which a step takes them: small ones first, so that they run beside the first big prologue and the
+    // large chunks (last, routers alone were a 400 us tail with the machine idle), the longest chain of them first.
     std::vector<int> order;
     std::vector<int> desc_bucket;          // bucket of descriptor i
     std::vector<int64_t> desc_pos;         // position of descriptor i's matrix 0 inside its bucket
     std::vector<int64_t> desc_first_gid;   // global matrix index (descriptor order) of matrix 0
     bool all_small = true;                 // no large bucket: small ones use all slots
+    int64_t n_small = 0;
     size_t state_bytes = 0, workspace_bytes = 0;
     size_t slot_off[NSLOTS] = {};          // bytes from the workspace base
 };
@@ -212,20 +213,24 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         b.off32_a = off32; off32 += align_up((size_t)b.Cf * b.s * b.s * 4, 1024);
         b.off32_b = off32; off32 += align_up((size_t)b.Cf * b.s * b.s * 4, 1024);
         b.data_bytes = std::max(off, off32);
-        b.small = bucket_is_small(b.s, b.e, count, b.tc_ok, !b.tc_ok && small_ns_eligible(b.rows, b.cols)) && cb == count;
+        b.small = bucket_is_small(b.s, b.e, count, b.tc_ok, !b.tc_ok && small_ns_eligible(b.rows, b.cols)) && (b.tc_ok ? b.Cb : b.Cf) == count;
         plan.all_small = plan.all_small && b.small;
+        {   // a five-step chain: about 100 us on the tensor cores, 25 in one block cluster, three products per iteration in fp32
+            const double ts = (double)((b.s + 63) / 64), tl = (double)((b.l + 63) / 64), waves = (double)count / 148.0;
+            const double product = std::max(1.0, ts * (ts + 1) / 2 * waves) * (double)(b.l + b.s) / 32 + std::max(1.0, ts * tl * waves) * (double)b.s / 32;
+            b.chain_us = b.tc_ok ? 100.0 : small_ns_eligible(b.rows, b.cols) ? 25.0 : 5.0 * (1.2 * product + 20.0);
+        }
         max_data[0] = std::max(max_data[0], b.data_bytes);
         if (b.small) max_data[1] = std::max(max_data[1], b.data_bytes);
     }
     // slots 2 and 3 exist when there are small buckets to fill them with
-    int64_t n_small = 0;
-    for (const Bucket& b : plan.buckets) n_small += b.small ? 1 : 0;
-    const int64_t extra = plan.all_small ? std::max<int64_t>(0, n_small - BIG_SLOTS) : n_small;
-    for (int small = 1; small >= 0; --small)
-        for (int i = 0; i < (int)plan.buckets.size(); ++i) {
-            const Bucket& b = plan.buckets[i];
-            if ((!b.tc_ok && small_ns_eligible(b.rows, b.cols)) == (small != 0)) plan.order.push_back(i);
-        }
+    for (const Bucket& b : plan.buckets) plan.n_small += b.small ? 1 : 0;
+    const int64_t extra = plan.all_small ? std::max<int64_t>(0, plan.n_small - BIG_SLOTS) : plan.n_small;
+    for (int i = 0; i < (int)plan.buckets.size(); ++i) plan.order.push_back(i);
+    std::stable_sort(plan.order.begin(), plan.order.end(), [&](int x, int y) {
+        const Bucket &a = plan.buckets[x], &b = plan.buckets[y];
+        return a.small != b.small ? a.small : a.small && a.chain_us > b.chain_us;
+    });
     plan.state_bytes = state_bytes;
     plan.workspace_bytes = WS_DATA_OFF;
     for (int sl = 0; sl < NSLOTS; ++sl) {
@@ -423,6 +428,7 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
     }
     MONA_CUDA(h, ns_configure(&h->max_pairs));
     MONA_CUDA(h, small_ns_configure());
+    MONA_CUDA(h, sgemm_configure());
     MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
     for (int sl = 1; sl < NSLOTS; ++sl) {
         MONA_CUDA(h, cudaStreamCreateWithFlags(&h->side[sl], cudaStreamNonBlocking));
@@ -568,7 +574,8 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
     bool slot_used[NSLOTS] = {true};
     for (int sl = 1; sl < NSLOTS; ++sl) slot_stream[sl] = overlap ? h->side[sl] : (cudaStream_t)stream_v;
     if (overlap) MONA_CUDA(h, cudaEventRecord(h->ev_fork, slot_stream[0]));
-    int64_t big_index = 0, small_index = 0;
+    int64_t big_index = 0;
+    double slot_load[NSLOTS] = {};
     // estimated tensor work of the buckets, by which chunks that run side by side share the SM pairs
     double work_total = 0.0;
     for (const Bucket& b : plan.buckets)
@@ -610,7 +617,12 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             int slot = 0;
             if (overlap) {
                 if (!small) slot = (int)(big_index++ % BIG_SLOTS);
-                else slot = plan.all_small ? (int)(small_index++ % NSLOTS) : BIG_SLOTS + (int)(small_index++ % (NSLOTS - BIG_SLOTS));
+                else {      // the slot with the least in it so far (slots past the second exist for as many small buckets as there are)
+                    const int lo = plan.all_small ? 0 : BIG_SLOTS, hi = (int)std::min<int64_t>(NSLOTS, lo + plan.n_small);
+                    slot = lo;
+                    for (int sl = lo; sl < hi; ++sl) if (slot_load[sl] < slot_load[slot]) slot = sl;
+                    slot_load[slot] += b.chain_us;
+                }
                 if (!slot_used[slot]) MONA_CUDA(h, cudaStreamWaitEvent(slot_stream[slot], h->ev_fork, 0));
                 slot_used[slot] = true;
             }
@@ -705,15 +717,15 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                         if (!b.tall) { g1.a_si = b.cols; g1.a_sk = 1; g1.b_sk = 1; g1.b_sj = b.cols; }
                         else         { g1.a_si = 1; g1.a_sk = b.cols; g1.b_sk = b.cols; g1.b_sj = 1; }
                         g1.cin = nullptr; g1.d = af; g1.ldd = b.s; g1.d_batch = b.s * b.s;
-                        g1.M = g1.N = (int)b.s; g1.K = (int)b.l; g1.batch = C; g1.c1 = 0.f; g1.c2 = 1.f;
+                        g1.M = g1.N = (int)b.s; g1.K = (int)b.l; g1.batch = C; g1.c1 = 0.f; g1.c2 = 1.f; g1.symmetric = 1;
                         MONA_CUDA(h, launch_sgemm(g1, stream));
-                        SgemmArgs g2{};   // B = b A + c A A
+                        SgemmArgs g2{};   // B' = b A + c A A + a I
                         g2.a = af; g2.b = af; g2.a_batch = g2.b_batch = b.s * b.s;
                         g2.a_si = b.s; g2.a_sk = 1; g2.b_sk = b.s; g2.b_sj = 1;
                         g2.cin = af; g2.d = bf; g2.ldd = b.s; g2.d_batch = b.s * b.s;
-                        g2.M = g2.N = g2.K = (int)b.s; g2.batch = C; g2.c1 = ns_b; g2.c2 = ns_c;
+                        g2.M = g2.N = g2.K = (int)b.s; g2.batch = C; g2.c1 = ns_b; g2.c2 = ns_c; g2.diag_add = ns_a; g2.symmetric = 1;
                         MONA_CUDA(h, launch_sgemm(g2, stream));
-                        SgemmArgs g3{};   // X' = a X + B X (wide) or a X + X B (tall)
+                        SgemmArgs g3{};   // X' = B' X (wide) or X B' (tall)
                         if (!b.tall) {
                             g3.a = bf; g3.a_si = b.s; g3.a_sk = 1; g3.a_batch = b.s * b.s;
                             g3.b = xf[cur]; g3.b_sk = b.cols; g3.b_sj = 1; g3.b_batch = b.e;
@@ -723,8 +735,8 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                             g3.b = bf; g3.b_sk = b.s; g3.b_sj = 1; g3.b_batch = b.s * b.s;
                             g3.M = (int)b.l; g3.N = (int)b.s;
                         }
-                        g3.K = (int)b.s; g3.cin = xf[cur]; g3.d = xf[nxt]; g3.ldd = b.cols; g3.d_batch = b.e;
-                        g3.batch = C; g3.c1 = ns_a; g3.c2 = 1.f;
+                        g3.K = (int)b.s; g3.cin = nullptr; g3.d = xf[nxt]; g3.ldd = b.cols; g3.d_batch = b.e;
+                        g3.batch = C; g3.c1 = 0.f; g3.c2 = 1.f;
                         MONA_CUDA(h, launch_sgemm(g3, stream));
                         h->launches += 3;
                         h->flops_dense += (double)C * (4.0 * b.s * b.s * b.l + 2.0 * (double)b.s * b.s * b.s);

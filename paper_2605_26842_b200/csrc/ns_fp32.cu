@@ -1,6 +1,6 @@
 // fp32 validation path of Eq. newton_schulz: a plain shared-memory tiled SGEMM with generic operand
 // strides, so that X X^T, X^T X, A A and B X / X B all go through the same kernel without any
-// transposed copy.  Accumulation is sequential fp32 FMA; this path exists to separate algorithmic
+// transposed copy.  Products and sums are fp32 FMA throughout; this path exists to separate algorithmic
 // errors from bf16 rounding, and to serve shapes the tensor-core path does not take.
 #include "ns_fp32.cuh"
 
@@ -8,66 +8,171 @@ namespace mona {
 
 namespace {
 
-constexpr int TS = 64;   // tile of D per block
-constexpr int TK = 16;   // k-slice
-// 256 threads, each owns a 4x4 patch of the 64x64 tile.
-__global__ void __launch_bounds__(256) sgemm_kernel(SgemmArgs g) {
-    __shared__ float As[TK][TS + 4];
-    __shared__ float Bs[TK][TS + 4];
+// A block computes a 64 x 64 tile of D with four groups of 64 threads.  Each group takes a quarter of every k-slab (16 of 64) and
+// each thread 8 x 8 elements of the whole tile, so that 64 FMAs cost four 16-byte shared-memory reads (4 x 4 per thread cost
+// eight 4-byte reads per 16); the groups' sums are added through shared memory at the end, in group order.  The k split, not
+// a larger tile, fills the block: these matrices have few tiles (1001 x 1001: 136 of 64 x 64 in the lower triangle, 36 of
+// 128 x 128), so the tile stays small and eight warps share it.  Slabs are fetched with 4-byte asynchronous copies - odd row
+// lengths leave no wider alignment - two slabs ahead of the arithmetic.
+// Bound: fp32 FMA issue while there is a tile for every SM, the chain of dependent products below that.  Symmetric products
+// compute the tiles on and below the diagonal and write each twice.
+// Measured (T = 5 products of one 1001 x 1500 matrix, X X^T / A A / B' X): 154 / 100 / 122 us with the 4 x 4 kernel and both halves
+// of the symmetric products, 83 / 59 / 158 with these tiles, 54 / 38 / 101 with packed FMAs, unchecked copies of interior slabs
+// and no register cap (an SM holds one block then, but a capped one spilled), slabs of 64 instead of 32 another 7 %; five odd
+// matrices, 1001 x 1500 the largest: 2.91 -> 1.21 ms per step.
+constexpr int TS = 64;                   // tile of D per block
+constexpr int TK = 64;                   // k-slab
+constexpr int SG_GROUPS = 4;             // thread groups, TK / SG_GROUPS k each
+constexpr int SG_THREADS = 64 * SG_GROUPS;
+constexpr int PITCH = TS + 4;            // 4 mod 32: see copy_slab
+constexpr int SLAB = TK * PITCH;         // floats of one operand's slab
+constexpr int SG_STAGES = 3;             // slabs in flight or in use
+constexpr size_t SG_SMEM = sizeof(float) * (2 * SG_STAGES * SLAB > SG_GROUPS * TS * PITCH ? 2 * SG_STAGES * SLAB : SG_GROUPS * TS * PITCH);
+
+__device__ __forceinline__ void cp_async4(uint32_t d, const float* src, bool valid) {
+    const int bytes = valid ? 4 : 0;                       // 0: the word is zero-filled and nothing is read
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+// One thread's share of fetching an operand: slab n becomes dst[k][r] (pitch PITCH) = src(r0 + r, n TK + k) for r < 64, k < TK, zero
+// outside rows x K, src(r, k) = src[r * s_r + k * s_k].  When k is contiguous, a warp's lanes cover 8 k of 4 rows: whole 32-byte
+// sectors, and with PITCH = 4 mod 32 the 32 words fall into different banks; otherwise they cover 32 consecutive rows.  Either way a
+// thread's elements differ in one coordinate only, so that each costs an addition and a comparison.
+struct SlabCopy {
+    static constexpr int ROWS = 4 * (SG_THREADS / 32) / (TK / 8);    // rows all warps cover at once when k is contiguous
+    const float* src;           // this thread's first element of slab 0
+    long long step, slab_step;  // in elements: to its next element, to the next slab
+    int first, limit, stride;   // row of its first element, bound, change per element
+    int k, k_stride;            // k of its first element in slab 0, change per element
+    int dst, dst_step;          // position in the slab, change per element
+    __device__ __forceinline__ SlabCopy(const float* base, long long s_r, long long s_k, int r0, int rows) {
+        const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+        const bool k_fast = s_k == 1;
+        constexpr int KW = TK / 8;       // warps side by side along k when k is contiguous
+        const int r = k_fast ? (warp / KW) * 4 + (lane >> 3) : (warp & 1) * 32 + lane;
+        k = k_fast ? (warp % KW) * 8 + (lane & 7) : warp >> 1;
+        src = base + (long long)(r0 + r) * s_r + (long long)k * s_k;
+        step = k_fast ? ROWS * s_r : 4 * s_k;
+        slab_step = (long long)TK * s_k;
+        dst = k * PITCH + r;
+        dst_step = k_fast ? ROWS : 4 * PITCH;
+        first = r0 + r; limit = rows; stride = k_fast ? ROWS : 0;
+        k_stride = k_fast ? 0 : 4;
+    }
+    // `inside`: the whole slab lies inside rows x K (the same for all threads of the block)
+    __device__ __forceinline__ void fetch(float* buf, const float* safe, int n, int K, bool inside) const {
+        const float* p = src + (long long)n * slab_step;
+        const uint32_t d = (uint32_t)__cvta_generic_to_shared(buf + dst);
+        if (inside) {
+            #pragma unroll
+            for (int q = 0; q < TS * TK / SG_THREADS; ++q) {
+                asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(d + (uint32_t)(q * dst_step * 4)), "l"(p) : "memory");
+                p += step;
+            }
+            return;
+        }
+        int r = first, kk = n * TK + k;
+        #pragma unroll
+        for (int q = 0; q < TS * TK / SG_THREADS; ++q) {
+            const bool valid = r < limit && kk < K;
+            cp_async4(d + (uint32_t)(q * dst_step * 4), valid ? p : safe, valid);
+            p += step; r += stride; kk += k_stride;
+        }
+    }
+};
+
+// Two independent fp32 FMAs (round to nearest) in one instruction: half the issue slots of the scalar form.
+__device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a, unsigned long long b) {
+    asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+
+__global__ void __launch_bounds__(SG_THREADS, 1) sgemm_kernel(const __grid_constant__ SgemmArgs g) {
+    extern __shared__ __align__(16) float sg[];
     const int z = blockIdx.z;
     const float* __restrict__ A = g.a + (long long)z * g.a_batch;
     const float* __restrict__ B = g.b + (long long)z * g.b_batch;
-    const int i0 = blockIdx.y * TS, j0 = blockIdx.x * TS;
-    const int tx = threadIdx.x & 15, ty = threadIdx.x >> 4;
-    float acc[4][4];
-    #pragma unroll
-    for (int r = 0; r < 4; ++r)
-        #pragma unroll
-        for (int c = 0; c < 4; ++c) acc[r][c] = 0.f;
-
-    for (int k0 = 0; k0 < g.K; k0 += TK) {
-        // each thread brings 4 elements of each operand slice
-        #pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            int idx = threadIdx.x + q * 256;          // 0..1023 = TK*TS
-            int kk, mm;
-            if (g.a_sk == 1) { kk = idx % TK; mm = idx / TK; } else { mm = idx % TS; kk = idx / TS; }
-            int gi = i0 + mm, gk = k0 + kk;
-            As[kk][mm] = (gi < g.M && gk < g.K) ? A[(long long)gi * g.a_si + (long long)gk * g.a_sk] : 0.f;
-            int kb, nn;
-            if (g.b_sk == 1) { kb = idx % TK; nn = idx / TK; } else { nn = idx % TS; kb = idx / TS; }
-            int gj = j0 + nn, gk2 = k0 + kb;
-            Bs[kb][nn] = (gj < g.N && gk2 < g.K) ? B[(long long)gk2 * g.b_sk + (long long)gj * g.b_sj] : 0.f;
-        }
-        __syncthreads();
-        #pragma unroll
-        for (int kk = 0; kk < TK; ++kk) {
-            float a[4], b[4];
-            #pragma unroll
-            for (int r = 0; r < 4; ++r) a[r] = As[kk][ty * 4 + r];
-            #pragma unroll
-            for (int c = 0; c < 4; ++c) b[c] = Bs[kk][tx * 4 + c];
-            #pragma unroll
-            for (int r = 0; r < 4; ++r)
-                #pragma unroll
-                for (int c = 0; c < 4; ++c) acc[r][c] = fmaf(a[r], b[c], acc[r][c]);
-        }
-        __syncthreads();
+    int ti = blockIdx.y, tj = blockIdx.x;
+    if (g.symmetric) {                                     // lower triangle, row by row
+        ti = 0;
+        while ((ti + 1) * (ti + 2) / 2 <= (int)blockIdx.x) ++ti;
+        tj = blockIdx.x - ti * (ti + 1) / 2;
     }
+    const int i0 = ti * TS, j0 = tj * TS;
+    const int group = threadIdx.x >> 6, tx = threadIdx.x & 7, ty = (threadIdx.x >> 3) & 7;
+    const int slabs = (g.K + TK - 1) / TK;
+    const SlabCopy copy_a(A, g.a_si, g.a_sk, i0, g.M), copy_b(B, g.b_sj, g.b_sk, j0, g.N);
+    auto fetch = [&](int n, int stage) {
+        float* buf = sg + stage * 2 * SLAB;
+        const bool k_inside = (n + 1) * TK <= g.K;
+        if (n < slabs) { copy_a.fetch(buf, A, n, g.K, k_inside && i0 + TS <= g.M); copy_b.fetch(buf + SLAB, B, n, g.K, k_inside && j0 + TS <= g.N); }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    unsigned long long acc[8][4];                          // 8 x 8 sums, two neighbouring columns per register pair
+    #pragma unroll
+    for (int r = 0; r < 8; ++r)
+        #pragma unroll
+        for (int c = 0; c < 4; ++c) acc[r][c] = 0ull;
+    #pragma unroll
+    for (int n = 0; n < SG_STAGES - 1; ++n) fetch(n, n);
+    int stage = 0;
+    for (int n = 0; n < slabs; ++n) {
+        asm volatile("cp.async.wait_group %0;" ::"n"(SG_STAGES - 2) : "memory");
+        __syncthreads();                                   // the slab is here, and everyone is done with the one before it
+        fetch(n + SG_STAGES - 1, stage == 0 ? SG_STAGES - 1 : stage - 1);
+        const float* as = sg + stage * 2 * SLAB + group * (TK / SG_GROUPS) * PITCH;
+        const float* bs = as + SLAB;
+        #pragma unroll
+        for (int kk = 0; kk < TK / SG_GROUPS; ++kk) {
+            float a[8];
+            ulonglong2 b[2];
+            *reinterpret_cast<float4*>(a) = *reinterpret_cast<const float4*>(as + kk * PITCH + 4 * ty);
+            *reinterpret_cast<float4*>(a + 4) = *reinterpret_cast<const float4*>(as + kk * PITCH + 32 + 4 * ty);
+            b[0] = *reinterpret_cast<const ulonglong2*>(bs + kk * PITCH + 4 * tx);
+            b[1] = *reinterpret_cast<const ulonglong2*>(bs + kk * PITCH + 32 + 4 * tx);
+            #pragma unroll
+            for (int r = 0; r < 8; ++r) {
+                unsigned long long aa;
+                asm("mov.b64 %0, {%1, %1};" : "=l"(aa) : "f"(a[r]));
+                fma2(acc[r][0], aa, b[0].x); fma2(acc[r][1], aa, b[0].y);
+                fma2(acc[r][2], aa, b[1].x); fma2(acc[r][3], aa, b[1].y);
+            }
+        }
+        stage = stage + 1 == SG_STAGES ? 0 : stage + 1;
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();                                       // the slabs' memory becomes the groups' partial tiles
+    float* part = sg + group * TS * PITCH;
+    #pragma unroll
+    for (int r = 0; r < 8; ++r) {
+        const int row = (r >> 2) * 32 + 4 * ty + (r & 3);
+        #pragma unroll
+        for (int h = 0; h < 2; ++h)
+            *reinterpret_cast<ulonglong2*>(part + row * PITCH + 32 * h + 4 * tx) = make_ulonglong2(acc[r][2 * h], acc[r][2 * h + 1]);
+    }
+    __syncthreads();
     float* __restrict__ D = g.d + (long long)z * g.d_batch;
     const float* __restrict__ Cin = g.cin ? g.cin + (long long)z * g.d_batch : nullptr;
-    #pragma unroll
-    for (int r = 0; r < 4; ++r) {
-        int gi = i0 + ty * 4 + r;
-        if (gi >= g.M) continue;
+    const bool mirror = g.symmetric && ti != tj;
+    #pragma unroll 4
+    for (int idx = threadIdx.x; idx < TS * TS; idx += SG_THREADS) {
+        const int r = idx >> 6, c = idx & 63, gi = i0 + r, gj = j0 + c;
+        float v = sg[r * PITCH + c];
         #pragma unroll
-        for (int c = 0; c < 4; ++c) {
-            int gj = j0 + tx * 4 + c;
-            if (gj >= g.N) continue;
-            long long off = (long long)gi * g.ldd + gj;
-            float v = g.c2 * acc[r][c];
+        for (int q = 1; q < SG_GROUPS; ++q) v += sg[q * TS * PITCH + r * PITCH + c];
+        v *= g.c2;
+        if (gi < g.M && gj < g.N) {
+            const long long off = (long long)gi * g.ldd + gj;
             if (Cin) v = fmaf(g.c1, Cin[off], v);
+            if (gi == gj) v += g.diag_add;
             D[off] = v;
+        }
+        if (mirror) sg[r * PITCH + c] = v;                 // (each thread rewrites only words it alone has read)
+    }
+    if (mirror) {
+        __syncthreads();
+        #pragma unroll 4
+        for (int idx = threadIdx.x; idx < TS * TS; idx += SG_THREADS) {
+            const int c = idx >> 6, r = idx & 63, gi = i0 + r, gj = j0 + c;
+            if (gi < g.M && gj < g.N) D[(long long)gj * g.ldd + gi] = sg[r * PITCH + c];
         }
     }
 }
@@ -301,9 +406,12 @@ cudaError_t launch_small_ns(const float* M, float* O, const float* inv_norm, int
                    : cudaLaunchKernelEx(&cfg, small_ns_kernel<64>, M, O, inv_norm, rows, cols, T, a, b, c);
 }
 
+cudaError_t sgemm_configure() { return cudaFuncSetAttribute(sgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SG_SMEM); }
+
 cudaError_t launch_sgemm(const SgemmArgs& g, cudaStream_t stream) {
-    dim3 grid((g.N + TS - 1) / TS, (g.M + TS - 1) / TS, g.batch);
-    sgemm_kernel<<<grid, 256, 0, stream>>>(g);
+    const int tm = (g.M + TS - 1) / TS, tn = (g.N + TS - 1) / TS;
+    dim3 grid(g.symmetric ? tm * (tm + 1) / 2 : tn, g.symmetric ? 1 : tm, g.batch);
+    sgemm_kernel<<<grid, SG_THREADS, SG_SMEM, stream>>>(g);
     return cudaGetLastError();
 }
 

@@ -4,7 +4,7 @@
 
 namespace mona {
 
-// Batched D = c1 * Cin + c2 * (A x B) with generic strides, plain fp32 FMA (no tensor cores, no TF32):
+// Batched D = c1 * Cin + c2 * (A x B) + diag_add * I with generic strides, plain fp32 FMA (no tensor cores, no TF32):
 //   A(i,k) = a[i*a_si + k*a_sk], B(k,j) = b[k*b_sk + j*b_sj], D(i,j) = d[i*ldd + j], Cin(i,j) = cin[i*ldd + j].
 // Matrix z of the batch is offset by z*a_batch / z*b_batch / z*d_batch elements.  cin may be null.
 struct SgemmArgs {
@@ -13,7 +13,10 @@ struct SgemmArgs {
     const float* cin; float* d; long long ldd, d_batch;
     int M, N, K, batch;
     float c1, c2;
+    float diag_add;
+    int symmetric;      // D = D^T (and M = N): computed on and below the diagonal 64 x 64 tiles, written on both sides
 };
+cudaError_t sgemm_configure();      // once per device, before the first launch
 cudaError_t launch_sgemm(const SgemmArgs& g, cudaStream_t stream);
 
 // Whole Newton-Schulz iteration (Eq. newton_schulz, T steps, fp32 FMA) of `batch` small matrices, one cluster of blocks per

@@ -75,6 +75,7 @@ struct Bucket {
     int grad_dtype = 0, state_dtype = 0;
     bool tall = false, tc_ok = false;
     double chain_us = 0.0;      // rough time of a small bucket's step, for ordering and slots only
+    int slot = 0;               // of a small bucket: where it always runs (large ones alternate between slots 0 and 1)
     bool small = false;         // its products do not fill the machine: runs beside other chunks (see bucket_is_small)
     bool paired = false;        // takes its first two iterations together on the s x s side (see ns_pair_pays)
     std::vector<MatRef> mats;
@@ -138,7 +139,7 @@ struct Plan {
     std::vector<int64_t> desc_pos;         // position of descriptor i's matrix 0 inside its bucket
     std::vector<int64_t> desc_first_gid;   // global matrix index (descriptor order) of matrix 0
     bool all_small = true;                 // no large bucket: small ones use all slots
-    int64_t n_small = 0;
+    int n_slots = 1;                       // slots that hold something
     size_t state_bytes = 0, workspace_bytes = 0;
     size_t slot_off[NSLOTS] = {};          // bytes from the workspace base
 };
@@ -180,7 +181,6 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         gid += d.batch;
     }
     size_t state_bytes = 0;
-    size_t max_data[2] = {0, 0};        // of all buckets, of the small ones
     for (Bucket& b : plan.buckets) {
         const int64_t count = (int64_t)b.mats.size();
         const size_t aux = b.state_dtype == MONA_BF16 ? 2 : 4;              // every block starts 256-byte aligned
@@ -194,8 +194,8 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         cb = std::max<int64_t>(1, std::min<int64_t>(std::min<int64_t>(cb, MAXC), count));
         b.Cb = (int)cb;
         // fp32 iterates take twice the bytes.  A bucket that has no other path gets whole chunks; in validation mode one that
-        // also has the bf16 path must not make the workspace larger than that path needs.
-        const int64_t cf = b.tc_ok ? cb / 2 : std::min<int64_t>(cb, (int64_t)(chunk_budget / (2 * per_mat_bf16)));
+        // also has the bf16 path must not make a large workspace larger than that path needs.
+        const int64_t cf = b.tc_ok && per_mat_bf16 * cb > (32u << 20) ? cb / 2 : std::min<int64_t>(cb, (int64_t)(chunk_budget / (2 * per_mat_bf16)));
         b.Cf = (int)std::max<int64_t>(1, cf);
         long long slab = 0;
         slab_plan(b.e, cb, PROLOGUE_UNIT, &slab, &b.slabs);
@@ -220,22 +220,33 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
             const double product = std::max(1.0, ts * (ts + 1) / 2 * waves) * (double)(b.l + b.s) / 32 + std::max(1.0, ts * tl * waves) * (double)b.s / 32;
             b.chain_us = b.tc_ok ? 100.0 : small_ns_eligible(b.rows, b.cols) ? 25.0 : 5.0 * (1.2 * product + 20.0);
         }
-        max_data[0] = std::max(max_data[0], b.data_bytes);
-        if (b.small) max_data[1] = std::max(max_data[1], b.data_bytes);
     }
-    // slots 2 and 3 exist when there are small buckets to fill them with
-    for (const Bucket& b : plan.buckets) plan.n_small += b.small ? 1 : 0;
-    const int64_t extra = plan.all_small ? std::max<int64_t>(0, plan.n_small - BIG_SLOTS) : plan.n_small;
     for (int i = 0; i < (int)plan.buckets.size(); ++i) plan.order.push_back(i);
     std::stable_sort(plan.order.begin(), plan.order.end(), [&](int x, int y) {
         const Bucket &a = plan.buckets[x], &b = plan.buckets[y];
         return a.small != b.small ? a.small : a.small && a.chain_us > b.chain_us;
     });
     plan.state_bytes = state_bytes;
+    // Every small bucket gets the slot with the least in it so far, and a slot is as large as the largest bucket it ever holds.
+    size_t slot_bytes[NSLOTS] = {};
+    double slot_load[NSLOTS] = {};
+    const int first_small = plan.all_small ? 0 : BIG_SLOTS;
+    for (int i : plan.order) {
+        Bucket& b = plan.buckets[i];
+        if (!b.small) {
+            for (int sl = 0; sl < BIG_SLOTS; ++sl) slot_bytes[sl] = std::max(slot_bytes[sl], b.data_bytes);
+            continue;
+        }
+        b.slot = first_small;
+        for (int sl = first_small; sl < NSLOTS; ++sl) if (slot_load[sl] < slot_load[b.slot]) b.slot = sl;
+        slot_load[b.slot] += b.chain_us;
+        slot_bytes[b.slot] = std::max(slot_bytes[b.slot], b.data_bytes);
+    }
     plan.workspace_bytes = WS_DATA_OFF;
     for (int sl = 0; sl < NSLOTS; ++sl) {
         plan.slot_off[sl] = plan.workspace_bytes;
-        plan.workspace_bytes += align_up(sl < BIG_SLOTS ? max_data[0] : sl - BIG_SLOTS < extra ? max_data[1] : 0, 1024);
+        plan.workspace_bytes += align_up(slot_bytes[sl], 1024);
+        if (slot_bytes[sl]) plan.n_slots = sl + 1;
     }
     return MONA_OK;
 }
@@ -273,11 +284,11 @@ struct mona_handle {
     uint8_t* ws = nullptr;
     cudaStream_t side[NSLOTS] = {};        // stream of slot 1 .. NSLOTS - 1 (slot 0 uses the caller's)
     cudaEvent_t ev_fork = nullptr, ev_join[NSLOTS] = {};
-    // host-to-host pipeline of mona_step_host(): copy streams and per-descriptor events, created on first use
+    // host-to-host pipeline of mona_step_host(): copy streams and per-chunk events, created on first use
     cudaStream_t h2d = nullptr, d2h = nullptr;
     cudaEvent_t ev_hfork = nullptr, ev_hjoin = nullptr;
-    std::vector<cudaEvent_t> ev_in;     // gradient of descriptor i has arrived on the device
-    std::vector<cudaEvent_t> ev_out;    // NSLOTS per descriptor: its chunks on that slot's stream have been updated
+    std::vector<cudaEvent_t> ev_in;     // the gradients of chunk i have arrived on the device
+    std::vector<cudaEvent_t> ev_out;    // chunk i has been updated
     DeviceStatus* host_status = nullptr;   // pinned
     std::string last_error;
     int64_t launches = 0;
@@ -412,7 +423,7 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
         if (!b.tc_ok) continue;
         bool ok = true;
         for (int sl = 0; sl < NSLOTS; ++sl) {
-            if (sl >= BIG_SLOTS && !b.small) continue;
+            if (b.small ? sl != b.slot : sl >= BIG_SLOTS) continue;
             uint8_t* data = h->ws + h->plan.slot_off[sl];
             for (int big = 0; big < 2; ++big) {     // 64-row boxes, then 128-row boxes
                 const int rows = big ? 2 * TC_BOX : TC_BOX, at = big * NS_TENSORS;
@@ -430,7 +441,7 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
     MONA_CUDA(h, small_ns_configure());
     MONA_CUDA(h, sgemm_configure());
     MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
-    for (int sl = 1; sl < NSLOTS; ++sl) {
+    for (int sl = 1; sl < h->plan.n_slots; ++sl) {
         MONA_CUDA(h, cudaStreamCreateWithFlags(&h->side[sl], cudaStreamNonBlocking));
         MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_join[sl], cudaEventDisableTiming));
     }
@@ -530,11 +541,23 @@ static void ns_fit_launch(NsProgram& g, int pairs, bool shared) {
     g.max_pairs = std::min(pairs, most);
 }
 
-// One optimizer step.  With `params_host` set (mona_step_host) every chunk first waits for the gradient copies of
-// the descriptors it touches, and a descriptor whose last matrix has been updated is copied back right away
-// on the handle's device-to-host stream, so transfers in both directions overlap the remaining chunks.
+// Bytes of parameters per chunk in mona_step_host(): a sixteenth of the set, so that the copy back starts early and little of either
+// direction is left alone at the ends, but not so few that a chunk is all launch latency (8 MiB are 150 us of the link).
+// One layer of 512 x 1024 experts, 218 MB each way: with chunks as large as the workspace holds the copy back started when two thirds
+// of the gradients had arrived, 7.2 ms per step; with sixteenths 5.7
+// (eighths 5.7, thirty-seconds 5.9, sixty-fourths 8.9).
+static size_t host_chunk_bytes(const Plan& plan) {
+    size_t total = 0;
+    for (const Bucket& b : plan.buckets) total += b.mats.size() * (size_t)b.e * 4;
+    return std::max<size_t>(8u << 20, total / 16);
+}
+
+// One optimizer step.  With `params_host` set (mona_step_host) every chunk's gradients are copied in on the handle's host-to-device
+// stream before it runs, and its parameters are copied back on the device-to-host stream as soon as it is updated, so
+// transfers in both directions overlap the remaining chunks.
 static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const* params, const void* const* grads,
-                             void* const* o_out, uint32_t phase_mask, void* stream_v, void* const* params_host) {
+                             void* const* o_out, uint32_t phase_mask, void* stream_v, void* const* params_host,
+                             const void* const* grads_host) {
     if (!h) return MONA_ERR_INVALID_ARG;
     if (!hp || !params || !grads) return h->fail(MONA_ERR_INVALID_ARG, "hp, params or grads is null");
     if (hp->ns_steps < 0 || hp->ns_steps > 64) return h->fail(MONA_ERR_INVALID_ARG, "ns_steps out of range");
@@ -564,24 +587,28 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
     DeviceStatus* dstatus = (DeviceStatus*)(h->ws + WS_STATUS_OFF);
     // chunks alternate between the caller's stream (slot 0) and the handle's own stream (slot 1)
     int64_t total_chunks = 0;
+    const size_t host_bytes = params_host ? host_chunk_bytes(plan) : 0;
+    auto chunk_cap = [&](const Bucket& b) {
+        const int cap = hp->ns_precision == 0 && b.tc_ok && T >= 1 ? b.Cb : b.Cf;
+        return params_host ? (int)std::min<size_t>(cap, std::max<size_t>(1, host_bytes / ((size_t)b.e * 4))) : cap;
+    };
     for (const Bucket& b : plan.buckets) {
-        const bool tcb = (hp->ns_precision == 0) && b.tc_ok && T >= 1;
-        const int capb = tcb ? b.Cb : b.Cf;
+        const int capb = chunk_cap(b);
         total_chunks += ((int64_t)b.mats.size() + capb - 1) / capb;
     }
     const bool overlap = h->opt.chunk_overlap && total_chunks > 1;
     cudaStream_t slot_stream[NSLOTS] = {(cudaStream_t)stream_v};
     bool slot_used[NSLOTS] = {true};
-    for (int sl = 1; sl < NSLOTS; ++sl) slot_stream[sl] = overlap ? h->side[sl] : (cudaStream_t)stream_v;
+    for (int sl = 1; sl < NSLOTS; ++sl) slot_stream[sl] = overlap && h->side[sl] ? h->side[sl] : (cudaStream_t)stream_v;
     if (overlap) MONA_CUDA(h, cudaEventRecord(h->ev_fork, slot_stream[0]));
     int64_t big_index = 0;
-    double slot_load[NSLOTS] = {};
     // estimated tensor work of the buckets, by which chunks that run side by side share the SM pairs
     double work_total = 0.0;
     for (const Bucket& b : plan.buckets)
         if (hp->ns_precision == 0 && b.tc_ok) work_total += bucket_work(b);
-    std::vector<char> out_recorded(params_host ? NSLOTS * plan.descs.size() : 0, 0);
-    std::vector<int> chunk_descs;
+    struct DescRange { int desc; int64_t b0, b1; };      // matrices [b0, b1) of a descriptor
+    std::vector<DescRange> ranges;                       // of the chunk (host pipeline only)
+    size_t host_chunk = 0;
     h->launches = 0;
     h->flops_exec = 0.0;
     h->flops_dense = 0.0;
@@ -590,7 +617,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
     for (int bucket_index : plan.order) {
         const Bucket& b = plan.buckets[bucket_index];
         const bool tc = (hp->ns_precision == 0) && b.tc_ok && T >= 1;
-        const int cap = tc ? b.Cb : b.Cf;
+        const int cap = chunk_cap(b);
         const int64_t count = (int64_t)b.mats.size();
         const bool small = b.small && cap >= count;       // one chunk: the extra slots are made for whole buckets
         const double gamma = hp->scale_mode == 0 ? hp->scale_value * std::sqrt((double)b.l) : hp->scale_value;
@@ -603,26 +630,22 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             const int C = (int)std::min<int64_t>(cap, count - start);
             ChunkPtrs ptrs;
             bool vec4 = (b.e % 4 == 0);
-            chunk_descs.clear();
+            ranges.clear();
             for (int c = 0; c < C; ++c) {
                 const MatRef& mr = b.mats[start + c];
                 const mona_matrix_desc& d = plan.descs[mr.desc];
-                if (chunk_descs.empty() || chunk_descs.back() != mr.desc) chunk_descs.push_back(mr.desc);
+                if (params_host) {
+                    if (ranges.empty() || ranges.back().desc != mr.desc) ranges.push_back({mr.desc, mr.b, mr.b});
+                    ranges.back().b1 = mr.b + 1;
+                }
                 if ((d.batch_stride * (int64_t)gsz) % 16 != 0 || (d.batch_stride * 4) % 16 != 0) vec4 = false;
                 ptrs.g[c] = (const uint8_t*)grads[mr.desc] + (size_t)mr.b * d.batch_stride * gsz;
                 ptrs.w[c] = (float*)params[mr.desc] + mr.b * d.batch_stride;
                 ptrs.o[c] = (o_out && o_out[mr.desc]) ? (float*)o_out[mr.desc] + mr.b * d.batch_stride : nullptr;
                 ptrs.gid[c] = (int)(plan.desc_first_gid[mr.desc] + mr.b);
             }
-            int slot = 0;
+            const int slot = b.small ? b.slot : overlap ? (int)(big_index++ % BIG_SLOTS) : 0;
             if (overlap) {
-                if (!small) slot = (int)(big_index++ % BIG_SLOTS);
-                else {      // the slot with the least in it so far (slots past the second exist for as many small buckets as there are)
-                    const int lo = plan.all_small ? 0 : BIG_SLOTS, hi = (int)std::min<int64_t>(NSLOTS, lo + plan.n_small);
-                    slot = lo;
-                    for (int sl = lo; sl < hi; ++sl) if (slot_load[sl] < slot_load[slot]) slot = sl;
-                    slot_load[slot] += b.chain_us;
-                }
                 if (!slot_used[slot]) MONA_CUDA(h, cudaStreamWaitEvent(slot_stream[slot], h->ev_fork, 0));
                 slot_used[slot] = true;
             }
@@ -642,8 +665,29 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             float* af = (float*)(data + b.off32_a);
             float* bf = (float*)(data + b.off32_b);
 
-            if (params_host)
-                for (int dsc : chunk_descs) MONA_CUDA(h, cudaStreamWaitEvent(stream, h->ev_in[dsc], 0));
+            // elements [first, last) of a descriptor's buffer that belong to a range (padding up to the next matrix included)
+            auto span = [&](const DescRange& r, int64_t& first, int64_t& last) {
+                const mona_matrix_desc& d = plan.descs[r.desc];
+                first = r.b0 * d.batch_stride;
+                last = r.b1 == d.batch ? (d.batch - 1) * d.batch_stride + d.rows * d.cols : r.b1 * d.batch_stride;
+            };
+            if (params_host) {
+                if (host_chunk == h->ev_in.size()) {
+                    cudaEvent_t in = nullptr, out = nullptr;
+                    MONA_CUDA(h, cudaEventCreateWithFlags(&in, cudaEventDisableTiming));
+                    h->ev_in.push_back(in);
+                    MONA_CUDA(h, cudaEventCreateWithFlags(&out, cudaEventDisableTiming));
+                    h->ev_out.push_back(out);
+                }
+                for (const DescRange& r : ranges) {
+                    int64_t first, last;
+                    span(r, first, last);
+                    MONA_CUDA(h, cudaMemcpyAsync((uint8_t*)const_cast<void*>(grads[r.desc]) + first * gsz, (const uint8_t*)grads_host[r.desc] + first * gsz,
+                                                 (size_t)(last - first) * gsz, cudaMemcpyHostToDevice, h->h2d));
+                }
+                MONA_CUDA(h, cudaEventRecord(h->ev_in[host_chunk], h->h2d));
+                MONA_CUDA(h, cudaStreamWaitEvent(stream, h->ev_in[host_chunk], 0));
+            }
             const bool cleared_by_prologue = tc && small;
             if (phase_mask & 1u) {
                 NvtxRange range("mona.prologue");
@@ -750,24 +794,20 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                 ++h->launches;
             }
             if (params_host) {
-                for (int dsc : chunk_descs) {
-                    MONA_CUDA(h, cudaEventRecord(h->ev_out[NSLOTS * dsc + slot], stream));
-                    out_recorded[NSLOTS * dsc + slot] = 1;
+                MONA_CUDA(h, cudaEventRecord(h->ev_out[host_chunk], stream));
+                MONA_CUDA(h, cudaStreamWaitEvent(h->d2h, h->ev_out[host_chunk], 0));
+                for (const DescRange& r : ranges) {
+                    int64_t first, last;
+                    span(r, first, last);
+                    MONA_CUDA(h, cudaMemcpyAsync((float*)params_host[r.desc] + first, (const float*)params[r.desc] + first, (size_t)(last - first) * 4,
+                                                 cudaMemcpyDeviceToHost, h->d2h));
                 }
-                const MatRef& last = b.mats[start + C - 1];
-                for (int dsc : chunk_descs) {
-                    const mona_matrix_desc& d = plan.descs[dsc];
-                    if (dsc == last.desc && last.b != d.batch - 1) continue;    // descriptor continues in the next chunk
-                    for (int sl = 0; sl < NSLOTS; ++sl)
-                        if (out_recorded[NSLOTS * dsc + sl]) MONA_CUDA(h, cudaStreamWaitEvent(h->d2h, h->ev_out[NSLOTS * dsc + sl], 0));
-                    const size_t bytes = (size_t)((d.batch - 1) * d.batch_stride + d.rows * d.cols) * 4;
-                    MONA_CUDA(h, cudaMemcpyAsync(params_host[dsc], params[dsc], bytes, cudaMemcpyDeviceToHost, h->d2h));
-                }
+                ++host_chunk;
             }
         }
     }
     for (int sl = 1; sl < NSLOTS; ++sl) {
-        if (!slot_used[sl]) continue;
+        if (!overlap || !slot_used[sl]) continue;
         MONA_CUDA(h, cudaEventRecord(h->ev_join[sl], slot_stream[sl]));
         MONA_CUDA(h, cudaStreamWaitEvent(slot_stream[0], h->ev_join[sl], 0));
     }
@@ -778,11 +818,11 @@ extern "C" {
 
 mona_status mona_step_ex(mona_handle* h, const mona_hparams* hp, void* const* params, const void* const* grads,
                          void* const* o_out, uint32_t phase_mask, void* stream_v) {
-    return step_impl(h, hp, params, grads, o_out, phase_mask, stream_v, nullptr);
+    return step_impl(h, hp, params, grads, o_out, phase_mask, stream_v, nullptr, nullptr);
 }
 
 mona_status mona_step(mona_handle* h, const mona_hparams* hp, void* const* params, const void* const* grads, void* stream) {
-    return step_impl(h, hp, params, grads, nullptr, 7u, stream, nullptr);
+    return step_impl(h, hp, params, grads, nullptr, 7u, stream, nullptr, nullptr);
 }
 
 mona_status mona_step_host(mona_handle* h, const mona_hparams* hp, void* const* params, void* const* grads,
@@ -800,29 +840,12 @@ mona_status mona_step_host(mona_handle* h, const mona_hparams* hp, void* const* 
         MONA_CUDA(h, cudaStreamCreateWithFlags(&h->d2h, cudaStreamNonBlocking));
         MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_hfork, cudaEventDisableTiming));
         MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_hjoin, cudaEventDisableTiming));
-        h->ev_in.assign((size_t)n_desc, nullptr);
-        h->ev_out.assign((size_t)(NSLOTS * n_desc), nullptr);
-        for (auto& e : h->ev_in) MONA_CUDA(h, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
-        for (auto& e : h->ev_out) MONA_CUDA(h, cudaEventCreateWithFlags(&e, cudaEventDisableTiming));
     }
     // both copy streams start after whatever the caller's stream holds so far
     MONA_CUDA(h, cudaEventRecord(h->ev_hfork, stream));
     MONA_CUDA(h, cudaStreamWaitEvent(h->h2d, h->ev_hfork, 0));
     MONA_CUDA(h, cudaStreamWaitEvent(h->d2h, h->ev_hfork, 0));
-    // gradients travel in the order in which the chunks will want them: bucket by bucket, descriptor by descriptor
-    for (int bucket_index : h->plan.order) {
-        const Bucket& b = h->plan.buckets[bucket_index];
-        int prev = -1;
-        for (const MatRef& mr : b.mats) {
-            if (mr.desc == prev) continue;
-            prev = mr.desc;
-            const mona_matrix_desc& d = h->plan.descs[mr.desc];
-            const size_t bytes = (size_t)((d.batch - 1) * d.batch_stride + d.rows * d.cols) * (d.grad_dtype == MONA_BF16 ? 2 : 4);
-            MONA_CUDA(h, cudaMemcpyAsync(grads[mr.desc], grads_host[mr.desc], bytes, cudaMemcpyHostToDevice, h->h2d));
-            MONA_CUDA(h, cudaEventRecord(h->ev_in[mr.desc], h->h2d));
-        }
-    }
-    mona_status st = step_impl(h, hp, params, (const void* const*)grads, nullptr, 7u, stream_v, params_host);
+    mona_status st = step_impl(h, hp, params, (const void* const*)grads, nullptr, 7u, stream_v, params_host, grads_host);
     // join the copy streams back into the caller's stream whether or not the step was enqueued completely
     const std::string step_error = h->last_error;
     MONA_CUDA(h, cudaEventRecord(h->ev_hjoin, h->h2d));
@@ -850,7 +873,7 @@ mona_status mona_selftest_timeout(mona_handle* h, void* stream_v) {
         ns_phase_plan(p);
         ns_program_plan(g);
         MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(1, 1), (cudaStream_t)stream_v));
-        MONA_CUDA(h, launch_ns_program(b.maps[0], g, NsUpdatePtrs{}, h->max_pairs, (DeviceStatus*)(h->ws + WS_STATUS_OFF), (cudaStream_t)stream_v));
+        MONA_CUDA(h, launch_ns_program(b.maps[b.small ? b.slot : 0], g, NsUpdatePtrs{}, h->max_pairs, (DeviceStatus*)(h->ws + WS_STATUS_OFF), (cudaStream_t)stream_v));
         return MONA_OK;
     }
     return h->fail(MONA_ERR_UNSUPPORTED_SHAPE, "no descriptor of this handle takes the tensor-core path");

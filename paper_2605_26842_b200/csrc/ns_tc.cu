@@ -213,6 +213,8 @@ __device__ __forceinline__ unsigned ld_acquire_gpu(const unsigned int* p) {
     return v;
 }
 // Bounded wait until a dependency counter in global memory has reached `need` (acquire at device scope).
+// SLEEP: the pause between attempts that keeps many waiting pairs off the memory system.
+template <bool SLEEP = true>
 __device__ __forceinline__ bool wait_counter(const unsigned int* ctr, unsigned need, volatile int* abort_flag,
                                              DeviceStatus* status, unsigned site, uint32_t* waited = nullptr) {
     TRACE_ONLY(const uint32_t t_in = trace_clock();)
@@ -227,7 +229,7 @@ __device__ __forceinline__ bool wait_counter(const unsigned int* ctr, unsigned n
             TRACE_ONLY(if (waited) *waited += trace_clock() - t_in;)
             return true;
         }
-        __nanosleep(64);
+        if (SLEEP) __nanosleep(64);
         if ((++spins & 63u) == 0u) {
             if (*abort_flag) return false;
             if (clock64() - t0 > WAIT_BUDGET_CYCLES) {
@@ -468,6 +470,22 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
         return true;
     };
 
+    // The phase before an item must be complete for its matrix: its outputs are the item's operands, and the buffers
+    // the item overwrites were last read two phases further back.
+    auto dependency = [&](const Item& it, const unsigned int*& ctr, unsigned& need) {
+        ctr = nullptr; need = 0u;
+        if (!it.stop && it.q > 0) { ctr = g.done + (size_t)it.c * P + (it.q - 1); need = 2u * (phase_first[it.q] - phase_first[it.q - 1]); }
+    };
+    // In a launch of few tiles the chain of phases is the time: there the scheduler publishes an item at once, and those who read what
+    // the phase before has written wait for it themselves - the producers and, for the axpy operand, the epilogue warps (every
+    // other role follows the producers' copies) - so that publication and set-up lie before the wait, not behind it
+    // (one 256 x 512 matrix 99.7 -> 92.2 us per step, a mixed small set 123.6 -> 115.5).
+    auto wait_dependency = [&](const Item& it) -> bool {
+        const unsigned int* ctr; unsigned need;
+        dependency(it, ctr, need);
+        return !ctr || wait_counter<false>(ctr, need, abort_flag, status, 6);
+    };
+
     // TMA loads of all k-slices of one item into the stage ring (both CTAs run this, each for its own rows).
     // producer's view of the slab ring: next entry, next slab, oldest entry not yet known to be free, free slabs, and
     // the slabs every entry in flight took (3 bits each, wrap-around gap included)
@@ -560,7 +578,8 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             for (unsigned n = 0; ok; ++n) {
                 Item it;
                 if (!(ok = take_item(n, it, 8, true, TRACE_PTR(w_ring))) || it.stop) break;
-                fence_proxy_async_global();       // the scheduler's acquire of the dependency precedes these copies
+                if (FEW && !(ok = wait_dependency(it))) break;
+                fence_proxy_async_global();       // the acquire of the dependency (the scheduler's, or the one above) precedes these copies
                 ok = produce(it);
                 TRACE_ONLY(trace_add(NS_TRACE_PRODUCER_EMPTY, w_empty); trace_add(NS_TRACE_PRODUCER_RING, w_ring); w_empty = w_ring = 0;)
             }
@@ -724,12 +743,6 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 if (it.stop) return true;
                 return cursor.find(idx, phase_first, it.c, it.q, it.t);      // false: the item count and the walk disagree
             };
-            // The phase before an item must be complete for its matrix: its outputs are the item's operands, and the buffers
-            // the item overwrites were last read two phases further back.
-            auto dependency = [&](const Item& it, const unsigned int*& ctr, unsigned& need) {
-                ctr = nullptr; need = 0u;
-                if (!it.stop && it.q > 0) { ctr = g.done + (size_t)it.c * P + (it.q - 1); need = 2u * (phase_first[it.q] - phase_first[it.q - 1]); }
-            };
             unsigned published = 0;
             TRACE_ONLY(const uint32_t t_role0 = trace_clock(); uint32_t w_slot = 0, w_dep = 0;)
             bool ok = true;
@@ -756,7 +769,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 }
                 const unsigned int* ctr; unsigned need;
                 dependency(it, ctr, need);
-                if (ctr && !(ok = wait_counter(ctr, need, abort_flag, status, 6, TRACE_PTR(w_dep)))) break;
+                if (!FEW && ctr && !(ok = wait_counter(ctr, need, abort_flag, status, 6, TRACE_PTR(w_dep)))) break;
                 // (no proxy fence here: this thread issues no copy; the producers fence after they have taken the item)
                 asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring_items + 16 * slot), "r"(it.c), "r"(it.q), "r"(it.t), "r"(it.stop) : "memory");
                 asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring_items_peer + 16 * slot), "r"(it.c), "r"(it.q), "r"(it.t), "r"(it.stop) : "memory");
@@ -824,6 +837,11 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             const int gr = m0 + row_in_cta;
             const bool row_ok = gr < p.M;
             const long long row_off = (long long)it.c * p.mat_stride + (long long)gr * p.ld;
+            if (FEW && p.cin) {
+                bool there = true;
+                if (lane == 0) there = wait_dependency(it);
+                if (!__shfl_sync(0xffffffffu, there, 0)) break;      // (also orders the other lanes' loads behind the acquire)
+            }
             float post = 1.0f;
             if (p.post_mode) { const float sc = g.inv_norm[it.c]; post = p.post_mode == 2 ? sc * sc : sc; }
             // correction of this row's diagonal element of A (written earlier in this launch by another CTA: read from L2)

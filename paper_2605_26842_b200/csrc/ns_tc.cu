@@ -1080,9 +1080,11 @@ double ns_phase_executed_flops(const NsPhase& p) {
     return 2.0 * TC_BM * ns_tile_cols(p) * kpad * tiles;
 }
 
-// Figures: a k-slice takes the tensor pipe 512 cycles per 256 x 256 x 64; a narrow tile's is bound by its copies (24 KiB per CTA), not
-// its 256.  The constant is what an item adds on a pair with nothing else to do - first copies, epilogue, stores, completion count,
-// the next claim - from the wait breakdown (an epilogue of 4400 cycles per plain tile, half of it per 128 columns).
+// Figures: a k-slice takes the tensor pipe 512 cycles per 256 x 256 x 64 and half of that per narrow tile, 340 with some loss.  The
+// constant is what an item adds on a pair with nothing else to do - first copies, epilogue, stores, completion count, the next
+// claim - from the wait breakdown (an epilogue of 4400 cycles per plain tile, half of it per 128 columns).  In a launch of one
+// small matrix a narrow k-slice was seen to take ~575 cycles like a plain one, but with 575 and 590 here the choices measured equal
+// within the noise on every case (one matrix 92.2 us either way, a dense block 368 against 367): the constants decide.
 double ns_phase_cycles(const NsPhase& p, double rounds) {
     const double ks = (p.K + TC_BK - 1) / TC_BK;
     return rounds * (p.wide ? 1024.0 * ks + 9000.0 : p.narrow ? 340.0 * ks + 4500.0 : 512.0 * ks + 6500.0);

@@ -840,7 +840,8 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             if (FEW && p.cin) {
                 bool there = true;
                 if (lane == 0) there = wait_dependency(it);
-                if (!__shfl_sync(0xffffffffu, there, 0)) break;      // (also orders the other lanes' loads behind the acquire)
+                if (!__shfl_sync(0xffffffffu, there, 0)) break;
+                __syncwarp();        // orders the other lanes' loads of the operand and of delta behind lane 0's acquire (a shuffle orders nothing)
             }
             float post = 1.0f;
             if (p.post_mode) { const float sc = g.inv_norm[it.c]; post = p.post_mode == 2 ? sc * sc : sc; }

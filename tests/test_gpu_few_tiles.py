@@ -47,3 +47,27 @@ def test_small_buckets_beside_a_large_one_match_a_single_stream():
             return out
         for x, y in zip(run(1), run(0)):
             assert torch.equal(x, y)
+
+
+def test_repeated_steps_agree_bit_for_bit():
+    """The operands that the epilogue and the copies of a phase read were written by other blocks moments before."""
+    dev = torch.device("cuda", 0)
+    gen = torch.Generator().manual_seed(54)
+    shapes = [(1, 256, 512), (2, 512, 264), (1, 776, 520), (3, 136, 200)]
+    W0 = [(torch.randn(s, generator=gen) * 0.02).to(dev) for s in shapes]
+    G = [(torch.randn(s, generator=gen) * 1e-3).to(dev) for s in shapes]
+    p = [w.clone() for w in W0]
+    opt = pkg.MonaOptimizer(p)
+    hp = pkg.default_hparams()
+    first = None
+    for _ in range(100):
+        opt.state.zero_()
+        for w, w0 in zip(p, W0):
+            w.copy_(w0)
+        opt.step(hp, p, G)
+        if first is None:
+            first = [w.clone() for w in p]
+        for x, y in zip(p, first):
+            assert torch.equal(x, y)
+    assert opt.poll_status()[0] == 0
+    opt.close()

@@ -105,13 +105,21 @@ bool ns_pair_pays(int64_t s, int64_t l, int64_t count) {
     const int64_t plain = 2 * (sym * kl + sym * ks + ts * tl * ks), paired = sym * kl + 5 * sym * ks + ts * tl * ks;
     return paired * 100 <= plain * 80 && sym * count >= 150;
 }
-// Whether a T-step run takes its first two iterations together.  Rounding A to bf16 perturbs A' by up to a^2 |A| 2^-9 in the
-// directions of small singular values, so only the first two are, where |A| is small (the iterate has Frobenius norm 1).
-// Relative error of O_5 against fp64 at 256 x 768 (bf16 emulation; every iteration apart -> first two together, both with the
-// diagonal correction): Gaussian 0.0081 -> 0.0082, training-like 0.0085 -> 0.0085, condition number 100 0.0279 -> 0.0228, 1000
-// 0.0536 -> 0.0424 (without the correction, apart: 0.0086, 0.0097, 0.0279, 0.0536).  With the last two together as well the
-// ill-conditioned ones get worse (0.030), and for T < 4 an error of the first two has no iterations left to shrink in.
-bool ns_first_two_together(const bool pair_pays, int T) { return pair_pays && T >= 4; }
+// The quintic of Eq. newton_schulz as the paper gives it.
+constexpr double NS_A = 3.4445, NS_B = -4.7750, NS_C = 2.0315;
+// Whether a run takes its first two iterations together: the paper's coefficients and at least four iterations only.  Rounding A
+// to bf16 perturbs A' by up to a^2 |A| 2^-9 in the directions of small singular values, so only the first two are, where |A| is
+// small (the iterate has Frobenius norm 1).  Relative error of O_5 against fp64 at 256 x 768 (bf16 emulation, mean of twelve
+// draws; plain iterations -> every iteration apart with the diagonal correction -> first two together with it): Gaussian 0.0088 ->
+// 0.0081 -> 0.0082, rows scaled over a factor of ten 0.0093 -> 0.0085 -> 0.0089, training-like 0.0091 -> 0.0085 -> 0.0084,
+// condition number 100 0.0279 -> 0.0278 -> 0.0228; with all singular values equal, or all but one, it goes either way (0.0046 ->
+// 0.0066, 0.0079 -> 0.0056).  Other coefficients can lose: (4.0848, -6.8946, 2.9270) 0.0304 -> 0.0301 -> 0.0457 on Gaussian and
+// 0.0532 -> 0.0474 -> 0.0700 on scaled rows, (1.5, -0.5, 0) 0.0048 -> 0.0048 -> 0.0050; none but the paper's were found to be safe
+// by a bound, so every other set iterates plainly.  With the last two together as well the ill-conditioned ones get worse
+// (0.030), and for T < 4 an error of the first two has no iterations left to shrink in.
+bool ns_first_two_together(bool pair_pays, const mona_hparams& hp) {
+    return pair_pays && hp.ns_steps >= 4 && hp.ns_a == NS_A && hp.ns_b == NS_B && hp.ns_c == NS_C;
+}
 
 // A bucket whose symmetric products are at most four waves of tiles over the machine's 74 CTA pairs, and whose iterates are
 // small enough to hold twice more, does not get the machine to itself: a launch of it is a chain of dependent products with many
@@ -317,7 +325,7 @@ mona_status mona_default_hparams(mona_hparams* hp) {
     if (!hp) return MONA_ERR_INVALID_ARG;
     memset(hp, 0, sizeof *hp);
     hp->lr = 1e-3; hp->momentum = 0.95; hp->accel_beta = 0.99; hp->accel_alpha = -1.0 / (2.0 * (1.0 - 0.99));
-    hp->weight_decay = 0.1; hp->ns_a = 3.4445; hp->ns_b = -4.7750; hp->ns_c = 2.0315; hp->norm_eps = 1e-7;
+    hp->weight_decay = 0.1; hp->ns_a = NS_A; hp->ns_b = NS_B; hp->ns_c = NS_C; hp->norm_eps = 1e-7;
     hp->scale_value = 0.2; hp->ns_steps = 5; hp->scale_mode = 0; hp->ns_precision = 0;
     return MONA_OK;
 }
@@ -700,7 +708,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             const void* o_final = nullptr;
             bool update_fused = false;
             if (tc) {
-                const bool together = ns_first_two_together(b.paired, T);
+                const bool together = ns_first_two_together(b.paired, *hp);
                 const int groups = together ? T - 1 : T;      // each reads one iterate and writes the other
                 if (phase_mask & 2u) {
                     NvtxRange range("mona.newton_schulz");

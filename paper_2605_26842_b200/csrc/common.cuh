@@ -10,20 +10,27 @@ namespace mona {
 // A chunk is the unit that goes through prologue -> Newton-Schulz -> update together: up to MAXC
 // same-shape matrices whose bf16 iterates fit the chunk budget (sized for full machine occupancy, not for cache).
 constexpr int MAXC = 512;   // per-matrix pointers travel as kernel arguments (at most 8 KiB of the 32 KiB CUDA 12 allows)
-// Each matrix is cut into at most MAX_SLABS contiguous slabs for the prologue; every slab
-// owns one partial sum of squares, so the Frobenius norm is reduced in a fixed order.
-constexpr int MAX_SLABS = 256;
+// The Frobenius norm is the sum, in a fixed order, of at most MAX_UNITS partial sums of squares per matrix.  A unit's length follows
+// from the matrix size alone, so the norm's bits do not depend on how many matrices share a launch.
+constexpr int MAX_UNITS = 256;
+inline long long norm_unit(long long e) {
+    const long long least = (e + MAX_UNITS - 1) / MAX_UNITS;
+    return (least + 1023) / 1024 * 1024;                 // a multiple of the prologue's loop trip
+}
 
-// Slab decomposition of `count` matrices of e elements that go through one launch.  A slab is one block's work: a multiple of
-// `unit` elements (one trip of its loop), 16 K of them at most (longer slabs leave fewer blocks than the device holds at
-// once), as short as it takes to give every SM its eleven blocks - with 16 K always, a 256 x 512 matrix ran on 8 blocks and its
-// prologue took 10.6 us, 128 blocks take 4.1 - and long enough for at most MAX_SLABS per matrix.
+// Slab decomposition of `count` matrices of e elements that go through one elementwise launch.  A slab is one block's work: a
+// multiple of `unit` elements (the prologue: norm units; otherwise one trip of the loop), 16 K of them at most where a unit is not
+// longer (longer slabs leave fewer blocks than the device holds at once), as short as it takes to give every SM its eleven
+// blocks - with 16 K always, a 256 x 512 matrix ran on 8 blocks and its prologue took 10.6 us, 128 blocks take 4.1 - and long
+// enough for at most MAX_UNITS per matrix.
 inline void slab_plan(long long e, long long count, long long unit, long long* slab_len, int* slabs) {
-    const long long resident = 148 * 11;
+    const long long resident = 148 * 11, longest = 16384;
     long long slab = (e * count + resident - 1) / resident;
-    slab = slab < 16384 ? slab : 16384;
-    if ((e + slab - 1) / slab > MAX_SLABS) slab = (e + MAX_SLABS - 1) / MAX_SLABS;
+    slab = slab < longest ? slab : longest;
+    if ((e + slab - 1) / slab > MAX_UNITS) slab = (e + MAX_UNITS - 1) / MAX_UNITS;
+    const bool shorter = slab <= longest;
     slab = (slab + unit - 1) / unit * unit;
+    if (shorter && slab > longest && slab > unit) slab -= unit;
     *slab_len = slab;
     *slabs = (int)((e + slab - 1) / slab);
 }

@@ -135,21 +135,6 @@ __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi) {
     return *reinterpret_cast<uint32_t*>(&v);
 }
 
-__device__ __forceinline__ float block_sum(float v, float* smem /* >= 8 floats */) {
-    #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    if (lane == 0) smem[warp] = v;
-    __syncthreads();
-    float t = 0.f;
-    if (warp == 0) {
-        t = (lane < (EW_THREADS >> 5)) ? smem[lane] : 0.f;
-        #pragma unroll
-        for (int o = 4; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
-    }
-    return t;   // valid in warp 0 (all lanes)
-}
-
 // Pointers of up to CAP matrices as the kernels take them.  The driver copies a launch's arguments on the host, and a table
 // sized for the largest chunk (14 KiB with all pointers of 512 matrices) cost about 10 us per launch (19 -> 10 us of host time
 // for one call that launches the prologue), more than the kernel of a small set runs: chunks of up to SMALL_TABLE matrices
@@ -166,83 +151,112 @@ struct ParamTable {
     float* o[CAP];
 };
 
-// grid = (slabs, C).  Block (p, c) owns elements [p*slab_len, min(e, (p+1)*slab_len)) of matrix c.
-// The last block of a matrix to finish adds the slab partials in index order, so ||M||_F does not
-// depend on scheduling; it then resets the arrival counter for the next call.
+// grid = (slabs, C).  Block (p, c) owns elements [p*slab_len, min(e, (p+1)*slab_len)) of matrix c: one or more units of the norm,
+// each with a partial sum of its own (thread sums in the order of the trips, added over the warp and then over the block's
+// warps).  The last block of a matrix to finish adds the partials in index order, so ||M||_F depends neither on scheduling nor
+// on the length of the slabs; it then resets the arrival counter for the next call.
+// A unit's sum is added over the warp while the next unit's loads are under way, so that short units cost the pass nothing (512 matrices of
+// 256 x 768, units of one trip: 503 us with one sum per 16 K slab, 505 so; 93 of 768 x 2048 736 -> 720).
 template <typename GT, typename ST, int VEC, int CAP>
-__global__ void __launch_bounds__(EW_THREADS)
+__global__ void __launch_bounds__(EW_THREADS, 9)      // 56 registers at most: what is free beside a Newton-Schulz CTA
 prologue_kernel(const __grid_constant__ GradTable<CAP> ptrs, float* __restrict__ Mst, void* __restrict__ Ast, void* __restrict__ Gpst,
                 __nv_bfloat16* __restrict__ xhat, float* __restrict__ partials, unsigned int* __restrict__ counters,
                 float* __restrict__ inv_norm, DeviceStatus* __restrict__ status, long long e, long long slab_len,
-                int slabs, PrologueScalars k, unsigned int* __restrict__ zero, int zero_words) {
+                int unit_len, int slab_units, int units, PrologueScalars k, unsigned int* __restrict__ zero, int zero_words) {
     for (unsigned i = (blockIdx.y * gridDim.x + blockIdx.x) * EW_THREADS + threadIdx.x; i < (unsigned)zero_words; i += gridDim.x * gridDim.y * EW_THREADS) zero[i] = 0u;
-    __shared__ float red[8];
+    constexpr int WARPS = EW_THREADS / 32, MAX_SLAB_UNITS = 16;      // (a slab of several units is at most 16 K elements long)
+    __shared__ float red[MAX_SLAB_UNITS * WARPS];
     __shared__ int is_last;
-    const int c = blockIdx.y, p = blockIdx.x;
+    const int c = blockIdx.y, p = blockIdx.x, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long lo = (long long)p * slab_len;
     const long long hi = (lo + slab_len < e) ? lo + slab_len : e;
-    if (!MONA_IN_BOUNDS(c < MAXC && p < slabs && p < MAX_SLABS && lo < e && (VEC == 1 || (lo % 4 == 0 && e % 4 == 0)), status, 201)) return;
-    const GT* __restrict__ g = reinterpret_cast<const GT*>(ptrs.g[c]);
-    float* __restrict__ M = Mst + (long long)c * e;
+    if (!MONA_IN_BOUNDS(c < MAXC && lo < e && slab_len == slab_units * (long long)unit_len && slab_units <= MAX_SLAB_UNITS && units <= MAX_UNITS && e <= units * (long long)unit_len && (VEC == 1 || (lo % 4 == 0 && e % 4 == 0)), status, 201)) return;
+    const long long at = (long long)c * e + lo;             // the block's elements of the state; below, positions are within the slab
+    const int n = (int)(hi - lo);
+    const GT* __restrict__ g = reinterpret_cast<const GT*>(ptrs.g[c]) + lo;
+    float* __restrict__ M = Mst + at;
     using AuxT = typename StateIO<ST>::elem;
-    AuxT* __restrict__ A = reinterpret_cast<AuxT*>(Ast) + (long long)c * e;      // never dereferenced by formats without it
-    AuxT* __restrict__ Gp = reinterpret_cast<AuxT*>(Gpst) + (long long)c * e;
-    __nv_bfloat16* __restrict__ X = xhat ? xhat + (long long)c * e : nullptr;
+    AuxT* __restrict__ A = reinterpret_cast<AuxT*>(Ast) + at;      // never dereferenced by formats without it
+    AuxT* __restrict__ Gp = reinterpret_cast<AuxT*>(Gpst) + at;
+    __nv_bfloat16* __restrict__ X = xhat ? xhat + at : nullptr;
 
-    float acc = 0.f;
+    float acc = 0.f, full = 0.f;          // sums of the present unit, and of one that is complete
+    int units_done = 0;
+    int unit_end = unit_len;
+    auto unit_boundary = [&](int trip) -> bool {            // (the same for all threads)
+        if (trip != unit_end) return false;
+        full = acc; acc = 0.f; unit_end += unit_len;
+        return true;
+    };
+    auto keep_sum = [&](float v) {
+        #pragma unroll
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) red[units_done * WARPS + warp] = v;
+        ++units_done;
+    };
     if (VEC == 4) {
-        constexpr long long STEP = (long long)EW_THREADS * 4;
-        long long i = lo + (long long)threadIdx.x * 4;
-        // two independent vectors per trip keep ~128 B per thread in flight
-        for (; i + STEP < hi; i += 2 * STEP) {
-            float4 g0 = GradLoad<GT>::load4(g + i), g1 = GradLoad<GT>::load4(g + i + STEP);
-            float4 p0 = gp_load4<ST>(Gp + i), p1 = gp_load4<ST>(Gp + i + STEP);
-            float4 a0 = StateIO<ST>::load4(A + i), a1 = StateIO<ST>::load4(A + i + STEP);
-            float4 m0 = __ldcs(reinterpret_cast<const float4*>(M + i)), m1 = __ldcs(reinterpret_cast<const float4*>(M + i + STEP));
-            mona_elem<ST>(g0.x, p0.x, a0.x, m0.x, k); mona_elem<ST>(g0.y, p0.y, a0.y, m0.y, k);
-            mona_elem<ST>(g0.z, p0.z, a0.z, m0.z, k); mona_elem<ST>(g0.w, p0.w, a0.w, m0.w, k);
-            mona_elem<ST>(g1.x, p1.x, a1.x, m1.x, k); mona_elem<ST>(g1.y, p1.y, a1.y, m1.y, k);
-            mona_elem<ST>(g1.z, p1.z, a1.z, m1.z, k); mona_elem<ST>(g1.w, p1.w, a1.w, m1.w, k);
-            gp_store4<ST>(Gp + i, p0); gp_store4<ST>(Gp + i + STEP, p1);
-            StateIO<ST>::store4(A + i, a0);  StateIO<ST>::store4(A + i + STEP, a1);
-            __stcs(reinterpret_cast<float4*>(M + i), m0);  __stcs(reinterpret_cast<float4*>(M + i + STEP), m1);
-            if (X) {
-                *reinterpret_cast<uint2*>(X + i) = make_uint2(pack_bf16x2(m0.x, m0.y), pack_bf16x2(m0.z, m0.w));
-                *reinterpret_cast<uint2*>(X + i + STEP) = make_uint2(pack_bf16x2(m1.x, m1.y), pack_bf16x2(m1.z, m1.w));
+        constexpr int STEP = EW_THREADS * 4;
+        static_assert(2 * STEP == PROLOGUE_UNIT, "a unit is a whole number of trips");
+        for (int trip = 0; trip < n; trip += 2 * STEP) {
+            const int i = trip + (int)threadIdx.x * 4;
+            const bool boundary = unit_boundary(trip);
+            if (trip + 2 * STEP <= n) {
+                // two independent vectors per trip keep ~128 B per thread in flight
+                float4 g0 = GradLoad<GT>::load4(g + i), g1 = GradLoad<GT>::load4(g + i + STEP);
+                float4 p0 = gp_load4<ST>(Gp + i), p1 = gp_load4<ST>(Gp + i + STEP);
+                float4 a0 = StateIO<ST>::load4(A + i), a1 = StateIO<ST>::load4(A + i + STEP);
+                float4 m0 = __ldcs(reinterpret_cast<const float4*>(M + i)), m1 = __ldcs(reinterpret_cast<const float4*>(M + i + STEP));
+                if (boundary) keep_sum(full);
+                mona_elem<ST>(g0.x, p0.x, a0.x, m0.x, k); mona_elem<ST>(g0.y, p0.y, a0.y, m0.y, k);
+                mona_elem<ST>(g0.z, p0.z, a0.z, m0.z, k); mona_elem<ST>(g0.w, p0.w, a0.w, m0.w, k);
+                mona_elem<ST>(g1.x, p1.x, a1.x, m1.x, k); mona_elem<ST>(g1.y, p1.y, a1.y, m1.y, k);
+                mona_elem<ST>(g1.z, p1.z, a1.z, m1.z, k); mona_elem<ST>(g1.w, p1.w, a1.w, m1.w, k);
+                gp_store4<ST>(Gp + i, p0); gp_store4<ST>(Gp + i + STEP, p1);
+                StateIO<ST>::store4(A + i, a0);  StateIO<ST>::store4(A + i + STEP, a1);
+                __stcs(reinterpret_cast<float4*>(M + i), m0);  __stcs(reinterpret_cast<float4*>(M + i + STEP), m1);
+                if (X) {
+                    *reinterpret_cast<uint2*>(X + i) = make_uint2(pack_bf16x2(m0.x, m0.y), pack_bf16x2(m0.z, m0.w));
+                    *reinterpret_cast<uint2*>(X + i + STEP) = make_uint2(pack_bf16x2(m1.x, m1.y), pack_bf16x2(m1.z, m1.w));
+                }
+                acc = fmaf(m0.x, m0.x, acc); acc = fmaf(m0.y, m0.y, acc); acc = fmaf(m0.z, m0.z, acc); acc = fmaf(m0.w, m0.w, acc);
+                acc = fmaf(m1.x, m1.x, acc); acc = fmaf(m1.y, m1.y, acc); acc = fmaf(m1.z, m1.z, acc); acc = fmaf(m1.w, m1.w, acc);
+            } else {                       // the last trip of a matrix
+                if (boundary) keep_sum(full);
+                for (int j = i; j < n; j += STEP) {
+                    float4 g0 = GradLoad<GT>::load4(g + j);
+                    float4 p0 = gp_load4<ST>(Gp + j);
+                    float4 a0 = StateIO<ST>::load4(A + j);
+                    float4 m0 = __ldcs(reinterpret_cast<const float4*>(M + j));
+                    mona_elem<ST>(g0.x, p0.x, a0.x, m0.x, k); mona_elem<ST>(g0.y, p0.y, a0.y, m0.y, k);
+                    mona_elem<ST>(g0.z, p0.z, a0.z, m0.z, k); mona_elem<ST>(g0.w, p0.w, a0.w, m0.w, k);
+                    gp_store4<ST>(Gp + j, p0);
+                    StateIO<ST>::store4(A + j, a0);
+                    __stcs(reinterpret_cast<float4*>(M + j), m0);
+                    if (X) *reinterpret_cast<uint2*>(X + j) = make_uint2(pack_bf16x2(m0.x, m0.y), pack_bf16x2(m0.z, m0.w));
+                    acc = fmaf(m0.x, m0.x, acc); acc = fmaf(m0.y, m0.y, acc); acc = fmaf(m0.z, m0.z, acc); acc = fmaf(m0.w, m0.w, acc);
+                }
             }
-            acc = fmaf(m0.x, m0.x, acc); acc = fmaf(m0.y, m0.y, acc); acc = fmaf(m0.z, m0.z, acc); acc = fmaf(m0.w, m0.w, acc);
-            acc = fmaf(m1.x, m1.x, acc); acc = fmaf(m1.y, m1.y, acc); acc = fmaf(m1.z, m1.z, acc); acc = fmaf(m1.w, m1.w, acc);
-        }
-        for (; i < hi; i += STEP) {
-            float4 g0 = GradLoad<GT>::load4(g + i);
-            float4 p0 = gp_load4<ST>(Gp + i);
-            float4 a0 = StateIO<ST>::load4(A + i);
-            float4 m0 = __ldcs(reinterpret_cast<const float4*>(M + i));
-            mona_elem<ST>(g0.x, p0.x, a0.x, m0.x, k); mona_elem<ST>(g0.y, p0.y, a0.y, m0.y, k);
-            mona_elem<ST>(g0.z, p0.z, a0.z, m0.z, k); mona_elem<ST>(g0.w, p0.w, a0.w, m0.w, k);
-            gp_store4<ST>(Gp + i, p0);
-            StateIO<ST>::store4(A + i, a0);
-            __stcs(reinterpret_cast<float4*>(M + i), m0);
-            if (X) *reinterpret_cast<uint2*>(X + i) = make_uint2(pack_bf16x2(m0.x, m0.y), pack_bf16x2(m0.z, m0.w));
-            acc = fmaf(m0.x, m0.x, acc); acc = fmaf(m0.y, m0.y, acc); acc = fmaf(m0.z, m0.z, acc); acc = fmaf(m0.w, m0.w, acc);
         }
     } else {
         // single elements (an odd matrix size leaves the matrices of a stack unaligned): eight per thread and trip, all loads
         // first, or the pass is one dependent round trip after the other (five odd matrices, 1023 x 511 the largest bucket:
         // the whole step 3.15 -> 2.91 ms with this, the update's unrolling and the shorter slabs)
         constexpr int UNROLL = PROLOGUE_UNIT / EW_THREADS;
-        for (long long i = lo + threadIdx.x; i < hi; i += UNROLL * EW_THREADS) {
+        for (int trip = 0; trip < n; trip += PROLOGUE_UNIT) {
+            const int i = trip + (int)threadIdx.x;
+            const bool boundary = unit_boundary(trip);
             float gv[UNROLL], pv[UNROLL], av[UNROLL], mv[UNROLL];
             #pragma unroll
             for (int u = 0; u < UNROLL; ++u) {
-                const long long j = i + u * EW_THREADS;
+                const int j = i + u * EW_THREADS;
                 gv[u] = pv[u] = av[u] = mv[u] = 0.f;
-                if (j < hi) { gv[u] = GradLoad<GT>::load1(g + j); pv[u] = gp_load1<ST>(Gp + j); av[u] = StateIO<ST>::load1(A + j); mv[u] = M[j]; }
+                if (j < n) { gv[u] = GradLoad<GT>::load1(g + j); pv[u] = gp_load1<ST>(Gp + j); av[u] = StateIO<ST>::load1(A + j); mv[u] = M[j]; }
             }
+            if (boundary) keep_sum(full);
             #pragma unroll
             for (int u = 0; u < UNROLL; ++u) {
-                const long long j = i + u * EW_THREADS;
-                if (j < hi) {
+                const int j = i + u * EW_THREADS;
+                if (j < n) {
                     mona_elem<ST>(gv[u], pv[u], av[u], mv[u], k);
                     gp_store1<ST>(Gp + j, pv[u]); StateIO<ST>::store1(A + j, av[u]); M[j] = mv[u];
                     if (X) X[j] = __float2bfloat16_rn(mv[u]);
@@ -251,19 +265,32 @@ prologue_kernel(const __grid_constant__ GradTable<CAP> ptrs, float* __restrict__
             }
         }
     }
+    keep_sum(acc);
 
-    float total = block_sum(acc, red);
-    if (threadIdx.x == 0) {
-        __stcg(partials + (long long)c * MAX_SLABS + p, total);
-        __threadfence();
-        unsigned int prev = atomicAdd(counters + c, 1u);
-        is_last = (prev == (unsigned int)(slabs - 1));
+    __syncthreads();
+    if (warp == 0) {
+        if (lane < units_done) {
+            float total = red[lane * WARPS];
+            #pragma unroll
+            for (int w = 1; w < WARPS; ++w) total += red[lane * WARPS + w];
+            __stcg(partials + (long long)c * MAX_UNITS + p * slab_units + lane, total);
+        }
+        __syncwarp();
+        if (lane == 0) {
+            __threadfence();               // the block's partials, all written by this warp, precede its arrival
+            unsigned int prev = atomicAdd(counters + c, 1u);
+            is_last = (prev == gridDim.x - 1);
+        }
     }
     __syncthreads();
     if (is_last && threadIdx.x < 32) {
         __threadfence();
         double s = 0.0;
-        for (int j = threadIdx.x; j < slabs; j += 32) s += (double)__ldcg(partials + (long long)c * MAX_SLABS + j);
+        float part[MAX_UNITS / 32];        // all loads first: one round trip (in a loop they were eight, 2 us of a small launch)
+        #pragma unroll
+        for (int q = 0; q < MAX_UNITS / 32; ++q) part[q] = lane + 32 * q < units ? __ldcg(partials + (long long)c * MAX_UNITS + lane + 32 * q) : 0.f;
+        #pragma unroll
+        for (int q = 0; q < MAX_UNITS / 32; ++q) s += (double)part[q];
         #pragma unroll
         for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (threadIdx.x == 0) {
@@ -360,18 +387,18 @@ namespace {
 template <typename GT, typename ST, int CAP>
 void launch_prologue_cap(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, const ChunkPtrs& ptrs, float* M, void* A, void* Gp,
                          __nv_bfloat16* xhat, float* partials, unsigned int* counters, float* inv_norm, DeviceStatus* status,
-                         long long e, long long slab_len, int slabs, const PrologueScalars& k, unsigned int* zero, int zero_words) {
+                         long long e, long long slab_len, const PrologueScalars& k, unsigned int* zero, int zero_words) {
     GradTable<CAP> t;
     for (unsigned c = 0; c < grid.y; ++c) { t.g[c] = ptrs.g[c]; t.gid[c] = ptrs.gid[c]; }
-    if (vec4) prologue_kernel<GT, ST, 4, CAP><<<grid, block, 0, stream>>>(t, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, slabs, k, zero, zero_words);
-    else      prologue_kernel<GT, ST, 1, CAP><<<grid, block, 0, stream>>>(t, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, slabs, k, zero, zero_words);
+    if (vec4) prologue_kernel<GT, ST, 4, CAP><<<grid, block, 0, stream>>>(t, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, (int)norm_unit(e), (int)(slab_len / norm_unit(e)), (int)((e + norm_unit(e) - 1) / norm_unit(e)), k, zero, zero_words);
+    else      prologue_kernel<GT, ST, 1, CAP><<<grid, block, 0, stream>>>(t, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, (int)norm_unit(e), (int)(slab_len / norm_unit(e)), (int)((e + norm_unit(e) - 1) / norm_unit(e)), k, zero, zero_words);
 }
 template <typename GT, typename ST>
 void launch_prologue_t(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, const ChunkPtrs& ptrs, float* M, void* A, void* Gp,
                        __nv_bfloat16* xhat, float* partials, unsigned int* counters, float* inv_norm, DeviceStatus* status,
-                       long long e, long long slab_len, int slabs, const PrologueScalars& k, unsigned int* zero, int zero_words) {
-    if (grid.y <= SMALL_TABLE) launch_prologue_cap<GT, ST, SMALL_TABLE>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, slabs, k, zero, zero_words);
-    else                       launch_prologue_cap<GT, ST, MAXC>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, slabs, k, zero, zero_words);
+                       long long e, long long slab_len, const PrologueScalars& k, unsigned int* zero, int zero_words) {
+    if (grid.y <= SMALL_TABLE) launch_prologue_cap<GT, ST, SMALL_TABLE>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words);
+    else                       launch_prologue_cap<GT, ST, MAXC>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words);
 }
 template <typename OT, int CAP>
 void launch_update_cap(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, const ChunkPtrs& ptrs, const void* O, long long e,
@@ -388,7 +415,7 @@ cudaError_t launch_prologue(const ChunkPtrs& ptrs, int C, bool grad_bf16, int st
                             DeviceStatus* status, long long e, long long slab_len, int slabs,
                             const PrologueScalars& k, unsigned int* zero, int zero_words, cudaStream_t stream) {
     dim3 grid(slabs, C), block(EW_THREADS);
-#define MONA_PROLOGUE_CASE(GT, ST) launch_prologue_t<GT, ST>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, slabs, k, zero, zero_words)
+#define MONA_PROLOGUE_CASE(GT, ST) launch_prologue_t<GT, ST>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words)
     if (grad_bf16) {
         if (state_kind == PROLOGUE_NO_AUX) MONA_PROLOGUE_CASE(__nv_bfloat16, NoAux);
         else if (state_kind == PROLOGUE_AUX_COMBINED) MONA_PROLOGUE_CASE(__nv_bfloat16, Combined);
@@ -427,7 +454,7 @@ cudaError_t launch_scale(const float* M, float* X, const float* inv_norm, int C,
 // ---------------------------------------------------------------------------------------------------
 // Allocation-free single-matrix prologue (mona_prologue_noalloc, declared in include/mona.h).
 //
-// The fused prologue needs a little global scratch: one partial sum of squares per slab and a counter
+// The fused prologue needs a little global scratch: a partial sum of squares per unit of the norm and a counter
 // that tells the last slab to finish that it must add them up.  The handle-based path keeps that
 // scratch in the caller's workspace.  Some callers have no workspace to give and cannot create one:
 // a process whose framework allocator has already claimed the whole device, or a hook that must not
@@ -445,7 +472,7 @@ constexpr long long NOALLOC_MAX_ELEMS = 1ll << 24;      // one 4096 x 4096 matri
 constexpr int NOALLOC_MAX_DEVICES = 64;
 
 struct NoAllocScratch {
-    float partials[MAX_SLABS];     // slab sums of squares (fully rewritten by every call)
+    float partials[MAX_UNITS];     // partial sums of squares (fully rewritten by every call)
     unsigned int counter;          // slab arrival counter; must be 0 when a call starts
     unsigned int pad[3];
     DeviceStatus status;           // sink of the kernel's non-finite flag; the caller reads inv_norm_out instead
@@ -517,7 +544,7 @@ extern "C" mona_status mona_prologue_noalloc(const void* grad, int32_t grad_dtyp
     const long long e = rows * cols;
     long long slab = 0;
     int slabs = 0;
-    slab_plan(e, 1, PROLOGUE_UNIT, &slab, &slabs);
+    slab_plan(e, 1, norm_unit(e), &slab, &slabs);
     // the array keeps whatever the previous call left: the counter has to start from zero
     ce = cudaMemsetAsync(&scratch->counter, 0, sizeof(unsigned int), stream);
     if (ce != cudaSuccess) { set_msg(err, err_len, cudaGetErrorString(ce)); return MONA_ERR_CUDA; }

@@ -12,7 +12,7 @@ constexpr int PROLOGUE_UNIT = 1024, UPDATE_UNIT = 2048;
 // and leaves 1/(||M||_F + eps) of matrix c in inv_norm[c].  `state_kind` says how the acceleration state is kept:
 // fp32, bfloat16 (MONA-Lite storage), as the single fp32 buffer Z = beta_a A - (1 - beta_a) G passed in `A`
 // (`Gp` ignored), or not at all (plain Muon step, M = mu M + G; A and Gp are ignored).
-// M is always fp32.  `partials` holds C*MAX_SLABS floats and
+// M is always fp32.  `partials` holds C*MAX_UNITS floats and
 // `counters` C zero-initialised words of scratch.  Also clears `zero_words` words at `zero` (the scheduler words of the
 // Newton-Schulz launch that follows: a separate memset is one more operation in a short chain).
 enum { PROLOGUE_AUX_F32 = 0, PROLOGUE_AUX_BF16 = 1, PROLOGUE_NO_AUX = 2, PROLOGUE_AUX_COMBINED = 3 };

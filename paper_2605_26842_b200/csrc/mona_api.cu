@@ -39,7 +39,7 @@ constexpr size_t WS_CTRL_BYTES = 1024 * 1024;        // per slot
 constexpr size_t CTRL_COUNTERS_OFF = 0;
 constexpr size_t CTRL_INVNORM_OFF = 4096;
 constexpr size_t CTRL_PARTIALS_OFF = 8192;
-constexpr size_t CTRL_SCHED_OFF = CTRL_PARTIALS_OFF + sizeof(float) * MAXC * MAX_SLABS;   // work counter + done counters of the NS kernel
+constexpr size_t CTRL_SCHED_OFF = CTRL_PARTIALS_OFF + sizeof(float) * MAXC * MAX_UNITS;   // work counter + done counters of the NS kernel
 constexpr size_t WS_DATA_OFF = WS_CTRL_OFF + NSLOTS * WS_CTRL_BYTES;
 static_assert(CTRL_SCHED_OFF + sizeof(unsigned int) * (64 + (size_t)MAXC * NS_MAX_PHASES) <= WS_CTRL_BYTES, "control block overflow");
 static_assert(sizeof(unsigned int) * MAXC <= CTRL_INVNORM_OFF && sizeof(float) * MAXC <= CTRL_PARTIALS_OFF - CTRL_INVNORM_OFF, "control block overflow");
@@ -206,7 +206,7 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         const int64_t cf = b.tc_ok && per_mat_bf16 * cb > (32u << 20) ? cb / 2 : std::min<int64_t>(cb, (int64_t)(chunk_budget / (2 * per_mat_bf16)));
         b.Cf = (int)std::max<int64_t>(1, cf);
         long long slab = 0;
-        slab_plan(b.e, cb, PROLOGUE_UNIT, &slab, &b.slabs);
+        slab_plan(b.e, cb, norm_unit(b.e), &slab, &b.slabs);
         b.slab_len = slab;
         slab_plan(b.e, cb, UPDATE_UNIT, &slab, &b.up_slabs);
         b.up_slab_len = slab;

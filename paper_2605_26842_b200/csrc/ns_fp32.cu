@@ -180,27 +180,30 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sgemm_kernel(const __grid_const
 // ---------------------------------------------------------------------------------------------------
 // Small matrices (shorter side <= 64, e.g. a 32 x 1024 router): the whole Newton-Schulz iteration of one matrix in ONE
 // cluster of 1 to 8 blocks.  The matrix lives in shared memory in its wide orientation Y (s x l, tall inputs are transposed
-// while loading), every block holding a contiguous range of its columns.  An iteration forms the block's share of A = Y Y^T,
-// adds the shares of all blocks through distributed shared memory (in rank order, so that all blocks hold the same bits), forms
-// B' = b A + c A^2 + a I in every block and overwrites the block's columns with B' Y, in plain fp32 FMA throughout.
+// while loading).  Its columns are cut into 1, 2, 4 or 8 parts by the shape alone; every block holds one or several neighbouring
+// parts.  An iteration forms the share of A = Y Y^T of each part, adds the shares as a binary tree over the parts - inside the
+// block first, then over the blocks through distributed shared memory, the same tree whatever the number of blocks, so that a
+// matrix's result does not depend on how many are in the launch - forms B' = b A + c A^2 + a I in every block and overwrites the
+// block's columns with B' Y, in plain fp32 FMA throughout.
 //
 // Bound: latency - a few thousand FMAs per thread and iteration, one cluster barrier each.  A matrix has 4 s^2 l FMAs' worth of work
 // per iteration, too much for one block; split by columns the only exchange is the s x s sum.  The two products read shared
 // memory 16 bytes at a time: Y Y^T as 4 x 4 register tiles whose k range is dealt to four neighbouring lanes (20 wavefronts
 // per 64 FMAs and lane), B' Y with a column of Y in registers and the rows of B' as broadcasts.
-// Measured against one block per matrix with scalar shared-memory reads: a 32 x 512 matrix 182 -> 39 us (five iterations, 4
-// blocks); the step of four layers of 512 x 1024 experts with their 32 x 1024 routers 4.26 -> 3.87 ms.
-constexpr int SMALL_THREADS = 256;
+// Measured against one block per matrix with scalar shared-memory reads, five iterations: one 32 x 512 matrix 180 -> 31 us, 512 of
+// 32 x 1024 1247 -> 664, one 63 x 1000 459 -> 111.
+constexpr int SMALL_THREADS = 256, SMALL_THREADS64 = 384;    // s up to 32, up to 64 (512 leave a thread too few registers for its column)
 constexpr int SMALL_KGROUPS = 4;             // lanes that share a 4 x 4 block of A
 constexpr int SMALL_MAX_CLUSTER = 8;         // the largest portable cluster
-constexpr int SMALL_MIN_COLS = 64;           // a block with fewer columns spends its time in barriers
+constexpr int SMALL_MIN_COLS = 64;           // a part with fewer columns spends its time in barriers
 constexpr size_t SMALL_MAX_SMEM = 200 * 1024;
 
 struct SmallLayout {                         // of one block's shared memory, in floats
-    int s4, cols, lp, sp;                    // padded rows, columns per block, pitch of Y, pitch of the s x s matrices
-    __host__ __device__ SmallLayout(int s, int l, int cluster) {
+    int s4, part, cols, lp, sp;              // padded rows, columns per part and per block, pitch of Y, pitch of the s x s matrices
+    __host__ __device__ SmallLayout(int s, int l, int parts, int cluster) {
         s4 = (s + 3) & ~3;
-        cols = ((l + cluster - 1) / cluster + 4 * SMALL_KGROUPS - 1) / (4 * SMALL_KGROUPS) * (4 * SMALL_KGROUPS);
+        part = ((l + parts - 1) / parts + 4 * SMALL_KGROUPS - 1) / (4 * SMALL_KGROUPS) * (4 * SMALL_KGROUPS);
+        cols = parts / cluster * part;
         lp = cols + 4;                       // 4 mod 16: rows 4 apart start 16 banks apart, two rows of four lanes per wavefront
         sp = s4 + 4;
     }
@@ -217,17 +220,19 @@ __device__ __forceinline__ void small_cluster_sync() {
     asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
 }
 
-template <int SMAX>   // upper bound of the padded shorter side: 32 or 64 (a thread holds a column of Y in registers)
-__global__ void __launch_bounds__(SMALL_THREADS)
+__device__ __forceinline__ float4 add4(const float4& a, const float4& b) { return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w); }
+
+template <int SMAX, int THREADS>   // SMAX: upper bound of the padded shorter side, 32 or 64 (a thread holds a column of Y in registers)
+__global__ void __launch_bounds__(THREADS, SMAX <= 32 ? 2 : 1)
 small_ns_kernel(const float* __restrict__ M, float* __restrict__ O, const float* __restrict__ inv_norm, int rows, int cols,
-                int T, float ca, float cb, float cc) {
+                int parts, int T, float ca, float cb, float cc) {
     extern __shared__ __align__(16) float sm[];
     uint32_t rank, n;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
     const bool tall = rows > cols;
     const int s = tall ? cols : rows, l = tall ? rows : cols;
-    const SmallLayout L(s, l, (int)n);
+    const SmallLayout L(s, l, parts, (int)n);
     const int s4 = L.s4, lp = L.lp, sp = L.sp, nc = L.cols;
     float* Y = sm;
     float* share[2] = {Y + (size_t)s4 * lp, Y + (size_t)s4 * lp + s4 * sp};
@@ -242,9 +247,9 @@ small_ns_kernel(const float* __restrict__ M, float* __restrict__ O, const float*
     const int c_n = max(0, min(nc, l - c_lo));
 
     // X_0 = M / (||M||_F + eps); rows and columns of the padding are zero and stay zero
-    for (int idx = tid; idx < s4 * lp; idx += SMALL_THREADS) Y[idx] = 0.f;
+    for (int idx = tid; idx < s4 * lp; idx += THREADS) Y[idx] = 0.f;
     __syncthreads();
-    for (int idx = tid; idx < s * c_n; idx += SMALL_THREADS) {
+    for (int idx = tid; idx < s * c_n; idx += THREADS) {
         if (!tall) { const int r = idx / c_n, q = idx - r * c_n; Y[r * lp + q] = Mz[(long long)r * cols + c_lo + q] * scale; }
         else       { const int q = idx / s, r = idx - q * s;     Y[r * lp + q] = Mz[(long long)c_lo * cols + idx] * scale; }
     }
@@ -256,67 +261,91 @@ small_ns_kernel(const float* __restrict__ M, float* __restrict__ O, const float*
     for (int t = 0; t < T; ++t) {
         float* mine = share[t & 1];       // two, so that one cluster barrier per iteration is enough
         // (the loop bound is the same for all threads of a warp's group of four; the shuffles stay inside the group)
-        for (int blk0 = 0; blk0 < nblocks; blk0 += SMALL_THREADS / SMALL_KGROUPS) {
+        for (int blk0 = 0; blk0 < nblocks; blk0 += THREADS / SMALL_KGROUPS) {
             const int blk = blk0 + tid / SMALL_KGROUPS;
             int bi = 0;
             while ((bi + 1) * (bi + 2) / 2 <= blk) ++bi;
             const int bj = blk - bi * (bi + 1) / 2;
-            float acc[4][4];
-            #pragma unroll
-            for (int r = 0; r < 4; ++r)
+            float4 sum, level0, level1, level2;       // of the parts so far: complete groups of 1, 2 and 4
+            const int block_parts = parts / (int)n;
+            for (int pt = 0; pt < block_parts; ++pt) {
+                float acc[4][4];
                 #pragma unroll
-                for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
-            if (blk < nblocks) {
-                const float* ya = Y + (size_t)4 * bi * lp + 4 * kg;
-                const float* yb = Y + (size_t)4 * bj * lp + 4 * kg;
-                for (int k = 0; k < nc; k += 4 * SMALL_KGROUPS) {
-                    float4 a[4], b[4];
+                for (int r = 0; r < 4; ++r)
                     #pragma unroll
-                    for (int r = 0; r < 4; ++r) {
-                        a[r] = *reinterpret_cast<const float4*>(ya + r * lp + k);
-                        b[r] = *reinterpret_cast<const float4*>(yb + r * lp + k);
-                    }
-                    #pragma unroll
-                    for (int r = 0; r < 4; ++r)
+                    for (int q = 0; q < 4; ++q) acc[r][q] = 0.f;
+                if (blk < nblocks) {
+                    const float* ya = Y + (size_t)4 * bi * lp + pt * L.part + 4 * kg;
+                    const float* yb = Y + (size_t)4 * bj * lp + pt * L.part + 4 * kg;
+                    for (int k = 0; k < L.part; k += 4 * SMALL_KGROUPS) {
+                        float4 a[4], b[4];
                         #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            acc[r][q] = fmaf(a[r].x, b[q].x, acc[r][q]);
-                            acc[r][q] = fmaf(a[r].y, b[q].y, acc[r][q]);
-                            acc[r][q] = fmaf(a[r].z, b[q].z, acc[r][q]);
-                            acc[r][q] = fmaf(a[r].w, b[q].w, acc[r][q]);
+                        for (int r = 0; r < 4; ++r) {
+                            a[r] = *reinterpret_cast<const float4*>(ya + r * lp + k);
+                            b[r] = *reinterpret_cast<const float4*>(yb + r * lp + k);
                         }
+                        #pragma unroll
+                        for (int r = 0; r < 4; ++r)
+                            #pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                acc[r][q] = fmaf(a[r].x, b[q].x, acc[r][q]);
+                                acc[r][q] = fmaf(a[r].y, b[q].y, acc[r][q]);
+                                acc[r][q] = fmaf(a[r].z, b[q].z, acc[r][q]);
+                                acc[r][q] = fmaf(a[r].w, b[q].w, acc[r][q]);
+                            }
+                    }
+                }
+                // added over the four lanes so that lane kg is left with row kg of the block
+                const bool up2 = kg & 2, up1 = kg & 1;
+                float half[2][4], v[4];
+                #pragma unroll
+                for (int r = 0; r < 2; ++r)
+                    #pragma unroll
+                    for (int q = 0; q < 4; ++q)
+                        half[r][q] = (up2 ? acc[2 + r][q] : acc[r][q]) + __shfl_xor_sync(0xffffffffu, up2 ? acc[r][q] : acc[2 + r][q], 2);
+                #pragma unroll
+                for (int q = 0; q < 4; ++q) v[q] = (up1 ? half[1][q] : half[0][q]) + __shfl_xor_sync(0xffffffffu, up1 ? half[0][q] : half[1][q], 1);
+                sum = make_float4(v[0], v[1], v[2], v[3]);
+                if (!(pt & 1)) level0 = sum;
+                else {
+                    sum = add4(level0, sum);
+                    if (!(pt & 2)) level1 = sum;
+                    else {
+                        sum = add4(level1, sum);
+                        if (!(pt & 4)) level2 = sum; else sum = add4(level2, sum);
+                    }
                 }
             }
-            #pragma unroll
-            for (int r = 0; r < 4; ++r)
-                #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    float v = acc[r][q];
-                    #pragma unroll
-                    for (int o = SMALL_KGROUPS / 2; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-                    if (kg == r && blk < nblocks) {      // lane kg of the four writes row kg of the block and its mirror image
-                        mine[(4 * bi + r) * sp + 4 * bj + q] = v;
-                        mine[(4 * bj + q) * sp + 4 * bi + r] = v;
-                    }
-                }
+            if (blk < nblocks) {                     // row kg of the block and its mirror image
+                *reinterpret_cast<float4*>(mine + (4 * bi + kg) * sp + 4 * bj) = sum;
+                mine[(4 * bj) * sp + 4 * bi + kg] = sum.x; mine[(4 * bj + 1) * sp + 4 * bi + kg] = sum.y;
+                mine[(4 * bj + 2) * sp + 4 * bi + kg] = sum.z; mine[(4 * bj + 3) * sp + 4 * bi + kg] = sum.w;
+            }
         }
-        // A = the sum of all blocks' shares
+        // A = the sum of all blocks' shares, the tree over the parts carried on
         if (n > 1) small_cluster_sync(); else __syncthreads();
         const uint32_t mine_addr = (uint32_t)__cvta_generic_to_shared(mine);
-        for (int idx = tid; idx < s4 * nb; idx += SMALL_THREADS) {
+        for (int idx = tid; idx < s4 * nb; idx += THREADS) {
             const int off = (idx / nb) * sp + 4 * (idx % nb);
-            float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
-            for (uint32_t r = 0; r < n; ++r) {
-                uint32_t addr;
-                asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(mine_addr + 4u * off), "r"(r));
-                const float4 v = ld_cluster4(addr);
-                sum.x += v.x; sum.y += v.y; sum.z += v.z; sum.w += v.w;
+            float4 v[SMALL_MAX_CLUSTER];
+            #pragma unroll
+            for (uint32_t r = 0; r < SMALL_MAX_CLUSTER; ++r) {
+                if (r < n) {
+                    uint32_t addr;
+                    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(addr) : "r"(mine_addr + 4u * off), "r"(r));
+                    v[r] = ld_cluster4(addr);
+                }
             }
-            *reinterpret_cast<float4*>(A + off) = sum;
+            #pragma unroll
+            for (uint32_t w = 1; w < SMALL_MAX_CLUSTER; w *= 2)
+                #pragma unroll
+                for (uint32_t r = 0; r < SMALL_MAX_CLUSTER; r += 2 * w)
+                    if (r + w < n) v[r] = add4(v[r], v[r + w]);
+            *reinterpret_cast<float4*>(A + off) = v[0];
         }
         __syncthreads();
         // B' = b A + c A A + a I
-        for (int idx = tid; idx < s4 * nb; idx += SMALL_THREADS) {
+        for (int idx = tid; idx < s4 * nb; idx += THREADS) {
             const int i = idx / nb, j = 4 * (idx - i * nb);
             float4 sum = make_float4(0.f, 0.f, 0.f, 0.f);
             #pragma unroll 8
@@ -334,9 +363,9 @@ small_ns_kernel(const float* __restrict__ M, float* __restrict__ O, const float*
             *reinterpret_cast<float4*>(B + i * sp + j) = o;
         }
         __syncthreads();
-        // Y <- B' Y: two threads own a column, each half of its rows; both hold the old column in registers
-        constexpr int COLS = SMALL_THREADS / 2;
-        const int row0 = (tid / COLS) * (nb + 1) / 2 * 4, row1 = tid / COLS ? s4 : (nb + 1) / 2 * 4;
+        // Y <- B' Y: THREADS / 128 threads own a column, each a range of its rows; all hold the old column in registers
+        constexpr int COLS = 128, ROW_GROUPS = THREADS / COLS;
+        const int row0 = nb * (tid / COLS) / ROW_GROUPS * 4, row1 = nb * (tid / COLS + 1) / ROW_GROUPS * 4;
         for (int c0 = 0; c0 < nc; c0 += COLS) {
             const int q = c0 + tid % COLS;
             float y[SMAX];
@@ -348,11 +377,13 @@ small_ns_kernel(const float* __restrict__ M, float* __restrict__ O, const float*
                     float o[4] = {0.f, 0.f, 0.f, 0.f};
                     #pragma unroll
                     for (int k = 0; k < SMAX; k += 4) {
-                        if (k < s4) {
-                            const float4 v = *reinterpret_cast<const float4*>(B + i * sp + k);
-                            o[0] = fmaf(v.x, y[k], o[0]); o[1] = fmaf(v.y, y[k + 1], o[1]);
-                            o[2] = fmaf(v.z, y[k + 2], o[2]); o[3] = fmaf(v.w, y[k + 3], o[3]);
-                        }
+                        // s > 32: the load is predicated and zeros are added, since behind branches a row's loads wait for one
+                        // another (a 63 x 1000 matrix 137 -> 117 us); below that the additions saved weigh more
+                        if (SMAX <= 32 && k >= s4) continue;
+                        float4 v = make_float4(0.f, 0.f, 0.f, 0.f);
+                        if (k < s4) v = *reinterpret_cast<const float4*>(B + i * sp + k);
+                        o[0] = fmaf(v.x, y[k], o[0]); o[1] = fmaf(v.y, y[k + 1], o[1]);
+                        o[2] = fmaf(v.z, y[k + 2], o[2]); o[3] = fmaf(v.w, y[k + 3], o[3]);
                     }
                     Y[i * lp + q] = (o[0] + o[1]) + (o[2] + o[3]);
                 }
@@ -360,50 +391,62 @@ small_ns_kernel(const float* __restrict__ M, float* __restrict__ O, const float*
         }
         __syncthreads();
     }
-    for (int idx = tid; idx < s * c_n; idx += SMALL_THREADS) {          // O = X_T, back in the input's orientation
+    for (int idx = tid; idx < s * c_n; idx += THREADS) {          // O = X_T, back in the input's orientation
         if (!tall) { const int r = idx / c_n, q = idx - r * c_n; Oz[(long long)r * cols + c_lo + q] = Y[r * lp + q]; }
         else       { const int q = idx / s, r = idx - q * s;     Oz[(long long)c_lo * cols + idx] = Y[r * lp + q]; }
     }
     if (n > 1) small_cluster_sync();      // no block leaves while another may still read its share
 }
 
-// Blocks per matrix: as many as leave each SMALL_MIN_COLS columns and all matrices together about one block per SM, and at
-// least as many as the matrix needs to fit.
-int small_ns_cluster(int s, int l, int batch) {
+// Parts of a matrix, by its shape alone: as many as leave each SMALL_MIN_COLS columns.
+int small_ns_parts(int l) {
     int n = 1;
-    while (n < SMALL_MAX_CLUSTER && (SmallLayout(s, l, n).bytes() > SMALL_MAX_SMEM || (l >= 2 * n * SMALL_MIN_COLS && 2 * n * batch <= 148))) n *= 2;
+    while (n < SMALL_MAX_CLUSTER && l >= 2 * n * SMALL_MIN_COLS) n *= 2;
+    return n;
+}
+// Blocks per matrix: as many as there are parts while all matrices together have about one block per SM, and at least as many as
+// the matrix needs to fit.
+int small_ns_cluster(int s, int l, int parts, int batch) {
+    int n = 1;
+    while (n < parts && (SmallLayout(s, l, parts, n).bytes() > SMALL_MAX_SMEM || 2 * n * batch <= 148)) n *= 2;
     return n;
 }
 
 }  // namespace
 
+// Every shape whose parts fit takes this path, however many there are: from a few hundred long matrices of s > 32 on the tiled
+// products would be faster (512 of 63 x 2500: 4.8 ms against 7.3; 48: 1.24 against 0.82; one: 0.98 against 0.20), but they add in
+// another order, and which path a matrix takes must not depend on its neighbours.
 bool small_ns_eligible(long long rows, long long cols) {
     const long long s = rows < cols ? rows : cols, l = rows < cols ? cols : rows;
-    return s <= 64 && l <= (1 << 16) && SmallLayout((int)s, (int)l, SMALL_MAX_CLUSTER).bytes() <= SMALL_MAX_SMEM;
+    if (s > 64 || l > (1 << 16)) return false;
+    const int parts = small_ns_parts((int)l);
+    return SmallLayout((int)s, (int)l, parts, parts).bytes() <= SMALL_MAX_SMEM;
 }
 
 cudaError_t small_ns_configure() {
-    cudaError_t e = cudaFuncSetAttribute(small_ns_kernel<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_MAX_SMEM);
+    cudaError_t e = cudaFuncSetAttribute(small_ns_kernel<32, SMALL_THREADS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_MAX_SMEM);
     if (e != cudaSuccess) return e;
-    return cudaFuncSetAttribute(small_ns_kernel<64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_MAX_SMEM);
+    return cudaFuncSetAttribute(small_ns_kernel<64, SMALL_THREADS64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMALL_MAX_SMEM);
 }
 
 cudaError_t launch_small_ns(const float* M, float* O, const float* inv_norm, int batch, int rows, int cols, int T,
                             float a, float b, float c, cudaStream_t stream) {
     const int s = rows < cols ? rows : cols, l = rows < cols ? cols : rows;
-    const int n = small_ns_cluster(s, l, batch);
+    const int parts = small_ns_parts(l), n = small_ns_cluster(s, l, parts, batch);
+    const size_t smem = SmallLayout(s, l, parts, n).bytes();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(batch * n));
-    cfg.blockDim = dim3(SMALL_THREADS);
-    cfg.dynamicSmemBytes = SmallLayout(s, l, n).bytes();
+    cfg.blockDim = dim3(s > 32 ? SMALL_THREADS64 : SMALL_THREADS);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeClusterDimension;
     attr.val.clusterDim.x = (unsigned)n; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
-    return s <= 32 ? cudaLaunchKernelEx(&cfg, small_ns_kernel<32>, M, O, inv_norm, rows, cols, T, a, b, c)
-                   : cudaLaunchKernelEx(&cfg, small_ns_kernel<64>, M, O, inv_norm, rows, cols, T, a, b, c);
+    return s <= 32 ? cudaLaunchKernelEx(&cfg, small_ns_kernel<32, SMALL_THREADS>, M, O, inv_norm, rows, cols, parts, T, a, b, c)
+                   : cudaLaunchKernelEx(&cfg, small_ns_kernel<64, SMALL_THREADS64>, M, O, inv_norm, rows, cols, parts, T, a, b, c);
 }
 
 cudaError_t sgemm_configure() { return cudaFuncSetAttribute(sgemm_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SG_SMEM); }

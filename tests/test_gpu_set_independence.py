@@ -28,6 +28,9 @@ def two_steps(W0, G, grad_dtype, state_dtype, hp, beside=()):
     ((40, 256, 512), (1, 2, 17, 40), torch.float32, torch.float32),      # slabs of one trip to slabs of sixteen
     ((300, 136, 264), (1, 150, 300), torch.bfloat16, torch.bfloat16),
     ((9, 1032, 1160), (1, 4, 9), torch.float32, torch.float32),
+    ((100, 32, 1024), (1, 37, 64, 100), torch.float32, torch.float32),   # one block cluster per matrix
+    ((300, 520, 24), (2, 300), torch.float32, torch.bfloat16),
+    ((150, 63, 1000), (1, 20, 150), torch.float32, torch.float32),
     ((23, 257, 1001), (1, 8, 23), torch.bfloat16, torch.float32),        # fp32 products, scalar elementwise passes
 ])
 def test_a_part_of_a_set_gives_the_bits_of_the_whole(shape, cuts, grad, state):

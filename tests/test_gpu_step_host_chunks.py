@@ -10,7 +10,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("shapes,pad", [([(1, 64, 128)], 0), ([(7, 512, 520), (13, 512, 520), (3, 520, 512), (1, 33, 1001), (1, 32, 256)], 0),
-                                        ([(9, 512, 512), (2, 512, 512)], 64)])
+                                        ([(9, 512, 512), (2, 512, 512)], 64), ([(100, 32, 1024), (1, 256, 512)], 0)])
 def test_step_host_equals_step(shapes, pad):
     dev = torch.device("cuda", 0)
     gen = torch.Generator().manual_seed(71)

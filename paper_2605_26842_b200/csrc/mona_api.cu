@@ -96,14 +96,17 @@ constexpr int MAP_X0 = 0, MAP_A = 2, MAP_B = 3, MAP_C = 4;
 // (A, P and their products are polynomials in A: they commute and are symmetric, lower-triangle tiles all).  Against two plain
 // iterations this saves one X X^T and one B' X and costs three s x s products.  It pays where that is clearly less tensor work
 // (tile-k-slices of the pair against two plain iterations, one step before -> after: 1024 x 4096 0.68, 21.7 -> 20.1 ms; 768 x 2048
-// 0.76, 20.2 -> 19.6 ms; 256 x 768 0.79, 3.87 -> 3.79 ms; but 512 x 1024 0.85, 4.05 -> 4.12 ms; 1024 x 1536 0.91, 6.93 -> 6.95 ms),
-// and only with enough tiles per product to fill the machine twice over: on a few tiles the launch is bound by its chain of
-// dependent products, which gets one longer (16 instead of 15).
-bool ns_pair_pays(int64_t s, int64_t l, int64_t count) {
+// 0.76, 20.2 -> 19.6 ms; 256 x 768 0.79, 3.87 -> 3.79 ms; but 512 x 1024 0.85, 4.05 -> 4.12 ms; 1024 x 1536 0.91, 6.93 -> 6.95 ms).
+// By the shape alone: the pair rounds elsewhere than two plain iterations, and what a matrix gets must not depend on how many others
+// of its shape there are.  On a few tiles, where the launch is bound by its chain of dependent products, the chain gets one longer
+// (16 instead of 15) and its links shorter: one 256 x 768 97.9 -> 99.0 us per step, eight 107.7 -> 110.1, one 1024 x 2816 234 -> 236,
+// 256 x 4096 171 -> 157, eight 1024 x 4096 716 -> 677, a block of 2048 and 8192 2498 -> 2250, sixteen of 1160 x 3096 and four of
+// its square 2023 -> 1976.
+bool ns_pair_pays(int64_t s, int64_t l) {
     const int64_t ts = (s + TC_BM - 1) / TC_BM, tl = (l + TC_BM - 1) / TC_BM, ks = (s + TC_BK - 1) / TC_BK, kl = (l + TC_BK - 1) / TC_BK;
     const int64_t sym = ts * (ts + 1) / 2;
     const int64_t plain = 2 * (sym * kl + sym * ks + ts * tl * ks), paired = sym * kl + 5 * sym * ks + ts * tl * ks;
-    return paired * 100 <= plain * 80 && sym * count >= 150;
+    return paired * 100 <= plain * 80;
 }
 // The quintic of Eq. newton_schulz as the paper gives it.
 constexpr double NS_A = 3.4445, NS_B = -4.7750, NS_C = 2.0315;
@@ -210,7 +213,7 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         b.slab_len = slab;
         slab_plan(b.e, cb, UPDATE_UNIT, &slab, &b.up_slabs);
         b.up_slab_len = slab;
-        b.paired = b.tc_ok && ns_pair_pays(b.s, b.l, count);
+        b.paired = b.tc_ok && ns_pair_pays(b.s, b.l);
         size_t off = 0;
         for (int i = 0; i < 2; ++i) { b.off_x[i] = off; off += align_up((size_t)b.Cb * b.e * 2, 1024); }
         b.off_a = off; off += align_up((size_t)b.Cb * b.s * b.s * 2, 1024);

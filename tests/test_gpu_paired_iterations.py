@@ -1,6 +1,6 @@
-"""The first two Newton-Schulz iterations taken together on the short side: sets wide and numerous enough for the rule that
-selects it (tile work of the pair at most 0.8 of two plain iterations, at least 150 tiles per product), with ragged tiles, both
-orientations, and iteration counts around the smallest that takes it."""
+"""The first two Newton-Schulz iterations taken together on the short side: shapes wide enough for the rule that selects it (tile
+work of the pair at most 0.8 of two plain iterations), with ragged tiles, both orientations, one matrix and many, and iteration
+counts around the smallest that takes it."""
 import pytest
 import torch
 
@@ -64,3 +64,20 @@ def test_no_further_from_64_bits_than_plain_iterations(coefficients):
                 errs[k] += float((got.double() - X).norm() / X.norm()) / 4
         assert errs[0] <= 1.2 * errs[1], (first, errs)
     opt.close()
+
+
+@pytest.mark.parametrize("shape,T,coefficient,paired", [((50, 264, 1048), 5, 3.4445, True), ((1, 264, 1048), 5, 3.4445, True), ((2, 1048, 264), 4, 3.4445, True),
+                                                        ((50, 264, 1048), 3, 3.4445, False), ((50, 264, 1048), 5, 3.4446, False),
+                                                        ((50, 264, 520), 5, 3.4445, False), ((1, 256, 768), 7, 3.4445, True)])
+def test_which_launches_take_the_pair(shape, T, coefficient, paired):
+    """Plain iterations all execute the same number of flops; the pair executes fewer than two of them."""
+    dev = torch.device("cuda", 0)
+    p, g = [torch.zeros(shape, device=dev)], [torch.full(shape, 1e-3, device=dev)]
+    opt = pkg.MonaOptimizer(p)
+    flops = []
+    for steps in (1, T):
+        opt.step(pkg.default_hparams(ns_steps=steps, ns_a=coefficient), p, g)
+        flops.append(opt.last_ns_flops()[0])
+    assert opt.poll_status()[0] == 0
+    opt.close()
+    assert (flops[1] < 0.999 * T * flops[0]) == paired and flops[1] <= 1.001 * T * flops[0], flops

@@ -25,6 +25,8 @@ def two_steps(W0, G, grad_dtype, state_dtype, hp, beside=()):
 
 
 @pytest.mark.parametrize("shape,cuts,grad,state", [
+    ((50, 264, 1048), (1, 20, 50), torch.float32, torch.float32),        # two iterations taken together, one tile row and a bit
+    ((20, 2056, 520), (3, 20), torch.bfloat16, pkg.MONA_STATE_COMBINED),
     ((40, 256, 512), (1, 2, 17, 40), torch.float32, torch.float32),      # slabs of one trip to slabs of sixteen
     ((300, 136, 264), (1, 150, 300), torch.bfloat16, torch.bfloat16),
     ((9, 1032, 1160), (1, 4, 9), torch.float32, torch.float32),

@@ -121,9 +121,13 @@ mona_status mona_default_hparams(mona_hparams* hp);
  *                        (tens of MiB) hold too few tiles for the machine and were measured 1.5-2x slower.
  *   chunk_overlap      : 1 (default) pipelines consecutive chunks over two streams - the caller's and one the
  *                        handle owns, joined by events before mona_step*() returns to the caller's stream - so
- *                        that the start and the tail of one chunk's kernels are filled by the other chunk's;
- *                        0 keeps every launch on the caller's stream.  Results are identical either way; the
- *                        workspace holds two chunks.
+ *                        that the start and the tail of one chunk's kernels are filled by the other chunk's, and
+ *                        runs buckets too small to fill the machine beside them on up to two further streams (on
+ *                        all four when there is nothing else); 0 keeps every launch on the caller's stream.
+ *                        Results are identical either way.
+ *                        The workspace holds two chunks and the small buckets that run beside them: at most 2.25
+ *                        times the budget (or the iterates of the largest matrix in fp32, where that is more), and
+ *                        some 4 MiB.
  *   fuse_update        : 0 (default): O_k is stored in bf16 and a separate elementwise kernel applies Eq. muon_update.
  *                        1: on the tensor-core path the last X' = B' X of a step applies the update in its epilogue
  *                        (fp32 O_k straight from the accumulator, no bf16 copy of O_k written and re-read, one launch
@@ -183,7 +187,7 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
 /* One optimizer step for all descriptors, enqueued on `stream` (a cudaStream_t passed as void*;
  * NULL = the legacy default stream).  params[i] / grads[i] are the device base pointers of
  * descriptor i (16-byte aligned).  Reads grads, updates params and the state in place.  Allocates
- * nothing and does not synchronise; work also runs on the handle's internal stream, ordered with
+ * nothing and does not synchronise; work also runs on the handle's internal streams, ordered with
  * `stream` by events, so synchronising `stream` is enough to observe the result. */
 mona_status mona_step(mona_handle* h, const mona_hparams* hp,
                       void* const* params, const void* const* grads, void* stream);
@@ -325,7 +329,7 @@ mona_status mona_prologue_noalloc(const void* grad, int32_t grad_dtype, float* M
 /* Human-readable detail of the last failing call on this handle (never NULL). */
 const char* mona_last_error(const mona_handle* h);
 
-/* Frees the handle's tables, stream and events.  The caller's buffers are untouched. */
+/* Frees the handle's tables, streams and events.  The caller's buffers are untouched. */
 void mona_destroy(mona_handle* h);
 
 #ifdef __cplusplus

@@ -12,6 +12,7 @@
 #include <cstdio>
 #include <cstring>
 #include <map>
+#include <numeric>
 #include <string>
 #include <tuple>
 #include <vector>
@@ -125,18 +126,21 @@ bool ns_first_two_together(bool pair_pays, const mona_hparams& hp) {
 }
 
 // A bucket whose symmetric products are at most four waves of tiles over the machine's 74 CTA pairs, and whose iterates are
-// small enough to hold twice more, does not get the machine to itself: a launch of it is a chain of dependent products with many
+// few enough to hold once more, does not get the machine to itself: a launch of it is a chain of dependent products with many
 // pairs idle at the end of each, so such buckets run side by side on streams and SM pairs of their own.  Measured: buckets of four
 // 1024 x 1024, two 2816 x 1024 and one 1024 x 2816 928 -> 372 us per step; sixteen, eight and four of 1160 and 3096 (240, 120 and 60
 // tiles; with the line at two waves 2.03 ms) -> 1.75 ms; from five waves on (six tried) nothing changes.  Everything on the
-// fp32 path that takes one block cluster per matrix is small too.
-constexpr size_t SMALL_BUCKET_BYTES = 400ull << 20;
+// fp32 path that takes one block cluster per matrix is small too.  The line in bytes: with 64 MiB the set of 1160 and 3096 takes
+// 2121 us instead of 1911 and a block of 2048 and 8192 2987 instead of 2250; with 400 instead of 200 nothing changes but the
+// workspace (twelve blocks of 1024 and 2816, whose tall bucket has 360 MiB: 3470 us with 200, 3450 with 400, 952 and 1313 MiB).
+constexpr size_t SMALL_BUCKET_BYTES = 200ull << 20;
 bool bucket_is_small(int64_t s, int64_t e, int64_t count, bool tc_ok, bool one_cluster) {
     const int64_t tile = tc_ok ? TC_BM : 64, ts = (s + tile - 1) / tile;       // the fp32 GEMM: 64 x 64 tiles, one block per SM
     return (one_cluster || ts * (ts + 1) / 2 * count <= 4 * (tc_ok ? 74 : 148)) && (size_t)(2 * e + 2 * s * s) * (tc_ok ? 2 : 4) * count <= SMALL_BUCKET_BYTES;
 }
-// NARROW_ROUNDS: a launch on a share of the pairs looks at other tile widths for phases of at most this many rounds of items (1 to 8
-// measured equal within 2 %).  GATE_ROUNDS: the claim gate (NsProgram::gate) pays while a phase leaves pairs idle (mixed small set 151 ->
+// NARROW_ROUNDS: a launch on a share of the pairs looks at other tile widths for phases of at most this many rounds of items (with 1
+// instead of 4 a dense block of 1024 and 2816 takes 407 us instead of 373, but one of 768 and 3072 254 instead of 276; the other sets
+// tried are the same).  GATE_ROUNDS: the claim gate (NsProgram::gate) pays while a phase leaves pairs idle (mixed small set 151 ->
 // 124 us) and costs a round trip per item where every pair has several (12 dense blocks, a bucket at 1.6 rounds: 1-2 %).
 constexpr double NARROW_ROUNDS = 4.0, GATE_ROUNDS = 1.5;
 
@@ -225,7 +229,6 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         b.off32_b = off32; off32 += align_up((size_t)b.Cf * b.s * b.s * 4, 1024);
         b.data_bytes = std::max(off, off32);
         b.small = bucket_is_small(b.s, b.e, count, b.tc_ok, !b.tc_ok && small_ns_eligible(b.rows, b.cols)) && (b.tc_ok ? b.Cb : b.Cf) == count;
-        plan.all_small = plan.all_small && b.small;
         {   // a five-step chain: about 100 us on the tensor cores, 25 in one block cluster, three products per iteration in fp32
             const double ts = (double)((b.s + 63) / 64), tl = (double)((b.l + 63) / 64), waves = (double)count / 148.0;
             const double product = std::max(1.0, ts * (ts + 1) / 2 * waves) * (double)(b.l + b.s) / 32 + std::max(1.0, ts * tl * waves) * (double)b.s / 32;
@@ -233,25 +236,39 @@ mona_status build_plan(const mona_matrix_desc* descs, int64_t n_desc, size_t chu
         }
     }
     for (int i = 0; i < (int)plan.buckets.size(); ++i) plan.order.push_back(i);
-    std::stable_sort(plan.order.begin(), plan.order.end(), [&](int x, int y) {
-        const Bucket &a = plan.buckets[x], &b = plan.buckets[y];
-        return a.small != b.small ? a.small : a.small && a.chain_us > b.chain_us;
-    });
     plan.state_bytes = state_bytes;
-    // Every small bucket gets the slot with the least in it so far, and a slot is as large as the largest bucket it ever holds.
-    size_t slot_bytes[NSLOTS] = {};
-    double slot_load[NSLOTS] = {};
-    const int first_small = plan.all_small ? 0 : BIG_SLOTS;
-    for (int i : plan.order) {
-        Bucket& b = plan.buckets[i];
-        if (!b.small) {
-            for (int sl = 0; sl < BIG_SLOTS; ++sl) slot_bytes[sl] = std::max(slot_bytes[sl], b.data_bytes);
-            continue;
+    // Every small bucket gets the slot with the least in it so far, and a slot is as large as the largest bucket it ever holds.  All
+    // slots together hold no more than two chunks (of the budget, or of the largest matrix) and an eighth of that: where they
+    // would, the largest small bucket runs as a large one, until they do.  The eighth is for sets whose large buckets fill two
+    // chunks: four layers of 512 x 1024 experts with their sixteen 1024 x 1024 beside them 3.79 ms per step, behind them 3.83, with
+    // chunks shortened by as much 3 % more.
+    size_t slot_bytes[NSLOTS], limit = chunk_budget;
+    for (const Bucket& b : plan.buckets) limit = std::max(limit, b.data_bytes);
+    limit = 2 * limit + limit / 4;
+    while (true) {
+        plan.all_small = std::all_of(plan.buckets.begin(), plan.buckets.end(), [](const Bucket& b) { return b.small; });
+        std::stable_sort(plan.order.begin(), plan.order.end(), [&](int x, int y) {
+            const Bucket &a = plan.buckets[x], &b = plan.buckets[y];
+            return a.small != b.small ? a.small : a.small && a.chain_us > b.chain_us;
+        });
+        double slot_load[NSLOTS] = {};
+        const int first_small = plan.all_small ? 0 : BIG_SLOTS;
+        Bucket* largest = nullptr;
+        std::fill_n(slot_bytes, NSLOTS, (size_t)0);
+        for (int i : plan.order) {
+            Bucket& b = plan.buckets[i];
+            if (!b.small) {
+                for (int sl = 0; sl < BIG_SLOTS; ++sl) slot_bytes[sl] = std::max(slot_bytes[sl], b.data_bytes);
+                continue;
+            }
+            b.slot = first_small;
+            for (int sl = first_small; sl < NSLOTS; ++sl) if (slot_load[sl] < slot_load[b.slot]) b.slot = sl;
+            slot_load[b.slot] += b.chain_us;
+            slot_bytes[b.slot] = std::max(slot_bytes[b.slot], b.data_bytes);
+            if (!largest || b.data_bytes > largest->data_bytes) largest = &b;
         }
-        b.slot = first_small;
-        for (int sl = first_small; sl < NSLOTS; ++sl) if (slot_load[sl] < slot_load[b.slot]) b.slot = sl;
-        slot_load[b.slot] += b.chain_us;
-        slot_bytes[b.slot] = std::max(slot_bytes[b.slot], b.data_bytes);
+        if (!largest || std::accumulate(slot_bytes, slot_bytes + NSLOTS, (size_t)0) <= limit) break;
+        largest->small = false;
     }
     plan.workspace_bytes = WS_DATA_OFF;
     for (int sl = 0; sl < NSLOTS; ++sl) {
@@ -518,7 +535,8 @@ static double bucket_work(const Bucket& b) {
 }
 // SM pairs of a small chunk: its share of the work when only small chunks run; beside large ones four times that, and eight
 // at least, so that it is through long before they are.  (Pairs that a launch does not find free simply come later: items are
-// handed out to whichever pairs run.)
+// handed out to whichever pairs run.)  Twelve blocks of 1024 and 2816: 3433 us per step, 3599 with the share alone, 3472 with all
+// pairs; four layers of 512 x 1024 experts the same with all three; a drawn set of experts 2571, 2421 and 2630.
 static int pairs_share(int max_pairs, double work, double work_total, bool all_small) {
     const double share = max_pairs * work / work_total;
     return std::max(1, std::min(max_pairs, (int)(all_small ? share + 0.5 : std::max(8.0, 4.0 * share))));

@@ -99,3 +99,16 @@ def test_binding_fails_loudly_without_the_library(monkeypatch, L):
     monkeypatch.setattr(binding, "_LIB_PATH", "/nonexistent/libmona.so")
     with pytest.raises(ImportError):
         binding.lib()
+
+
+@pytest.mark.parametrize("budget_mib", [1, 16, 100, 400, 768])
+@pytest.mark.parametrize("shapes", [[(1, 256, 512)], [(4, 1024, 1024), (2, 2816, 1024), (1, 1024, 2816)], [(48, 1024, 1024), (24, 2816, 1024), (12, 1024, 2816)],
+                                    [(192, 768, 2048), (96, 2048, 768), (12, 2048, 2048), (3, 1536, 2048)], [(300, 256, 256), (30, 512, 256), (3, 264, 520), (9, 32, 512)],
+                                    [(2, 1023, 511), (1, 257, 1025), (1, 1001, 1500), (1, 10, 768)], [(1, s, s) for s in range(64, 1100, 64)]])
+def test_workspace_holds_little_more_than_two_chunks(L, shapes, budget_mib):
+    """Twice the budget - or the iterates of the largest matrix in fp32, where that is more - and an eighth of that for small buckets
+    beside them, besides the control blocks and what alignment and the diagonal corrections add."""
+    descs = [pkg.MatrixDesc(r, c, b, 0, 0, 0) for b, r, c in shapes]
+    largest = max(8 * (r * c + min(r, c) ** 2) for _, r, c in shapes)
+    bound = 2.25 * max(budget_mib << 20, largest)
+    assert pkg.query_sizes(descs, pkg.default_options(chunk_budget_bytes=budget_mib << 20))[1] <= 1.01 * bound + (5 << 20)

@@ -249,7 +249,7 @@ mona_status mona_last_ns_useful_flops(const mona_handle* h, double* useful);
  * the kernel's scheduler uses; no device is needed.  The paper has no counterpart: this exposes the property the
  * kernel's freedom from deadlock rests on - every item comes after all items it depends on (GEMM q of a matrix after
  * all items of GEMM q - 1 of that matrix) - so that it can be tested for any launch shape.
- *   n_matrices, n_phases (1..15), delay (>= 1, see mona_options.ns_delay), items_per_phase[n_phases]: items per matrix.
+ *   n_matrices, n_phases (1..16: five iterations, the first two taken together), delay (>= 1, see mona_options.ns_delay), items_per_phase[n_phases]: items per matrix.
  * Writes (matrix, phase, item) triples of the items start, start + stride, start + 2 stride, ... (one CTA pair sees such
  * a subsequence) into the HOST array out_cqt (3 int32 per item), at most `capacity` items; *n_written receives the
  * count.  MONA_ERR_INVALID_ARG for null pointers or non-positive sizes. */

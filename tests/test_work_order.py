@@ -18,6 +18,9 @@ CASES = [  # (matrices, delay, items per phase)
     (5, 2, [1, 1, 2] * 5),
     (512, 7, [1, 1, 1] * 5),
     (3, 1024, [10, 10, 8]),
+    (93, 20, [6] * 6 + [12] + [6, 6, 12] * 3),      # the first two iterations together: the longest launch
+    (1, 1, [6] * 6 + [12] + [6, 6, 12] * 3),
+    (5, 3, [3] * 6 + [10] + [3, 3, 10] * 3),
 ]
 
 
@@ -58,7 +61,7 @@ def test_a_pair_decodes_its_subsequence_to_the_same_items(C, delay, items):
 
 
 def test_bad_arguments_are_refused():
-    for args in ((0, 1, [1]), (1, 0, [1]), (1, 1, []), (1, 1, [1] * 16)):
+    for args in ((0, 1, [1]), (1, 0, [1]), (1, 1, []), (1, 1, [1] * 17)):      # (17: one phase more than a launch holds)
         with pytest.raises(binding.MonaError) as e:
             binding.work_order(*args, capacity=4)
         assert e.value.status == 1

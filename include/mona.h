@@ -219,11 +219,13 @@ mona_status mona_step_host(mona_handle* h, const mona_hparams* hp,
  * reported a problem, or -1.  The word is cleared by the call. */
 mona_status mona_poll_status(mona_handle* h, void* stream, int64_t* first_bad_matrix);
 
-/* Failure-detection self-test: enqueues one Newton-Schulz launch (a single X X^T phase) whose shared-memory stages are made to
- * expect 16 bytes more than their copies deliver.  Nothing faults - every copy completes - but the wait for a
- * full stage can never end, so it must run out after its bound (about half a second), latch the time-out in the
+/* Failure-detection self-test: enqueues one Newton-Schulz launch (one iteration of one matrix of the first bucket on the
+ * tensor-core path, in the form in which that bucket's steps run: for a bucket of few tiles with early publication and the
+ * claim gate) whose shared-memory stages are made to expect 16 bytes more than their copies deliver.  Nothing faults
+ * - every copy completes - but neither the wait for a full stage nor the waits for the product it belongs to can end, so
+ * they must run out after their bound (about half a second), latch the time-out in the
  * status word and leave the kernel cleanly.  Afterwards mona_poll_status() returns MONA_ERR_TIMEOUT once and
- * the handle works as before.  Only the first workspace slot is written (with meaningless values); parameters
+ * the handle works as before.  Only the bucket's workspace slot is written (with meaningless values); parameters
  * and state are not touched.  Needs at least one descriptor that takes the tensor-core path. */
 mona_status mona_selftest_timeout(mona_handle* h, void* stream);
 

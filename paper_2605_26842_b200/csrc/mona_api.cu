@@ -890,18 +890,19 @@ mona_status mona_selftest_timeout(mona_handle* h, void* stream_v) {
     MONA_CUDA(h, cudaSetDevice(h->device));
     for (const Bucket& b : h->plan.buckets) {
         if (!b.tc_ok) continue;
-        // one X X^T phase over the first matrix slot of the workspace whose stages expect 16 bytes too many
+        // one iteration of the first matrix of the workspace slot, in the kernel instance that the bucket's steps run in, with stages
+        // that expect 16 bytes too many: the first product never gets its operands, the others never get the first
         uint8_t* ctrl = h->ws + WS_CTRL_OFF;
+        uint8_t* data = h->ws + h->plan.slot_off[b.small ? b.slot : 0];
         unsigned int* sched = (unsigned int*)(ctrl + CTRL_SCHED_OFF);
         NsProgram g{};
-        g.C = 1; g.P = 1; g.delay = 1; g.inv_norm = (const float*)(ctrl + CTRL_INVNORM_OFF); g.work_counter = sched; g.done = sched + 64;
+        g.C = 1; g.delay = 1; g.inv_norm = (const float*)(ctrl + CTRL_INVNORM_OFF); g.work_counter = sched; g.done = sched + 64;
         g.selftest_extra_tx = 16;
-        NsPhase& p = g.ph[0];
-        p.M = p.N = (int)b.s; p.K = (int)b.l; p.a_map = p.b_map = MAP_X0; p.a_mn = p.b_mn = b.tall ? 1 : 0; p.symmetric = 1; p.ab_same = 1;
-        p.d_map = MAP_A; p.ld = b.s; p.mat_stride = b.s * b.s; p.c1 = 0.f; p.c2 = 1.f;
-        ns_phase_plan(p);
+        ns_plan_group(g, b, false, false, 0, (const __nv_bfloat16*)(data + b.off_a), (float*)(data + b.off_delta), (float)NS_A, (float)NS_B, (float)NS_C,
+                      h->opt.macro_tile_min_k, false);
+        if (b.small) ns_fit_launch(g, h->max_pairs, true);
         ns_program_plan(g);
-        MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(1, 1), (cudaStream_t)stream_v));
+        MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(g.C, g.P), (cudaStream_t)stream_v));
         MONA_CUDA(h, launch_ns_program(b.maps[b.small ? b.slot : 0], g, NsUpdatePtrs{}, h->max_pairs, (DeviceStatus*)(h->ws + WS_STATUS_OFF), (cudaStream_t)stream_v));
         return MONA_OK;
     }

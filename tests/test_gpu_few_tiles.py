@@ -71,3 +71,41 @@ def test_repeated_steps_agree_bit_for_bit():
             assert torch.equal(x, y)
     assert opt.poll_status()[0] == 0
     opt.close()
+
+
+@pytest.mark.parametrize("shape", [(1, 256, 512), (2, 136, 200), (1, 1032, 1160), (400, 256, 256)])
+def test_waits_that_cannot_end_time_out_in_every_form_of_the_launch(shape):
+    """Few tiles (early publication, claim gate, narrow tiles; one pair and several) and many: the launch reports the time-out, leaves,
+    and the next step on the same handle gives the bits that it gives on a fresh one."""
+    dev = torch.device("cuda", 0)
+    gen = torch.Generator().manual_seed(55)
+    W0 = (torch.randn(shape, generator=gen) * 0.02).to(dev)
+    G = (torch.randn(shape, generator=gen) * 1e-3).to(dev)
+    out = []
+    for selftest in (False, True):
+        p = [W0.clone()]
+        opt = pkg.MonaOptimizer(p)
+        if selftest:
+            opt.selftest_timeout()
+            assert pkg.STATUS_NAMES[opt.poll_status()[0]] == "MONA_ERR_TIMEOUT"
+        opt.step(pkg.default_hparams(), p, [G])
+        assert opt.poll_status()[0] == 0
+        opt.close()
+        out.append(p[0])
+    assert torch.equal(out[0], out[1])
+
+
+@pytest.mark.parametrize("shape,columns", [((1, 256, 264), 384), ((1, 136, 136), 256), ((400, 256, 264), 512)])
+def test_which_launches_take_narrow_tiles(shape, columns):
+    """Executed flops of one iteration: the two symmetric products of one 256-row tile (two narrow tiles or one whole one, less where
+    the second narrow tile has no columns) and B' X over `columns` columns, with the inner dimension padded to 64."""
+    dev = torch.device("cuda", 0)
+    p, g = [torch.zeros(shape, device=dev)], [torch.full(shape, 1e-3, device=dev)]
+    opt = pkg.MonaOptimizer(p)
+    opt.step(pkg.default_hparams(ns_steps=1), p, g)
+    assert opt.poll_status()[0] == 0
+    executed = opt.last_ns_flops()[0]
+    opt.close()
+    s, l = min(shape[1:]), max(shape[1:])
+    ks, kl = -(-s // 64) * 64, -(-l // 64) * 64
+    assert executed == shape[0] * 2.0 * 256 * (256 * kl + 256 * ks + columns * ks), executed

@@ -48,14 +48,17 @@ def test_profiling_build_matches_the_oracle_and_counts_exactly():
     assert d["again_sum"] == 0                      # the reset cleared the table
     assert len(rows) % 2 == 0 and 2 <= len(rows) <= 148
     lead = rows[0::2]
-    mats, iters = 7, 5
-    # 768 x 768 symmetric products: 3 diagonal + 3 off-diagonal tiles; X X^T has 2048 / 64 = 32 k-slices, A A has 768 / 64 = 12;
-    # X' = B' X: 3 tile rows x 4 macro-tiles of 512 columns, 12 k-slices each
-    expect = {0: 3 * 32, 1: 3 * 32, 2: 3 * 12, 3: 3 * 12, 4: 12 * 12, 5: 0}
-    for kind, per_matrix_iteration in expect.items():
+    mats = 7
+    # 768 x 768 symmetric products: 3 diagonal + 3 off-diagonal tiles; X X^T has 2048 / 64 = 32 k-slices, products of 768 x 768
+    # matrices have 768 / 64 = 12; X' = B' X: 3 tile rows x 4 macro-tiles of 512 columns, 12 k-slices each.  768 x 2048 takes its
+    # first two iterations together: one X X^T, P, P A, P (P A), P', P' P and one Q X; of the s x s products only P and P' have the
+    # same operand on both sides, so the diagonal tiles of the other three count with the off-diagonal ones.  Three plain
+    # iterations follow.
+    expect = {0: 4 * 3 * 32, 1: 4 * 3 * 32, 2: (5 + 3) * 3 * 12 + 3 * 3 * 12, 3: (2 + 3) * 3 * 12, 4: 4 * 12 * 12, 5: 0}
+    for kind, per_matrix in expect.items():
         got = sum(r[16 + 4 * kind + 1] for r in lead)
-        assert got == per_matrix_iteration * mats * iters, (kind, got)
-    assert sum(r[15] for r in rows) == 2 * (6 + 6 + 12) * mats * iters       # every item is counted once by each CTA of its pair
+        assert got == per_matrix * mats, (kind, got)
+    assert sum(r[15] for r in rows) == 2 * ((6 * 6 + 12) + 3 * (6 + 6 + 12)) * mats       # every item is counted once by each CTA of its pair
     for r in lead:
         for kind in range(5):
             cyc, ks, wf, wa = r[16 + 4 * kind:16 + 4 * kind + 4]

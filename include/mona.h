@@ -144,7 +144,8 @@ mona_status mona_default_hparams(mona_hparams* hp);
  *                        accumulators below it (0 = the default, 1: always macro-tiles.  Plain tiles keep the tensor
  *                        cores busier per clock on short inner dimensions, but the step runs at the power cap and
  *                        macro-tiles move fewer bytes per flop: measured 3-7 % faster on every benchmark set).
- *                        Results do not depend on it. */
+ *                        Launches of few tiles choose among 256 x 512, 256 x 256 and 256 x 128 by an estimate of
+ *                        their time, whatever it says.  Results do not depend on it. */
 typedef struct {
     size_t chunk_budget_bytes;
     int32_t chunk_overlap;
@@ -188,7 +189,12 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
  * NULL = the legacy default stream).  params[i] / grads[i] are the device base pointers of
  * descriptor i (16-byte aligned).  Reads grads, updates params and the state in place.  Allocates
  * nothing and does not synchronise; work also runs on the handle's internal streams, ordered with
- * `stream` by events, so synchronising `stream` is enough to observe the result. */
+ * `stream` by events, so synchronising `stream` is enough to observe the result.
+ * What a matrix receives follows from its shape, its data, the state format and hp: not from how many others of its
+ * shape the handle holds, how they are cut into chunks or what runs beside them, so a set split over several handles
+ * gives the bits of the whole.  (Two exceptions, both through alignment: a descriptor whose batch_stride is not a multiple
+ * of 16 bytes makes the chunks it shares with others of its shape take the scalar elementwise kernels, which add up the
+ * norm in another order; and with fuse_update a parameter off a 32-byte boundary keeps its chunk's update separate.) */
 mona_status mona_step(mona_handle* h, const mona_hparams* hp,
                       void* const* params, const void* const* grads, void* stream);
 
@@ -240,8 +246,8 @@ mona_status mona_state_layout(const mona_handle* h, int64_t desc,
 int64_t mona_last_launch_count(const mona_handle* h);
 
 /* Counts of executed tensor-core work of the most recent step: bf16 multiply-add flops actually
- * issued (2 * M * N * K summed over issued 256 x 256 tile MMAs: padding and the upper halves of diagonal tiles
- * count) and the dense-equivalent figure (4 s^2 l + 2 s^3 per matrix and iteration).  Either pointer may be NULL. */
+ * issued (2 * M * N * K summed over issued 256 x 256 and 256 x 128 tile MMAs: padding and the upper halves of diagonal
+ * tiles count) and the dense-equivalent figure (4 s^2 l + 2 s^3 per matrix and iteration).  Either pointer may be NULL. */
 mona_status mona_last_ns_flops(const mona_handle* h, double* executed, double* dense_equivalent);
 /* The work the iteration itself needs when both symmetric products are computed once per pair of entries:
  * 3 s^2 l + s^3 per matrix and iteration (tensor-core path only). */
@@ -301,7 +307,8 @@ mona_status mona_trace_read(unsigned long long* out, size_t rows, int reset);
  * for integration reasons only.  It performs lines 4-7 and 10 of Algorithm 1 on a rows x cols matrix
  * (A, M, G_prev updated in place from `grad`, all device pointers, 16-byte aligned, dense row-major),
  * writes 1 / (||M_k||_F + eps) to inv_norm_out[0] (device) and, when xhat_bf16 is not NULL, the bf16
- * copy of M_k there.  Results equal those of the prologue phase of mona_step_ex().
+ * copy of M_k there.  Results equal those of the prologue phase of mona_step_ex() bit for bit (stacks whose stride
+ * is no multiple of 16 bytes: up to the rounding of the norm).
  *
  * Who needs it: callers that cannot get device memory when they call us - for instance a trainer whose
  * framework allocator already owns all of HBM, or a hook running where the device-wide stall of

@@ -1,5 +1,5 @@
 """The fp32 products (sizes the tensor-core path does not take, and the validation mode): remainders of the 64 x 64 tile and of the
-32-wide k-slab, one tile and many, both orientations, stacks."""
+64-wide k-slab, one tile and many, both orientations, stacks."""
 import pytest
 
 import paper_2605_26842_b200 as pkg

@@ -486,26 +486,31 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
 }  // extern "C"
 
 // Appends to `g` the phases of one iteration (or of two taken together) of a chunk of bucket `b`.  X is read from tensor
-// MAP_X0 + x_cur and written to the other one; `first`: X is still un-normalised.
-static void ns_plan_group(NsProgram& g, const Bucket& b, bool together, bool first, int x_cur, const __nv_bfloat16* a_data, float* delta,
-                          float ns_a, float ns_b, float ns_c, int macro_tile_min_k, bool fuse_update) {
+// MAP_X0 + x_cur and written to the other one, or over itself with `in_place`; `first`: X is still un-normalised.
+static void ns_plan_group(NsProgram& g, const Bucket& b, bool together, bool first, int x_cur, uint8_t* data, float* delta,
+                          float ns_a, float ns_b, float ns_c, int macro_tile_min_k, bool fuse_update, bool in_place) {
     const int s = (int)b.s, l = (int)b.l;
+    const size_t offset[NS_TENSORS] = {b.off_x[0], b.off_x[1], b.off_a, b.off_b, b.off_x[1]};
+    auto output = [&](NsPhase& p, int d_map, int64_t ld) {
+        p.d_map = d_map; p.d = (__nv_bfloat16*)(data + offset[d_map]); p.ld = ld;
+        p.mat_stride = d_map == MAP_A || d_map == MAP_B ? (int64_t)s * s : b.e;
+    };
     // D = product of two symmetric s x s matrices, operands and result lower-block-stored
     auto small = [&](int a_map, int b_map, int d_map) -> NsPhase& {
         NsPhase& p = g.ph[g.P++];
         p.M = p.N = p.K = s; p.a_map = a_map; p.b_map = b_map; p.a_sym = p.b_sym = 1; p.symmetric = p.small_sym = 1; p.ab_same = a_map == b_map;
-        p.d_map = d_map; p.ld = s; p.mat_stride = (long long)s * s; p.c2 = 1.f;
+        output(p, d_map, s); p.c2 = 1.f;
         ns_phase_plan(p);
         return p;
     };
     // D = b A + c A A + a I
     auto poly = [&](int d_map) {
         NsPhase& p = small(MAP_A, MAP_A, d_map);
-        p.cin = a_data; p.c1 = ns_b; p.c2 = ns_c; p.diag_add = ns_a; p.delta_in = delta;
+        p.cin = (const __nv_bfloat16*)(data + b.off_a); p.cin_stride = (long long)s * s; p.c1 = ns_b; p.c2 = ns_c; p.diag_add = ns_a; p.delta_in = delta;
     };
     NsPhase& g1 = g.ph[g.P++];      // A = X X^T (wide) or X^T X (tall): lower-triangle tiles only
     g1.M = g1.N = s; g1.K = l; g1.a_map = g1.b_map = MAP_X0 + x_cur; g1.a_mn = g1.b_mn = b.tall ? 1 : 0;
-    g1.symmetric = 1; g1.ab_same = 1; g1.d_map = MAP_A; g1.ld = s; g1.mat_stride = (long long)s * s;
+    g1.symmetric = 1; g1.ab_same = 1; output(g1, MAP_A, s);
     g1.c2 = 1.f; g1.post_mode = first ? 2 : 0; g1.delta_out = delta;
     ns_phase_plan(g1);
     poly(MAP_B);                                        // P
@@ -517,7 +522,7 @@ static void ns_plan_group(NsProgram& g, const Bucket& b, bool together, bool fir
     }
     const int q_map = together ? MAP_A : MAP_B;
     NsPhase& g3 = g.ph[g.P++];      // X' = Q X (wide) or X Q (tall); 256 x 512 macro-tiles when the inner dimension is long
-    g3.K = s; g3.wide = s >= macro_tile_min_k ? 1 : 0; g3.d_map = MAP_X0 + (x_cur ^ 1); g3.ld = b.cols; g3.mat_stride = b.e;
+    g3.K = s; g3.wide = s >= macro_tile_min_k ? 1 : 0; output(g3, MAP_X0 + (in_place ? x_cur : x_cur ^ 1), b.cols);
     g3.c2 = 1.f; g3.post_mode = first ? 1 : 0; g3.fuse_update = fuse_update ? 1 : 0;
     if (!b.tall) {   // Q is the symmetric "A" operand, X the MN-major "B" operand
         g3.M = s; g3.N = l; g3.a_map = q_map; g3.a_sym = 1; g3.b_map = MAP_X0 + x_cur; g3.b_mn = 1;
@@ -540,6 +545,19 @@ static double bucket_work(const Bucket& b) {
 static int pairs_share(int max_pairs, double work, double work_total, bool all_small) {
     const double share = max_pairs * work / work_total;
     return std::max(1, std::min(max_pairs, (int)(all_small ? share + 0.5 : std::max(8.0, 4.0 * share))));
+}
+// Whether a launch over C matrices deals them whole to its SM pairs (NsForm::Whole).  Only where the shorter side is one tile.
+// Matrices of one tile (l <= 256 too) from eight on, where spreading a product over pairs buys nothing and handing it over inside a
+// pair is quicker: forty of 64 x 64 117 -> 72 us per step, forty of 256 x 256 151 -> 121, sixteen of 256 x 128 113 -> 84, but
+// four of 64 x 64 66 against 72 and four of 256 x 256 96 against 88.  Longer ones once every pair has one, and by the rounds that C makes of two
+// matrices per pair: a full round of 256 x 768 takes 217 us, one in which no pair has a second 167, and spread over all pairs as many
+// matrices take 1.1 times a full round's share (C = 148: 421 against 453 us per step, 256: 828 against 755, 370: 1020 against 1061,
+// 512: 1397 against 1448; 60 of 200 x 4096 767 against 698, 74 of 256 x 512 210 against 233).
+static bool whole_matrices(const Bucket& b, int C, int pairs) {
+    if (b.s > TC_BM) return false;
+    if (b.l <= TC_BN) return C >= 8;
+    const int rest = C % (2 * pairs);
+    return C >= pairs && C / (2 * pairs) + (rest == 0 ? 0.0 : rest <= pairs ? 0.77 : 1.0) <= 1.1 * C / (2.0 * pairs);
 }
 // Fits a launch to `pairs` SM pairs: tile widths by estimated time, the claim gate, no more pairs than a phase has items.
 // (`shared`: beside other launches on a part of the pairs.)  A launch that has all pairs looks at other tile widths only for phases
@@ -565,8 +583,8 @@ static void ns_fit_launch(NsProgram& g, int pairs, bool shared) {
         most = std::max(most, p.items_per_mat * g.C);
     }
     g.gate = !fused && most < GATE_ROUNDS * pairs ? 1 : 0;
-    g.few = g.gate;
-    for (int q = 0; q < g.P; ++q) g.few |= g.ph[q].narrow;
+    if (g.gate) g.form = NsForm::Few;
+    for (int q = 0; q < g.P; ++q) if (g.ph[q].narrow) g.form = NsForm::Few;
     g.max_pairs = std::min(pairs, most);
 }
 
@@ -689,7 +707,6 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             void* Ac = h->state + b.off_A + (size_t)start * b.e * aux;
             void* Gc = h->state + b.off_G + (size_t)start * b.e * aux;
             __nv_bfloat16* xb[2] = {(__nv_bfloat16*)(data + b.off_x[0]), (__nv_bfloat16*)(data + b.off_x[1])};
-            __nv_bfloat16* ab = (__nv_bfloat16*)(data + b.off_a);
             float* xf[2] = {(float*)(data + b.off32_x[0]), (float*)(data + b.off32_x[1])};
             float* af = (float*)(data + b.off32_a);
             float* bf = (float*)(data + b.off32_b);
@@ -730,7 +747,10 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             bool update_fused = false;
             if (tc) {
                 const bool together = ns_first_two_together(b.paired, *hp);
-                const int groups = together ? T - 1 : T;      // each reads one iterate and writes the other
+                const int groups = together ? T - 1 : T;      // each reads one iterate and writes the other (a pair's own matrices: the same)
+                const bool shared = overlap && small;
+                const int pairs = shared ? pairs_share(h->max_pairs, bucket_work(b), work_total, plan.all_small) : h->max_pairs;
+                const bool whole = !h->opt.fuse_update && whole_matrices(b, C, pairs);
                 if (phase_mask & 2u) {
                     NvtxRange range("mona.newton_schulz");
                     // the last X' = B' X applies the parameter update in its epilogue when this call runs both phases and the
@@ -747,11 +767,11 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                         bool last = false;
                         for (; gi < groups && g.P + (gi == 0 && together ? 7 : 3) <= NS_MAX_PHASES; ++gi) {
                             last = gi + 1 == groups;
-                            ns_plan_group(g, b, gi == 0 && together, gi == 0, gi & 1, ab, (float*)(data + b.off_delta), ns_a, ns_b, ns_c,
-                                          h->opt.macro_tile_min_k, update_fused && last);
+                            ns_plan_group(g, b, gi == 0 && together, gi == 0, whole ? 0 : gi & 1, data, (float*)(data + b.off_delta), ns_a, ns_b, ns_c,
+                                          h->opt.macro_tile_min_k, update_fused && last, whole);
                         }
-                        const bool shared = overlap && small;
-                        ns_fit_launch(g, shared ? pairs_share(h->max_pairs, bucket_work(b), work_total, plan.all_small) : h->max_pairs, shared);
+                        if (whole) { g.form = NsForm::Whole; g.max_pairs = pairs; g.lane_tensors = C >= 2 * pairs; }
+                        else ns_fit_launch(g, pairs, shared);
                         for (int q = 0; q < g.P; ++q) h->flops_exec += (double)C * ns_phase_executed_flops(g.ph[q]);
                         ns_program_plan(g);
                         // For a small chunk the prologue of this call has cleared the scheduler words of the first launch: one
@@ -768,7 +788,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                     h->flops_dense += (double)T * C * (4.0 * b.s * b.s * b.l + 2.0 * (double)b.s * b.s * b.s);
                     h->flops_useful += (double)T * C * (3.0 * b.s * b.s * b.l + (double)b.s * b.s * b.s);
                 }
-                o_final = xb[groups & 1];
+                o_final = xb[whole ? 0 : groups & 1];
             } else if (small_ns_eligible(b.rows, b.cols)) {
                 // short side <= 64 (routers): the whole iteration in one launch, one block cluster per matrix
                 if (phase_mask & 2u) {
@@ -898,9 +918,11 @@ mona_status mona_selftest_timeout(mona_handle* h, void* stream_v) {
         NsProgram g{};
         g.C = 1; g.delay = 1; g.inv_norm = (const float*)(ctrl + CTRL_INVNORM_OFF); g.work_counter = sched; g.done = sched + 64;
         g.selftest_extra_tx = 16;
-        ns_plan_group(g, b, false, false, 0, (const __nv_bfloat16*)(data + b.off_a), (float*)(data + b.off_delta), (float)NS_A, (float)NS_B, (float)NS_C,
-                      h->opt.macro_tile_min_k, false);
-        if (b.small) ns_fit_launch(g, h->max_pairs, true);
+        const bool whole = !h->opt.fuse_update && whole_matrices(b, (int)std::min<int64_t>(b.Cb, (int64_t)b.mats.size()), h->max_pairs);
+        ns_plan_group(g, b, false, false, 0, data, (float*)(data + b.off_delta), (float)NS_A, (float)NS_B, (float)NS_C,
+                      h->opt.macro_tile_min_k, false, whole);
+        if (whole) g.form = NsForm::Whole;
+        else if (b.small) ns_fit_launch(g, h->max_pairs, true);
         ns_program_plan(g);
         MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(g.C, g.P), (cudaStream_t)stream_v));
         MONA_CUDA(h, launch_ns_program(b.maps[b.small ? b.slot : 0], g, NsUpdatePtrs{}, h->max_pairs, (DeviceStatus*)(h->ws + WS_STATUS_OFF), (cudaStream_t)stream_v));

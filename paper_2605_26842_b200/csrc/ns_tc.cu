@@ -23,12 +23,20 @@
 //              the "empty" barriers of both CTAs (multicast commit),
 //   warps 4-11 epilogue: tcgen05.ld the CTA's 128 x 256 fp32 accumulator, apply the polynomial term
 //              (b A + c A^2 + a I) and the deferred 1/||M||_F scale, pack to bf16 into swizzled shared
-//              memory and hand the boxes to TMA stores (a thread owns one row, so storing from registers
-//              would touch 32 lines per warp instruction; the TMA writes whole lines);
+//              memory (a thread owns one row, so storing from registers would touch 32 lines per warp instruction) and
+//              hand the boxes to TMA stores, or read them back four lines at a time and store them themselves:
+//              TMA stores in the spread form, where their fewer instructions are 1-2 % of the energy of the large sets, own
+//              stores in the others, where a hand-over less is 2 % of a short chain and 6 % of 256 x 768 experts;
 //              for the last X' = B' X of a step the same warps apply the parameter update of Eq. muon_update
 //              to the fp32 weights instead,
-//   warp 3     store warp: turns each staged phase into TMA stores, frees the staging buffer, and counts the item as
-//              done once its stores have completed, so that no epilogue warp ever waits for global memory.
+//   warp 3     store warp: turns each staged phase into TMA stores and frees the staging buffer (spread form), and counts the item
+//              as done once its stores have completed, so that no epilogue warp ever waits for global memory.
+//
+// A launch comes in one of three forms (NsForm).  The spread form above is the one of many tiles per phase.  Launches of few tiles add
+// narrow tiles, early publication and the claim gate.  Where a matrix has one row of tiles (s <= 256) a pair can own whole
+// matrices: each of its two lanes walks the phases of one, a lane's phases are ordered by a counter in the pair's shared memory
+// instead of one in global memory, X' overwrites X, and A, B' and C are the lane's, so that what is written stays in L2
+// (512 of 256 x 768: 3.0 -> 1.75 GB of DRAM traffic, and 790 -> 840 TFLOP/s executed).
 // Tensor memory holds two 256-column accumulators.  Plain tiles alternate between them, so the epilogue of one
 // tile overlaps the main loop of the next.  A macro-tile uses both at once, two neighbouring tiles computed
 // from ONE staged slice of the A operand: 96 KiB instead of 128 KiB cross from L2 per k-slice and pair.
@@ -65,7 +73,9 @@ constexpr uint32_t BOX_BYTES = TC_BOX * TC_BOX * 2;               // 8 KiB
 constexpr uint32_t A_STAGE_BYTES = CTA_M * TC_BK * 2;             // 16 KiB
 constexpr uint32_t B_SUB_BYTES = CTA_N * TC_BK * 2;               // 16 KiB per 256-column tile
 constexpr int EPI_COLS = 128;                                     // output columns per epilogue phase
-constexpr uint32_t EPI_BUF_BYTES = CTA_M * EPI_COLS * 2;          // 32 KiB = 2 x 2 boxes: staging buffer of the store epilogue
+constexpr uint32_t EPI_WARP_BYTES = 32 * 128;                     // staging of an epilogue warp: 64 bf16 columns of its 32 rows
+constexpr uint32_t EPI_BUF_BYTES = TC_EPI_WARPS * EPI_WARP_BYTES;
+constexpr int DONE_RING = 4;                                      // completion barriers: an epilogue warp can be two items ahead of another
 constexpr uint32_t TMEM_COLS = 512;                               // 2 accumulators x 256 fp32 columns
 // Operand staging: a ring of 16 KiB slabs.  A k-slice takes one slab per operand part it stages (1: diagonal tile whose
 // operands coincide, 2: plain tile, 3: macro-tile), contiguous (a k-slice that does not fit before the end of the ring
@@ -83,7 +93,7 @@ constexpr long long WAIT_BUDGET_CYCLES = 1000000000ll;            // ~0.5 s
 // epilogue warps in the peer
 constexpr uint32_t RING_READERS = 3 + TC_EPI_WARPS + 2 + TC_EPI_WARPS;
 static_assert(SMEM_TOTAL <= 232448, "shared memory budget");
-static_assert(8 * (2 * NENT + 4 + 2 * RING + 4) + 16 + 16 * RING + 4 * (NS_MAX_PHASES + 1) <= SMEM_CTRL_BYTES, "control block");
+static_assert(8 * (2 * NENT + 4 + 2 * RING + 4 + DONE_RING) + 16 + 16 * RING + 4 * (NS_MAX_PHASES + 1) <= SMEM_CTRL_BYTES, "control block");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -240,6 +250,28 @@ __device__ __forceinline__ bool wait_counter(const unsigned int* ctr, unsigned n
     }
 }
 
+// Completion counts of the whole-matrix form live in shared memory, one copy per CTA of the pair.
+__device__ __forceinline__ void red_add_release_cluster(uint32_t cluster_addr, unsigned v) {
+    asm volatile("red.release.cluster.shared::cluster.add.u32 [%0], %1;" ::"r"(cluster_addr), "r"(v) : "memory");
+}
+// Bounded wait until a counter in this CTA's shared memory has reached `need` (acquire at cluster scope).
+__device__ __forceinline__ bool wait_shared_counter(uint32_t addr, unsigned need, volatile int* abort_flag, DeviceStatus* status, unsigned site) {
+    long long t0 = 0;
+    for (unsigned spins = 0;; ++spins) {
+        unsigned v;
+        asm volatile("ld.acquire.cluster.shared::cta.u32 %0, [%1];" : "=r"(v) : "r"(addr) : "memory");
+        if ((int)(v - need) >= 0) return true;
+        if (spins == 0) t0 = clock64();
+        if ((spins & 63u) == 63u) {
+            if (*abort_flag) return false;
+            if (clock64() - t0 > WAIT_BUDGET_CYCLES) {
+                latch_timeout(abort_flag, status, site);
+                return false;
+            }
+        }
+    }
+}
+
 // ---- TMA ------------------------------------------------------------------------------------------
 // Box load into this CTA's shared memory; completion bytes are counted on `bar`, a cluster-wide
 // address that may name the barrier of the peer CTA of the pair (cta_group::2 form).
@@ -332,7 +364,8 @@ __device__ __forceinline__ void tmem_ld32(uint32_t taddr, float* v) {
 }
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
-// A published work item: item `t` of phase `q` for matrix `c`; stop != 0 ends the role loops.
+// A published work item: item `t` of phase `q` for matrix `c`.  Bit 0 of `stop` ends the role loops; in the whole-matrix form bit 1
+// is the lane and the bits above are the arrivals its counter must show before the item's operands are complete.
 struct Item {
     int c, q, t, stop;
 };
@@ -380,12 +413,6 @@ __device__ __forceinline__ void ld8(const float* p, float* v) {
                  : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
                  : "l"(p));
 }
-// 32 bytes of bf16 data written earlier in this launch by other CTAs: from L2 (.cg), never from a line L1 may still hold
-__device__ __forceinline__ void ld8cg(const void* p, uint32_t* w) {
-    asm volatile("ld.global.cg.v8.b32 {%0, %1, %2, %3, %4, %5, %6, %7}, [%8];"
-                 : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]), "=r"(w[4]), "=r"(w[5]), "=r"(w[6]), "=r"(w[7])
-                 : "l"(p));
-}
 __device__ __forceinline__ void st8(float* p, const float* v) {
     asm volatile("st.global.cs.v8.f32 [%8], {%0, %1, %2, %3, %4, %5, %6, %7};"
                  ::"f"(v[0]), "f"(v[1]), "f"(v[2]), "f"(v[3]), "f"(v[4]), "f"(v[5]), "f"(v[6]), "f"(v[7]), "l"(p)
@@ -401,12 +428,13 @@ struct UpdateTable {
     float* o[CAP];
 };
 
-// FEW: the instance for launches of few tiles per phase, which knows narrow tiles and the claim gate.  As run-time branches in the one
-// kernel they cost the large launches 3-7 % (more live values in the single-thread loops of the producer and the MMA issuer).
-template <int CAP, bool FEW>
+// FORM is a template parameter because its branches, taken at run time in the one kernel, cost the large launches 3-7 % (more live
+// values in the single-thread loops of the producer and the MMA issuer).
+template <int CAP, NsForm FORM>
 __global__ void __cluster_dims__(2, 1, 1) __maxnreg__(TC_MAX_REGS)
 ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsProgram g,
                 const __grid_constant__ UpdateTable<CAP> upd, DeviceStatus* __restrict__ status) {
+    constexpr bool FEW = FORM == NsForm::Few, WHOLE = FORM == NsForm::Whole, BULK_STORES = FORM == NsForm::Spread;
     extern __shared__ uint8_t smem_raw[];
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;       // swizzle atoms need 1024-byte alignment
     const uint32_t epi_buf = base + NSLAB * SLAB_BYTES;
@@ -417,9 +445,11 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     const uint32_t bar_acc_empty = bar_acc_full + 16;           // 2 x 8 B (used in the leader)
     const uint32_t bar_ring_full = bar_acc_empty + 16;          // RING x 8 B
     const uint32_t bar_ring_empty = bar_ring_full + 8 * RING;   // RING x 8 B (used in the leader)
-    const uint32_t bar_stg_full = bar_ring_empty + 8 * RING;    // 2 x 8 B: a 64-column half of the staging buffer written (its 4 warps)
+    const uint32_t bar_stored = bar_ring_empty + 8 * RING;      // DONE_RING x 8 B: an item stored by the CTA's epilogue warps
+    const uint32_t bar_stg_full = bar_stored + 8 * DONE_RING;   // 2 x 8 B: a 64-column half of the staging buffer written (its 4 warps)
     const uint32_t bar_stg_empty = bar_stg_full + 16;           // 2 x 8 B: that half read by its store (store warp)
-    const uint32_t tmem_slot = bar_stg_empty + 16;              // 4 B + abort flag 4 B + 8 B pad
+    const uint32_t tmem_slot = bar_stg_empty + 16;              // 4 B + abort flag 4 B
+    const uint32_t lane_done = tmem_slot + 8;                   // 2 x 4 B: arrivals of the completed items of a lane (two per item)
     const uint32_t ring_items = tmem_slot + 16;                 // RING x 16 B
     // items per matrix of the phases before phase q (q = 0 .. P): phase q has phase_first[q + 1] - phase_first[q] items
     volatile unsigned int* phase_first = reinterpret_cast<volatile unsigned int*>(smem_raw + (ring_items + 16 * RING - smem_u32(smem_raw)));   // (NS_MAX_PHASES + 1) x 4 B
@@ -439,12 +469,14 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
 
     if (threadIdx.x == 0) {
         *abort_flag = 0;
+        asm volatile("st.shared.v2.b32 [%0], {%1, %1};" ::"r"(lane_done), "r"(0) : "memory");
         unsigned first = 0u;
         for (int q = 0; q <= NS_MAX_PHASES; ++q) { phase_first[q] = first; if (q < P) first += (unsigned)g.ph[q].items_per_mat; }
         for (int s = 0; s < NENT; ++s) { mbar_init(bar_full + 8 * s, 1); mbar_init(bar_empty + 8 * s, 1); }
         for (int a = 0; a < 2; ++a) { mbar_init(bar_acc_full + 8 * a, 1); mbar_init(bar_acc_empty + 8 * a, 2 * TC_EPI_WARPS); }
         for (int r = 0; r < RING; ++r) { mbar_init(bar_ring_full + 8 * r, 1); mbar_init(bar_ring_empty + 8 * r, RING_READERS); }
         for (int b = 0; b < 2; ++b) { mbar_init(bar_stg_full + 8 * b, TC_EPI_WARPS / 2); mbar_init(bar_stg_empty + 8 * b, 1); }
+        for (int b = 0; b < DONE_RING; ++b) mbar_init(bar_stored + 8 * b, TC_EPI_WARPS);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         #pragma unroll
         for (int i = 0; i < NS_MAPS; ++i) asm volatile("prefetch.tensormap [%0];" ::"l"(&maps.m[i]) : "memory");
@@ -485,6 +517,14 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
         dependency(it, ctr, need);
         return !ctr || wait_counter<false>(ctr, need, abort_flag, status, 6);
     };
+    // The same where a pair owns its matrices.  The first phase of a lane's next matrix waits for nothing: its iterate is its own, and
+    // the lane's A and B' are overwritten only by phases that wait for its own earlier ones, whose MMAs follow those of the
+    // matrix before.
+    auto wait_lane = [&](const Item& it) -> bool {
+        return wait_shared_counter(lane_done + 2 * (it.stop & 2), (unsigned)it.stop >> 2, abort_flag, status, 6);
+    };
+    // Index of the matrix in the tensors A, B' and C: the lane's where the pair owns its matrices, the matrix's own otherwise.
+    auto small_index = [&](const Item& it) -> int { return WHOLE && g.lane_tensors ? (int)(blockIdx.x & ~1u) + ((it.stop >> 1) & 1) : it.c; };
 
     // TMA loads of all k-slices of one item into the stage ring (both CTAs run this, each for its own rows).
     // producer's view of the slab ring: next entry, next slab, oldest entry not yet known to be free, free slabs, and
@@ -497,6 +537,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     auto produce = [&](const Item& it) -> bool {
         const NsPhase& p = g.ph[it.q];
         const TileCoord tc = decode_tile<FEW>(p, it.t);
+        const int za = p.a_map >= NS_TENSOR_A ? small_index(it) : it.c, zb = p.b_map >= NS_TENSOR_A ? small_index(it) : it.c;
         // K-major operands come as one box of 128 rows, MN-major ones as two boxes of 64 (the swizzle row is 64 elements)
         const CUtensorMap* a_box64 = &maps.m[p.a_map];
         const CUtensorMap* a_box128 = &maps.m[p.a_map + NS_TENSORS];
@@ -538,28 +579,28 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             const int k0 = kb * TC_BK;
             if (rank == 0) mbar_arrive_expect_tx(bar_full + 8 * e, tx_bytes);   // both CTAs' copies land here
             if (kb >= a_switch) {
-                tma_load_3d(sa, a_box64, full, m0, k0, it.c);
-                tma_load_3d(sa + BOX_BYTES, a_box64, full, m0 + TC_BOX, k0, it.c);
+                tma_load_3d(sa, a_box64, full, m0, k0, za);
+                tma_load_3d(sa + BOX_BYTES, a_box64, full, m0 + TC_BOX, k0, za);
             } else {
-                tma_load_3d(sa, a_box128, full, k0, m0, it.c);
+                tma_load_3d(sa, a_box128, full, k0, m0, za);
             }
             if (nb > 0) {
                 const uint32_t sb = sa + A_STAGE_BYTES;
                 if (narrow) {                 // 64 rows of B per CTA: one box in either form
                     const bool mn = kb >= b_switch0;
-                    tma_load_3d(sb, b_box64, full, mn ? n0 : k0, mn ? k0 : n0, it.c);
+                    tma_load_3d(sb, b_box64, full, mn ? n0 : k0, mn ? k0 : n0, zb);
                 } else if (kb >= b_switch0) {
-                    tma_load_3d(sb, b_box64, full, n0, k0, it.c);
-                    tma_load_3d(sb + BOX_BYTES, b_box64, full, n0 + TC_BOX, k0, it.c);
+                    tma_load_3d(sb, b_box64, full, n0, k0, zb);
+                    tma_load_3d(sb + BOX_BYTES, b_box64, full, n0 + TC_BOX, k0, zb);
                 } else {
-                    tma_load_3d(sb, b_box128, full, k0, n0, it.c);
+                    tma_load_3d(sb, b_box128, full, k0, n0, zb);
                 }
                 if (nb > 1) {
                     if (kb >= b_switch1) {
-                        tma_load_3d(sb + B_SUB_BYTES, b_box64, full, n0 + TC_BN, k0, it.c);
-                        tma_load_3d(sb + B_SUB_BYTES + BOX_BYTES, b_box64, full, n0 + TC_BN + TC_BOX, k0, it.c);
+                        tma_load_3d(sb + B_SUB_BYTES, b_box64, full, n0 + TC_BN, k0, zb);
+                        tma_load_3d(sb + B_SUB_BYTES + BOX_BYTES, b_box64, full, n0 + TC_BN + TC_BOX, k0, zb);
                     } else {
-                        tma_load_3d(sb + B_SUB_BYTES, b_box128, full, k0, n0 + TC_BN, it.c);
+                        tma_load_3d(sb + B_SUB_BYTES, b_box128, full, k0, n0 + TC_BN, zb);
                     }
                 }
             }
@@ -577,8 +618,9 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             bool ok = true;
             for (unsigned n = 0; ok; ++n) {
                 Item it;
-                if (!(ok = take_item(n, it, 8, true, TRACE_PTR(w_ring))) || it.stop) break;
+                if (!(ok = take_item(n, it, 8, true, TRACE_PTR(w_ring))) || (it.stop & 1)) break;
                 if (FEW && !(ok = wait_dependency(it))) break;
+                if (WHOLE && !(ok = wait_lane(it))) break;
                 fence_proxy_async_global();       // the acquire of the dependency (the scheduler's, or the one above) precedes these copies
                 ok = produce(it);
                 TRACE_ONLY(trace_add(NS_TRACE_PRODUCER_EMPTY, w_empty); trace_add(NS_TRACE_PRODUCER_RING, w_ring); w_empty = w_ring = 0;)
@@ -598,7 +640,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             bool ok = true;
             for (unsigned n = 0; ok; ++n) {
                 Item it;
-                if (!(ok = take_item(n, it, 9, true, TRACE_PTR(w_ring))) || it.stop) break;
+                if (!(ok = take_item(n, it, 9, true, TRACE_PTR(w_ring))) || (it.stop & 1)) break;
                 TRACE_ONLY(const uint32_t t_item0 = trace_clock(); uint32_t w_full = 0, w_acc = 0;)
                 const NsPhase& p = g.ph[it.q];
                 const TileCoord tc = decode_tile<FEW>(p, it.t);
@@ -681,52 +723,63 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     } else if (warp == STORE_WARP) {
         if (lane == 0) {
             // ---------------- store warp (both CTAs) ----------------
-            // Sends every staged phase of the epilogue to D with TMA stores (this thread owns the bulk-copy groups, so it is
-            // the one that can wait for them), frees the staging buffer when a phase has been read, and counts the item as
-            // done for its matrix and phase once all of its stores have completed.  The epilogue warps never wait for global
-            // memory.  It walks the items and their phases in the epilogue's order.
-            uint32_t staged = 0;
+            // Counts an item as done for its matrix and phase once it is in global memory, so that no epilogue warp waits for that.
+            // BULK_STORES: it also sends every staged phase of the epilogue to D with TMA stores (this thread owns the bulk-copy groups, so
+            // it is the one that can wait for them) and frees the staging buffer when a phase has been read; it walks the items
+            // and their phases in the epilogue's order.  Otherwise its fence covers the warps' own stores, which it has observed
+            // through the barrier.
+            uint32_t staged = 0, stored = 0;
             TRACE_ONLY(const uint32_t t_role0 = trace_clock(); uint32_t w_stg = 0;)
             bool ok = true;
             for (unsigned n = 0; ok; ++n) {
                 Item it;
-                if (!(ok = take_item(n, it, 12, true)) || it.stop) break;
+                if (!(ok = take_item(n, it, 12, true)) || (it.stop & 1)) break;
                 const NsPhase& p = g.ph[it.q];
-                if (p.fuse_update) continue;               // the epilogue writes the parameters itself; nothing is staged
-                const CUtensorMap* tma_d = &maps.m[p.d_map + NS_TENSORS];     // 64 columns x 128 rows per store
-                const TileCoord tc = decode_tile<FEW>(p, it.t);
-                const int m0 = tc.tm * TC_BM + (int)rank * CTA_M;
-                // The two 64-column halves of the staging buffer are separate buffers with their own barriers, filled by
-                // different warps: each half is stored as soon as it is full and handed back as soon as its own store has
-                // read it, the first half while the second store is still reading.
-                for (int u = 0; u < tc.nsub && ok; ++u) {
-                    for (int ph = 0; ph < 2 && ok; ++ph) {
-                        const int x0 = (tc.tn + u) * (FEW ? ns_tile_cols(p) : TC_BN) + ph * EPI_COLS;
-                        if (x0 >= p.N || (FEW && ph && p.narrow)) continue;
-                        if (!MONA_IN_BOUNDS(m0 < p.M + CTA_M && it.c < g.C && tc.tm < p.tiles_m, status, 106)) { ok = false; break; }
-                        #pragma unroll
-                        for (int bx = 0; bx < 2; ++bx) {
-                            if (!(ok = mbar_wait(bar_stg_full + 8 * bx, staged & 1u, abort_flag, status, 13, TRACE_PTR(w_stg)))) break;
-                            const int x = x0 + bx * TC_BOX;
-                            if (x < p.N && m0 < p.M) tma_store_3d(tma_d, epi_buf + bx * 2 * BOX_BYTES, x, m0, it.c);   // clipped at the extents
-                            bulk_commit();
+                if (p.fuse_update) continue;               // the epilogue writes the parameters itself; nothing waits for them
+                if (BULK_STORES) {
+                    const CUtensorMap* tma_d = &maps.m[p.d_map + NS_TENSORS];     // 64 columns x 128 rows per store
+                    const TileCoord tc = decode_tile<FEW>(p, it.t);
+                    const int m0 = tc.tm * TC_BM + (int)rank * CTA_M, zd = p.d_map >= NS_TENSOR_A ? small_index(it) : it.c;
+                    // The two 64-column halves of the staging buffer are separate buffers with their own barriers, filled by
+                    // different warps: each half is stored as soon as it is full and handed back as soon as its own store has
+                    // read it, the first half while the second store is still reading.
+                    for (int u = 0; u < tc.nsub && ok; ++u) {
+                        for (int ph = 0; ph < 2 && ok; ++ph) {
+                            const int x0 = (tc.tn + u) * (FEW ? ns_tile_cols(p) : TC_BN) + ph * EPI_COLS;
+                            if (x0 >= p.N || (FEW && ph && p.narrow)) continue;
+                            if (!MONA_IN_BOUNDS(m0 < p.M + CTA_M && it.c < g.C && tc.tm < p.tiles_m, status, 106)) { ok = false; break; }
+                            #pragma unroll
+                            for (int bx = 0; bx < 2; ++bx) {
+                                if (!(ok = mbar_wait(bar_stg_full + 8 * bx, staged & 1u, abort_flag, status, 13, TRACE_PTR(w_stg)))) break;
+                                const int x = x0 + bx * TC_BOX;
+                                if (x < p.N && m0 < p.M) tma_store_3d(tma_d, epi_buf + bx * 2 * BOX_BYTES, x, m0, zd);   // clipped at the extents
+                                bulk_commit();
+                            }
+                            if (!ok) break;
+                            bulk_wait_read<1>();               // the first store has read its half: its warps may refill it
+                            mbar_arrive_local(bar_stg_empty);
+                            bulk_wait_read<0>();
+                            mbar_arrive_local(bar_stg_empty + 8);
+                            ++staged;
                         }
-                        if (!ok) break;
-                        bulk_wait_read<1>();               // the first store has read its half: its warps may refill it
-                        mbar_arrive_local(bar_stg_empty);
-                        bulk_wait_read<0>();
-                        mbar_arrive_local(bar_stg_empty + 8);
-                        ++staged;
                     }
+                    if (!ok) break;
+                    bulk_wait_all();                           // the item's output is in global memory
+                } else {
+                    if (!(ok = mbar_wait(bar_stored + 8 * (stored % DONE_RING), (stored / DONE_RING) & 1u, abort_flag, status, 13, TRACE_PTR(w_stg)))) break;
+                    ++stored;
                 }
-                if (!ok) break;
-                bulk_wait_all();                           // the item's output is in global memory
-                fence_proxy_async_global();
-                __threadfence();
-                atomicAdd(g.done + (size_t)it.c * P + it.q, 1u);
+                fence_proxy_async_global();                // the copies that read the item go through the asynchronous proxy
+                if (WHOLE) {
+                    red_add_release_cluster(map_to_cta(lane_done + 2 * (it.stop & 2), 0), 1u);
+                    red_add_release_cluster(map_to_cta(lane_done + 2 * (it.stop & 2), 1), 1u);
+                } else {
+                    __threadfence();
+                    atomicAdd(g.done + (size_t)it.c * P + it.q, 1u);
+                }
                 TRACE_ONLY(trace_add(NS_TRACE_STORE_STAGED, w_stg); w_stg = 0; trace_add(NS_TRACE_ITEMS, 1u);)
             }
-            bulk_wait_all();           // shared memory must outlive the stores that read it
+            if (BULK_STORES) bulk_wait_all();           // shared memory must outlive the stores that read it
             TRACE_ONLY(trace_add(NS_TRACE_STORE_ROLE, trace_clock() - t_role0);)
         }
     } else if (warp == SCHED_WARP) {
@@ -746,6 +799,40 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             unsigned published = 0;
             TRACE_ONLY(const uint32_t t_role0 = trace_clock(); uint32_t w_slot = 0, w_dep = 0;)
             bool ok = true;
+            auto publish = [&](uint32_t slot, const Item& it) {
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring_items + 16 * slot), "r"(it.c), "r"(it.q), "r"(it.t), "r"(it.stop) : "memory");
+                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring_items_peer + 16 * slot), "r"(it.c), "r"(it.q), "r"(it.t), "r"(it.stop) : "memory");
+                fence_release_cluster();       // the item, and the acquire of its dependency before it, precede both arrivals
+                mbar_arrive_relaxed_cluster(ring_full_own + 8 * slot);
+                mbar_arrive_relaxed_cluster(ring_full_peer + 8 * slot);
+                ++published;
+            };
+            if constexpr (WHOLE) {
+                // Two lanes take turns, a phase each: while a phase of one matrix is finished and stored, the other lane's is
+                // computed.  A lane without a matrix claims the next one (asked for ahead, at the claim before).
+                struct Lane { int c, q, arrivals, live; } lane_a = {0, 0, 0, 1}, lane_b = {0, 0, 0, 1};
+                unsigned next = atomicAdd(g.work_counter, 1u);
+                auto turn = [&](Lane& l, int w) {
+                    if (!ok || !l.live) return;
+                    if (l.q == 0) {
+                        if (!(l.live = next < (unsigned)g.C)) return;
+                        l.c = (int)next;
+                        next = atomicAdd(g.work_counter, 1u);
+                    }
+                    const int items = (int)(phase_first[l.q + 1] - phase_first[l.q]);
+                    const int mark = (l.q ? l.arrivals << 2 : 0) | w << 1;
+                    for (int t = 0; t < items && ok; ++t) {
+                        const uint32_t slot = published % RING, par = (published / RING) & 1u;
+                        if ((ok = mbar_wait<true>(bar_ring_empty + 8 * slot, par ^ 1u, abort_flag, status, 7, TRACE_PTR(w_slot)))) publish(slot, Item{l.c, l.q, t, mark});
+                    }
+                    l.arrivals += 2 * items;
+                    if (++l.q == P) l.q = 0;
+                    TRACE_ONLY(trace_add(NS_TRACE_SCHED_SLOT, w_slot); w_slot = 0;)
+                };
+                while (ok && (lane_a.live | lane_b.live)) { turn(lane_a, 0); turn(lane_b, 1); }
+                const uint32_t slot = published % RING, par = (published / RING) & 1u;
+                if (ok && mbar_wait<true>(bar_ring_empty + 8 * slot, par ^ 1u, abort_flag, status, 7)) publish(slot, Item{0, 0, 0, 1});
+            } else {
             // The counter is always asked for one item more than has been published, so that its round trip (as long as that
             // of the dependency check) runs beside the dependency wait of the item before.  An item claimed early is still
             // published in order and only after everything it depends on, all of it with smaller indices, is complete.
@@ -771,12 +858,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 dependency(it, ctr, need);
                 if (!FEW && ctr && !(ok = wait_counter(ctr, need, abort_flag, status, 6, TRACE_PTR(w_dep)))) break;
                 // (no proxy fence here: this thread issues no copy; the producers fence after they have taken the item)
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring_items + 16 * slot), "r"(it.c), "r"(it.q), "r"(it.t), "r"(it.stop) : "memory");
-                asm volatile("st.shared::cluster.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(ring_items_peer + 16 * slot), "r"(it.c), "r"(it.q), "r"(it.t), "r"(it.stop) : "memory");
-                fence_release_cluster();       // the item, and the acquire of its dependency before it, precede both arrivals
-                mbar_arrive_relaxed_cluster(ring_full_own + 8 * slot);
-                mbar_arrive_relaxed_cluster(ring_full_peer + 8 * slot);
-                ++published;
+                publish(slot, it);
                 if (FEW && g.gate && !it.stop) {
                     const int nsub = decode_tile<FEW>(g.ph[it.q], it.t).nsub;
                     last_acc = nsub == 2 ? 1u : acc_next;
@@ -785,6 +867,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 }
                 TRACE_ONLY(trace_add(NS_TRACE_SCHED_SLOT, w_slot); trace_add(NS_TRACE_SCHED_DEPENDENCY, w_dep); w_slot = w_dep = 0;)
                 if (it.stop) break;
+            }
             }
             TRACE_ONLY(trace_add(NS_TRACE_SCHED_ROLE, trace_clock() - t_role0);)
         }
@@ -802,51 +885,75 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
         const int row_in_cta = quad * 32 + lane;
         const uint32_t lane_base = (uint32_t)(quad * 32) << 16;
         const uint32_t acc_empty_leader = map_to_cta(bar_acc_empty, 0);
-        // position of this thread's row inside the staging buffer: one 128-row box per column half, 128-byte rows
-        const uint32_t stage_off = (uint32_t)half * (2u * BOX_BYTES) + (uint32_t)row_in_cta * 128u;
-        const uint32_t swz = (uint32_t)row_in_cta & 7u;
+        // A warp's own staging, 32 rows of 128 bytes whose 16-byte chunks are permuted by the row: a thread writes or reads its own
+        // row, or the warp four rows at a time, eight lanes to a row, without bank conflicts either way.
+        // (The four warps of a column half are neighbours: their rows together are one box of a TMA store with the 128-byte swizzle.)
+        const uint32_t stage = epi_buf + (uint32_t)(half * 4 + quad) * EPI_WARP_BYTES;
+        const uint32_t own_row = stage + (uint32_t)lane * 128u + (((uint32_t)lane & 7u) << 4);
+        auto own_addr = [&](int q) -> uint32_t { return own_row ^ (uint32_t)(q << 4); };
+        const int line_row = lane >> 3, line_chunk = lane & 7;     // the warp's view: instruction i covers rows 4 i + line_row
+        const uint32_t line = stage + (uint32_t)line_row * 128u + (uint32_t)((line_chunk ^ line_row) << 4);
+        auto line_addr = [&](int i) -> uint32_t { return (i & 1 ? line ^ 64u : line) + (uint32_t)i * 512u; };
         uint32_t acc_next = 0, acc_par = 0;   // acc_par: one use-parity bit per accumulator
-        uint32_t staged = 0;                  // staging phases handed to the store warp so far
+        uint32_t stored = 0, staged = 0;      // items stored, phases handed to the store warp so far
         TRACE_ONLY(const uint32_t t_role0 = trace_clock(); uint32_t w_ring = 0, w_accf = 0, w_stge = 0;)
         bool alive = true;
-        // 128 packed columns of this thread's row go to the staging buffer; the store warp sends them on
-        auto put_phase = [&](const uint4* pk) -> bool {
-            if (!mbar_wait(bar_stg_empty + 8 * half, (staged & 1u) ^ 1u, abort_flag, status, 11, TRACE_PTR(w_stge))) return false;   // the previous phase of this half has been read
-            if (!MONA_IN_BOUNDS(stage_off + 128u <= EPI_BUF_BYTES, status, 104)) return false;
+        // The staging is this warp's to write (with TMA stores: the previous phase of its half has been read).
+        auto staging_free = [&]() -> bool {
+            return !BULK_STORES || mbar_wait(bar_stg_empty + 8 * half, (staged & 1u) ^ 1u, abort_flag, status, 11, TRACE_PTR(w_stge));
+        };
+        // 64 packed columns of the warp's rows, from column `col` on, go to D through the staging, which is free: by the store warp, or
+        // here, four whole lines per store instruction.  (A thread owns a row: from registers an instruction would touch 32 lines.)
+        auto put_columns = [&](const uint4* pk, __nv_bfloat16* d, int row0, int col, const NsPhase& p) {
             #pragma unroll
-            for (int q = 0; q < 8; ++q) {
-                const uint32_t addr = epi_buf + stage_off + (((uint32_t)q ^ swz) << 4);
-                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(addr), "r"(pk[q].x), "r"(pk[q].y), "r"(pk[q].z), "r"(pk[q].w) : "memory");
+            for (int q = 0; q < 8; ++q)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(own_addr(q)), "r"(pk[q].x), "r"(pk[q].y), "r"(pk[q].z), "r"(pk[q].w) : "memory");
+            if (BULK_STORES) {
+                fence_proxy_async_shared();            // generic-proxy writes above must be visible to the TMA engine
+                __syncwarp();
+                if (lane == 0) mbar_arrive_local(bar_stg_full + 8 * half);
+                ++staged;
+                return;
             }
-            fence_proxy_async_shared();            // generic-proxy writes above must be visible to the TMA engine
             __syncwarp();
-            if (lane == 0) mbar_arrive_local(bar_stg_full + 8 * half);
-            ++staged;
-            return true;
+            const int c = col + 8 * line_chunk;
+            __nv_bfloat16* at = d + (long long)(row0 + line_row) * p.ld + c;
+            uint4 r[8];
+            #pragma unroll
+            for (int i = 0; i < 8; ++i)
+                asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(r[i].x), "=r"(r[i].y), "=r"(r[i].z), "=r"(r[i].w) : "r"(line_addr(i)) : "memory");
+            #pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                if (row0 + 4 * i + line_row < p.M && c < p.N && MONA_IN_BOUNDS(at + 8 <= p.d + (long long)g.C * p.mat_stride, status, 104)) *reinterpret_cast<uint4*>(at) = r[i];
+                at += 4 * p.ld;
+            }
+            __syncwarp();
         };
         for (unsigned n = 0; alive; ++n) {
             Item it;
             if (!take_item(n, it, 10, false, TRACE_PTR(w_ring))) break;
             __syncwarp();
             if (lane == 0) mbar_arrive_slot_read(ring_empty_leader + 8 * (n % RING), it.c, it.q, it.t, it.stop);   // every lane has its copy of the item
-            if (it.stop) break;
+            if (it.stop & 1) break;
             TRACE_ONLY(const uint32_t t_item0 = trace_clock();)
             const NsPhase& p = g.ph[it.q];
             const TileCoord tc = decode_tile<FEW>(p, it.t);
             const int m0 = tc.tm * TC_BM + (int)rank * CTA_M;
             const int gr = m0 + row_in_cta;
             const bool row_ok = gr < p.M;
-            const long long row_off = (long long)it.c * p.mat_stride + (long long)gr * p.ld;
-            if (FEW && p.cin) {
+            const int zs = small_index(it);          // of the axpy operand and of delta
+            const int row0 = m0 + quad * 32;         // the warp's rows
+            __nv_bfloat16* const d = p.d ? p.d + (long long)(p.d_map >= NS_TENSOR_A ? zs : it.c) * p.mat_stride : nullptr;
+            if ((WHOLE || FEW) && p.cin) {
                 bool there = true;
-                if (lane == 0) there = wait_dependency(it);
+                if (lane == 0) there = WHOLE ? wait_lane(it) : wait_dependency(it);
                 if (!__shfl_sync(0xffffffffu, there, 0)) break;
                 __syncwarp();        // orders the other lanes' loads of the operand and of delta behind lane 0's acquire (a shuffle orders nothing)
             }
             float post = 1.0f;
             if (p.post_mode) { const float sc = g.inv_norm[it.c]; post = p.post_mode == 2 ? sc * sc : sc; }
             // correction of this row's diagonal element of A (written earlier in this launch by another CTA: read from L2)
-            const float delta = row_ok && p.delta_in ? __ldcg(p.delta_in + (size_t)it.c * p.M + gr) : 0.0f;
+            const float delta = row_ok && p.delta_in ? __ldcg(p.delta_in + (size_t)zs * p.M + gr) : 0.0f;
             const float c2 = p.c2 * post, c1 = fmaf(2.0f * c2, delta, p.c1 * post);
             const uint32_t acc0 = tc.nsub == 2 ? 0u : acc_next;
             if (!p.cin && !p.fuse_update) {
@@ -870,25 +977,23 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                         const uint32_t t_base = tmem_base + lane_base + acc * TC_BN + half * 64;
                         #pragma unroll
                         for (int ph = 0; ph < NPH; ++ph) {
+                            float v[64];
+                            tmem_ld32(t_base + ph * EPI_COLS, v);
+                            tmem_ld32(t_base + ph * EPI_COLS + 32, v + 32);
+                            tmem_ld_wait();
                             #pragma unroll
-                            for (int h = 0; h < 2; ++h) {
-                                float v[32];
-                                tmem_ld32(t_base + ph * EPI_COLS + 32 * h, v);
-                                tmem_ld_wait();
-                                #pragma unroll
-                                for (int j = 0; j < 32; ++j) v[j] *= c2;
-                                if (NSUB == 1 && p.delta_out) {
-                                    const int dj = gr - ((tc.tn + u) * (EPI_COLS * NPH) + ph * EPI_COLS + half * 64 + 32 * h);
-                                    if (row_ok && dj >= 0 && dj < 32) {       // this row's diagonal element is among the 32
-                                        float d = 0.f;
-                                        #pragma unroll
-                                        for (int j = 0; j < 32; ++j) d = j == dj ? v[j] : d;
-                                        p.delta_out[(size_t)it.c * p.M + gr] = d - __bfloat162float(__float2bfloat16_rn(d));
-                                    }
+                            for (int j = 0; j < 64; ++j) v[j] *= c2;
+                            if (NSUB == 1 && p.delta_out) {
+                                const int dj = gr - ((tc.tn + u) * (EPI_COLS * NPH) + ph * EPI_COLS + half * 64);
+                                if (row_ok && dj >= 0 && dj < 64) {       // this row's diagonal element is among the 64
+                                    float dg = 0.f;
+                                    #pragma unroll
+                                    for (int j = 0; j < 64; ++j) dg = j == dj ? v[j] : dg;
+                                    p.delta_out[(size_t)zs * p.M + gr] = dg - __bfloat162float(__float2bfloat16_rn(dg));
                                 }
-                                #pragma unroll
-                                for (int q = 0; q < 4; ++q) pk[u][ph][4 * h + q] = pack8(v + 8 * q);
                             }
+                            #pragma unroll
+                            for (int q = 0; q < 8; ++q) pk[u][ph][q] = pack8(v + 8 * q);
                         }
                         tc_fence_before();
                         __syncwarp();
@@ -897,102 +1002,131 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                     #pragma unroll
                     for (int u = 0; u < NSUB; ++u)
                         #pragma unroll
-                        for (int ph = 0; ph < NPH; ++ph)
-                            if ((tc.tn + u) * (EPI_COLS * NPH) + ph * EPI_COLS < p.N && !put_phase(pk[u][ph])) return false;
+                        for (int ph = 0; ph < NPH; ++ph) {
+                            const int c0 = (tc.tn + u) * (EPI_COLS * NPH) + ph * EPI_COLS;
+                            if (c0 >= p.N) continue;
+                            if (!staging_free()) return false;
+                            put_columns(pk[u][ph], d, row0, c0 + half * 64, p);
+                        }
                     return true;
                 };
                 using std::integral_constant;
                 if (tc.nsub == 2) alive = pack_and_stage(integral_constant<int, 2>{}, integral_constant<int, 2>{});
                 else if (!(FEW && p.narrow)) alive = pack_and_stage(integral_constant<int, 1>{}, integral_constant<int, 2>{});
                 else alive = pack_and_stage(integral_constant<int, 1>{}, integral_constant<int, FEW ? 1 : 2>{});
-            } else
-            for (int u = 0; u < tc.nsub && alive; ++u) {
-                const uint32_t acc = acc0 + u;
-                const int n0 = (tc.tn + u) * (FEW ? ns_tile_cols(p) : TC_BN);
-                const int nphases = (p.N - n0 > EPI_COLS && !(FEW && p.narrow)) ? 2 : 1;
-                // Operand of the axpy term: this thread's 64 values of a phase (128 bytes), requested before the accumulator is
-                // ready (first phase) or before the previous phase is staged (second), so that the round trip is hidden.  It was written by other CTAs of this
-                // launch, so it is read from L2 (.cg), never from a line L1 may still hold from an earlier iteration.  A thread
-                // owns a row, so a warp's load touches 32 lines whatever its width: 32-byte accesses halve the requests.
-                uint32_t cin_w[32];
-                const bool cin_v8 = p.cin && ((p.ld | p.mat_stride | (long long)p.N) & 15) == 0 && (reinterpret_cast<uintptr_t>(p.cin) & 31) == 0;
-                auto load_cin = [&](int ph) {
-                    const int gc0 = n0 + ph * EPI_COLS + half * 64;
-                    if (cin_v8) {
+            } else if (p.cin) {
+                // b A + c A^2 + a I.  The axpy operand, A of the same tile, is requested before the accumulator is awaited, in whole lines
+                // like the stores, and handed to the rows' owners through the staging.  It was written by other CTAs of this launch,
+                // so it is read from L2 (.cg), never from a line L1 may still hold from an earlier iteration.
+                auto poly = [&](auto nph_c) -> bool {
+                    constexpr int NPH = decltype(nph_c)::value;
+                    const uint32_t acc = acc0;
+                    const int n0 = tc.tn * (EPI_COLS * NPH) + half * 64;
+                    uint4 cin[NPH][8];
+                    #pragma unroll
+                    for (int ph = 0; ph < NPH; ++ph) {
+                        const int c = n0 + ph * EPI_COLS + 8 * line_chunk;
+                        const __nv_bfloat16* at = p.cin + (long long)zs * p.cin_stride + (long long)(row0 + line_row) * p.ld + c;
                         #pragma unroll
-                        for (int q = 0; q < 4; ++q) {
-                            if (row_ok && gc0 + 16 * q < p.N && MONA_IN_BOUNDS(row_off + gc0 + 16 * q + 16 <= (long long)g.C * p.mat_stride, status, 105)) ld8cg(p.cin + row_off + gc0 + 16 * q, cin_w + 8 * q);
-                            else {
-                                #pragma unroll
-                                for (int j = 0; j < 8; ++j) cin_w[8 * q + j] = 0u;
-                            }
-                        }
-                    } else {
-                        #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            uint4 r = make_uint4(0u, 0u, 0u, 0u);
-                            if (row_ok && gc0 + 8 * q < p.N && MONA_IN_BOUNDS(row_off + gc0 + 8 * q + 8 <= (long long)g.C * p.mat_stride, status, 105)) r = __ldcg(reinterpret_cast<const uint4*>(p.cin + row_off + gc0 + 8 * q));
-                            cin_w[4 * q] = r.x; cin_w[4 * q + 1] = r.y; cin_w[4 * q + 2] = r.z; cin_w[4 * q + 3] = r.w;
+                        for (int i = 0; i < 8; ++i) {
+                            cin[ph][i] = make_uint4(0u, 0u, 0u, 0u);
+                            if (row0 + 4 * i + line_row < p.M && c < p.N && MONA_IN_BOUNDS(at + 8 <= p.cin + (long long)g.C * p.cin_stride, status, 105)) cin[ph][i] = __ldcg(reinterpret_cast<const uint4*>(at));
+                            at += 4 * p.ld;
                         }
                     }
+                    if (!mbar_wait(bar_acc_full + 8 * acc, (acc_par >> acc) & 1u, abort_flag, status, 4, TRACE_PTR(w_accf))) return false;
+                    tc_fence_after();
+                    acc_par ^= 1u << acc;
+                    const uint32_t t_base = tmem_base + lane_base + acc * TC_BN + half * 64;
+                    #pragma unroll
+                    for (int ph = 0; ph < NPH; ++ph) {
+                        const bool any = n0 - half * 64 + ph * EPI_COLS < p.N;        // (a phase beyond N has nothing to store)
+                        if (any && !staging_free()) return false;
+                        float v[64];
+                        tmem_ld32(t_base + ph * EPI_COLS, v);
+                        tmem_ld32(t_base + ph * EPI_COLS + 32, v + 32);
+                        #pragma unroll
+                        for (int i = 0; i < 8; ++i) if (any)
+                            asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(line_addr(i)), "r"(cin[ph][i].x), "r"(cin[ph][i].y), "r"(cin[ph][i].z), "r"(cin[ph][i].w) : "memory");
+                        __syncwarp();
+                        tmem_ld_wait();
+                        if (ph == NPH - 1) {
+                            // this warp has read all it needs from the accumulator: hand it back to the MMA issuer
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive_remote(acc_empty_leader + 8 * acc);
+                        }
+                        const int gc0 = n0 + ph * EPI_COLS;
+                        uint4 pk[8];
+                        #pragma unroll
+                        for (int q = 0; q < 8; ++q) {
+                            uint32_t w[4];
+                            asm volatile("ld.shared.v4.b32 {%0, %1, %2, %3}, [%4];" : "=r"(w[0]), "=r"(w[1]), "=r"(w[2]), "=r"(w[3]) : "r"(own_addr(q)) : "memory");
+                            #pragma unroll
+                            for (int h = 0; h < 4; ++h) {
+                                v[8 * q + 2 * h] = fmaf(c1, __uint_as_float(w[h] << 16), c2 * v[8 * q + 2 * h]);
+                                v[8 * q + 2 * h + 1] = fmaf(c1, __uint_as_float(w[h] & 0xffff0000u), c2 * v[8 * q + 2 * h + 1]);
+                            }
+                        }
+                        if (gr >= gc0 && gr < gc0 + 64) {
+                            // the row's diagonal element: + a, and b A(i,i) with the exact A(i,i)
+                            const float dg = fmaf(p.c1, delta, p.diag_add);
+                            #pragma unroll
+                            for (int j = 0; j < 64; ++j) v[j] += (gc0 + j == gr) ? dg : 0.f;
+                        }
+                        #pragma unroll
+                        for (int q = 0; q < 8; ++q) pk[q] = pack8(v + 8 * q);
+                        __syncwarp();
+                        if (any) put_columns(pk, d, row0, gc0, p);
+                    }
+                    return true;
                 };
-                if (p.cin) load_cin(0);
+                if (FEW && p.narrow) alive = poly(std::integral_constant<int, 1>{});
+                else alive = poly(std::integral_constant<int, 2>{});
+            } else
+            for (int u = 0; u < tc.nsub && alive; ++u) {
+                // Eq. muon_update on this thread's parameters, 64 columns at a time: W <- (W - eta lambda W) - eta gamma O.  Nothing in the
+                // launch reads these stores (the phase is the last one of the step), so they need no completion signal.
+                const uint32_t acc = acc0 + u;
+                const int n0 = (tc.tn + u) * TC_BN;
+                const int nphases = p.N - n0 > EPI_COLS ? 2 : 1;
                 if (!mbar_wait(bar_acc_full + 8 * acc, (acc_par >> acc) & 1u, abort_flag, status, 4, TRACE_PTR(w_accf))) { alive = false; break; }
                 tc_fence_after();
                 acc_par ^= 1u << acc;
                 const uint32_t t_base = tmem_base + lane_base + acc * TC_BN + half * 64;
-                for (int ph = 0; ph < nphases && alive; ++ph) {
+                for (int ph = 0; ph < nphases; ++ph) {
                     float v[64];
                     tmem_ld32(t_base + ph * EPI_COLS, v);
                     tmem_ld32(t_base + ph * EPI_COLS + 32, v + 32);
                     tmem_ld_wait();
                     if (ph == nphases - 1) {
-                        // this warp has read all it needs from the accumulator: hand it back to the MMA issuer
                         tc_fence_before();
                         __syncwarp();
                         if (lane == 0) mbar_arrive_remote(acc_empty_leader + 8 * acc);
                     }
                     const int gc0 = n0 + ph * EPI_COLS + half * 64;
-                    if (p.cin) {
-                        #pragma unroll
-                        for (int h = 0; h < 32; ++h) {
-                            v[2 * h] = fmaf(c1, __uint_as_float(cin_w[h] << 16), c2 * v[2 * h]);
-                            v[2 * h + 1] = fmaf(c1, __uint_as_float(cin_w[h] & 0xffff0000u), c2 * v[2 * h + 1]);
-                        }
-                        if (gr >= gc0 && gr < gc0 + 64) {
-                            // the row's diagonal element: + a, and b A(i,i) with the exact A(i,i)
-                            const float d = fmaf(p.c1, delta, p.diag_add);
+                    if (!row_ok) continue;
+                    #pragma unroll
+                    for (int j = 0; j < 64; ++j) v[j] *= c2;
+                    float* wrow = upd.w[it.c] + (long long)gr * p.ld + gc0;
+                    float* orow = upd.o[it.c] ? upd.o[it.c] + (long long)gr * p.ld + gc0 : nullptr;
+                    #pragma unroll
+                    for (int q = 0; q < 8; ++q) {
+                        if (gc0 + 8 * q < p.N) {
+                            float w8[8];
+                            ld8(wrow + 8 * q, w8);
                             #pragma unroll
-                            for (int j = 0; j < 64; ++j) v[j] += (gc0 + j == gr) ? d : 0.f;
-                        }
-                        if (ph + 1 < nphases) load_cin(ph + 1);
-                    } else {
-                        #pragma unroll
-                        for (int j = 0; j < 64; ++j) v[j] *= c2;
-                    }
-                    if (!p.fuse_update) {
-                        uint4 pk[8];
-                        #pragma unroll
-                        for (int q = 0; q < 8; ++q) pk[q] = pack8(v + 8 * q);
-                        alive = put_phase(pk);
-                    } else if (row_ok) {
-                        // Eq. muon_update on this thread's 64 parameters: W <- (W - eta lambda W) - eta gamma O.  Nothing in the
-                        // launch reads these stores (the phase is the last one of the step), so they need no completion signal.
-                        float* wrow = upd.w[it.c] + (long long)gr * p.ld + gc0;
-                        float* orow = upd.o[it.c] ? upd.o[it.c] + (long long)gr * p.ld + gc0 : nullptr;
-                        #pragma unroll
-                        for (int q = 0; q < 8; ++q) {
-                            if (gc0 + 8 * q < p.N) {
-                                float w8[8];
-                                ld8(wrow + 8 * q, w8);
-                                #pragma unroll
-                                for (int j = 0; j < 8; ++j) w8[j] = fmaf(-g.eta_gamma, v[8 * q + j], fmaf(-g.eta_lambda, w8[j], w8[j]));
-                                st8(wrow + 8 * q, w8);
-                                if (orow) st8(orow + 8 * q, v + 8 * q);
-                            }
+                            for (int j = 0; j < 8; ++j) w8[j] = fmaf(-g.eta_gamma, v[8 * q + j], fmaf(-g.eta_lambda, w8[j], w8[j]));
+                            st8(wrow + 8 * q, w8);
+                            if (orow) st8(orow + 8 * q, v + 8 * q);
                         }
                     }
                 }
+            }
+            if (!BULK_STORES) {
+                __syncwarp();
+                if (lane == 0) mbar_arrive_local(bar_stored + 8 * (stored % DONE_RING));
+                ++stored;
             }
             if (tc.nsub == 1) acc_next ^= 1u;
 #ifdef MONA_TRACE
@@ -1102,9 +1236,10 @@ cudaError_t ns_configure(int* max_pairs) {
     cudaError_t e;
     if ((e = cudaGetDevice(&dev)) != cudaSuccess) return e;
     if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<1, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<1, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<MAXC, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<1, NsForm::Spread>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<1, NsForm::Few>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<1, NsForm::Whole>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(ns_chunk_kernel<MAXC, NsForm::Spread>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_TOTAL)) != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(sms / 2 * 2));
     cfg.blockDim = dim3(TC_THREADS);
@@ -1115,7 +1250,7 @@ cudaError_t ns_configure(int* max_pairs) {
     cfg.attrs = &attr;
     cfg.numAttrs = 1;
     int clusters = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(&clusters, ns_chunk_kernel<1, false>, &cfg)) != cudaSuccess) return e;
+    if ((e = cudaOccupancyMaxActiveClusters(&clusters, ns_chunk_kernel<1, NsForm::Spread>, &cfg)) != cudaSuccess) return e;
     if (clusters < 1) return cudaErrorInvalidConfiguration;
     *max_pairs = clusters < sms / 2 ? clusters : sms / 2;
     return cudaSuccess;
@@ -1125,15 +1260,18 @@ cudaError_t launch_ns_program(const NsMaps& maps, const NsProgram& g, const NsUp
                               DeviceStatus* status, cudaStream_t stream) {
     if (g.total_items == 0) return cudaSuccess;
     if (g.max_pairs > 0 && g.max_pairs < max_pairs) max_pairs = g.max_pairs;
-    const int pairs = (long long)g.total_items < (long long)max_pairs ? (int)g.total_items : max_pairs;
+    const long long units = g.form == NsForm::Whole ? g.C : (long long)g.total_items;
+    const int pairs = units < (long long)max_pairs ? (int)units : max_pairs;
     if (up.w) {
         UpdateTable<MAXC> table;
         for (int c = 0; c < g.C; ++c) { table.w[c] = up.w[c]; table.o[c] = up.o ? up.o[c] : nullptr; }
-        ns_chunk_kernel<MAXC, false><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, table, status);
-    } else if (g.few) {
-        ns_chunk_kernel<1, true><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
+        ns_chunk_kernel<MAXC, NsForm::Spread><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, table, status);
+    } else if (g.form == NsForm::Few) {
+        ns_chunk_kernel<1, NsForm::Few><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
+    } else if (g.form == NsForm::Whole) {
+        ns_chunk_kernel<1, NsForm::Whole><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
     } else {
-        ns_chunk_kernel<1, false><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
+        ns_chunk_kernel<1, NsForm::Spread><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
     }
     return cudaGetLastError();
 }

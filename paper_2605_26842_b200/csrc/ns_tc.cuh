@@ -14,6 +14,7 @@ constexpr int TC_BK = 64;       // k-slice per pipeline stage: 64 bf16 = one 128
 constexpr int TC_BOX = 64;      // every TMA box is 64 bf16 wide (one 128-byte swizzle row) and 64 or 128 rows high
 constexpr int NS_MAX_PHASES = 16;   // five iterations: 3 GEMMs each, 7 for two iterations taken together; longer ones take several launches
 constexpr int NS_TENSORS = 5;       // operand tensors of a chunk: X ping, X pong, A, B', C (in the memory of X pong)
+constexpr int NS_TENSOR_A = 2;      // the first of the s x s ones
 constexpr int NS_MAPS = 2 * NS_TENSORS;   // each with 64-row boxes (index t) and with 128-row boxes (index t + NS_TENSORS)
 
 // One batched GEMM ("phase") of the iteration of Eq. newton_schulz over the C matrices of a chunk:
@@ -43,9 +44,11 @@ struct NsPhase {
                                 //    one staged slice of the A operand, one per tensor-memory accumulator
     int narrow;                 // 1: tiles of 128 instead of 256 columns (not with `wide`)
     int tiles_m, tiles_n, items_per_mat;   // filled by ns_phase_plan(); items are macro-tiles when `wide`
+    __nv_bfloat16* d;           // tensor d_map; null when fuse_update
     const __nv_bfloat16* cin;   // may be null; [C][M][N] like D; lower-block-stored when D is symmetric
-    long long ld, mat_stride;   // leading dimension and per-matrix stride of cin (and of the fp32 parameter when
-                                // fuse_update), in elements
+    long long ld, mat_stride;   // leading dimension (of cin, and of the fp32 parameter when fuse_update, too) and per-matrix stride of
+                                // D, in elements
+    long long cin_stride;       // per-matrix stride of cin
     float c1, c2;
     float diag_add;             // added to D(i,i): folds the a*X term of the quintic into B' = b A + c A^2 + a I
     int post_mode;              // 0: post = 1, 1: post = inv_norm[c], 2: post = inv_norm[c]^2
@@ -56,6 +59,13 @@ struct NsPhase {
     float* delta_out;
     const float* delta_in;
 };
+
+// How a launch deals its work to the CTA pairs; each form is a kernel instance of its own.
+//   Spread : items of all matrices in the order of NsItemCursor, from one counter
+//   Few    : the same for launches of few tiles per phase; knows narrow phases and the claim gate (not with fuse_update)
+//   Whole  : a pair takes whole matrices, two at a time (its two lanes); X' overwrites X (not with fuse_update or narrow phases).
+//            Only for s <= 256, where a tile of X' reads no columns of X but its own
+enum class NsForm : int { Spread = 0, Few = 1, Whole = 2 };
 
 // Everything one launch needs: the phases in execution order and the scheduler state.  Work items are handed
 // out through one atomic counter in a fixed order in which every item comes after the items it depends on
@@ -72,7 +82,8 @@ struct NsProgram {
     unsigned int* work_counter; // zero at launch
     unsigned int* done;         // C * P words, zero at launch
     float eta_lambda, eta_gamma;    // fuse_update: eta * lambda and eta * gamma
-    int few;                    // 1: the launch runs the kernel instance that knows narrow phases and the gate (not with fuse_update)
+    NsForm form;
+    int lane_tensors;           // Whole: 1: A, B' and C are indexed by pair and lane (2 per pair) instead of by matrix
     int gate;                   // 1: a pair takes its next item only when the MMAs of the last one are complete.  0: a few items
                                 //    ahead.  For launches of about one round of items per phase, where pairs that come first
                                 //    would hoard items that others are idle for

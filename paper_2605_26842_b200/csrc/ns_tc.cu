@@ -186,6 +186,18 @@ __device__ __forceinline__ bool mbar_try_wait(uint32_t bar, uint32_t parity) {
     }
     return ok != 0;
 }
+// Whether the phase is complete, without waiting.
+__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ void latch_timeout(volatile int* abort_flag, DeviceStatus* status, unsigned site) {
     *abort_flag = 1;
     atomicOr(&status->flags, STATUS_TIMEOUT);
@@ -663,6 +675,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 tc_fence_after();
                 const uint32_t d0 = tmem_base + acc0 * TC_BN, d1 = d0 + TC_BN;
                 uint32_t accum = 0u;
+                bool ready = mbar_test(bar_full + 8 * ment_e, ment_par);
                 const uint32_t nslab = shared_ab ? 1u : 1u + (uint32_t)tc.nsub;
                 for (int kb = 0; kb < num_kb; ++kb) {
                     // same slab walk as the producer's
@@ -672,8 +685,12 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                     if (!MONA_IN_BOUNDS(pos + nslab <= NSLAB && tc.tm < p.tiles_m && tc.tn + tc.nsub <= p.tiles_n, status, 103)) { ok = false; break; }
                     const uint32_t stage_lo = (base + pos * SLAB_BYTES) >> 4;
                     // no tcgen05 fence here: the operands arrive through the asynchronous proxy and the barrier orders them
-                    if (!(ok = mbar_wait(bar_full + 8 * e, ment_par, abort_flag, status, 3, TRACE_PTR(w_full)))) break;
+                    if (!ready && !(ok = mbar_wait(bar_full + 8 * e, ment_par, abort_flag, status, 3, TRACE_PTR(w_full)))) break;
                     if (++ment_e == NENT) { ment_e = 0; ment_par ^= 1u; }
+                    // The next slice's barrier is asked before this one's MMAs are issued: on its own a successful wait is 130 cycles of the
+                    // 430 that four N = 128 MMAs, their commit and the wait take one thread to issue (47 per MMA, 45 the commit), where
+                    // the tensor pipe needs 256 (one 256 x 512 matrix 88 -> 85 us per step, a mixed small set 116 -> 112).
+                    ready = kb + 1 < num_kb && mbar_test(bar_full + 8 * ment_e, ment_par);
                     const uint32_t a_mn = kb >= a_switch ? 1u : 0u, b_mn0 = kb >= b_switch[0] ? 1u : 0u;
                     // one k-step of 16 advances 32 B inside the swizzle row (K-major) or 16 rows = 2048 B (MN-major)
                     const uint32_t a_step = a_mn ? (2048u >> 4) : (32u >> 4), b_step0 = b_mn0 ? (2048u >> 4) : (32u >> 4);

@@ -128,12 +128,14 @@ mona_status mona_default_hparams(mona_hparams* hp);
  *                        The workspace holds two chunks and the small buckets that run beside them: at most 2.25
  *                        times the budget (or the iterates of the largest matrix in fp32, where that is more), and
  *                        some 4 MiB.
- *   fuse_update        : 0 (default): O_k is stored in bf16 and a separate elementwise kernel applies Eq. muon_update.
+ *   fuse_update        : 0 (default): Eq. muon_update is applied from O_k rounded to bf16: inside the last X' = B' X of a whole step
+ *                        on the tensor-core path, by a separate elementwise kernel where O_k is asked for, phases run apart or a
+ *                        stride is no multiple of 16 bytes.  The results are the same bits.
  *                        1: on the tensor-core path the last X' = B' X of a step applies the update in its epilogue
  *                        (fp32 O_k straight from the accumulator, no bf16 copy of O_k written and re-read, one launch
  *                        fewer per chunk).  The two differ by the bf16 rounding of O_k only.  Measured slower on the
- *                        benchmark sets: a thread owns a row of the accumulator, so its fp32 read-modify-write of W
- *                        touches 32 lines per warp instruction and sits, unhidden, in the macro-tile's epilogue.
+ *                        benchmark sets: a thread owns a row of the accumulator, and its fp32 read-modify-write of W
+ *                        touches 32 lines per warp instruction.
  *   ns_delay           : how many matrices apart consecutive Newton-Schulz GEMMs of one matrix sit in the kernel's
  *                        work order (0 = the default, 20; at most 1024; a value >= the chunk's matrix count
  *                        runs the chunk GEMM by GEMM).  Larger values hide the dependency latency

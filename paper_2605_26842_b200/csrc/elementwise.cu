@@ -143,6 +143,7 @@ constexpr int SMALL_TABLE = 32;
 template <int CAP>
 struct GradTable {
     const void* g[CAP];
+    float* w[CAP];
     int gid[CAP];
 };
 template <int CAP>
@@ -162,7 +163,9 @@ __global__ void __launch_bounds__(EW_THREADS, 9)      // 56 registers at most: w
 prologue_kernel(const __grid_constant__ GradTable<CAP> ptrs, float* __restrict__ Mst, void* __restrict__ Ast, void* __restrict__ Gpst,
                 __nv_bfloat16* __restrict__ xhat, float* __restrict__ partials, unsigned int* __restrict__ counters,
                 float* __restrict__ inv_norm, DeviceStatus* __restrict__ status, long long e, long long slab_len,
-                int unit_len, int slab_units, int units, PrologueScalars k, unsigned int* __restrict__ zero, int zero_words) {
+                int unit_len, int slab_units, int units, PrologueScalars k, unsigned int* __restrict__ zero, int zero_words,
+                float** __restrict__ params) {
+    if (params && blockIdx.x == 0 && threadIdx.x == 0) params[blockIdx.y] = ptrs.w[blockIdx.y];
     for (unsigned i = (blockIdx.y * gridDim.x + blockIdx.x) * EW_THREADS + threadIdx.x; i < (unsigned)zero_words; i += gridDim.x * gridDim.y * EW_THREADS) zero[i] = 0u;
     constexpr int WARPS = EW_THREADS / 32, MAX_SLAB_UNITS = 16;      // (a slab of several units is at most 16 K elements long)
     __shared__ float red[MAX_SLAB_UNITS * WARPS];
@@ -387,18 +390,18 @@ namespace {
 template <typename GT, typename ST, int CAP>
 void launch_prologue_cap(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, const ChunkPtrs& ptrs, float* M, void* A, void* Gp,
                          __nv_bfloat16* xhat, float* partials, unsigned int* counters, float* inv_norm, DeviceStatus* status,
-                         long long e, long long slab_len, const PrologueScalars& k, unsigned int* zero, int zero_words) {
+                         long long e, long long slab_len, const PrologueScalars& k, unsigned int* zero, int zero_words, float** params) {
     GradTable<CAP> t;
-    for (unsigned c = 0; c < grid.y; ++c) { t.g[c] = ptrs.g[c]; t.gid[c] = ptrs.gid[c]; }
-    if (vec4) prologue_kernel<GT, ST, 4, CAP><<<grid, block, 0, stream>>>(t, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, (int)norm_unit(e), (int)(slab_len / norm_unit(e)), (int)((e + norm_unit(e) - 1) / norm_unit(e)), k, zero, zero_words);
-    else      prologue_kernel<GT, ST, 1, CAP><<<grid, block, 0, stream>>>(t, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, (int)norm_unit(e), (int)(slab_len / norm_unit(e)), (int)((e + norm_unit(e) - 1) / norm_unit(e)), k, zero, zero_words);
+    for (unsigned c = 0; c < grid.y; ++c) { t.g[c] = ptrs.g[c]; t.w[c] = ptrs.w[c]; t.gid[c] = ptrs.gid[c]; }
+    if (vec4) prologue_kernel<GT, ST, 4, CAP><<<grid, block, 0, stream>>>(t, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, (int)norm_unit(e), (int)(slab_len / norm_unit(e)), (int)((e + norm_unit(e) - 1) / norm_unit(e)), k, zero, zero_words, params);
+    else      prologue_kernel<GT, ST, 1, CAP><<<grid, block, 0, stream>>>(t, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, (int)norm_unit(e), (int)(slab_len / norm_unit(e)), (int)((e + norm_unit(e) - 1) / norm_unit(e)), k, zero, zero_words, params);
 }
 template <typename GT, typename ST>
 void launch_prologue_t(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, const ChunkPtrs& ptrs, float* M, void* A, void* Gp,
                        __nv_bfloat16* xhat, float* partials, unsigned int* counters, float* inv_norm, DeviceStatus* status,
-                       long long e, long long slab_len, const PrologueScalars& k, unsigned int* zero, int zero_words) {
-    if (grid.y <= SMALL_TABLE) launch_prologue_cap<GT, ST, SMALL_TABLE>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words);
-    else                       launch_prologue_cap<GT, ST, MAXC>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words);
+                       long long e, long long slab_len, const PrologueScalars& k, unsigned int* zero, int zero_words, float** params) {
+    if (grid.y <= SMALL_TABLE) launch_prologue_cap<GT, ST, SMALL_TABLE>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words, params);
+    else                       launch_prologue_cap<GT, ST, MAXC>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words, params);
 }
 template <typename OT, int CAP>
 void launch_update_cap(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, const ChunkPtrs& ptrs, const void* O, long long e,
@@ -413,9 +416,9 @@ void launch_update_cap(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, co
 cudaError_t launch_prologue(const ChunkPtrs& ptrs, int C, bool grad_bf16, int state_kind, bool vec4, float* M, void* A, void* Gp,
                             __nv_bfloat16* xhat, float* partials, unsigned int* counters, float* inv_norm,
                             DeviceStatus* status, long long e, long long slab_len, int slabs,
-                            const PrologueScalars& k, unsigned int* zero, int zero_words, cudaStream_t stream) {
+                            const PrologueScalars& k, unsigned int* zero, int zero_words, float** params, cudaStream_t stream) {
     dim3 grid(slabs, C), block(EW_THREADS);
-#define MONA_PROLOGUE_CASE(GT, ST) launch_prologue_t<GT, ST>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words)
+#define MONA_PROLOGUE_CASE(GT, ST) launch_prologue_t<GT, ST>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words, params)
     if (grad_bf16) {
         if (state_kind == PROLOGUE_NO_AUX) MONA_PROLOGUE_CASE(__nv_bfloat16, NoAux);
         else if (state_kind == PROLOGUE_AUX_COMBINED) MONA_PROLOGUE_CASE(__nv_bfloat16, Combined);
@@ -557,7 +560,7 @@ extern "C" mona_status mona_prologue_noalloc(const void* grad, int32_t grad_dtyp
     k.mu = split_double(hp->momentum);
     k.eps = (float)hp->norm_eps;
     ce = launch_prologue(ptrs, 1, grad_dtype == MONA_BF16, PROLOGUE_AUX_F32, e % 4 == 0, M, A, G_prev, (__nv_bfloat16*)xhat_bf16, scratch->partials,
-                         &scratch->counter, inv_norm_out, &scratch->status, e, slab, slabs, k, nullptr, 0, stream);
+                         &scratch->counter, inv_norm_out, &scratch->status, e, slab, slabs, k, nullptr, 0, nullptr, stream);
     if (ce != cudaSuccess) { set_msg(err, err_len, cudaGetErrorString(ce)); return MONA_ERR_CUDA; }
     set_msg(err, err_len, "");
     return MONA_OK;

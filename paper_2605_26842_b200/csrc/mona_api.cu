@@ -41,8 +41,9 @@ constexpr size_t CTRL_COUNTERS_OFF = 0;
 constexpr size_t CTRL_INVNORM_OFF = 4096;
 constexpr size_t CTRL_PARTIALS_OFF = 8192;
 constexpr size_t CTRL_SCHED_OFF = CTRL_PARTIALS_OFF + sizeof(float) * MAXC * MAX_UNITS;   // work counter + done counters of the NS kernel
+constexpr size_t CTRL_PARAMS_OFF = (CTRL_SCHED_OFF + sizeof(unsigned int) * (64 + (size_t)MAXC * NS_MAX_PHASES) + 255) / 256 * 256;   // parameter pointers of the chunk
 constexpr size_t WS_DATA_OFF = WS_CTRL_OFF + NSLOTS * WS_CTRL_BYTES;
-static_assert(CTRL_SCHED_OFF + sizeof(unsigned int) * (64 + (size_t)MAXC * NS_MAX_PHASES) <= WS_CTRL_BYTES, "control block overflow");
+static_assert(CTRL_PARAMS_OFF + sizeof(float*) * MAXC <= WS_CTRL_BYTES, "control block overflow");
 static_assert(sizeof(unsigned int) * MAXC <= CTRL_INVNORM_OFF && sizeof(float) * MAXC <= CTRL_PARTIALS_OFF - CTRL_INVNORM_OFF, "control block overflow");
 
 // Process-wide defaults behind mona_set_chunk_budget() / mona_set_chunk_overlap().  They only seed
@@ -488,7 +489,7 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
 // Appends to `g` the phases of one iteration (or of two taken together) of a chunk of bucket `b`.  X is read from tensor
 // MAP_X0 + x_cur and written to the other one, or over itself with `in_place`; `first`: X is still un-normalised.
 static void ns_plan_group(NsProgram& g, const Bucket& b, bool together, bool first, int x_cur, uint8_t* data, float* delta,
-                          float ns_a, float ns_b, float ns_c, int macro_tile_min_k, bool fuse_update, bool in_place) {
+                          float ns_a, float ns_b, float ns_c, int macro_tile_min_k, bool fuse_update, bool update, bool in_place) {
     const int s = (int)b.s, l = (int)b.l;
     const size_t offset[NS_TENSORS] = {b.off_x[0], b.off_x[1], b.off_a, b.off_b, b.off_x[1]};
     auto output = [&](NsPhase& p, int d_map, int64_t ld) {
@@ -523,7 +524,7 @@ static void ns_plan_group(NsProgram& g, const Bucket& b, bool together, bool fir
     const int q_map = together ? MAP_A : MAP_B;
     NsPhase& g3 = g.ph[g.P++];      // X' = Q X (wide) or X Q (tall); 256 x 512 macro-tiles when the inner dimension is long
     g3.K = s; g3.wide = s >= macro_tile_min_k ? 1 : 0; output(g3, MAP_X0 + (in_place ? x_cur : x_cur ^ 1), b.cols);
-    g3.c2 = 1.f; g3.post_mode = first ? 1 : 0; g3.fuse_update = fuse_update ? 1 : 0;
+    g3.c2 = 1.f; g3.post_mode = first ? 1 : 0; g3.fuse_update = fuse_update ? 1 : 0; g3.update = update ? 1 : 0;
     if (!b.tall) {   // Q is the symmetric "A" operand, X the MN-major "B" operand
         g3.M = s; g3.N = l; g3.a_map = q_map; g3.a_sym = 1; g3.b_map = MAP_X0 + x_cur; g3.b_mn = 1;
     } else {         // X is K-major, the symmetric Q serves as its own transpose
@@ -735,12 +736,18 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                 MONA_CUDA(h, cudaStreamWaitEvent(stream, h->ev_in[host_chunk], 0));
             }
             const bool cleared_by_prologue = tc && small;
+            // The last X' = B' X updates the parameters, from O rounded to bf16 as the separate pass would read it: O is neither written
+            // nor read back, 4 of 12 bytes per element.
+            bool asked_for_o = false;
+            for (int c = 0; c < C; ++c) asked_for_o = asked_for_o || ptrs.o[c];
+            const bool update_inside = tc && phase_mask == 7u && vec4 && !asked_for_o && !h->opt.fuse_update;
+            float** param_table = (float**)(ctrl + CTRL_PARAMS_OFF);
             if (phase_mask & 1u) {
                 NvtxRange range("mona.prologue");
                 MONA_CUDA(h, launch_prologue(ptrs, C, b.grad_dtype == MONA_BF16,
                                              hp->algorithm == 1 ? PROLOGUE_NO_AUX : (b.state_dtype == MONA_BF16 ? PROLOGUE_AUX_BF16 :
                                                  b.state_dtype == MONA_STATE_COMBINED ? PROLOGUE_AUX_COMBINED : PROLOGUE_AUX_F32), vec4, Mc, Ac, Gc, tc ? xb[0] : nullptr, partials,
-                                             counters, inv_norm, dstatus, b.e, b.slab_len, b.slabs, ps, sched, cleared_by_prologue ? (int)ns_sched_words(C, NS_MAX_PHASES) : 0, stream));
+                                             counters, inv_norm, dstatus, b.e, b.slab_len, b.slabs, ps, sched, cleared_by_prologue ? (int)ns_sched_words(C, NS_MAX_PHASES) : 0, update_inside ? param_table : nullptr, stream));
                 ++h->launches;
             }
             const void* o_final = nullptr;
@@ -763,12 +770,12 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                         NsProgram g{};
                         g.C = C; g.delay = std::min(h->opt.ns_delay, C);       // beyond C matrices the order is the same
                         g.inv_norm = inv_norm; g.work_counter = sched; g.done = sched + 64;
-                        g.eta_lambda = eta_lambda; g.eta_gamma = eta_gamma;
+                        g.eta_lambda = eta_lambda; g.eta_gamma = eta_gamma; g.params = param_table;
                         bool last = false;
                         for (; gi < groups && g.P + (gi == 0 && together ? 7 : 3) <= NS_MAX_PHASES; ++gi) {
                             last = gi + 1 == groups;
                             ns_plan_group(g, b, gi == 0 && together, gi == 0, whole ? 0 : gi & 1, data, (float*)(data + b.off_delta), ns_a, ns_b, ns_c,
-                                          h->opt.macro_tile_min_k, update_fused && last, whole);
+                                          h->opt.macro_tile_min_k, update_fused && last, update_inside && last, whole);
                         }
                         if (whole) { g.form = NsForm::Whole; g.max_pairs = pairs; g.lane_tensors = C >= 2 * pairs; }
                         else ns_fit_launch(g, pairs, shared);
@@ -837,7 +844,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                 }
                 o_final = xf[T & 1];
             }
-            if ((phase_mask & 4u) && !update_fused) {
+            if ((phase_mask & 4u) && !update_fused && !update_inside) {
                 NvtxRange range("mona.update");
                 MONA_CUDA(h, launch_update(ptrs, C, tc, vec4, o_final, b.e, b.up_slab_len, b.up_slabs, eta_lambda, eta_gamma, stream));
                 ++h->launches;
@@ -920,7 +927,7 @@ mona_status mona_selftest_timeout(mona_handle* h, void* stream_v) {
         g.selftest_extra_tx = 16;
         const bool whole = !h->opt.fuse_update && whole_matrices(b, (int)std::min<int64_t>(b.Cb, (int64_t)b.mats.size()), h->max_pairs);
         ns_plan_group(g, b, false, false, 0, data, (float*)(data + b.off_delta), (float)NS_A, (float)NS_B, (float)NS_C,
-                      h->opt.macro_tile_min_k, false, whole);
+                      h->opt.macro_tile_min_k, false, false, whole);
         if (whole) g.form = NsForm::Whole;
         else if (b.small) ns_fit_launch(g, h->max_pairs, true);
         ns_program_plan(g);

@@ -28,7 +28,8 @@
 //              TMA stores in the spread form, where their fewer instructions are 1-2 % of the energy of the large sets, own
 //              stores in the others, where a hand-over less is 2 % of a short chain and 6 % of 256 x 768 experts;
 //              for the last X' = B' X of a step the same warps apply the parameter update of Eq. muon_update
-//              to the fp32 weights instead,
+//              to the fp32 weights instead (a separate pass reads O back and the weights at the end of the launch: three layers
+//              of 768 x 2048 experts 19.72 -> 19.42 ms per step, 256 x 768 experts 3.64 -> 3.56, one 256 x 512 85.0 -> 83.4 us),
 //   warp 3     store warp: turns each staged phase into TMA stores and frees the staging buffer (spread form), and counts the item
 //              as done once its stores have completed, so that no epilogue warp ever waits for global memory.
 //
@@ -752,7 +753,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 Item it;
                 if (!(ok = take_item(n, it, 12, true)) || (it.stop & 1)) break;
                 const NsPhase& p = g.ph[it.q];
-                if (p.fuse_update) continue;               // the epilogue writes the parameters itself; nothing waits for them
+                if (p.fuse_update || (BULK_STORES && p.update)) continue;      // the epilogue writes the parameters itself; nothing waits for them
                 if (BULK_STORES) {
                     const CUtensorMap* tma_d = &maps.m[p.d_map + NS_TENSORS];     // 64 columns x 128 rows per store
                     const TileCoord tc = decode_tile<FEW>(p, it.t);
@@ -946,6 +947,37 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             }
             __syncwarp();
         };
+        // The same columns, rounded to bf16 like those, update the parameters instead: W <- (W - eta lambda W) - eta gamma O.  An instruction
+        // covers two rows, 16 lanes of 16 bytes each.
+        auto update_columns = [&](const uint4* pk, float* w, int row0, int col, const NsPhase& p) {
+            #pragma unroll
+            for (int q = 0; q < 8; ++q)
+                asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(own_addr(q)), "r"(pk[q].x), "r"(pk[q].y), "r"(pk[q].z), "r"(pk[q].w) : "memory");
+            __syncwarp();
+            const int r0 = lane >> 4, c = col + 4 * (lane & 15);
+            float* at = w + (long long)(row0 + r0) * p.ld + c;
+            constexpr int AHEAD = 8;
+            #pragma unroll 1
+            for (int i0 = 0; i0 < 16; i0 += AHEAD) {
+                float4 v[AHEAD];
+                #pragma unroll
+                for (int i = 0; i < AHEAD; ++i)
+                    if (row0 + 2 * (i0 + i) + r0 < p.M && c < p.N) v[i] = __ldcs(reinterpret_cast<const float4*>(at + (long long)(2 * i) * p.ld));
+                #pragma unroll
+                for (int i = 0; i < AHEAD; ++i) {
+                    const int r = 2 * (i0 + i) + r0;
+                    uint32_t lo, hi;
+                    asm volatile("ld.shared.v2.b32 {%0, %1}, [%2];" : "=r"(lo), "=r"(hi) : "r"(stage + (uint32_t)r * 128u + (uint32_t)((((lane & 15) >> 1) ^ (r & 7)) << 4) + 8u * (lane & 1)) : "memory");
+                    v[i].x = fmaf(-g.eta_gamma, __uint_as_float(lo << 16), fmaf(-g.eta_lambda, v[i].x, v[i].x));
+                    v[i].y = fmaf(-g.eta_gamma, __uint_as_float(lo & 0xffff0000u), fmaf(-g.eta_lambda, v[i].y, v[i].y));
+                    v[i].z = fmaf(-g.eta_gamma, __uint_as_float(hi << 16), fmaf(-g.eta_lambda, v[i].z, v[i].z));
+                    v[i].w = fmaf(-g.eta_gamma, __uint_as_float(hi & 0xffff0000u), fmaf(-g.eta_lambda, v[i].w, v[i].w));
+                    if (row0 + r < p.M && c < p.N) __stcs(reinterpret_cast<float4*>(at + (long long)(2 * i) * p.ld), v[i]);
+                }
+                at += (long long)(2 * AHEAD) * p.ld;
+            }
+            __syncwarp();
+        };
         for (unsigned n = 0; alive; ++n) {
             Item it;
             if (!take_item(n, it, 10, false, TRACE_PTR(w_ring))) break;
@@ -973,7 +1005,13 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             const float delta = row_ok && p.delta_in ? __ldcg(p.delta_in + (size_t)zs * p.M + gr) : 0.0f;
             const float c2 = p.c2 * post, c1 = fmaf(2.0f * c2, delta, p.c1 * post);
             const uint32_t acc0 = tc.nsub == 2 ? 0u : acc_next;
-            if (!p.cin && !p.fuse_update) {
+            if (p.update && row_ok) {
+                // the parameters that this thread's row will need: half of the item's columns, one request (a main loop ahead of their use)
+                const int n0 = tc.tn * (FEW ? ns_tile_cols(p) : TC_BN), share = tc.nsub == 2 ? TC_BN : (FEW ? ns_tile_cols(p) : TC_BN) / 2;
+                const int c0 = n0 + half * share, bytes = 4 * min(share, p.N - c0);
+                if (bytes > 0) asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(g.params[it.c] + (long long)gr * p.ld + c0), "r"(bytes) : "memory");
+            }
+            if (!p.cin && !p.fuse_update && !p.update) {
                 // No axpy operand, no diagonal term (X X^T, products of s x s matrices, X' = B' X).  A thread's share of an accumulator is 128 values,
                 // 64 registers once packed: read and pack every accumulator of the item first, handing each back to the MMA
                 // issuer as soon as it has been read, and only then stage.  Nothing hides the epilogue of a macro-tile, so
@@ -1031,6 +1069,36 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 if (tc.nsub == 2) alive = pack_and_stage(integral_constant<int, 2>{}, integral_constant<int, 2>{});
                 else if (!(FEW && p.narrow)) alive = pack_and_stage(integral_constant<int, 1>{}, integral_constant<int, 2>{});
                 else alive = pack_and_stage(integral_constant<int, 1>{}, integral_constant<int, FEW ? 1 : 2>{});
+            } else if (p.update) {
+                // The last X' = B' X of a step.  64 columns at a time, each accumulator handed back when its last are read: keeping all of
+                // them packed, as above, leaves registers for four loads of the parameters in flight instead of eight, and it is
+                // their latency that counts here.
+                float* const w = g.params[it.c];
+                const int bn = FEW ? ns_tile_cols(p) : TC_BN;
+                for (int u = 0; u < tc.nsub && alive; ++u) {
+                    const uint32_t acc = acc0 + u;
+                    if (!(alive = mbar_wait(bar_acc_full + 8 * acc, (acc_par >> acc) & 1u, abort_flag, status, 4, TRACE_PTR(w_accf)))) break;
+                    tc_fence_after();
+                    acc_par ^= 1u << acc;
+                    for (int x = 0; x < bn && alive; x += EPI_COLS) {
+                        float v[64];
+                        tmem_ld32(tmem_base + lane_base + acc * TC_BN + x + half * 64, v);
+                        tmem_ld32(tmem_base + lane_base + acc * TC_BN + x + half * 64 + 32, v + 32);
+                        tmem_ld_wait();
+                        if (x + EPI_COLS == bn) {
+                            tc_fence_before();
+                            __syncwarp();
+                            if (lane == 0) mbar_arrive_remote(acc_empty_leader + 8 * acc);
+                        }
+                        const int col = (tc.tn + u) * bn + x + half * 64;
+                        uint4 pk[8];
+                        #pragma unroll
+                        for (int j = 0; j < 64; ++j) v[j] *= c2;
+                        #pragma unroll
+                        for (int q = 0; q < 8; ++q) pk[q] = pack8(v + 8 * q);
+                        if (col < p.N && (alive = staging_free())) update_columns(pk, w, row0, col, p);
+                    }
+                }
             } else if (p.cin) {
                 // b A + c A^2 + a I.  The axpy operand, A of the same tile, is requested before the accumulator is awaited, in whole lines
                 // like the stores, and handed to the rows' owners through the staging.  It was written by other CTAs of this launch,

@@ -28,7 +28,8 @@ constexpr int NS_MAPS = 2 * NS_TENSORS;   // each with 64-row boxes (index t) an
 // written (diagonal tiles completely).  A consumer that needs a block above the diagonal fetches the
 // stored block below it as an MN-major operand instead (`a_sym` / `b_sym`), so nothing is mirrored.
 //
-// With `fuse_update` set (the last X' = B' X of a step) D is not stored: the epilogue applies
+// With `update` set (the last X' = B' X of a step) D is not stored: the epilogue applies Eq. muon_update to the fp32 parameter of the
+// same matrix from D rounded to bf16, in whole lines of both.  With `fuse_update` set D is not stored either: the epilogue applies
 // Eq. muon_update, W <- (W - eta lambda W) - eta gamma D, to the fp32 parameter of the same matrix
 // straight from the fp32 accumulator, and writes D itself (fp32) only where an output pointer is given.
 struct NsPhase {
@@ -52,7 +53,8 @@ struct NsPhase {
     float c1, c2;
     float diag_add;             // added to D(i,i): folds the a*X term of the quintic into B' = b A + c A^2 + a I
     int post_mode;              // 0: post = 1, 1: post = inv_norm[c], 2: post = inv_norm[c]^2
-    int fuse_update;            // 1: epilogue applies the parameter update instead of storing D
+    int fuse_update;            // 1: epilogue applies the parameter update, from the fp32 accumulator, instead of storing D
+    int update;                 // 1: the same from D rounded to bf16 (what a separate pass over a stored D gives, bit for bit)
     // Diagonal correction of A, null or [C][M] fp32.  The diagonal of A is its largest entry by far, so its rounding to bf16 is
     // most of what rounding A costs.  The phase that stores A keeps delta_out[i] = exact - stored diagonal element; the phase
     // that forms b A + c A^2 + a I from it uses A + diag(delta) to first order (in A^2 the row's delta stands for both sides).
@@ -81,7 +83,8 @@ struct NsProgram {
     const float* inv_norm;      // per-matrix 1/(||M||_F + eps), used when post_mode != 0
     unsigned int* work_counter; // zero at launch
     unsigned int* done;         // C * P words, zero at launch
-    float eta_lambda, eta_gamma;    // fuse_update: eta * lambda and eta * gamma
+    float eta_lambda, eta_gamma;    // update and fuse_update: eta * lambda and eta * gamma
+    float* const* params;       // update: C parameter pointers in device memory
     NsForm form;
     int lane_tensors;           // Whole: 1: A, B' and C are indexed by pair and lane (2 per pair) instead of by matrix
     int gate;                   // 1: a pair takes its next item only when the MMAs of the last one are complete.  0: a few items

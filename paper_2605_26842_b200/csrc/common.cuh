@@ -64,6 +64,25 @@ constexpr unsigned STATUS_BOUNDS = 4u;       // debug build only: an index check
 #define MONA_IN_BOUNDS(cond, status, site) true
 #endif
 
+// Programmatic dependent launch: a kernel launched with `early` may be set up, and its blocks placed, while the kernel before it in
+// the stream still runs.  It calls wait_for_stream() before it touches global memory; a kernel that others follow early calls
+// let_next_start() when its own work is all placed.  Without the attribute both are free.  Where a chain of launches is the time
+// this takes the launch gaps out (one 256 x 512 matrix 83.4 -> 79.5 us per step, a mixed small set 108.3 -> 104.0, a dense block of 1024 and
+// 2816 370 -> 362, fp32: one 501 x 303 269 -> 239, one 1001 x 1500 945 -> 922).
+__device__ __forceinline__ void wait_for_stream() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P, typename... Q>
+cudaError_t launch_kernel(void (*kernel)(P...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, bool early, Q&&... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid; cfg.blockDim = block; cfg.dynamicSmemBytes = smem; cfg.stream = stream;
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &attr;
+    cfg.numAttrs = early ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
 // A scalar hyper-parameter carried as an unevaluated sum of two floats, hi + lo, so that products with
 // it are accurate to ~2^-45 instead of 2^-24: rounding beta_a = 0.99 to one float would by itself
 // cost 3e-8 per step in the EMA, which accumulates over its ~1/(1-beta_a) step memory.

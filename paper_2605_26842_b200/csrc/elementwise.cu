@@ -165,6 +165,7 @@ prologue_kernel(const __grid_constant__ GradTable<CAP> ptrs, float* __restrict__
                 float* __restrict__ inv_norm, DeviceStatus* __restrict__ status, long long e, long long slab_len,
                 int unit_len, int slab_units, int units, PrologueScalars k, unsigned int* __restrict__ zero, int zero_words,
                 float** __restrict__ params) {
+    let_next_start();
     if (params && blockIdx.x == 0 && threadIdx.x == 0) params[blockIdx.y] = ptrs.w[blockIdx.y];
     for (unsigned i = (blockIdx.y * gridDim.x + blockIdx.x) * EW_THREADS + threadIdx.x; i < (unsigned)zero_words; i += gridDim.x * gridDim.y * EW_THREADS) zero[i] = 0u;
     constexpr int WARPS = EW_THREADS / 32, MAX_SLAB_UNITS = 16;      // (a slab of several units is at most 16 K elements long)
@@ -313,6 +314,7 @@ template <typename OT, int VEC, int CAP>
 __global__ void __launch_bounds__(EW_THREADS)
 update_kernel(const __grid_constant__ ParamTable<CAP> ptrs, const OT* __restrict__ O, long long e, long long slab_len, float eta_lambda,
               float eta_gamma) {
+    wait_for_stream();
     const int c = blockIdx.y, p = blockIdx.x;
     const long long lo = (long long)p * slab_len;
     const long long hi = (lo + slab_len < e) ? lo + slab_len : e;
@@ -377,6 +379,8 @@ update_kernel(const __grid_constant__ ParamTable<CAP> ptrs, const OT* __restrict
 __global__ void __launch_bounds__(EW_THREADS)
 scale_kernel(const float* __restrict__ M, float* __restrict__ X, const float* __restrict__ inv_norm, long long e,
              long long slab_len) {
+    let_next_start();
+    wait_for_stream();
     const int c = blockIdx.y;
     const long long lo = (long long)blockIdx.x * slab_len;
     const long long hi = (lo + slab_len < e) ? lo + slab_len : e;
@@ -404,12 +408,11 @@ void launch_prologue_t(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, co
     else                       launch_prologue_cap<GT, ST, MAXC>(grid, block, stream, vec4, ptrs, M, A, Gp, xhat, partials, counters, inv_norm, status, e, slab_len, k, zero, zero_words, params);
 }
 template <typename OT, int CAP>
-void launch_update_cap(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, const ChunkPtrs& ptrs, const void* O, long long e,
-                       long long slab_len, float eta_lambda, float eta_gamma) {
+cudaError_t launch_update_cap(dim3 grid, dim3 block, cudaStream_t stream, bool vec4, const ChunkPtrs& ptrs, const void* O, long long e,
+                              long long slab_len, float eta_lambda, float eta_gamma, bool early) {
     ParamTable<CAP> t;
     for (unsigned c = 0; c < grid.y; ++c) { t.w[c] = ptrs.w[c]; t.o[c] = ptrs.o[c]; }
-    if (vec4) update_kernel<OT, 4, CAP><<<grid, block, 0, stream>>>(t, (const OT*)O, e, slab_len, eta_lambda, eta_gamma);
-    else      update_kernel<OT, 1, CAP><<<grid, block, 0, stream>>>(t, (const OT*)O, e, slab_len, eta_lambda, eta_gamma);
+    return launch_kernel(vec4 ? update_kernel<OT, 4, CAP> : update_kernel<OT, 1, CAP>, grid, block, 0, stream, early, t, (const OT*)O, e, slab_len, eta_lambda, eta_gamma);
 }
 }  // namespace
 
@@ -435,21 +438,18 @@ cudaError_t launch_prologue(const ChunkPtrs& ptrs, int C, bool grad_bf16, int st
 }
 
 cudaError_t launch_update(const ChunkPtrs& ptrs, int C, bool o_is_bf16, bool vec4, const void* O, long long e,
-                          long long slab_len, int slabs, float eta_lambda, float eta_gamma, cudaStream_t stream) {
+                          long long slab_len, int slabs, float eta_lambda, float eta_gamma, bool early, cudaStream_t stream) {
     dim3 grid(slabs, C), block(EW_THREADS);
     const bool small = C <= SMALL_TABLE;
-#define MONA_UPDATE_CASE(OT, CAP) launch_update_cap<OT, CAP>(grid, block, stream, vec4, ptrs, O, e, slab_len, eta_lambda, eta_gamma)
+#define MONA_UPDATE_CASE(OT, CAP) return launch_update_cap<OT, CAP>(grid, block, stream, vec4, ptrs, O, e, slab_len, eta_lambda, eta_gamma, early)
     if (o_is_bf16) { if (small) MONA_UPDATE_CASE(__nv_bfloat16, SMALL_TABLE); else MONA_UPDATE_CASE(__nv_bfloat16, MAXC); }
     else           { if (small) MONA_UPDATE_CASE(float, SMALL_TABLE); else MONA_UPDATE_CASE(float, MAXC); }
 #undef MONA_UPDATE_CASE
-    return cudaGetLastError();
 }
 
 cudaError_t launch_scale(const float* M, float* X, const float* inv_norm, int C, long long e, long long slab_len,
                          int slabs, cudaStream_t stream) {
-    dim3 grid(slabs, C), block(EW_THREADS);
-    scale_kernel<<<grid, block, 0, stream>>>(M, X, inv_norm, e, slab_len);
-    return cudaGetLastError();
+    return launch_kernel(scale_kernel, dim3(slabs, C), dim3(EW_THREADS), 0, stream, true, M, X, inv_norm, e, slab_len);
 }
 
 }  // namespace mona

@@ -24,7 +24,7 @@ cudaError_t launch_prologue(const ChunkPtrs& ptrs, int C, bool grad_bf16, int st
 
 // Parameter update W <- (W - eta*lambda*W) - eta*gamma*O for a chunk; O is bf16 or fp32, dense, e per matrix.
 cudaError_t launch_update(const ChunkPtrs& ptrs, int C, bool o_is_bf16, bool vec4, const void* O, long long e,
-                          long long slab_len, int slabs, float eta_lambda, float eta_gamma, cudaStream_t stream);
+                          long long slab_len, int slabs, float eta_lambda, float eta_gamma, bool early, cudaStream_t stream);
 
 // X_0 = M * inv_norm for the fp32 validation path.
 cudaError_t launch_scale(const float* M, float* X, const float* inv_norm, int C, long long e, long long slab_len,

@@ -786,6 +786,8 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                         // Between a large prologue and its launch the memset stays: without it the launch takes the SMs
                         // before the other stream's prologue has started on them (12 dense blocks 3.20 -> 3.36 ms).
                         if (!(cleared_by_prologue && (phase_mask & 1u)) || launched) MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(C, g.P), stream));
+                        // Nothing stands between a small chunk's prologue and its first launch: launch and set-up overlap the prologue.
+                        g.early = cleared_by_prologue && (phase_mask & 1u) && !launched;
                         launched = true;
                         NsUpdatePtrs up{};
                         if (update_fused && last) { up.w = ptrs.w; up.o = ptrs.o; }
@@ -846,7 +848,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             }
             if ((phase_mask & 4u) && !update_fused && !update_inside) {
                 NvtxRange range("mona.update");
-                MONA_CUDA(h, launch_update(ptrs, C, tc, vec4, o_final, b.e, b.up_slab_len, b.up_slabs, eta_lambda, eta_gamma, stream));
+                MONA_CUDA(h, launch_update(ptrs, C, tc, vec4, o_final, b.e, b.up_slab_len, b.up_slabs, eta_lambda, eta_gamma, !tc, stream));
                 ++h->launches;
             }
             if (params_host) {

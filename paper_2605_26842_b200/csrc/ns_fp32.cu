@@ -87,6 +87,7 @@ __device__ __forceinline__ void fma2(unsigned long long& d, unsigned long long a
 
 __global__ void __launch_bounds__(SG_THREADS, 1) sgemm_kernel(const __grid_constant__ SgemmArgs g) {
     extern __shared__ __align__(16) float sg[];
+    wait_for_stream();
     const int z = blockIdx.z;
     const float* __restrict__ A = g.a + (long long)z * g.a_batch;
     const float* __restrict__ B = g.b + (long long)z * g.b_batch;
@@ -138,6 +139,7 @@ __global__ void __launch_bounds__(SG_THREADS, 1) sgemm_kernel(const __grid_const
         }
         stage = stage + 1 == SG_STAGES ? 0 : stage + 1;
     }
+    let_next_start();                                      // not earlier: waiting blocks would hold SMs that other streams' products need
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();                                       // the slabs' memory becomes the groups' partial tiles
     float* part = sg + group * TS * PITCH;
@@ -227,6 +229,7 @@ __global__ void __launch_bounds__(THREADS, SMAX <= 32 ? 2 : 1)
 small_ns_kernel(const float* __restrict__ M, float* __restrict__ O, const float* __restrict__ inv_norm, int rows, int cols,
                 int parts, int T, float ca, float cb, float cc) {
     extern __shared__ __align__(16) float sm[];
+    wait_for_stream();
     uint32_t rank, n;
     asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(rank));
     asm volatile("mov.u32 %0, %%cluster_nctarank;" : "=r"(n));
@@ -391,6 +394,7 @@ small_ns_kernel(const float* __restrict__ M, float* __restrict__ O, const float*
         }
         __syncthreads();
     }
+    let_next_start();
     for (int idx = tid; idx < s * c_n; idx += THREADS) {          // O = X_T, back in the input's orientation
         if (!tall) { const int r = idx / c_n, q = idx - r * c_n; Oz[(long long)r * cols + c_lo + q] = Y[r * lp + q]; }
         else       { const int q = idx / s, r = idx - q * s;     Oz[(long long)c_lo * cols + idx] = Y[r * lp + q]; }
@@ -440,11 +444,13 @@ cudaError_t launch_small_ns(const float* M, float* O, const float* inv_norm, int
     cfg.blockDim = dim3(s > 32 ? SMALL_THREADS64 : SMALL_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr;
-    attr.id = cudaLaunchAttributeClusterDimension;
-    attr.val.clusterDim.x = (unsigned)n; attr.val.clusterDim.y = 1; attr.val.clusterDim.z = 1;
-    cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cudaLaunchAttribute attr[2];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = (unsigned)n; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[1].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 2;
     return s <= 32 ? cudaLaunchKernelEx(&cfg, small_ns_kernel<32, SMALL_THREADS>, M, O, inv_norm, rows, cols, parts, T, a, b, c)
                    : cudaLaunchKernelEx(&cfg, small_ns_kernel<64, SMALL_THREADS64>, M, O, inv_norm, rows, cols, parts, T, a, b, c);
 }
@@ -454,8 +460,7 @@ cudaError_t sgemm_configure() { return cudaFuncSetAttribute(sgemm_kernel, cudaFu
 cudaError_t launch_sgemm(const SgemmArgs& g, cudaStream_t stream) {
     const int tm = (g.M + TS - 1) / TS, tn = (g.N + TS - 1) / TS;
     dim3 grid(g.symmetric ? tm * (tm + 1) / 2 : tn, g.symmetric ? 1 : tm, g.batch);
-    sgemm_kernel<<<grid, SG_THREADS, SG_SMEM, stream>>>(g);
-    return cudaGetLastError();
+    return launch_kernel(sgemm_kernel, grid, dim3(SG_THREADS), SG_SMEM, stream, true, g);
 }
 
 }  // namespace mona

@@ -502,6 +502,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     tc_fence_before();
     __syncthreads();
     cluster_sync();                    // both CTAs' barriers exist before either side signals the other
+    wait_for_stream();
     tc_fence_after();
     const uint32_t tmem_base = *tmem_slot_ptr;
 
@@ -1347,18 +1348,14 @@ cudaError_t launch_ns_program(const NsMaps& maps, const NsProgram& g, const NsUp
     if (g.max_pairs > 0 && g.max_pairs < max_pairs) max_pairs = g.max_pairs;
     const long long units = g.form == NsForm::Whole ? g.C : (long long)g.total_items;
     const int pairs = units < (long long)max_pairs ? (int)units : max_pairs;
+    const dim3 grid(2 * (unsigned)pairs), block(TC_THREADS);
     if (up.w) {
         UpdateTable<MAXC> table;
         for (int c = 0; c < g.C; ++c) { table.w[c] = up.w[c]; table.o[c] = up.o ? up.o[c] : nullptr; }
-        ns_chunk_kernel<MAXC, NsForm::Spread><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, table, status);
-    } else if (g.form == NsForm::Few) {
-        ns_chunk_kernel<1, NsForm::Few><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
-    } else if (g.form == NsForm::Whole) {
-        ns_chunk_kernel<1, NsForm::Whole><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
-    } else {
-        ns_chunk_kernel<1, NsForm::Spread><<<2 * pairs, TC_THREADS, SMEM_TOTAL, stream>>>(maps, g, UpdateTable<1>{}, status);
+        return launch_kernel(ns_chunk_kernel<MAXC, NsForm::Spread>, grid, block, SMEM_TOTAL, stream, g.early, maps, g, table, status);
     }
-    return cudaGetLastError();
+    auto kernel = g.form == NsForm::Few ? ns_chunk_kernel<1, NsForm::Few> : g.form == NsForm::Whole ? ns_chunk_kernel<1, NsForm::Whole> : ns_chunk_kernel<1, NsForm::Spread>;
+    return launch_kernel(kernel, grid, block, SMEM_TOTAL, stream, g.early, maps, g, UpdateTable<1>{}, status);
 }
 
 }  // namespace mona

@@ -90,6 +90,7 @@ struct NsProgram {
     int gate;                   // 1: a pair takes its next item only when the MMAs of the last one are complete.  0: a few items
                                 //    ahead.  For launches of about one round of items per phase, where pairs that come first
                                 //    would hoard items that others are idle for
+    int early;                  // 1: the launch may start, and set itself up, while the kernel before it in the stream still runs
     int max_pairs;              // CTA pairs the launch may use (0: all that the device holds)
     int selftest_extra_tx;      // 0 in normal use.  The time-out self-test sets it: every stage then expects this many
                                 //    bytes more than its copies deliver, so the "full" wait runs out and the kernel must

@@ -401,7 +401,7 @@ def run_workload(torch, pkg, synth, shard, args, dev, local_rank, rank, world, d
               "ns_tflops_executed": ns_tflops, "ns_tflops_useful": flops_useful / (ms_kernel * 1e-3) / 1e12,
               "ns_tflops_executed_without_update": flops_exec / (ms_ns * 1e-3) / 1e12,
               "separate_update_gbs": upd_gbs, "separate_update_frac_of_hbm_peak": upd_gbs / peaks["hbm_gbs"],
-              "update": "in the epilogue of the last GEMM of the Newton-Schulz kernel" if fused else "separate kernel",
+              "update": "in the epilogue of the last GEMM of the Newton-Schulz kernel" if fused else "inside the last product of a whole step; timed apart as a kernel of its own",
               "hbm_peak_gbs": peaks["hbm_gbs"], "peak_source": peak_src}
     result = {"wl": wl, "fit_note": fit_note, "value": value, "ms_per_step": ms_per_step, "ms": ms, "clocks": clocks,
               "launches_per_step": launches_per_step, "phases": phases, "hp": hp, "options": opt.options}

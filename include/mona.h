@@ -129,8 +129,8 @@ mona_status mona_default_hparams(mona_hparams* hp);
  *                        times the budget (or the iterates of the largest matrix in fp32, where that is more), and
  *                        some 4 MiB.
  *   fuse_update        : 0 (default): Eq. muon_update is applied from O_k rounded to bf16: inside the last X' = B' X of a whole step
- *                        on the tensor-core path, by a separate elementwise kernel where O_k is asked for, phases run apart or a
- *                        stride is no multiple of 16 bytes.  The results are the same bits.
+ *                        on the tensor-core path, by a separate elementwise kernel where O_k is asked for, phases run apart,
+ *                        a stride is no multiple of 16 bytes or the step goes from host to host.  The results are the same bits.
  *                        1: on the tensor-core path the last X' = B' X of a step applies the update in its epilogue
  *                        (fp32 O_k straight from the accumulator, no bf16 copy of O_k written and re-read, one launch
  *                        fewer per chunk).  The two differ by the bf16 rounding of O_k only.  Measured slower on the

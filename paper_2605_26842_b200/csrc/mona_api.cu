@@ -560,6 +560,16 @@ static bool whole_matrices(const Bucket& b, int C, int pairs) {
     const int rest = C % (2 * pairs);
     return C >= pairs && C / (2 * pairs) + (rest == 0 ? 0.0 : rest <= pairs ? 0.77 : 1.0) <= 1.1 * C / (2.0 * pairs);
 }
+// The product that updates the parameters takes plain tiles where it has at least two rounds of macro-tiles.  Its epilogue is the
+// longest, 8 bytes per element in and out of the SM: behind a macro-tile nothing hides it, with plain tiles the next one's
+// products run beside it (12 dense blocks 3480 -> 3414 us per step, 1024 x 1536 experts 6778 -> 6650, three layers of 768 x 2048
+// 18.78 -> 18.48 ms, four of 512 x 1024 3875 -> 3827 us; 256 x 768, whole matrices, 3488 -> 3482).
+static void ns_plain_update_tiles(NsProgram& g, int pairs) {
+    for (int q = 0; q < g.P; ++q) {
+        NsPhase& p = g.ph[q];
+        if (p.update && p.wide && (long long)g.C * p.items_per_mat >= 2ll * pairs) { p.wide = 0; ns_phase_plan(p); }
+    }
+}
 // Fits a launch to `pairs` SM pairs: tile widths by estimated time, the claim gate, no more pairs than a phase has items.
 // (`shared`: beside other launches on a part of the pairs.)  A launch that has all pairs looks at other tile widths only for phases
 // that do not fill them once; macro-tiles move the fewest bytes per flop.
@@ -737,10 +747,11 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             }
             const bool cleared_by_prologue = tc && small;
             // The last X' = B' X updates the parameters, from O rounded to bf16 as the separate pass would read it: O is neither written
-            // nor read back, 4 of 12 bytes per element.
+            // nor read back, 4 of 12 bytes per element.  (Not host to host: its chunks are launches of few tiles, whose few SMs take longer for
+            // the update than a pass over all of them: 5.81 -> 5.77 ms for one layer of 512 x 1024 experts.)
             bool asked_for_o = false;
             for (int c = 0; c < C; ++c) asked_for_o = asked_for_o || ptrs.o[c];
-            const bool update_inside = tc && phase_mask == 7u && vec4 && !asked_for_o && !h->opt.fuse_update;
+            const bool update_inside = tc && phase_mask == 7u && !params_host && vec4 && !asked_for_o && !h->opt.fuse_update;
             float** param_table = (float**)(ctrl + CTRL_PARAMS_OFF);
             if (phase_mask & 1u) {
                 NvtxRange range("mona.prologue");
@@ -777,6 +788,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                             ns_plan_group(g, b, gi == 0 && together, gi == 0, whole ? 0 : gi & 1, data, (float*)(data + b.off_delta), ns_a, ns_b, ns_c,
                                           h->opt.macro_tile_min_k, update_fused && last, update_inside && last, whole);
                         }
+                        ns_plain_update_tiles(g, pairs);
                         if (whole) { g.form = NsForm::Whole; g.max_pairs = pairs; g.lane_tensors = C >= 2 * pairs; }
                         else ns_fit_launch(g, pairs, shared);
                         for (int q = 0; q < g.P; ++q) h->flops_exec += (double)C * ns_phase_executed_flops(g.ph[q]);

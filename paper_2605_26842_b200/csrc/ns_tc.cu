@@ -29,7 +29,7 @@
 //              stores in the others, where a hand-over less is 2 % of a short chain and 6 % of 256 x 768 experts;
 //              for the last X' = B' X of a step the same warps apply the parameter update of Eq. muon_update
 //              to the fp32 weights instead (a separate pass reads O back and the weights at the end of the launch: three layers
-//              of 768 x 2048 experts 19.72 -> 19.42 ms per step, 256 x 768 experts 3.64 -> 3.56, one 256 x 512 85.0 -> 83.4 us),
+//              of 768 x 2048 experts 19.06 -> 18.48 ms per step, 256 x 768 experts 3.63 -> 3.48, one 256 x 512 85.0 -> 83.4 us),
 //   warp 3     store warp: turns each staged phase into TMA stores and frees the staging buffer (spread form), and counts the item
 //              as done once its stores have completed, so that no epilogue warp ever waits for global memory.
 //
@@ -1097,7 +1097,9 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                         for (int j = 0; j < 64; ++j) v[j] *= c2;
                         #pragma unroll
                         for (int q = 0; q < 8; ++q) pk[q] = pack8(v + 8 * q);
-                        if (col < p.N && (alive = staging_free())) update_columns(pk, w, row0, col, p);
+                        if (col >= p.N) continue;
+                        alive = staging_free();
+                        if (alive) update_columns(pk, w, row0, col, p);
                     }
                 }
             } else if (p.cin) {

@@ -9,7 +9,7 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("shape,T", [((1, 64, 72), 5), ((1, 256, 512), 5), ((1, 264, 776), 7), ((2, 1032, 392), 1), ((80, 520, 648), 5),
-                                     ((80, 648, 520), 4), ((16, 128, 136), 5), ((150, 248, 520), 5), ((150, 520, 248), 6)])
+                                     ((80, 648, 520), 4), ((90, 264, 1160), 5), ((16, 128, 136), 5), ((150, 248, 520), 5), ((150, 520, 248), 6)])
 def test_update_inside_the_last_product(shape, T):
     dev = torch.device("cuda", 0)
     gen = torch.Generator(device=dev).manual_seed(23)

@@ -30,21 +30,28 @@ METRIC = "mona_optimizer_steps_per_s"
 UNIT = "steps/s"
 FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustained": 1400.0}
 # DRAM bytes (dram__bytes_read.sum + dram__bytes_write.sum) of one launch of the Newton-Schulz kernel from the ncu capture
-# summarised in profiles/ns_chunk_kernel_moe7b_1L.md: the launch over a 93-matrix 768x2048 chunk, the launch shape that
-# makes up most of the default workload (40 of its 56 launches per step are of this shape or its tall twin).  Valid only
-# for the kernel source the counters were taken with (hash of ns_tc.cu + ns_tc.cuh).
-NCU_TRAFFIC = {"source_sha256_16": "160982ecb797cc14", "bytes_per_launch": 5.754e9,
+# summarised in profiles/ns_chunk_kernel_counters.md: the launch over a 93-matrix 768x2048 chunk, parameter update included, the launch
+# shape that makes up most of the default workload (40 of its 56 launches per step are of this shape or its tall twin).  Valid only
+# for the kernel source the counters were taken with (hash of the code of ns_tc.cu + ns_tc.cuh).
+NCU_TRAFFIC = {"source_sha256_16": "449af8c0ab8d6db6", "bytes_per_launch": 6.627e9,
                "unit": "DRAM bytes of one launch over a 93-matrix 768x2048 chunk (ncu; 1.947 TFLOP executed in that launch)"}
+
+
+def kernel_source_hash(text: str) -> str:
+    """Hash of CUDA source without its comments and spacing: a comment makes no other kernel."""
+    import hashlib
+    import re
+    code = re.sub(r"/\*.*?\*/|//[^\n]*", " ", text, flags=re.S)
+    return hashlib.sha256(" ".join(code.split()).encode()).hexdigest()[:16]
 
 
 def kernel_traffic():
     """DRAM bytes per GEMM launch from the committed ncu capture, or None once the kernel source has changed."""
-    import hashlib
     try:
-        src = b"".join(open(os.path.join(ROOT, "paper_2605_26842_b200", "csrc", f), "rb").read() for f in ("ns_tc.cu", "ns_tc.cuh"))
+        src = "".join(open(os.path.join(ROOT, "paper_2605_26842_b200", "csrc", f)).read() for f in ("ns_tc.cu", "ns_tc.cuh"))
     except OSError:
         return None
-    return NCU_TRAFFIC["bytes_per_launch"] if hashlib.sha256(src).hexdigest()[:16] == NCU_TRAFFIC["source_sha256_16"] else None
+    return NCU_TRAFFIC["bytes_per_launch"] if kernel_source_hash(src) == NCU_TRAFFIC["source_sha256_16"] else None
 
 
 def load_peaks():

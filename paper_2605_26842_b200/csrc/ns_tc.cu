@@ -76,7 +76,6 @@ constexpr uint32_t B_SUB_BYTES = CTA_N * TC_BK * 2;               // 16 KiB per 
 constexpr int EPI_COLS = 128;                                     // output columns per epilogue phase
 constexpr uint32_t EPI_WARP_BYTES = 32 * 128;                     // staging of an epilogue warp: 64 bf16 columns of its 32 rows
 constexpr uint32_t EPI_BUF_BYTES = TC_EPI_WARPS * EPI_WARP_BYTES;
-constexpr int DONE_RING = 4;                                      // completion barriers: an epilogue warp can be two items ahead of another
 constexpr uint32_t TMEM_COLS = 512;                               // 2 accumulators x 256 fp32 columns
 // Operand staging: a ring of 16 KiB slabs.  A k-slice takes one slab per operand part it stages (1: diagonal tile whose
 // operands coincide, 2: plain tile, 3: macro-tile), contiguous (a k-slice that does not fit before the end of the ring
@@ -87,6 +86,11 @@ constexpr int NENT = 12;                                          // barrier ent
 constexpr uint32_t SLAB_BYTES = 16384;
 static_assert(SLAB_BYTES == A_STAGE_BYTES && SLAB_BYTES == B_SUB_BYTES, "one slab per operand part");
 constexpr int RING = 4;                                           // published-but-unfinished work items
+// Completion barriers, one per item stored: one more than the item ring has slots.  The store warp hands the slot of item n back before
+// it waits for the item to be stored, so items up to n + RING can be published and stored before it looks; n + RING + 1 needs
+// the slot that it hands back only after n.  With RING barriers n + RING could complete n's barrier a second time, whose parity would
+// then read "not yet" until the wait ran out.
+constexpr int DONE_RING = RING + 1;
 constexpr uint32_t SMEM_CTRL_BYTES = 512;
 constexpr uint32_t SMEM_TOTAL = NSLAB * SLAB_BYTES + EPI_BUF_BYTES + SMEM_CTRL_BYTES + 1024;
 constexpr long long WAIT_BUDGET_CYCLES = 1000000000ll;            // ~0.5 s
@@ -95,6 +99,7 @@ constexpr long long WAIT_BUDGET_CYCLES = 1000000000ll;            // ~0.5 s
 constexpr uint32_t RING_READERS = 3 + TC_EPI_WARPS + 2 + TC_EPI_WARPS;
 static_assert(SMEM_TOTAL <= 232448, "shared memory budget");
 static_assert(8 * (2 * NENT + 4 + 2 * RING + 4 + DONE_RING) + 16 + 16 * RING + 4 * (NS_MAX_PHASES + 1) <= SMEM_CTRL_BYTES, "control block");
+static_assert(DONE_RING > RING, "an item's completion must not be missed");
 
 __device__ __forceinline__ uint32_t smem_u32(const void* p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -452,7 +457,8 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     const uint32_t base = (smem_u32(smem_raw) + 1023u) & ~1023u;       // swizzle atoms need 1024-byte alignment
     const uint32_t epi_buf = base + NSLAB * SLAB_BYTES;
     const uint32_t ctrl = epi_buf + EPI_BUF_BYTES;
-    const uint32_t bar_full = ctrl;                             // NENT x 8 B (used in the leader)
+    const uint32_t ring_items = ctrl;                           // RING x 16 B, first: they are read and written 16 bytes at a time
+    const uint32_t bar_full = ring_items + 16 * RING;           // NENT x 8 B (used in the leader)
     const uint32_t bar_empty = bar_full + 8 * NENT;             // NENT x 8 B
     const uint32_t bar_acc_full = bar_empty + 8 * NENT;         // 2 x 8 B, one per accumulator
     const uint32_t bar_acc_empty = bar_acc_full + 16;           // 2 x 8 B (used in the leader)
@@ -463,9 +469,8 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
     const uint32_t bar_stg_empty = bar_stg_full + 16;           // 2 x 8 B: that half read by its store (store warp)
     const uint32_t tmem_slot = bar_stg_empty + 16;              // 4 B + abort flag 4 B
     const uint32_t lane_done = tmem_slot + 8;                   // 2 x 4 B: arrivals of the completed items of a lane (two per item)
-    const uint32_t ring_items = tmem_slot + 16;                 // RING x 16 B
     // items per matrix of the phases before phase q (q = 0 .. P): phase q has phase_first[q + 1] - phase_first[q] items
-    volatile unsigned int* phase_first = reinterpret_cast<volatile unsigned int*>(smem_raw + (ring_items + 16 * RING - smem_u32(smem_raw)));   // (NS_MAX_PHASES + 1) x 4 B
+    volatile unsigned int* phase_first = reinterpret_cast<volatile unsigned int*>(smem_raw + (tmem_slot + 16 - smem_u32(smem_raw)));   // (NS_MAX_PHASES + 1) x 4 B
     uint8_t* ctrl_ptr = smem_raw + (ctrl - smem_u32(smem_raw));
     volatile uint32_t* tmem_slot_ptr = reinterpret_cast<volatile uint32_t*>(ctrl_ptr + (tmem_slot - ctrl));
     volatile int* abort_flag = reinterpret_cast<volatile int*>(ctrl_ptr + (tmem_slot - ctrl) + 4);
@@ -747,7 +752,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             // it is the one that can wait for them) and frees the staging buffer when a phase has been read; it walks the items
             // and their phases in the epilogue's order.  Otherwise its fence covers the warps' own stores, which it has observed
             // through the barrier.
-            uint32_t staged = 0, stored = 0;
+            uint32_t staged = 0, done_e = 0, done_par = 0;
             TRACE_ONLY(const uint32_t t_role0 = trace_clock(); uint32_t w_stg = 0;)
             bool ok = true;
             for (unsigned n = 0; ok; ++n) {
@@ -785,8 +790,8 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                     if (!ok) break;
                     bulk_wait_all();                           // the item's output is in global memory
                 } else {
-                    if (!(ok = mbar_wait(bar_stored + 8 * (stored % DONE_RING), (stored / DONE_RING) & 1u, abort_flag, status, 13, TRACE_PTR(w_stg)))) break;
-                    ++stored;
+                    if (!(ok = mbar_wait(bar_stored + 8 * done_e, done_par, abort_flag, status, 13, TRACE_PTR(w_stg)))) break;
+                    if (++done_e == DONE_RING) { done_e = 0; done_par ^= 1u; }
                 }
                 fence_proxy_async_global();                // the copies that read the item go through the asynchronous proxy
                 if (WHOLE) {
@@ -914,7 +919,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
         const uint32_t line = stage + (uint32_t)line_row * 128u + (uint32_t)((line_chunk ^ line_row) << 4);
         auto line_addr = [&](int i) -> uint32_t { return (i & 1 ? line ^ 64u : line) + (uint32_t)i * 512u; };
         uint32_t acc_next = 0, acc_par = 0;   // acc_par: one use-parity bit per accumulator
-        uint32_t stored = 0, staged = 0;      // items stored, phases handed to the store warp so far
+        uint32_t done_e = 0, staged = 0;      // completion barrier of the present item, phases handed to the store warp so far
         TRACE_ONLY(const uint32_t t_role0 = trace_clock(); uint32_t w_ring = 0, w_accf = 0, w_stge = 0;)
         bool alive = true;
         // The staging is this warp's to write (with TMA stores: the previous phase of its half has been read).
@@ -1213,8 +1218,8 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             }
             if (!BULK_STORES) {
                 __syncwarp();
-                if (lane == 0) mbar_arrive_local(bar_stored + 8 * (stored % DONE_RING));
-                ++stored;
+                if (lane == 0) mbar_arrive_local(bar_stored + 8 * done_e);
+                if (++done_e == DONE_RING) done_e = 0;
             }
             if (tc.nsub == 1) acc_next ^= 1u;
 #ifdef MONA_TRACE

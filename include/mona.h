@@ -227,9 +227,8 @@ mona_status mona_step_host(mona_handle* h, const mona_hparams* hp,
  * reported a problem, or -1.  The word is cleared by the call. */
 mona_status mona_poll_status(mona_handle* h, void* stream, int64_t* first_bad_matrix);
 
-/* Failure-detection self-test: enqueues one Newton-Schulz launch (one iteration of one matrix of the first bucket on the
- * tensor-core path, in the form in which that bucket's steps run: for a bucket of few tiles with early publication and the
- * claim gate) whose shared-memory stages are made to expect 16 bytes more than their copies deliver.  Nothing faults
+/* Failure-detection self-test: enqueues one Newton-Schulz launch (the products of one matrix of the first bucket on the
+ * tensor-core path, in the form in which a step with the default hyper-parameters runs them) whose shared-memory stages are made to expect 16 bytes more than their copies deliver.  Nothing faults
  * - every copy completes - but neither the wait for a full stage nor the waits for the product it belongs to can end, so
  * they must run out after their bound (about half a second), latch the time-out in the
  * status word and leave the kernel cleanly.  Afterwards mona_poll_status() returns MONA_ERR_TIMEOUT once and
@@ -254,6 +253,24 @@ mona_status mona_last_ns_flops(const mona_handle* h, double* executed, double* d
 /* The work the iteration itself needs when both symmetric products are computed once per pair of entries:
  * 3 s^2 l + s^3 per matrix and iteration (tensor-core path only). */
 mona_status mona_last_ns_useful_flops(const mona_handle* h, double* useful);
+
+/* One launch of the Newton-Schulz kernel, as a step makes it. */
+typedef struct {
+    int64_t rows, cols;        /* of its matrices                                                      */
+    int32_t matrices;
+    int32_t sm_pairs;          /* SM pairs it may use                                                  */
+    int32_t slot;              /* workspace slot, which stands for the stream: launches of one slot follow one another */
+    int32_t form;              /* 0: many tiles per product, 1: few tiles, 2: whole matrices per SM pair */
+    int32_t products;          /* matrix products per matrix                                           */
+    int32_t update_columns;    /* columns of a work item of the product that updates the parameters (128, 256 or 512);
+                                  0: the launch does not update them                                   */
+} mona_launch_info;
+/* The tensor-core launches of a mona_step() over these descriptors on a device that holds `sm_pairs` pairs of SMs (74 on a B200), in
+ * the order in which they are enqueued, worked out on the HOST by the code that a step goes by; no device is needed.
+ * Parameters and gradients are taken to be 16-byte (with fuse_update 32-byte) aligned.  Writes at most `capacity` entries; *n_launches
+ * receives the number there are.  The paper has no counterpart: this is how tests know which form of the kernel a set runs in. */
+mona_status mona_describe_step(const mona_matrix_desc* descs, int64_t n_desc, const mona_options* options, const mona_hparams* hp,
+                               int32_t sm_pairs, mona_launch_info* out, size_t capacity, size_t* n_launches);
 
 /* The order in which the Newton-Schulz kernel hands out its work items (tiles), computed on the HOST with the cursor
  * the kernel's scheduler uses; no device is needed.  The paper has no counterpart: this exposes the property the

@@ -43,6 +43,14 @@ class Options(C.Structure):
                 ("ns_delay", C.c_int32), ("macro_tile_min_k", C.c_int32), ("reserved", C.c_int32 * 4)]
 
 
+class LaunchInfo(C.Structure):
+    """mona_launch_info: one Newton-Schulz launch of a step (see include/mona.h)."""
+    _fields_ = [("rows", C.c_int64), ("cols", C.c_int64), ("matrices", C.c_int32), ("sm_pairs", C.c_int32), ("slot", C.c_int32),
+                ("form", C.c_int32), ("products", C.c_int32), ("update_columns", C.c_int32)]
+
+
+FORM_MANY_TILES, FORM_FEW_TILES, FORM_WHOLE_MATRICES = 0, 1, 2
+
 _lib = None
 
 
@@ -67,6 +75,7 @@ def lib() -> C.CDLL:
     L.mona_trace_read.argtypes = [C.POINTER(C.c_ulonglong), C.c_size_t, C.c_int]
     L.mona_work_order.argtypes = [C.c_int32, C.c_int32, C.c_int32, C.POINTER(C.c_uint32), C.c_uint32, C.c_uint32,
                                   C.POINTER(C.c_int32), C.c_size_t, C.POINTER(C.c_size_t)]
+    L.mona_describe_step.argtypes = [C.POINTER(MatrixDesc), C.c_int64, C.POINTER(Options), C.POINTER(Hparams), C.c_int32, C.POINTER(LaunchInfo), C.c_size_t, C.POINTER(C.c_size_t)]
     L.mona_create.argtypes = [C.POINTER(vp), C.POINTER(MatrixDesc), C.c_int64, vp, C.c_size_t, vp, C.c_size_t, C.c_int]
     L.mona_step.argtypes = [vp, C.POINTER(Hparams), vpp, vpp, vp]
     L.mona_step_ex.argtypes = [vp, C.POINTER(Hparams), vpp, vpp, vpp, C.c_uint32, vp]
@@ -84,7 +93,7 @@ def lib() -> C.CDLL:
     L.mona_destroy.restype = None
     for name in ("mona_default_hparams", "mona_set_chunk_budget", "mona_set_chunk_overlap", "mona_query_sizes", "mona_create", "mona_step",
                  "mona_step_ex", "mona_step_host", "mona_poll_status", "mona_state_layout", "mona_last_ns_flops",
-                 "mona_default_options", "mona_query_sizes_opt", "mona_create_opt", "mona_last_ns_useful_flops", "mona_trace_read", "mona_work_order"):
+                 "mona_default_options", "mona_query_sizes_opt", "mona_create_opt", "mona_last_ns_useful_flops", "mona_trace_read", "mona_work_order", "mona_describe_step"):
         getattr(L, name).restype = C.c_int
     _lib = L
     return L
@@ -102,6 +111,21 @@ def work_order(n_matrices: int, delay: int, items_per_phase: Sequence[int], star
     if st:
         raise MonaError(st, "mona_work_order")
     return [(out[3 * i], out[3 * i + 1], out[3 * i + 2]) for i in range(n.value)]
+
+
+def describe_step(descs: Sequence[MatrixDesc], hp: Optional[Hparams] = None, options: Optional[Options] = None, sm_pairs: int = 74):
+    """mona_describe_step(): the Newton-Schulz launches of a step as a list of LaunchInfo."""
+    hp = hp if hp is not None else default_hparams()
+    n = C.c_size_t(0)
+    out, capacity = None, 0
+    while True:
+        st = lib().mona_describe_step(_desc_array(descs), len(descs), None if options is None else C.byref(options), C.byref(hp), sm_pairs, out, capacity, C.byref(n))
+        if st:
+            raise MonaError(st, "mona_describe_step")
+        if n.value <= capacity:
+            return list(out[:n.value]) if out is not None else []
+        capacity = n.value
+        out = (LaunchInfo * capacity)()
 
 
 def trace_read(reset: bool = True, rows: int = TRACE_ROWS):

@@ -309,6 +309,7 @@ struct mona_handle {
     Plan plan;
     mona_options opt = {};      // as resolved at creation; later changes of the process-wide defaults do not reach the handle
     int device = 0, max_pairs = 0;
+    std::vector<int> pairs_beside;   // per bucket: SM pairs of a small one beside others
     uint8_t* state = nullptr;
     uint8_t* ws = nullptr;
     cudaStream_t side[NSLOTS] = {};        // stream of slot 1 .. NSLOTS - 1 (slot 0 uses the caller's)
@@ -333,6 +334,8 @@ struct mona_handle {
         return st;
     }
 };
+
+static std::vector<int> share_pairs(const Plan& plan, int max_pairs);
 
 #define MONA_CUDA(h, call)                                                                                 \
     do {                                                                                                   \
@@ -467,6 +470,7 @@ mona_status mona_create_opt(mona_handle** out, const mona_matrix_desc* descs, in
         if (!ok) return h->fail(MONA_ERR_CUDA, "cuTensorMapEncodeTiled failed for bucket %lldx%lld", (long long)b.rows, (long long)b.cols);
     }
     MONA_CUDA(h, ns_configure(&h->max_pairs));
+    h->pairs_beside = share_pairs(h->plan, h->max_pairs);
     MONA_CUDA(h, small_ns_configure());
     MONA_CUDA(h, sgemm_configure());
     MONA_CUDA(h, cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming));
@@ -539,13 +543,19 @@ static double bucket_work(const Bucket& b) {
     const double ks = (double)((b.s + TC_BK - 1) / TC_BK), kl = (double)((b.l + TC_BK - 1) / TC_BK);
     return (double)b.mats.size() * (ts * (ts + 1) / 2 * (kl + ks) + ts * tl * ks);
 }
-// SM pairs of a small chunk: its share of the work when only small chunks run; beside large ones four times that, and eight
-// at least, so that it is through long before they are.  (Pairs that a launch does not find free simply come later: items are
-// handed out to whichever pairs run.)  Twelve blocks of 1024 and 2816: 3433 us per step, 3599 with the share alone, 3472 with all
-// pairs; four layers of 512 x 1024 experts the same with all three; a drawn set of experts 2571, 2421 and 2630.
-static int pairs_share(int max_pairs, double work, double work_total, bool all_small) {
-    const double share = max_pairs * work / work_total;
-    return std::max(1, std::min(max_pairs, (int)(all_small ? share + 0.5 : std::max(8.0, 4.0 * share))));
+// SM pairs of every bucket's launches when they run beside others: its share of the work when only small buckets run; beside large ones
+// four times that, and eight at least, so that it is through long before they are.  (Pairs that a launch does not find free
+// simply come later: items are handed out to whichever pairs run.)  Twelve blocks of 1024 and 2816: 3433 us per step, 3599 with
+// the share alone, 3472 with all pairs; four layers of 512 x 1024 experts the same with all three; a drawn set of experts 2571, 2421 and 2630.
+static std::vector<int> share_pairs(const Plan& plan, int max_pairs) {
+    double work_total = 0.0;
+    for (const Bucket& b : plan.buckets) if (b.tc_ok) work_total += bucket_work(b);
+    std::vector<int> pairs;
+    for (const Bucket& b : plan.buckets) {
+        const double share = b.tc_ok ? max_pairs * bucket_work(b) / work_total : 0.0;
+        pairs.push_back(std::max(1, std::min(max_pairs, (int)(plan.all_small ? share + 0.5 : std::max(8.0, 4.0 * share)))));
+    }
+    return pairs;
 }
 // Whether a launch over C matrices deals them whole to its SM pairs (NsForm::Whole).  Only where the shorter side is one tile.
 // Matrices of one tile (l <= 256 too) from eight on, where spreading a product over pairs buys nothing and handing it over inside a
@@ -599,6 +609,65 @@ static void ns_fit_launch(NsProgram& g, int pairs, bool shared) {
     g.max_pairs = std::min(pairs, most);
 }
 
+// How the launches of a chunk on the tensor-core path are made: what a step, the self-test and mona_describe_step() go by.
+struct NsChoice {
+    int pairs;              // SM pairs the launches may use
+    bool shared;            // beside other chunks, on a share of the pairs
+    bool whole;             // NsForm::Whole
+    bool together;          // the first two iterations on the s x s side
+    bool update_inside;     // the last X' = B' X updates the parameters
+    int groups;             // iterations, the first two counted as one when taken together
+};
+static NsChoice ns_choose(const mona_options& opt, int max_pairs, int pairs_beside, const Bucket& b, int C, bool beside, bool may_update, const mona_hparams& hp) {
+    NsChoice k;
+    k.shared = beside;
+    k.pairs = beside ? pairs_beside : max_pairs;
+    k.whole = !opt.fuse_update && whole_matrices(b, C, k.pairs);
+    k.together = ns_first_two_together(b.paired, hp);
+    k.groups = k.together ? hp.ns_steps - 1 : hp.ns_steps;
+    k.update_inside = may_update && !opt.fuse_update;
+    return k;
+}
+// The next launch of a chunk: the phases of group `gi` and of as many after it as one launch holds; moves `gi` behind them.
+static NsProgram ns_next_launch(const mona_options& opt, const Bucket& b, int C, const NsChoice& k, const mona_hparams& hp, bool update_fused, uint8_t* data, int& gi) {
+    NsProgram g{};
+    g.C = C; g.delay = std::min(opt.ns_delay, C);       // beyond C matrices the order is the same
+    for (; gi < k.groups && g.P + (gi == 0 && k.together ? 7 : 3) <= NS_MAX_PHASES; ++gi) {
+        const bool last = gi + 1 == k.groups;
+        ns_plan_group(g, b, gi == 0 && k.together, gi == 0, k.whole ? 0 : gi & 1, data, (float*)(data + b.off_delta), (float)hp.ns_a, (float)hp.ns_b,
+                      (float)hp.ns_c, opt.macro_tile_min_k, update_fused && last, k.update_inside && last, k.whole);
+    }
+    ns_plain_update_tiles(g, k.pairs);
+    if (k.whole) { g.form = NsForm::Whole; g.max_pairs = k.pairs; g.lane_tensors = C >= 2 * k.pairs; }
+    else ns_fit_launch(g, k.pairs, k.shared);
+    ns_program_plan(g);
+    return g;
+}
+
+// Matrices per chunk of a step (`host_bytes`: the bytes of parameters a chunk may hold in mona_step_host(), else 0).
+static int chunk_capacity(const Bucket& b, const mona_hparams& hp, size_t host_bytes) {
+    const int cap = hp.ns_precision == 0 && b.tc_ok && hp.ns_steps >= 1 ? b.Cb : b.Cf;
+    return host_bytes ? (int)std::min<size_t>(cap, std::max<size_t>(1, host_bytes / ((size_t)b.e * 4))) : cap;
+}
+// Whether a step's chunks run on several streams.
+static bool chunks_overlap(const Plan& plan, const mona_options& opt, const mona_hparams& hp, size_t host_bytes) {
+    int64_t chunks = 0;
+    for (const Bucket& b : plan.buckets) {
+        const int cap = chunk_capacity(b, hp, host_bytes);
+        chunks += ((int64_t)b.mats.size() + cap - 1) / cap;
+    }
+    return opt.chunk_overlap && chunks > 1;
+}
+// Whether the matrices [start, start + C) of a bucket can be accessed 16 bytes at a time (base pointers are aligned).
+static bool strides_aligned(const Plan& plan, const Bucket& b, int64_t start, int C) {
+    const int64_t gsz = b.grad_dtype == MONA_BF16 ? 2 : 4;
+    for (int c = 0; c < C; ++c) {
+        const int64_t stride = plan.descs[b.mats[start + c].desc].batch_stride;
+        if (stride * gsz % 16 != 0 || stride * 4 % 16 != 0) return false;
+    }
+    return b.e % 4 == 0;
+}
+
 // Bytes of parameters per chunk in mona_step_host(): a sixteenth of the set, so that the copy back starts early and little of either
 // direction is left alone at the ends, but not so few that a chunk is all launch latency (8 MiB are 150 us of the link).
 // One layer of 512 x 1024 experts, 218 MB each way: with chunks as large as the workspace holds the copy back started when two thirds
@@ -640,30 +709,17 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
     ps.eps = (float)hp->norm_eps;
     const float eta_lambda = (float)(hp->lr * hp->weight_decay);
     const int T = hp->ns_steps;
-    const float ns_a = (float)hp->ns_a, ns_b = (float)hp->ns_b, ns_c = (float)hp->ns_c;
+    const float ns_a = (float)hp->ns_a, ns_b = (float)hp->ns_b, ns_c = (float)hp->ns_c;     // fp32 path
 
     DeviceStatus* dstatus = (DeviceStatus*)(h->ws + WS_STATUS_OFF);
     // chunks alternate between the caller's stream (slot 0) and the handle's own stream (slot 1)
-    int64_t total_chunks = 0;
     const size_t host_bytes = params_host ? host_chunk_bytes(plan) : 0;
-    auto chunk_cap = [&](const Bucket& b) {
-        const int cap = hp->ns_precision == 0 && b.tc_ok && T >= 1 ? b.Cb : b.Cf;
-        return params_host ? (int)std::min<size_t>(cap, std::max<size_t>(1, host_bytes / ((size_t)b.e * 4))) : cap;
-    };
-    for (const Bucket& b : plan.buckets) {
-        const int capb = chunk_cap(b);
-        total_chunks += ((int64_t)b.mats.size() + capb - 1) / capb;
-    }
-    const bool overlap = h->opt.chunk_overlap && total_chunks > 1;
+    const bool overlap = chunks_overlap(plan, h->opt, *hp, host_bytes);
     cudaStream_t slot_stream[NSLOTS] = {(cudaStream_t)stream_v};
     bool slot_used[NSLOTS] = {true};
     for (int sl = 1; sl < NSLOTS; ++sl) slot_stream[sl] = overlap && h->side[sl] ? h->side[sl] : (cudaStream_t)stream_v;
     if (overlap) MONA_CUDA(h, cudaEventRecord(h->ev_fork, slot_stream[0]));
     int64_t big_index = 0;
-    // estimated tensor work of the buckets, by which chunks that run side by side share the SM pairs
-    double work_total = 0.0;
-    for (const Bucket& b : plan.buckets)
-        if (hp->ns_precision == 0 && b.tc_ok) work_total += bucket_work(b);
     struct DescRange { int desc; int64_t b0, b1; };      // matrices [b0, b1) of a descriptor
     std::vector<DescRange> ranges;                       // of the chunk (host pipeline only)
     size_t host_chunk = 0;
@@ -675,7 +731,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
     for (int bucket_index : plan.order) {
         const Bucket& b = plan.buckets[bucket_index];
         const bool tc = (hp->ns_precision == 0) && b.tc_ok && T >= 1;
-        const int cap = chunk_cap(b);
+        const int cap = chunk_capacity(b, *hp, host_bytes);
         const int64_t count = (int64_t)b.mats.size();
         const bool small = b.small && cap >= count;       // one chunk: the extra slots are made for whole buckets
         const double gamma = hp->scale_mode == 0 ? hp->scale_value * std::sqrt((double)b.l) : hp->scale_value;
@@ -687,7 +743,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
         for (int64_t start = 0; start < count; start += cap) {
             const int C = (int)std::min<int64_t>(cap, count - start);
             ChunkPtrs ptrs;
-            bool vec4 = (b.e % 4 == 0);
+            const bool vec4 = strides_aligned(plan, b, start, C);
             ranges.clear();
             for (int c = 0; c < C; ++c) {
                 const MatRef& mr = b.mats[start + c];
@@ -696,7 +752,6 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                     if (ranges.empty() || ranges.back().desc != mr.desc) ranges.push_back({mr.desc, mr.b, mr.b});
                     ranges.back().b1 = mr.b + 1;
                 }
-                if ((d.batch_stride * (int64_t)gsz) % 16 != 0 || (d.batch_stride * 4) % 16 != 0) vec4 = false;
                 ptrs.g[c] = (const uint8_t*)grads[mr.desc] + (size_t)mr.b * d.batch_stride * gsz;
                 ptrs.w[c] = (float*)params[mr.desc] + mr.b * d.batch_stride;
                 ptrs.o[c] = (o_out && o_out[mr.desc]) ? (float*)o_out[mr.desc] + mr.b * d.batch_stride : nullptr;
@@ -751,7 +806,8 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             // the update than a pass over all of them: 5.81 -> 5.77 ms for one layer of 512 x 1024 experts.)
             bool asked_for_o = false;
             for (int c = 0; c < C; ++c) asked_for_o = asked_for_o || ptrs.o[c];
-            const bool update_inside = tc && phase_mask == 7u && !params_host && vec4 && !asked_for_o && !h->opt.fuse_update;
+            const NsChoice k = ns_choose(h->opt, h->max_pairs, h->pairs_beside[bucket_index], b, C, overlap && small, phase_mask == 7u && !params_host && vec4 && !asked_for_o, *hp);
+            const bool update_inside = tc && k.update_inside;
             float** param_table = (float**)(ctrl + CTRL_PARAMS_OFF);
             if (phase_mask & 1u) {
                 NvtxRange range("mona.prologue");
@@ -764,11 +820,6 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             const void* o_final = nullptr;
             bool update_fused = false;
             if (tc) {
-                const bool together = ns_first_two_together(b.paired, *hp);
-                const int groups = together ? T - 1 : T;      // each reads one iterate and writes the other (a pair's own matrices: the same)
-                const bool shared = overlap && small;
-                const int pairs = shared ? pairs_share(h->max_pairs, bucket_work(b), work_total, plan.all_small) : h->max_pairs;
-                const bool whole = !h->opt.fuse_update && whole_matrices(b, C, pairs);
                 if (phase_mask & 2u) {
                     NvtxRange range("mona.newton_schulz");
                     // the last X' = B' X applies the parameter update in its epilogue when this call runs both phases and the
@@ -777,22 +828,11 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                     for (int c = 0; c < C && update_fused; ++c)
                         if (((uintptr_t)ptrs.w[c] & 31) || ((uintptr_t)ptrs.o[c] & 31)) update_fused = false;
                     bool launched = false;
-                    for (int gi = 0; gi < groups;) {
-                        NsProgram g{};
-                        g.C = C; g.delay = std::min(h->opt.ns_delay, C);       // beyond C matrices the order is the same
+                    for (int gi = 0; gi < k.groups;) {
+                        NsProgram g = ns_next_launch(h->opt, b, C, k, *hp, update_fused, data, gi);
                         g.inv_norm = inv_norm; g.work_counter = sched; g.done = sched + 64;
                         g.eta_lambda = eta_lambda; g.eta_gamma = eta_gamma; g.params = param_table;
-                        bool last = false;
-                        for (; gi < groups && g.P + (gi == 0 && together ? 7 : 3) <= NS_MAX_PHASES; ++gi) {
-                            last = gi + 1 == groups;
-                            ns_plan_group(g, b, gi == 0 && together, gi == 0, whole ? 0 : gi & 1, data, (float*)(data + b.off_delta), ns_a, ns_b, ns_c,
-                                          h->opt.macro_tile_min_k, update_fused && last, update_inside && last, whole);
-                        }
-                        ns_plain_update_tiles(g, pairs);
-                        if (whole) { g.form = NsForm::Whole; g.max_pairs = pairs; g.lane_tensors = C >= 2 * pairs; }
-                        else ns_fit_launch(g, pairs, shared);
                         for (int q = 0; q < g.P; ++q) h->flops_exec += (double)C * ns_phase_executed_flops(g.ph[q]);
-                        ns_program_plan(g);
                         // For a small chunk the prologue of this call has cleared the scheduler words of the first launch: one
                         // operation less in a short chain (one 256 x 512 matrix 102 -> 100 us, a mixed small set 126 -> 124).
                         // Between a large prologue and its launch the memset stays: without it the launch takes the SMs
@@ -802,14 +842,14 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                         g.early = cleared_by_prologue && (phase_mask & 1u) && !launched;
                         launched = true;
                         NsUpdatePtrs up{};
-                        if (update_fused && last) { up.w = ptrs.w; up.o = ptrs.o; }
+                        if (update_fused && gi == k.groups) { up.w = ptrs.w; up.o = ptrs.o; }
                         MONA_CUDA(h, launch_ns_program(b.maps[slot], g, up, h->max_pairs, dstatus, stream));
                         ++h->launches;
                     }
                     h->flops_dense += (double)T * C * (4.0 * b.s * b.s * b.l + 2.0 * (double)b.s * b.s * b.s);
                     h->flops_useful += (double)T * C * (3.0 * b.s * b.s * b.l + (double)b.s * b.s * b.s);
                 }
-                o_final = xb[whole ? 0 : groups & 1];
+                o_final = xb[k.whole ? 0 : k.groups & 1];
             } else if (small_ns_eligible(b.rows, b.cols)) {
                 // short side <= 64 (routers): the whole iteration in one launch, one block cluster per matrix
                 if (phase_mask & 2u) {
@@ -931,25 +971,62 @@ mona_status mona_selftest_timeout(mona_handle* h, void* stream_v) {
     MONA_CUDA(h, cudaSetDevice(h->device));
     for (const Bucket& b : h->plan.buckets) {
         if (!b.tc_ok) continue;
-        // one iteration of the first matrix of the workspace slot, in the kernel instance that the bucket's steps run in, with stages
-        // that expect 16 bytes too many: the first product never gets its operands, the others never get the first
+        // the first matrix of the workspace slot, in the launch that a step with the default hyper-parameters makes over the bucket's first
+        // chunk (O is stored instead of updating parameters), with stages that expect 16 bytes too many: the first product
+        // never gets its operands, the others never get the first
+        mona_hparams hp;
+        mona_default_hparams(&hp);
+        const int64_t i = &b - h->plan.buckets.data();
+        const int C = (int)std::min<int64_t>(b.Cb, (int64_t)b.mats.size());
         uint8_t* ctrl = h->ws + WS_CTRL_OFF;
         uint8_t* data = h->ws + h->plan.slot_off[b.small ? b.slot : 0];
         unsigned int* sched = (unsigned int*)(ctrl + CTRL_SCHED_OFF);
-        NsProgram g{};
-        g.C = 1; g.delay = 1; g.inv_norm = (const float*)(ctrl + CTRL_INVNORM_OFF); g.work_counter = sched; g.done = sched + 64;
+        int gi = 0;
+        NsProgram g = ns_next_launch(h->opt, b, C, ns_choose(h->opt, h->max_pairs, h->pairs_beside[i], b, C, b.small && chunks_overlap(h->plan, h->opt, hp, 0), false, hp),
+                                     hp, false, data, gi);
+        g.C = 1; g.delay = 1;
+        g.inv_norm = (const float*)(ctrl + CTRL_INVNORM_OFF); g.work_counter = sched; g.done = sched + 64;
         g.selftest_extra_tx = 16;
-        const bool whole = !h->opt.fuse_update && whole_matrices(b, (int)std::min<int64_t>(b.Cb, (int64_t)b.mats.size()), h->max_pairs);
-        ns_plan_group(g, b, false, false, 0, data, (float*)(data + b.off_delta), (float)NS_A, (float)NS_B, (float)NS_C,
-                      h->opt.macro_tile_min_k, false, false, whole);
-        if (whole) g.form = NsForm::Whole;
-        else if (b.small) ns_fit_launch(g, h->max_pairs, true);
         ns_program_plan(g);
         MONA_CUDA(h, cudaMemsetAsync(sched, 0, sizeof(unsigned int) * ns_sched_words(g.C, g.P), (cudaStream_t)stream_v));
         MONA_CUDA(h, launch_ns_program(b.maps[b.small ? b.slot : 0], g, NsUpdatePtrs{}, h->max_pairs, (DeviceStatus*)(h->ws + WS_STATUS_OFF), (cudaStream_t)stream_v));
         return MONA_OK;
     }
     return h->fail(MONA_ERR_UNSUPPORTED_SHAPE, "no descriptor of this handle takes the tensor-core path");
+}
+
+mona_status mona_describe_step(const mona_matrix_desc* descs, int64_t n_desc, const mona_options* options, const mona_hparams* hp, int32_t sm_pairs,
+                               mona_launch_info* out, size_t capacity, size_t* n_launches) {
+    if (!hp || !n_launches || sm_pairs < 1 || (capacity && !out) || hp->ns_steps < 0 || hp->ns_steps > 64) return MONA_ERR_INVALID_ARG;
+    mona_options opt;
+    if (resolve_options(options, opt) != MONA_OK) return MONA_ERR_INVALID_ARG;
+    Plan plan;
+    std::string err;
+    const mona_status st = build_plan(descs, n_desc, opt.chunk_budget_bytes, plan, err);
+    if (st != MONA_OK) return st;
+    const std::vector<int> pairs_beside = share_pairs(plan, sm_pairs);
+    const bool overlap = chunks_overlap(plan, opt, *hp, 0);
+    int64_t big_index = 0;
+    *n_launches = 0;
+    for (int bucket_index : plan.order) {
+        const Bucket& b = plan.buckets[bucket_index];
+        const int64_t count = (int64_t)b.mats.size();
+        const int cap = chunk_capacity(b, *hp, 0);
+        for (int64_t start = 0; start < count; start += cap) {
+            const int C = (int)std::min<int64_t>(cap, count - start);
+            const int slot = b.small ? b.slot : overlap ? (int)(big_index++ % BIG_SLOTS) : 0;
+            if (hp->ns_precision != 0 || !b.tc_ok) continue;
+            const NsChoice k = ns_choose(opt, sm_pairs, pairs_beside[bucket_index], b, C, overlap && b.small && cap >= count, strides_aligned(plan, b, start, C), *hp);
+            for (int gi = 0; gi < k.groups;) {
+                const NsProgram g = ns_next_launch(opt, b, C, k, *hp, opt.fuse_update != 0, nullptr, gi);
+                const NsPhase& p = g.ph[g.P - 1];
+                if (*n_launches < capacity)
+                    out[*n_launches] = {b.rows, b.cols, C, g.max_pairs, slot, opt.fuse_update ? 0 : (int32_t)g.form, g.P, p.update || p.fuse_update ? (p.wide ? 2 * TC_BN : ns_tile_cols(p)) : 0};
+                ++*n_launches;
+            }
+        }
+    }
+    return MONA_OK;
 }
 
 mona_status mona_poll_status(mona_handle* h, void* stream_v, int64_t* first_bad_matrix) {

@@ -1,0 +1,46 @@
+"""mona_describe_step(): the launches of a step, worked out on the host by the code the step itself goes by."""
+import pytest
+import torch
+
+import paper_2605_26842_b200 as pkg
+from paper_2605_26842_b200.binding import FORM_FEW_TILES, FORM_MANY_TILES, FORM_WHOLE_MATRICES, describe_step
+
+
+def descs(shapes):
+    return [pkg.MatrixDesc(r, c, b, 0, 0, 0) for b, r, c in shapes]
+
+
+@pytest.mark.parametrize("shape,T,form,products", [((1, 256, 512), 5, FORM_FEW_TILES, [15]), ((93, 768, 2048), 5, FORM_MANY_TILES, [16]), ((148, 256, 768), 5, FORM_WHOLE_MATRICES, [16]),
+                                                   ((93, 768, 2048), 7, FORM_MANY_TILES, [16, 6]), ((1, 256, 512), 0, None, []), ((1, 250, 512), 5, None, [])])
+def test_launches_of_one_bucket(shape, T, form, products):
+    got = describe_step(descs([shape]), pkg.default_hparams(ns_steps=T))
+    assert [g.products for g in got] == products
+    assert all((g.rows, g.cols, g.matrices, g.form) == (shape[1], shape[2], shape[0], form) for g in got)
+    assert [g.update_columns > 0 for g in got] == [i == len(products) - 1 for i in range(len(products))]
+
+
+def test_chunks_and_options():
+    got = describe_step(descs([(100, 768, 2048)]))
+    assert [(g.matrices, g.slot) for g in got] == [(93, 0), (7, 1)]
+    assert [g.slot for g in describe_step(descs([(100, 768, 2048)]), options=pkg.default_options(chunk_overlap=0))] == [0, 0]
+    assert describe_step(descs([(100, 768, 2048)]), pkg.default_hparams(ns_precision=1)) == []
+    odd = [pkg.MatrixDesc(256, 512, 2, 256 * 512 + 1, 0, 0)]                # a stride that no 16-byte access divides: a separate update
+    assert [g.update_columns for g in describe_step(odd)] == [0]
+    with pytest.raises(pkg.MonaError):
+        describe_step(descs([(1, 256, 512)]), sm_pairs=0)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("shapes,T", [([(1, 256, 512)], 5), ([(100, 768, 2048)], 7), ([(40, 256, 256), (4, 1024, 1024), (2, 2816, 1024)], 5), ([(60, 512, 512), (8, 256, 256)], 5)])
+def test_a_step_launches_what_is_described(shapes, T):
+    dev = torch.device("cuda", 0)
+    p, g = [torch.zeros(s, device=dev) for s in shapes], [torch.full(s, 1e-3, device=dev) for s in shapes]
+    hp = pkg.default_hparams(ns_steps=T)
+    opt = pkg.MonaOptimizer(p)
+    opt.step(hp, p, g)
+    assert opt.poll_status()[0] == 0
+    launches = describe_step(opt.descs, hp)
+    chunks = len({(x.rows, x.cols, x.slot, x.matrices) for x in launches})
+    updates = chunks - sum(x.update_columns > 0 for x in launches)
+    assert opt.last_launch_count() == chunks + len(launches) + updates        # a prologue per chunk, and an update where none is inside
+    opt.close()

@@ -1,4 +1,6 @@
 """mona_describe_step(): the launches of a step, worked out on the host by the code the step itself goes by."""
+import random
+
 import pytest
 import torch
 
@@ -28,6 +30,27 @@ def test_chunks_and_options():
     assert [g.update_columns for g in describe_step(odd)] == [0]
     with pytest.raises(pkg.MonaError):
         describe_step(descs([(1, 256, 512)]), sm_pairs=0)
+
+
+def random_small_set(rng):
+    shapes = {}
+    for _ in range(rng.randint(2, 9)):
+        r, c = (8 * int(8 * 32 ** rng.random()) for _ in range(2))
+        shapes[(r, c)] = rng.randint(1, 6)
+    return [(b, r, c) for (r, c), b in shapes.items()]
+
+
+@pytest.mark.parametrize("shapes", [[(13, 128, 128), (5, 2048, 2048), (3, 192, 128), (2, 448, 96)], [(40, 256, 256), (4, 1024, 1024), (2, 2816, 1024)]]
+                         + [random_small_set(random.Random(seed)) for seed in range(40)])
+def test_launches_that_run_side_by_side_fit_the_device(shapes):
+    """Where a set has small buckets only, one launch of every slot can run at a time: together they use no more SM pairs than there
+    are, so that none has to wait until another has ended."""
+    for sm_pairs in (74, 20, 5):
+        launches = describe_step(descs(shapes), sm_pairs=sm_pairs)
+        widest = {}
+        for g in launches:
+            widest[g.slot] = max(widest.get(g.slot, 0), g.sm_pairs)
+        assert all(w >= 1 for w in widest.values()) and sum(widest.values()) <= sm_pairs, [(g.rows, g.cols, g.slot, g.sm_pairs) for g in launches]
 
 
 @pytest.mark.gpu

@@ -130,7 +130,8 @@ mona_status mona_default_hparams(mona_hparams* hp);
  *                        some 4 MiB.
  *   fuse_update        : 0 (default): Eq. muon_update is applied from O_k rounded to bf16: inside the last X' = B' X of a whole step
  *                        on the tensor-core path, by a separate elementwise kernel where O_k is asked for, phases run apart,
- *                        a stride is no multiple of 16 bytes or the step goes from host to host.  The results are the same bits.
+ *                        a stride is no multiple of 16 bytes, the step goes from host to host, or the launch has so many tiles
+ *                        for its few SM pairs that a pass on all of them is quicker.  The results are the same bits.
  *                        1: on the tensor-core path the last X' = B' X of a step applies the update in its epilogue
  *                        (fp32 O_k straight from the accumulator, no bf16 copy of O_k written and re-read, one launch
  *                        fewer per chunk).  The two differ by the bf16 rounding of O_k only.  Measured slower on the

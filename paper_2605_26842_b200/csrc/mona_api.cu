@@ -583,6 +583,16 @@ static bool whole_matrices(const Bucket& b, int C, int pairs) {
     const int rest = C % (2 * pairs);
     return C >= pairs && C / (2 * pairs) + (rest == 0 ? 0.0 : rest <= pairs ? 0.77 : 1.0) <= 1.1 * C / (2.0 * pairs);
 }
+// Whether the last X' = B' X updates the parameters, or a pass of its own does: by estimated time.  Inside it lengthens the epilogue of every
+// 256 x 256 tile by some 3.5 us (8 x 64 KiB of parameters in and out of a pair), of half a tile's columns by half of that, however few
+// rows it has, and only the pairs of the launch work at it; apart it is a launch, 6 us, and 10 bytes per element at the bandwidth of the whole device.  One bucket on
+// 1, 8, 16 and 32 pairs, inside against apart, us per step: 40 of 256 x 256 2012 / 275 / 160 / 162 against 1868 / 262 / 158 / 165, 24 of
+// 512 x 512 4248 / 592 / 332 / 226 against 3928 / 567 / 325 / 227, 13 of 128 x 128 on 8 and 32 94 / 93 against 97 / 96; on all 74, 300 of
+// 72 x 648 439 against 428, but of 648 x 72 430 against 447.
+static bool update_pays_inside(const Bucket& b, int C, int pairs) {
+    const double tiles = 0.5 * (double)C * (double)((b.rows + TC_BM - 1) / TC_BM) * (double)((b.cols + TC_BN / 2 - 1) / (TC_BN / 2));
+    return 3.5 * std::max(1.0, tiles / pairs) <= 6.0 + (double)C * (double)b.e * 10.0 / 6.2e6;
+}
 // The product that updates the parameters takes plain tiles where it has at least two rounds of macro-tiles.  Its epilogue is the
 // longest, 8 bytes per element in and out of the SM: behind a macro-tile nothing hides it, with plain tiles the next one's
 // products run beside it (12 dense blocks 3480 -> 3414 us per step, 1024 x 1536 experts 6778 -> 6650, three layers of 768 x 2048
@@ -638,7 +648,7 @@ static NsChoice ns_choose(const mona_options& opt, int max_pairs, int pairs_besi
     k.whole = !opt.fuse_update && whole_matrices(b, C, k.pairs);
     k.together = ns_first_two_together(b.paired, hp);
     k.groups = k.together ? hp.ns_steps - 1 : hp.ns_steps;
-    k.update_inside = may_update && !opt.fuse_update;
+    k.update_inside = may_update && !opt.fuse_update && update_pays_inside(b, C, k.pairs);
     return k;
 }
 // The next launch of a chunk: the phases of group `gi` and of as many after it as one launch holds; moves `gi` behind them.

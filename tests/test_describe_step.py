@@ -32,6 +32,13 @@ def test_chunks_and_options():
         describe_step(descs([(1, 256, 512)]), sm_pairs=0)
 
 
+@pytest.mark.parametrize("shape,sm_pairs,inside", [((40, 256, 256), 8, False), ((24, 512, 512), 16, False), ((40, 1088, 256), 16, False), ((8, 1024, 1024), 4, False),
+                                                   ((300, 72, 648), 74, False), ((40, 256, 256), 32, True), ((13, 128, 128), 8, True), ((1, 64, 64), 1, True),
+                                                   ((93, 768, 2048), 74, True), ((512, 256, 768), 74, True), ((2, 2048, 2048), 74, True)])
+def test_few_pairs_leave_the_update_of_many_tiles_to_a_pass_of_its_own(shape, sm_pairs, inside):
+    assert [g.update_columns > 0 for g in describe_step(descs([shape]), sm_pairs=sm_pairs)] == [inside]
+
+
 def random_small_set(rng):
     shapes = {}
     for _ in range(rng.randint(2, 9)):

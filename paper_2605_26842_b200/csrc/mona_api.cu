@@ -570,18 +570,29 @@ static std::vector<int> share_pairs(const Plan& plan, int max_pairs) {
     }
     return pairs;
 }
-// Whether a launch over C matrices deals them whole to its SM pairs (NsForm::Whole).  Only where the shorter side is one tile.
-// Matrices of one tile (l <= 256 too) from eight on, where spreading a product over pairs buys nothing and handing it over inside a
-// pair is quicker: forty of 64 x 64 117 -> 72 us per step, forty of 256 x 256 151 -> 121, sixteen of 256 x 128 113 -> 84, but
-// four of 64 x 64 66 against 72 and four of 256 x 256 96 against 88.  Longer ones once every pair has one, and by the rounds that C makes of two
-// matrices per pair: a full round of 256 x 768 takes 217 us, one in which no pair has a second 167, and spread over all pairs as many
-// matrices take 1.1 times a full round's share (C = 148: 421 against 453 us per step, 256: 828 against 755, 370: 1020 against 1061,
-// 512: 1397 against 1448; 60 of 200 x 4096 767 against 698, 74 of 256 x 512 210 against 233).
-static bool whole_matrices(const Bucket& b, int C, int pairs) {
-    if (b.s > TC_BM) return false;
-    if (b.l <= TC_BN) return C >= 8;
+// Whether a launch over C matrices deals them whole to its SM pairs (NsForm::Whole) or spreads every product over the pairs.  Only where the
+// shorter side is one tile.  Time per step, whole against spread, us, on 74 pairs unless said otherwise:
+//  - one round, two matrices per pair at most: one-tile matrices (l <= 256) from nine on, 8 of 256 x 256 92 against 90, 12 93 against 101,
+//    74 121-133 against 172, 148 183 against 230 (up to 128 x 128 from eight, 8 of 64 x 64 60 against 74); up to l = 512 once every pair
+//    has one, 74 of 256 x 512 176-197 against 219; up to l = 1024 with one and a half, 90 of 256 x 768 296 against 287, 111 326 against 339,
+//    148 406 against 439, 148 of 1024 x 256 505 against 530; beyond that not, 111 of 256 x 1280 490 against 483, 148 656 against 640,
+//    74 of 192 x 2048 434 against 415;
+//  - more: a last round without second matrices counts half, a full one leaves a ragged end, and spread over all pairs as many matrices
+//    take 1.1 times a full round's share: 185, 222, 296, 370 and 512 of 256 x 768 550, 624, 861, 990 and 1377 against 532, 643, 820, 1037
+//    and 1425, of 256 x 256 277, 291, 418, 468 and 640 against 271, 312, 412, 500 and 690.  Not where one CTA of the pair has no rows
+//    and l > 512: 512 of 96 x 1024 950 against 917.  Always up to 128 x 128: 160, 300 and 512 167, 269 and 386 against 169, 284 and 446;
+//  - on a share of the pairs the iterates stay in L2 either way and spreading is quicker as soon as a pair needs a second matrix: 40 of 256 x
+//    256 on 32, 16 and 8 pairs 125, 206 and 313 against 162, 160 and 275; 42 beside two small buckets 187 against 162.  Longer ones never:
+//    40 of 1088 x 256 on 32 pairs 307 against 264.
+static bool whole_matrices(const Bucket& b, int C, int pairs, bool shared) {
+    const bool tiny = b.l <= TC_BN / 2, one_tile = b.l <= TC_BN;
+    if (b.s > TC_BM || C < (tiny ? 8 : 9)) return false;
+    if (shared) return one_tile && C <= pairs;
+    if (tiny) return true;
+    if (C <= 2 * pairs) return one_tile || (b.l <= 2 * TC_BN ? C >= pairs : b.l <= 4 * TC_BN && 2 * C >= 3 * pairs);
+    if (b.l > (b.s > TC_BM / 2 ? 3 : 2) * TC_BN) return false;
     const int rest = C % (2 * pairs);
-    return C >= pairs && C / (2 * pairs) + (rest == 0 ? 0.0 : rest <= pairs ? 0.77 : 1.0) <= 1.1 * C / (2.0 * pairs);
+    return C / (2 * pairs) + (rest == 0 ? 0.2 : rest <= pairs ? 0.5 : 1.0) < 1.1 * C / (2.0 * pairs);
 }
 // Whether the last X' = B' X updates the parameters, or a pass of its own does: by estimated time.  Inside it lengthens the epilogue of every
 // 256 x 256 tile by some 3.5 us (8 x 64 KiB of parameters in and out of a pair), of half a tile's columns by half of that, however few
@@ -645,7 +656,7 @@ static NsChoice ns_choose(const mona_options& opt, int max_pairs, int pairs_besi
     NsChoice k;
     k.shared = beside;
     k.pairs = beside ? pairs_beside : max_pairs;
-    k.whole = !opt.fuse_update && whole_matrices(b, C, k.pairs);
+    k.whole = !opt.fuse_update && whole_matrices(b, C, k.pairs, beside);
     k.together = ns_first_two_together(b.paired, hp);
     k.groups = k.together ? hp.ns_steps - 1 : hp.ns_steps;
     k.update_inside = may_update && !opt.fuse_update && update_pays_inside(b, C, k.pairs);

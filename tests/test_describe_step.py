@@ -39,6 +39,26 @@ def test_few_pairs_leave_the_update_of_many_tiles_to_a_pass_of_its_own(shape, sm
     assert [g.update_columns > 0 for g in describe_step(descs([shape]), sm_pairs=sm_pairs)] == [inside]
 
 
+WHOLE_PAYS = {(256, 256): [9, 12, 74, 100, 148, 222, 370, 512], (128, 128): [8, 100, 160, 222, 300, 512], (64, 64): [8, 40], (192, 256): [222, 370, 512],
+              (256, 512): [74, 100, 148, 222, 370, 512], (256, 768): [111, 148, 222, 370, 512], (768, 256): [148], (128, 1024): [148], (1024, 256): [148],
+              (72, 648): [148], (96, 1024): [148], (64, 512): [512]}
+SPREADING_PAYS = {(256, 256): [1, 4, 8, 160, 185, 260], (192, 256): [160], (64, 64): [4], (256, 768): [74, 90, 185, 296], (256, 1280): [74, 90, 111, 185],
+                  (72, 648): [300], (96, 1024): [512], (128, 1024): [512], (128, 1280): [300], (192, 2048): [74], (256, 4096): [74, 222], (264, 264): [8, 148]}
+
+
+@pytest.mark.parametrize("whole,shape,count", [(w, s, c) for w, table in ((True, WHOLE_PAYS), (False, SPREADING_PAYS)) for s, cs in table.items() for c in cs])
+def test_whole_matrices_where_they_were_measured_faster(whole, shape, count):
+    assert all((g.form == FORM_WHOLE_MATRICES) == whole for g in describe_step(descs([(count, *shape)])))
+
+
+@pytest.mark.parametrize("shapes,bucket,whole", [([(40, 256, 256), (4, 1024, 1024), (2, 2816, 1024)], 0, False), ([(8, 256, 200), (4, 1024, 1024)], 0, False),
+                                                 ([(2, 848, 608), (2, 320, 1472), (42, 256, 256)], 2, False), ([(37, 896, 192), (4, 576, 1024)], 0, False),
+                                                 ([(26, 192, 256), (8, 192, 128), (8, 448, 128)], 0, True), ([(6, 384, 128), (10, 256, 128)], 1, True)])
+def test_whole_matrices_on_a_share_of_the_pairs(shapes, bucket, whole):
+    got = {(g.rows, g.cols): g.form for g in describe_step(descs(shapes))}
+    assert (got[shapes[bucket][1:]] == FORM_WHOLE_MATRICES) == whole
+
+
 def random_small_set(rng):
     shapes = {}
     for _ in range(rng.randint(2, 9)):

@@ -592,7 +592,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             slab_head = pos + nslab == NSLAB ? 0u : pos + nslab;
             ++ent;
             if (++ent_e == NENT) { ent_e = 0; ent_par ^= 1u; }
-            if (!MONA_IN_BOUNDS(pos + nslab <= NSLAB && e < NENT && it.c < g.C, status, 102)) return false;
+            if (!MONA_IN_BOUNDS(pos + nslab <= NSLAB && e < NENT && it.c < g.C && za >= 0 && za < g.C && zb >= 0 && zb < g.C, status, 102)) return false;
             const uint32_t full = full_leader + 8 * e;
             const uint32_t sa = base + pos * SLAB_BYTES;
             const int k0 = kb * TC_BK;
@@ -962,13 +962,16 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             __syncwarp();
             const int r0 = lane >> 4, c = col + 4 * (lane & 15);
             float* at = w + (long long)(row0 + r0) * p.ld + c;
+            auto inside = [&](int r) -> bool {
+                return row0 + r < p.M && c < p.N && MONA_IN_BOUNDS(row0 + r >= 0 && c >= 0 && (long long)(row0 + r) * p.ld + c + 4 <= (long long)p.M * p.ld, status, 107);
+            };
             constexpr int AHEAD = 8;
             #pragma unroll 1
             for (int i0 = 0; i0 < 16; i0 += AHEAD) {
                 float4 v[AHEAD];
                 #pragma unroll
                 for (int i = 0; i < AHEAD; ++i)
-                    if (row0 + 2 * (i0 + i) + r0 < p.M && c < p.N) v[i] = __ldcs(reinterpret_cast<const float4*>(at + (long long)(2 * i) * p.ld));
+                    if (inside(2 * (i0 + i) + r0)) v[i] = __ldcs(reinterpret_cast<const float4*>(at + (long long)(2 * i) * p.ld));
                 #pragma unroll
                 for (int i = 0; i < AHEAD; ++i) {
                     const int r = 2 * (i0 + i) + r0;
@@ -978,7 +981,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                     v[i].y = fmaf(-g.eta_gamma, __uint_as_float(lo & 0xffff0000u), fmaf(-g.eta_lambda, v[i].y, v[i].y));
                     v[i].z = fmaf(-g.eta_gamma, __uint_as_float(hi << 16), fmaf(-g.eta_lambda, v[i].z, v[i].z));
                     v[i].w = fmaf(-g.eta_gamma, __uint_as_float(hi & 0xffff0000u), fmaf(-g.eta_lambda, v[i].w, v[i].w));
-                    if (row0 + r < p.M && c < p.N) __stcs(reinterpret_cast<float4*>(at + (long long)(2 * i) * p.ld), v[i]);
+                    if (inside(r)) __stcs(reinterpret_cast<float4*>(at + (long long)(2 * i) * p.ld), v[i]);
                 }
                 at += (long long)(2 * AHEAD) * p.ld;
             }
@@ -997,6 +1000,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             const int gr = m0 + row_in_cta;
             const bool row_ok = gr < p.M;
             const int zs = small_index(it);          // of the axpy operand and of delta
+            if (!MONA_IN_BOUNDS(zs >= 0 && zs < g.C, status, 108)) break;
             const int row0 = m0 + quad * 32;         // the warp's rows
             __nv_bfloat16* const d = p.d ? p.d + (long long)(p.d_map >= NS_TENSOR_A ? zs : it.c) * p.mat_stride : nullptr;
             if ((WHOLE || FEW) && p.cin) {
@@ -1205,7 +1209,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                     float* orow = upd.o[it.c] ? upd.o[it.c] + (long long)gr * p.ld + gc0 : nullptr;
                     #pragma unroll
                     for (int q = 0; q < 8; ++q) {
-                        if (gc0 + 8 * q < p.N) {
+                        if (gc0 + 8 * q < p.N && MONA_IN_BOUNDS((long long)gr * p.ld + gc0 + 8 * q + 8 <= (long long)p.M * p.ld, status, 109)) {
                             float w8[8];
                             ld8(wrow + 8 * q, w8);
                             #pragma unroll

@@ -82,12 +82,13 @@ def ar1_grads(shapes, steps, rho, sigma, seed, dtype=torch.float32, heavy_tail=F
 
 
 def run_case(shapes, steps=3, hp=None, grad_dtype=torch.float32, rho=0.9, sigma=1e-3, seed=0, heavy_tail=False,
-             pad=0, sample=None, lite=False, muon=False, combined=False, compare_aux=True, options=None, check_at=None):
+             pad=0, sample=None, lite=False, muon=False, combined=False, compare_aux=True, options=None, check_at=None, want_o=True):
     """shapes: list of (batch, rows, cols).  `pad` adds that many elements between stacked matrices
     (batch_stride > rows*cols).  `sample`: dict spec index -> list of batch indices the oracle follows
     (default: all).  `muon`: the oracle runs plain Muon; with `compare_aux=False` only M, O and W are compared
     (the library may then run MONA with alpha = 0, whose A and G_prev still evolve).  `options`: mona_options for
-    the handle.  `check_at`: steps (1-based) after which the comparison is made (default: every step).
+    the handle.  `check_at`: steps (1-based) after which the comparison is made (default: every step).  `want_o=False`: O is not
+    asked for, as in training, so that the kernels a plain step takes are the ones that run; its error is 0 then.
     Returns dict of max relative errors over the compared steps and sampled matrices."""
     dev = torch.device("cuda", 0)
     hp = hp or pkg.default_hparams()
@@ -123,7 +124,7 @@ def run_case(shapes, steps=3, hp=None, grad_dtype=torch.float32, rho=0.9, sigma=
     for k in range(steps):
         for gv, g in zip(gviews, grads_seq[k]):
             gv.copy_(g)
-        opt.step_ex(hp, pbufs, gbufs, obufs, 7)
+        opt.step_ex(hp, pbufs, gbufs, obufs if want_o else None, 7)
         st, bad = opt.poll_status()
         assert st == 0, (pkg.STATUS_NAMES[st], bad)
         compare = check_at is None or (k + 1) in check_at
@@ -182,6 +183,8 @@ def run_case(shapes, steps=3, hp=None, grad_dtype=torch.float32, rho=0.9, sigma=
                 w0 = W0[i][b].double().numpy()
                 errs["W"] = max(errs["W"], rel(got, Wn))
                 errs["dW"] = max(errs["dW"], rel(got - w0, Wn - w0))
+    if not want_o:
+        errs["O"] = errs["O_max"] = 0.0
     errs["launches"] = opt.last_launch_count()
     opt.close()
     return errs

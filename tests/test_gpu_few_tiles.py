@@ -5,6 +5,7 @@ import pytest
 import torch
 
 import paper_2605_26842_b200 as pkg
+from paper_2605_26842_b200.binding import FORM_FEW_TILES, FORM_MANY_TILES, FORM_WHOLE_MATRICES, describe_step
 from tests.parity_util import TOL_O_BF16, TOL_O_MAX_BF16, TOL_STATE, TOL_W, run_case
 
 pytestmark = pytest.mark.gpu
@@ -26,12 +27,15 @@ def test_more_buckets_than_slots():
     check(run_case(shapes, steps=3, seed=52))
 
 
-def test_small_buckets_beside_a_large_one_match_a_single_stream():
+@pytest.mark.parametrize("large,form", [((400, 256, 256), FORM_WHOLE_MATRICES), ((120, 264, 264), FORM_MANY_TILES)])
+def test_small_buckets_beside_a_large_one_match_a_single_stream(large, form):
     """Parameters and state agree bit for bit (a tile of any width accumulates over k in the same order), also in validation mode,
     whose chunks are smaller than a bucket."""
     dev = torch.device("cuda", 0)
     gen = torch.Generator().manual_seed(53)
-    shapes = [(400, 256, 256), (2, 264, 520), (1, 520, 264), (2, 32, 256)]
+    shapes = [large, (2, 264, 520), (1, 520, 264), (2, 32, 256)]
+    launches = describe_step([pkg.MatrixDesc(r, c, b, 0, 0, 0) for b, r, c in shapes], options=pkg.default_options(chunk_budget_bytes=64 << 20))
+    assert next(g for g in launches if (g.rows, g.cols) == large[1:]).form == form and any(g.form == FORM_FEW_TILES for g in launches)
     W0 = [torch.randn(s, generator=gen) * 0.02 for s in shapes]
     G = [[torch.randn(s, generator=gen) * 1e-3 for s in shapes] for _ in range(2)]
     for precision in (0, 1):
@@ -73,10 +77,13 @@ def test_repeated_steps_agree_bit_for_bit():
     opt.close()
 
 
-@pytest.mark.parametrize("shape", [(1, 256, 512), (2, 136, 200), (1, 1032, 1160), (400, 256, 256)])
-def test_waits_that_cannot_end_time_out_in_every_form_of_the_launch(shape):
-    """Few tiles (early publication, claim gate, narrow tiles; one pair and several) and many: the launch reports the time-out, leaves,
-    and the next step on the same handle gives the bits that it gives on a fresh one."""
+@pytest.mark.parametrize("shape,form", [((1, 256, 512), FORM_FEW_TILES), ((2, 136, 200), FORM_FEW_TILES), ((1, 1032, 1160), FORM_FEW_TILES), ((400, 256, 256), None),
+                                        ((100, 520, 648), FORM_MANY_TILES), ((20, 256, 256), FORM_WHOLE_MATRICES), ((148, 248, 1016), FORM_WHOLE_MATRICES)])
+def test_waits_that_cannot_end_time_out_in_every_form_of_the_launch(shape, form):
+    """Few tiles (early publication, claim gate, narrow tiles; one pair and several), many, and whole matrices (with and without tensors
+    of the lanes' own): the launch reports the time-out, leaves, and the next step on the same handle gives the bits that it
+    gives on a fresh one."""
+    assert form is None or describe_step([pkg.MatrixDesc(shape[1], shape[2], shape[0], 0, 0, 0)])[0].form == form
     dev = torch.device("cuda", 0)
     gen = torch.Generator().manual_seed(55)
     W0 = (torch.randn(shape, generator=gen) * 0.02).to(dev)

@@ -4,17 +4,26 @@ import pytest
 import torch
 
 import paper_2605_26842_b200 as pkg
+from paper_2605_26842_b200.binding import FORM_FEW_TILES, FORM_MANY_TILES, FORM_WHOLE_MATRICES, describe_step
 
 pytestmark = pytest.mark.gpu
 
 
-@pytest.mark.parametrize("shape,T", [((1, 64, 72), 5), ((1, 256, 512), 5), ((1, 264, 776), 7), ((2, 1032, 392), 1), ((80, 520, 648), 5),
+# form of the last launch and columns of its update's work items, by the shapes below
+KINDS = {(20, 520, 648): (FORM_MANY_TILES, 512), (10, 1032, 1000): (FORM_FEW_TILES, 512), (80, 520, 648): (FORM_MANY_TILES, 256), (1, 264, 776): (FORM_FEW_TILES, 128),
+         (148, 248, 1016): (FORM_WHOLE_MATRICES, 256), (100, 200, 72): (FORM_WHOLE_MATRICES, 256), (222, 712, 136): (FORM_WHOLE_MATRICES, 256)}
+
+
+@pytest.mark.parametrize("shape,T", [((20, 520, 648), 5), ((10, 1032, 1000), 5), ((148, 248, 1016), 5), ((100, 200, 72), 7), ((222, 712, 136), 5), ((1, 64, 72), 5), ((1, 256, 512), 5), ((1, 264, 776), 7), ((2, 1032, 392), 1), ((80, 520, 648), 5),
                                      ((80, 648, 520), 4), ((90, 264, 1160), 5), ((16, 128, 136), 5), ((150, 248, 520), 5), ((150, 520, 248), 6)])
 def test_update_inside_the_last_product(shape, T):
     dev = torch.device("cuda", 0)
     gen = torch.Generator(device=dev).manual_seed(23)
     n = shape[0] * shape[1] * shape[2]
     hp = pkg.default_hparams(ns_steps=T)
+    if shape in KINDS:
+        last = describe_step([pkg.MatrixDesc(shape[1], shape[2], shape[0], 0, 0, 0)], hp)[-1]
+        assert (last.form, last.update_columns) == KINDS[shape]
     W0 = torch.randn(n, generator=gen, device=dev) * 0.02
     G = [torch.randn(shape, generator=gen, device=dev) * 1e-3 for _ in range(2)]
     out = []

@@ -759,7 +759,10 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 Item it;
                 if (!(ok = take_item(n, it, 12, true)) || (it.stop & 1)) break;
                 const NsPhase& p = g.ph[it.q];
-                if (p.fuse_update || (BULK_STORES && p.update)) continue;      // the epilogue writes the parameters itself; nothing waits for them
+                if (p.fuse_update || (BULK_STORES && p.update)) {              // the epilogue writes the parameters itself; nothing waits for them
+                    TRACE_ONLY(trace_add(NS_TRACE_ITEMS, 1u);)
+                    continue;
+                }
                 if (BULK_STORES) {
                     const CUtensorMap* tma_d = &maps.m[p.d_map + NS_TENSORS];     // 64 columns x 128 rows per store
                     const TileCoord tc = decode_tile<FEW>(p, it.t);

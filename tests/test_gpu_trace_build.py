@@ -22,17 +22,20 @@ assert binding._LIB_PATH.endswith("libmona_trace.so"), binding._LIB_PATH
 errs = run_case(shapes=[(5, 256, 768), (2, 768, 256), (1, 1024, 1536)], steps=2, seed=4)
 assert errs["M"] <= TOL_STATE and errs["O"] <= TOL_O_BF16 and errs["dW"] <= TOL_W, errs
 binding.trace_read(reset=True, rows=0)
-# 7 matrices 768 x 2048 (3 x 3 tile rows/columns of the small side, 8 tile columns of X), one step, 5 iterations
+# 7 and 60 matrices 768 x 2048 (3 x 3 tile rows/columns of the small side, 8 tile columns of X), one step, 5 iterations
 dev = torch.device("cuda", 0)
-W = (torch.randn(7, 768, 2048, device=dev) * 0.02)
-G = torch.randn(7, 768, 2048, device=dev) * 1e-3
-opt = pkg.MonaOptimizer([W])
-opt.step(pkg.default_hparams(), [W], [G])
-torch.cuda.synchronize()
-assert opt.poll_status()[0] == 0
-rows = binding.trace_read(reset=True)
-again = binding.trace_read(reset=False)
-print("TRACE " + json.dumps({"rows": rows, "again_sum": sum(map(sum, again))}))
+for mats in (7, 60):
+    W = (torch.randn(mats, 768, 2048, device=dev) * 0.02)
+    G = torch.randn(mats, 768, 2048, device=dev) * 1e-3
+    opt = pkg.MonaOptimizer([W])
+    last = binding.describe_step(opt.descs)[-1]
+    opt.step(pkg.default_hparams(), [W], [G])
+    torch.cuda.synchronize()
+    assert opt.poll_status()[0] == 0
+    rows = binding.trace_read(reset=True)
+    again = binding.trace_read(reset=False)
+    print("TRACE " + json.dumps({"mats": mats, "form": last.form, "update_columns": last.update_columns, "rows": rows, "again_sum": sum(map(sum, again))}))
+    opt.close()
 """
 
 
@@ -42,23 +45,30 @@ def test_profiling_build_matches_the_oracle_and_counts_exactly():
     env = dict(os.environ, MONA_LIBRARY=lib, PYTHONPATH=ROOT + os.pathsep + os.environ.get("PYTHONPATH", ""))
     res = subprocess.run([sys.executable, "-c", CHILD], cwd=ROOT, env=env, capture_output=True, text=True, timeout=900)
     assert res.returncode == 0, res.stdout[-2000:] + res.stderr[-4000:]
-    line = [ln for ln in res.stdout.splitlines() if ln.startswith("TRACE ")][-1]
-    d = json.loads(line[len("TRACE "):])
+    runs = [json.loads(ln[len("TRACE "):]) for ln in res.stdout.splitlines() if ln.startswith("TRACE ")]
+    assert [(d["mats"], d["form"], d["update_columns"]) for d in runs] == [(7, 1, 512), (60, 0, 256)]     # few tiles; many, the last product in plain tiles
+    for d in runs:
+        check_counts(d)
+
+
+def check_counts(d):
     rows = [r for r in d["rows"] if r[0] > 0]
     assert d["again_sum"] == 0                      # the reset cleared the table
     assert len(rows) % 2 == 0 and 2 <= len(rows) <= 148
     lead = rows[0::2]
-    mats = 7
+    mats = d["mats"]
+    last_tiles = 12 if d["update_columns"] == 512 else 24          # work items of the product that updates the parameters
     # 768 x 768 symmetric products: 3 diagonal + 3 off-diagonal tiles; X X^T has 2048 / 64 = 32 k-slices, products of 768 x 768
     # matrices have 768 / 64 = 12; X' = B' X: 3 tile rows x 4 macro-tiles of 512 columns, 12 k-slices each.  768 x 2048 takes its
     # first two iterations together: one X X^T, P, P A, P (P A), P', P' P and one Q X; of the s x s products only P and P' have the
     # same operand on both sides, so the diagonal tiles of the other three count with the off-diagonal ones.  Three plain
     # iterations follow.
-    expect = {0: 4 * 3 * 32, 1: 4 * 3 * 32, 2: (5 + 3) * 3 * 12 + 3 * 3 * 12, 3: (2 + 3) * 3 * 12, 4: 4 * 12 * 12, 5: 0}
+    macro, plain = (4, 0) if last_tiles == 12 else (3, 24)
+    expect = {0: 4 * 3 * 32, 1: 4 * 3 * 32, 2: (5 + 3) * 3 * 12 + 3 * 3 * 12, 3: (2 + 3) * 3 * 12, 4: macro * 12 * 12, 5: plain * 12}
     for kind, per_matrix in expect.items():
         got = sum(r[16 + 4 * kind + 1] for r in lead)
         assert got == per_matrix * mats, (kind, got)
-    assert sum(r[15] for r in rows) == 2 * ((6 * 6 + 12) + 3 * (6 + 6 + 12)) * mats       # every item is counted once by each CTA of its pair
+    assert sum(r[15] for r in rows) == 2 * ((6 * 6 + 12) + 2 * (6 + 6 + 12) + (6 + 6 + last_tiles)) * mats       # every item is counted once by each CTA of its pair
     for r in lead:
         for kind in range(5):
             cyc, ks, wf, wa = r[16 + 4 * kind:16 + 4 * kind + 4]

@@ -366,14 +366,12 @@ def run_workload(torch, pkg, synth, shard, args, dev, local_rank, rank, world, d
     ns_clocks = None
     timed_steps(1, mask=1, refresh=False)
     ms_pro = statistics.median(timed_steps(n_phase, mask=1, refresh=False))
-    # The Newton-Schulz kernel alone (mask 2: O_k stored in bf16) and together with the update (mask 6: in the kernel's last
-    # epilogue when fuse_update is on, as a separate kernel otherwise).  The pass that times the kernel as it runs inside the
-    # step is the one whose clocks are sampled.
-    fused = bool(opt.options.fuse_update)
+    # The Newton-Schulz kernel as it runs inside a step, the parameters updated in the epilogue of its last GEMM (mask 6), and
+    # without the update (mask 2: O_k stored in bf16, macro-tiles in the last GEMM too).  The clocks of the first are sampled.
     passes = {}
-    for mask in ((2, 6) if fused else (6, 2)):
+    for mask in (2, 6):
         timed_steps(1, mask=mask, refresh=False)
-        sampled = full and mask == (6 if fused else 2)
+        sampled = full and mask == 6
         ns_sampler = ClockSampler(local_rank) if sampled else None
         if ns_sampler:
             ns_sampler.start()
@@ -400,7 +398,7 @@ def run_workload(torch, pkg, synth, shard, args, dev, local_rank, rank, world, d
         pro_elem = g_elem + 4 + 4 + 2                   # read G, M; write M, bf16 X
     pro_gbs = n * pro_elem / (ms_pro * 1e-3) / 1e9
     upd_gbs = n * (4 + 2 + 4) / (ms_upd * 1e-3) / 1e9   # read W, bf16 O; write W
-    ms_kernel = ms_nsu if fused else ms_ns
+    ms_kernel = ms_nsu
     ns_tflops = flops_exec / (ms_kernel * 1e-3) / 1e12
     phases = {"prologue_ms": ms_pro, "prologue_gbs": pro_gbs, "prologue_frac_of_hbm_peak": pro_gbs / peaks["hbm_gbs"],
               "prologue_frac_of_nominal_8000": pro_gbs / 8000.0, "prologue_bytes_per_elem": pro_elem,
@@ -408,7 +406,7 @@ def run_workload(torch, pkg, synth, shard, args, dev, local_rank, rank, world, d
               "ns_tflops_executed": ns_tflops, "ns_tflops_useful": flops_useful / (ms_kernel * 1e-3) / 1e12,
               "ns_tflops_executed_without_update": flops_exec / (ms_ns * 1e-3) / 1e12,
               "separate_update_gbs": upd_gbs, "separate_update_frac_of_hbm_peak": upd_gbs / peaks["hbm_gbs"],
-              "update": "in the epilogue of the last GEMM of the Newton-Schulz kernel" if fused else "inside the last product of a whole step; timed apart as a kernel of its own",
+              "update": "in the epilogue of the last GEMM of the Newton-Schulz kernel; the separate kernel is timed for comparison",
               "hbm_peak_gbs": peaks["hbm_gbs"], "peak_source": peak_src}
     result = {"wl": wl, "fit_note": fit_note, "value": value, "ms_per_step": ms_per_step, "ms": ms, "clocks": clocks,
               "launches_per_step": launches_per_step, "phases": phases, "hp": hp, "options": opt.options}
@@ -420,8 +418,7 @@ def run_workload(torch, pkg, synth, shard, args, dev, local_rank, rank, world, d
 
     # the Newton-Schulz kernel runs inside a long step: compare with the sustained GEMM peak
     mhz = (ns_clocks or {}).get("sm_mhz")
-    roofline = {"kernel": "ns_chunk_kernel (all Newton-Schulz GEMMs of a chunk in one launch"
-                          + (", parameter update in the last epilogue)" if fused else ")"), "bound": "tensor",
+    roofline = {"kernel": "ns_chunk_kernel (all Newton-Schulz GEMMs of a chunk in one launch, parameter update in the last epilogue)", "bound": "tensor",
                 "achieved": ns_tflops, "peak": peaks["bf16_tflops_sustained"], "unit": "TFLOP/s",
                 "frac": ns_tflops / peaks["bf16_tflops_sustained"], "peak_source": peak_src + " (sustained bf16 GEMM)",
                 "frac_of_burst_peak": ns_tflops / peaks["bf16_tflops"], "frac_of_nominal_2250": ns_tflops / 2250.0,
@@ -438,9 +435,9 @@ def run_workload(torch, pkg, synth, shard, args, dev, local_rank, rank, world, d
         # Diagnostic: the Newton-Schulz pass back to back for a few seconds with power sampling, to put joules per executed
         # TFLOP beside the library's on the same shapes (main() adds that leg).  Runs after every timed figure above.
         try:
-            roofline["energy"] = {"ns_kernel": sustained(torch, dev, local_rank, lambda: opt.step_ex(hp, params, gp.grads, None, 2), flops_exec),
+            roofline["energy"] = {"ns_kernel": sustained(torch, dev, local_rank, lambda: opt.step_ex(hp, params, gp.grads, None, 6), flops_exec),
                                   "power_field": power_field(local_rank),
-                                  "note": "Newton-Schulz pass (executed flops) and the library's dense products of the dominant bucket, "
+                                  "note": "Newton-Schulz pass with the update inside (executed flops) and the library's dense products of the dominant bucket, "
                                           "each run back to back for ~2.5 s; watts = median nvidia-smi sample after the first 0.5 s"}
             opt.poll_status()
         except Exception as exc:
@@ -520,7 +517,7 @@ def main():
     ap.add_argument("--no-yardstick", action="store_true", help="skip the library-GEMM diagnostic")
     ap.add_argument("--chunk-mb", type=int, default=None, help="override the chunk budget (MiB)")
     ap.add_argument("--no-overlap", action="store_true", help="keep all chunks on one stream")
-    ap.add_argument("--fuse", action="store_true", help="apply the parameter update in the epilogue of the last GEMM instead of a separate kernel")
+    ap.add_argument("--fuse", action="store_true", help="apply the parameter update from the fp32 accumulator instead of from O rounded to bf16")
     ap.add_argument("--ns-delay", type=int, default=None, help="work-order distance between consecutive GEMMs of one matrix")
     ap.add_argument("--macro-min-k", type=int, default=None, help="shortest inner dimension for which X' = B'X uses 256x512 macro-tiles")
     ap.add_argument("--shard", action="store_true", help="one parameter set partitioned over the ranks, parameters exchanged after the step")

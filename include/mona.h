@@ -129,7 +129,7 @@ mona_status mona_default_hparams(mona_hparams* hp);
  *                        times the budget (or the iterates of the largest matrix in fp32, where that is more), and
  *                        some 4 MiB.
  *   fuse_update        : 0 (default): Eq. muon_update is applied from O_k rounded to bf16: inside the last X' = B' X of a whole step
- *                        on the tensor-core path, by a separate elementwise kernel where O_k is asked for, phases run apart,
+ *                        on the tensor-core path, by a separate elementwise kernel where O_k is asked for, the two phases run apart,
  *                        a stride is no multiple of 16 bytes, the step goes from host to host, or the launch has so many tiles
  *                        for its few SM pairs that a pass on all of them is quicker.  The results are the same bits.
  *                        1: on the tensor-core path the last X' = B' X of a step applies the update in its epilogue

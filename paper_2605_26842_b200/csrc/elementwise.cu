@@ -309,6 +309,10 @@ prologue_kernel(const __grid_constant__ GradTable<CAP> ptrs, float* __restrict__
     }
 }
 
+__global__ void __launch_bounds__(EW_THREADS) param_table_kernel(const __grid_constant__ ParamTable<MAXC> ptrs, float** __restrict__ params, int C) {
+    for (int c = threadIdx.x; c < C; c += EW_THREADS) params[c] = ptrs.w[c];
+}
+
 // W <- W - eta (gamma O + lambda W), evaluated as (W - (eta lambda) W) - (eta gamma) O.
 template <typename OT, int VEC, int CAP>
 __global__ void __launch_bounds__(EW_THREADS)
@@ -435,6 +439,12 @@ cudaError_t launch_prologue(const ChunkPtrs& ptrs, int C, bool grad_bf16, int st
     }
 #undef MONA_PROLOGUE_CASE
     return cudaGetLastError();
+}
+
+cudaError_t launch_param_table(const ChunkPtrs& ptrs, int C, float** params, cudaStream_t stream) {
+    ParamTable<MAXC> t = {};
+    for (int c = 0; c < C; ++c) t.w[c] = ptrs.w[c];
+    return launch_kernel(param_table_kernel, dim3(1), dim3(EW_THREADS), 0, stream, false, t, params, C);
 }
 
 cudaError_t launch_update(const ChunkPtrs& ptrs, int C, bool o_is_bf16, bool vec4, const void* O, long long e,

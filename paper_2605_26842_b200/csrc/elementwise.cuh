@@ -22,6 +22,9 @@ cudaError_t launch_prologue(const ChunkPtrs& ptrs, int C, bool grad_bf16, int st
                             DeviceStatus* status, long long e, long long slab_len, int slabs,
                             const PrologueScalars& k, unsigned int* zero, int zero_words, float** params, cudaStream_t stream);
 
+// The same pointers written by a launch of their own, where the prologue does not run in the call.
+cudaError_t launch_param_table(const ChunkPtrs& ptrs, int C, float** params, cudaStream_t stream);
+
 // Parameter update W <- (W - eta*lambda*W) - eta*gamma*O for a chunk; O is bf16 or fp32, dense, e per matrix.
 cudaError_t launch_update(const ChunkPtrs& ptrs, int C, bool o_is_bf16, bool vec4, const void* O, long long e,
                           long long slab_len, int slabs, float eta_lambda, float eta_gamma, bool early, cudaStream_t stream);

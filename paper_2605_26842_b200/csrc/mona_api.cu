@@ -840,7 +840,7 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             // the update than a pass over all of them: 5.81 -> 5.77 ms for one layer of 512 x 1024 experts.)
             bool asked_for_o = false;
             for (int c = 0; c < C; ++c) asked_for_o = asked_for_o || ptrs.o[c];
-            const NsChoice k = ns_choose(h->opt, h->max_pairs, h->pairs_beside[bucket_index], b, C, overlap && small, phase_mask == 7u && !params_host && vec4 && !asked_for_o, *hp);
+            const NsChoice k = ns_choose(h->opt, h->max_pairs, h->pairs_beside[bucket_index], b, C, overlap && small, (phase_mask & 6u) == 6u && !params_host && vec4 && !asked_for_o, *hp);
             const bool update_inside = tc && k.update_inside;
             float** param_table = (float**)(ctrl + CTRL_PARAMS_OFF);
             if (phase_mask & 1u) {
@@ -849,6 +849,10 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
                                              hp->algorithm == 1 ? PROLOGUE_NO_AUX : (b.state_dtype == MONA_BF16 ? PROLOGUE_AUX_BF16 :
                                                  b.state_dtype == MONA_STATE_COMBINED ? PROLOGUE_AUX_COMBINED : PROLOGUE_AUX_F32), vec4, Mc, Ac, Gc, tc ? xb[0] : nullptr, partials,
                                              counters, inv_norm, dstatus, b.e, b.slab_len, b.slabs, ps, sched, cleared_by_prologue ? (int)ns_sched_words(C, NS_MAX_PHASES) : 0, update_inside ? param_table : nullptr, stream));
+                ++h->launches;
+            }
+            else if (update_inside) {
+                MONA_CUDA(h, launch_param_table(ptrs, C, param_table, stream));
                 ++h->launches;
             }
             const void* o_final = nullptr;

@@ -1,5 +1,5 @@
-"""Where the Newton-Schulz kernel's cycles go: runs the Newton-Schulz phase of a synthetic parameter set through the
-profiling build of the library (libmona_trace.so, compiled with -DMONA_TRACE) and prints what every role of the kernel
+"""Where the Newton-Schulz kernel's cycles go: runs the Newton-Schulz and update phases of a synthetic parameter set, which
+take the kernels of a whole step (the parameters updated in the last product), through the profiling build of the library (libmona_trace.so, compiled with -DMONA_TRACE) and prints what every role of the kernel
 waited for, and the MMA issuer's cycles per k-slice for every kind of tile.
 
     python -m paper_2605_26842_b200.trace_report --config 3 --layers 2 [--bucket wide|tall|square] [--json]
@@ -56,7 +56,7 @@ def collect(config: int, layers: int, bucket: str | None, steps: int, delay: int
     e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
     e0.record()
     for _ in range(steps):
-        opt.step_ex(hp, params, gp.grads, None, 2)      # phase mask 2: the Newton-Schulz phase alone
+        opt.step_ex(hp, params, gp.grads, None, 6)      # without the prologue
     e1.record()
     torch.cuda.synchronize()
     launches = opt.last_launch_count()

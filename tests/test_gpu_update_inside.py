@@ -42,3 +42,29 @@ def test_update_inside_the_last_product(shape, T):
         out.append((buf, launches))
     assert torch.equal(out[0][0], out[1][0])
     assert out[0][1] == out[1][1] - 1
+
+
+@pytest.mark.parametrize("shapes", [[(1, 256, 512)], [(100, 520, 648), (2, 264, 520), (1, 33, 17)], [(148, 248, 1016)]])
+def test_newton_schulz_and_update_without_the_prologue(shapes):
+    """The phases behind the prologue in a call of their own (as the benchmark times them) are the kernels of a whole step: the same bits,
+    and one launch more, which writes the parameters' addresses, for every chunk whose last product updates the parameters."""
+    dev = torch.device("cuda", 0)
+    gen = torch.Generator(device=dev).manual_seed(29)
+    W0 = [torch.randn(s, generator=gen, device=dev) * 0.02 for s in shapes]
+    G = [torch.randn(s, generator=gen, device=dev) * 1e-3 for s in shapes]
+    hp = pkg.default_hparams()
+    out = []
+    for masks in ((7,), (1, 6)):
+        p = [w.clone() for w in W0]
+        opt = pkg.MonaOptimizer(p)
+        for mask in masks:
+            opt.step_ex(hp, p, G, None, mask)
+            out.append(opt.last_launch_count())
+        assert opt.poll_status()[0] == 0
+        out.append(p + [opt.state.clone()])
+        inside = sum(g.update_columns > 0 for g in describe_step(opt.descs, hp))
+        opt.close()
+    whole, whole_out, prologue, rest, parts_out = out
+    assert rest == whole - prologue + inside
+    for x, y in zip(whole_out, parts_out):
+        assert torch.equal(x, y)

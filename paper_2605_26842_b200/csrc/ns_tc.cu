@@ -766,20 +766,20 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
                 if (BULK_STORES) {
                     const CUtensorMap* tma_d = &maps.m[p.d_map + NS_TENSORS];     // 64 columns x 128 rows per store
                     const TileCoord tc = decode_tile<FEW>(p, it.t);
-                    const int m0 = tc.tm * TC_BM + (int)rank * CTA_M, zd = p.d_map >= NS_TENSOR_A ? small_index(it) : it.c;
+                    const int m0 = tc.tm * TC_BM + (int)rank * CTA_M;
                     // The two 64-column halves of the staging buffer are separate buffers with their own barriers, filled by
                     // different warps: each half is stored as soon as it is full and handed back as soon as its own store has
                     // read it, the first half while the second store is still reading.
                     for (int u = 0; u < tc.nsub && ok; ++u) {
                         for (int ph = 0; ph < 2 && ok; ++ph) {
-                            const int x0 = (tc.tn + u) * (FEW ? ns_tile_cols(p) : TC_BN) + ph * EPI_COLS;
-                            if (x0 >= p.N || (FEW && ph && p.narrow)) continue;
+                            const int x0 = (tc.tn + u) * TC_BN + ph * EPI_COLS;
+                            if (x0 >= p.N) continue;
                             if (!MONA_IN_BOUNDS(m0 < p.M + CTA_M && it.c < g.C && tc.tm < p.tiles_m, status, 106)) { ok = false; break; }
                             #pragma unroll
                             for (int bx = 0; bx < 2; ++bx) {
                                 if (!(ok = mbar_wait(bar_stg_full + 8 * bx, staged & 1u, abort_flag, status, 13, TRACE_PTR(w_stg)))) break;
                                 const int x = x0 + bx * TC_BOX;
-                                if (x < p.N && m0 < p.M) tma_store_3d(tma_d, epi_buf + bx * 2 * BOX_BYTES, x, m0, zd);   // clipped at the extents
+                                if (x < p.N && m0 < p.M) tma_store_3d(tma_d, epi_buf + bx * 2 * BOX_BYTES, x, m0, it.c);   // clipped at the extents
                                 bulk_commit();
                             }
                             if (!ok) break;
@@ -1005,7 +1005,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             const int zs = small_index(it);          // of the axpy operand and of delta
             if (!MONA_IN_BOUNDS(zs >= 0 && zs < g.C, status, 108)) break;
             const int row0 = m0 + quad * 32;         // the warp's rows
-            __nv_bfloat16* const d = p.d ? p.d + (long long)(p.d_map >= NS_TENSOR_A ? zs : it.c) * p.mat_stride : nullptr;
+            __nv_bfloat16* const d = p.d + (long long)(p.d_map >= NS_TENSOR_A ? zs : it.c) * p.mat_stride;
             if ((WHOLE || FEW) && p.cin) {
                 bool there = true;
                 if (lane == 0) there = WHOLE ? wait_lane(it) : wait_dependency(it);

@@ -33,7 +33,7 @@ FALLBACK_PEAKS = {"hbm_gbs": 6650.0, "bf16_tflops": 1590.0, "bf16_tflops_sustain
 # summarised in profiles/ns_chunk_kernel_counters.md: the launch over a 93-matrix 768x2048 chunk, parameter update included, the launch
 # shape that makes up most of the default workload (40 of its 56 launches per step are of this shape or its tall twin).  Valid only
 # for the kernel source the counters were taken with (hash of the code of ns_tc.cu + ns_tc.cuh).
-NCU_TRAFFIC = {"source_sha256_16": "9beccc5c1b0bb0a9", "bytes_per_launch": 6.627e9,
+NCU_TRAFFIC = {"source_sha256_16": "ac2dc420bbf6b28a", "bytes_per_launch": 6.627e9,
                "unit": "DRAM bytes of one launch over a 93-matrix 768x2048 chunk (ncu; 1.947 TFLOP executed in that launch)"}
 
 

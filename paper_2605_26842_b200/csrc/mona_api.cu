@@ -534,6 +534,7 @@ static void ns_plan_group(NsProgram& g, const Bucket& b, bool together, bool fir
     } else {         // X is K-major, the symmetric Q serves as its own transpose
         g3.M = l; g3.N = s; g3.a_map = MAP_X0 + x_cur; g3.a_mn = 0; g3.b_map = q_map; g3.b_sym = 1;
     }
+    if (fuse_update || update) g3.d = nullptr;
     ns_phase_plan(g3);
 }
 

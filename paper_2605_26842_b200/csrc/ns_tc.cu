@@ -1005,7 +1005,7 @@ ns_chunk_kernel(const __grid_constant__ NsMaps maps, const __grid_constant__ NsP
             const int zs = small_index(it);          // of the axpy operand and of delta
             if (!MONA_IN_BOUNDS(zs >= 0 && zs < g.C, status, 108)) break;
             const int row0 = m0 + quad * 32;         // the warp's rows
-            __nv_bfloat16* const d = p.d + (long long)(p.d_map >= NS_TENSOR_A ? zs : it.c) * p.mat_stride;
+            __nv_bfloat16* const d = p.d ? p.d + (long long)(p.d_map >= NS_TENSOR_A ? zs : it.c) * p.mat_stride : nullptr;
             if ((WHOLE || FEW) && p.cin) {
                 bool there = true;
                 if (lane == 0) there = WHOLE ? wait_lane(it) : wait_dependency(it);

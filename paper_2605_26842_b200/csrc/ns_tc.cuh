@@ -45,7 +45,7 @@ struct NsPhase {
                                 //    one staged slice of the A operand, one per tensor-memory accumulator
     int narrow;                 // 1: tiles of 128 instead of 256 columns (not with `wide`)
     int tiles_m, tiles_n, items_per_mat;   // filled by ns_phase_plan(); items are macro-tiles when `wide`
-    __nv_bfloat16* d;           // tensor d_map
+    __nv_bfloat16* d;           // tensor d_map; null where the epilogue updates the parameters instead
     const __nv_bfloat16* cin;   // may be null; [C][M][N] like D; lower-block-stored when D is symmetric
     long long ld, mat_stride;   // leading dimension (of cin, and of the fp32 parameter when fuse_update, too) and per-matrix stride of
                                 // D, in elements

@@ -132,11 +132,11 @@ mona_status mona_default_hparams(mona_hparams* hp);
  *                        on the tensor-core path, by a separate elementwise kernel where O_k is asked for, the two phases run apart,
  *                        a stride is no multiple of 16 bytes, the step goes from host to host, or the launch has so many tiles
  *                        for its few SM pairs that a pass on all of them is quicker.  The results are the same bits.
- *                        1: on the tensor-core path the last X' = B' X of a step applies the update in its epilogue
- *                        (fp32 O_k straight from the accumulator, no bf16 copy of O_k written and re-read, one launch
- *                        fewer per chunk).  The two differ by the bf16 rounding of O_k only.  Measured slower on the
- *                        benchmark sets: a thread owns a row of the accumulator, and its fp32 read-modify-write of W
- *                        touches 32 lines per warp instruction.
+ *                        1: on the tensor-core path the last X' = B' X of every step applies the update from the fp32
+ *                        accumulator: O_k is not rounded to bf16 on its way into W, and o_out receives it in fp32.  That
+ *                        rounding is all that the two differ by.  Slower on the benchmark sets: a thread owns a row of
+ *                        the accumulator, its fp32 read-modify-write of W touches 32 lines per warp instruction, and the
+ *                        launch forms for few tiles and for whole matrices per SM pair do not know it.
  *   ns_delay           : how many matrices apart consecutive Newton-Schulz GEMMs of one matrix sit in the kernel's
  *                        work order (0 = the default, 20; at most 1024; a value >= the chunk's matrix count
  *                        runs the chunk GEMM by GEMM).  Larger values hide the dependency latency
@@ -144,11 +144,12 @@ mona_status mona_default_hparams(mona_hparams* hp);
  *   macro_tile_min_k   : X' = B' X runs as 256 x 512 macro-tiles (two tiles sharing one staged operand slice, both
  *                        accumulators in use, so nothing hides their epilogue) when its inner dimension - the shorter
  *                        side of the weight - is at least this, and as plain 256 x 256 tiles with alternating
- *                        accumulators below it (0 = the default, 1: always macro-tiles.  Plain tiles keep the tensor
+ *                        accumulators below it (0 = the default, 1: macro-tiles.  Plain tiles keep the tensor
  *                        cores busier per clock on short inner dimensions, but the step runs at the power cap and
- *                        macro-tiles move fewer bytes per flop: measured 3-7 % faster on every benchmark set).
- *                        Launches of few tiles choose among 256 x 512, 256 x 256 and 256 x 128 by an estimate of
- *                        their time, whatever it says.  Results do not depend on it. */
+ *                        macro-tiles move fewer bytes per flop: measured 1-4 % faster on the benchmark sets).
+ *                        Whatever it says, launches of few tiles choose among 256 x 512, 256 x 256 and 256 x 128 by an
+ *                        estimate of their time, and the product that updates the parameters takes plain tiles where
+ *                        it has two rounds of macro-tiles or more.  Results do not depend on it. */
 typedef struct {
     size_t chunk_budget_bytes;
     int32_t chunk_overlap;

@@ -9,7 +9,7 @@ namespace mona {
 
 // A chunk is the unit that goes through prologue -> Newton-Schulz -> update together: up to MAXC
 // same-shape matrices whose bf16 iterates fit the chunk budget (sized for full machine occupancy, not for cache).
-constexpr int MAXC = 512;   // per-matrix pointers travel as kernel arguments (at most 8 KiB of the 32 KiB CUDA 12 allows)
+constexpr int MAXC = 512;   // per-matrix pointers travel as kernel arguments (at most 10 KiB of the 32 KiB CUDA 12 allows)
 // The Frobenius norm is the sum, in a fixed order, of at most MAX_UNITS partial sums of squares per matrix.  A unit's length follows
 // from the matrix size alone, so the norm's bits do not depend on how many matrices share a launch.
 constexpr int MAX_UNITS = 256;

@@ -608,7 +608,10 @@ static bool update_pays_inside(const Bucket& b, int C, int pairs) {
 // The product that updates the parameters takes plain tiles where it has at least two rounds of macro-tiles.  Its epilogue is the
 // longest, 8 bytes per element in and out of the SM: behind a macro-tile nothing hides it, with plain tiles the next one's
 // products run beside it (12 dense blocks 3480 -> 3414 us per step, 1024 x 1536 experts 6778 -> 6650, three layers of 768 x 2048
-// 18.78 -> 18.48 ms, four of 512 x 1024 3875 -> 3827 us; 256 x 768, whole matrices, 3488 -> 3482).
+// 18.78 -> 18.48 ms; 512 x 1024 and 256 x 768 experts within the noise).  With fewer rounds it goes either way, by how well the last round fills:
+// rounds of macro-tiles and us with macro-tiles -> plain ones, 0.9: 8 of 1024 x 1024 260 -> 268, 2 of 2048 x 2048 388 -> 427; 1.5: 9 of
+// 768 x 2048 311 -> 322; 1.7: 4 of 1024 x 4096 424 -> 414, 16 of 1024 x 1024 460 -> 453, 4 of 2048 x 2048 702 -> 690; 2.2: 5 of 2048 x 2048
+// 874 -> 869; 2.6: 24 of 768 x 2048 708 -> 690.
 static void ns_plain_update_tiles(NsProgram& g, int pairs) {
     for (int q = 0; q < g.P; ++q) {
         NsPhase& p = g.ph[q];
@@ -837,8 +840,9 @@ static mona_status step_impl(mona_handle* h, const mona_hparams* hp, void* const
             }
             const bool cleared_by_prologue = tc && small;
             // The last X' = B' X updates the parameters, from O rounded to bf16 as the separate pass would read it: O is neither written
-            // nor read back, 4 of 12 bytes per element.  (Not host to host: its chunks are launches of few tiles, whose few SMs take longer for
-            // the update than a pass over all of them: 5.81 -> 5.77 ms for one layer of 512 x 1024 experts.)
+            // nor read back, 4 of 12 bytes per element.  (Not host to host, where the step waits for the link and the update inside goes either
+            // way: us apart -> inside, one 256 x 512 123 -> 115, 7 of 1024 x 2816 and 4 of its square 2455 -> 2411, 64 of 256 x 768 1357 -> 1402,
+            // 16 each of 384 x 768 and 768 x 384 1160 -> 1174, one layer of 512 x 1024 experts 5650 -> 5660.)
             bool asked_for_o = false;
             for (int c = 0; c < C; ++c) asked_for_o = asked_for_o || ptrs.o[c];
             const NsChoice k = ns_choose(h->opt, h->max_pairs, h->pairs_beside[bucket_index], b, C, overlap && small, (phase_mask & 6u) == 6u && !params_host && vec4 && !asked_for_o, *hp);
@@ -1060,7 +1064,7 @@ mona_status mona_describe_step(const mona_matrix_desc* descs, int64_t n_desc, co
                 const NsProgram g = ns_next_launch(opt, b, C, k, *hp, opt.fuse_update != 0, nullptr, gi);
                 const NsPhase& p = g.ph[g.P - 1];
                 if (*n_launches < capacity)
-                    out[*n_launches] = {b.rows, b.cols, C, g.max_pairs, slot, opt.fuse_update ? 0 : (int32_t)g.form, g.P, p.update || p.fuse_update ? (p.wide ? 2 * TC_BN : ns_tile_cols(p)) : 0};
+                    out[*n_launches] = {b.rows, b.cols, C, g.max_pairs, slot, p.fuse_update ? 0 : (int32_t)g.form, g.P, p.update || p.fuse_update ? (p.wide ? 2 * TC_BN : ns_tile_cols(p)) : 0};
                 ++*n_launches;
             }
         }

@@ -26,9 +26,9 @@
 //              memory (a thread owns one row, so storing from registers would touch 32 lines per warp instruction) and
 //              hand the boxes to TMA stores, or read them back four lines at a time and store them themselves:
 //              TMA stores in the spread form, where their fewer instructions are 1-2 % of the energy of the large sets, own
-//              stores in the others, where a hand-over less is 2 % of a short chain and 6 % of 256 x 768 experts;
+//              stores in the others, where a hand-over less is 2 % of a short chain and 3 % of 256 x 768 experts;
 //              for the last X' = B' X of a step the same warps apply the parameter update of Eq. muon_update
-//              to the fp32 weights instead (a separate pass reads O back and the weights at the end of the launch: three layers
+//              to the fp32 weights instead, where the launch has enough SM pairs for its tiles (a separate pass reads O back and the weights at the end of the launch: three layers
 //              of 768 x 2048 experts 19.06 -> 18.48 ms per step, 256 x 768 experts 3.63 -> 3.48, one 256 x 512 85.0 -> 83.4 us),
 //   warp 3     store warp: turns each staged phase into TMA stores and frees the staging buffer (spread form), and counts the item
 //              as done once its stores have completed, so that no epilogue warp ever waits for global memory.
